@@ -29,8 +29,8 @@
  * Tuning knobs (environment variables, decimal; unset = the default).  None
  * changes a result, only how the work is scheduled:
  *   LG_HEAVY_MIN     256   degrees above this go to the heavy-vertex schedule
- *                          (a warp per item; 0 = default); read at every
- *                          lg_encode
+ *                          (a warp per item; 0 = default, at most 4096); read
+ *                          at every lg_encode
  *   LG_HEAVY_SEG     4096  fields per heavy-schedule item (values below 32 =
  *                          default); read at every lg_encode
  *   LG_BFS_PULL_DIV  64    a BFS level runs bottom-up when its frontier holds
@@ -247,7 +247,7 @@ lg_status lg_pagerank(const lg_graph *g, float damping, uint32_t iters,
  * front under a fixed budget cannot add cudaMalloc calls of its own, and a
  * latency-sensitive loop cannot afford cudaFree's implicit synchronization;
  * this call runs the same kernels as lg_pagerank (same results) but keeps its
- * scratch in a fixed array inside liblg.so (9 MiB held on every GPU that loads
+ * scratch in a fixed array inside liblg.so (10.1 MiB held on every GPU that loads
  * the library, until the process exits) and calls no allocator.
  *   Limit: graphs of at most 1,048,576 vertices (and at most 262,144 schedule
  *   items for vertices split by the heavy-vertex schedule); larger graphs give

@@ -97,7 +97,7 @@ uint32_t env_u32(const char* name, uint32_t dflt) {
 // read at every encode (LG_HEAVY_MIN, LG_HEAVY_SEG).
 uint32_t heavy_min_env() {
   const uint32_t v = env_u32("LG_HEAVY_MIN", 256);
-  return v ? v : 256;
+  return v == 0 ? 256 : v > lg::PW_HEAVY_MAX ? lg::PW_HEAVY_MAX : v;
 }
 uint32_t heavy_seg_env() {
   const uint32_t v = env_u32("LG_HEAVY_SEG", 4096);
@@ -183,29 +183,13 @@ GView make_view(const lg_graph* g) {
   v.n_multi = g->n_multi;
   v.heavy_min = g->heavy_min;
   v.heavy_seg = g->heavy_seg;
+  v.heavy_prefix = g->heavy_prefix;
   return v;
 }
 
 // ---------------------------------------------------------------- split vertices
 // A vertex split into several heavy items: its items' partial sums are added
 // in item order (deterministic), then the vertex is finished.
-__global__ void k_pr_finish_multi(GView g, PrArgs a) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < g.n_multi; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t first = g.multi[i];
-    const HeavyItem h = g.items[first];
-    float s = 0.f;
-    for (uint32_t k = 0; k < h.nitems; k++) s += a.part[first + k];
-    pr_finish(g, a, h.v, h.deg, s);
-  }
-}
-
-cudaError_t pr_finish_multi(const GView& g, const PrArgs& a, cudaStream_t st) {
-  if (g.n_multi == 0) return cudaSuccess;
-  k_pr_finish_multi<<<grid_for(g.n_multi, 256, 4096), 256, 0, st>>>(g, a);
-  count_launch();
-  return cudaGetLastError();
-}
-
 __global__ void k_ppr_finish_multi(GView g, PprArgs a) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < g.n_multi; i += (uint64_t)gridDim.x * blockDim.x) {
     const uint32_t first = g.multi[i];
@@ -379,6 +363,34 @@ uint32_t hot_rows(const lg_graph* g, uint32_t elem_bytes) {
   return (uint32_t)(rows < all ? rows : all);
 }
 
+// Warp tiles hold 128 vertices, but fewer where that would make a long unit: in
+// a small graph (fewer than two tiles of 128 per resident warp), and for the
+// DM-ordered vertices of more than 32 arcs (a warp walks 256 fields in about
+// 2 us, so 128 x 256 fields ran 250 us on one warp).  The smaller tiles trade
+// the tile's own cost against the longest unit; measured per sweep at 4 / 8 /
+// 16 / 32 vertices: R-MAT 2^12 in DM order 8 / 10 / 13 / 19 us, community 2^15
+// 25 / 26 / 34 / 54, community 2^18 in DM order 133 / 80 / 58 / 80, R-MAT 2^18
+// not relabeled 110 / 72 / 53 / 47, R-MAT 900,000 287 / 173 / 114 / 85.  The shared-memory table
+// of contributions pays when it answers some of the gathers of a sweep that is
+// long enough to fill it (R-MAT 2^24 in DM order, 28 % of the arcs on the
+// first 16,384 labels: 1.78 -> 1.61 ms a sweep; community 2^23, 9 %: 0.94 ->
+// 0.91; 2^24, 6 %: equal; R-MAT 2^18, 76 %: 41 -> 43 us).
+PrPlan pr_plan(const lg_graph* g) {
+  PrPlan p;
+  const uint64_t warps = (uint64_t)PW_WARPS * PW_SMS;
+  const bool small = g->n < 2 * warps * PW_TV;
+  p.tile_a = g->heavy_prefix & ~31ull;
+  p.tile_nv = g->n < (1u << 14) ? 4 : g->n < (1u << 16) ? 8 : g->n < (1u << 19) && g->relabel == 1 ? 16 : 32;
+  const uint64_t end = small ? g->n : g->mid_prefix > p.tile_a ? g->mid_prefix : p.tile_a;
+  p.tile_b = (end + PW_TV - 1) & ~(uint64_t)(PW_TV - 1);
+  const uint64_t most = (PW_SMEM - PW_WARPS * sizeof(PrWarp)) / sizeof(float);
+  p.tabn = g->arcs >> 24 && 12 * g->top_arcs >= g->arcs ? (uint32_t)(g->n < most ? g->n : most) : 0;
+  p.part_floats = g->n_multi ? g->n_items : 0;
+  p.sync_words = 2 + g->n_multi;
+  p.aux_words = g->off_mode == OFF_EF ? (p.tile_b - p.tile_a) / p.tile_nv + g->n / PW_TV + 1 : 0;
+  return p;
+}
+
 cudaError_t pr_fill0(float* ranks, uint64_t n, int64_t personal_orig, cudaStream_t st) {
   k_pr_fill0<<<grid_for(n, 256, 152 * 32), 256, 0, st>>>(ranks, n, 1.0f / (float)n, personal_orig);
   count_launch();
@@ -539,7 +551,10 @@ static lg_status build_schedule(lg_graph* g, cudaStream_t st) {
   g->heavy_min = heavy_min_env();
   g->heavy_seg = heavy_seg_env();
   const uint64_t ntiles = (g->n + LG_TILE_V - 1) / LG_TILE_V;
-  Tmp t_cnt(st), t_mcnt(st), t_off(st), t_moff(st), t_stmp(st), t_seg(st);
+  Tmp t_cnt(st), t_mcnt(st), t_off(st), t_moff(st), t_stmp(st), t_seg(st), t_mid(st);
+  struct { unsigned long long top; uint32_t mid, pad; } first = {};
+  LG_TRY(t_mid.alloc(sizeof(first)));
+  LG_TRY(cudaMemsetAsync(t_mid.p, 0, sizeof(first), st));
   LG_TRY(t_cnt.alloc(ntiles * sizeof(uint32_t)));
   LG_TRY(t_mcnt.alloc(ntiles * sizeof(uint32_t)));
   LG_TRY(t_off.alloc((ntiles + 1) * sizeof(uint64_t)));
@@ -551,17 +566,23 @@ static lg_status build_schedule(lg_graph* g, cudaStream_t st) {
   p.multi_count = t_mcnt.as<uint32_t>();
   p.tile_off = t_off.as<uint64_t>();
   p.multi_off = t_moff.as<uint64_t>();
+  p.top = t_mid.as<unsigned long long>();
+  p.mid = reinterpret_cast<uint32_t*>(p.top + 1);
   GView v = make_view(g);
   const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
   LG_TRY(ops->plan_count(v, p, st));
   LG_TRY(scan_excl_u32(p.tile_count, ntiles, t_off.as<uint64_t>(), t_stmp.as<uint64_t>(), st));
   LG_TRY(scan_excl_u32(p.multi_count, ntiles, t_moff.as<uint64_t>(), t_stmp.as<uint64_t>(), st));
   uint64_t tot[2] = {0, 0};
+  LG_TRY(cudaMemcpyAsync(&first, t_mid.p, sizeof(first), cudaMemcpyDeviceToHost, st));
   LG_TRY(cudaMemcpyAsync(&tot[0], t_off.as<uint64_t>() + ntiles, 8, cudaMemcpyDeviceToHost, st));
   LG_TRY(cudaMemcpyAsync(&tot[1], t_moff.as<uint64_t>() + ntiles, 8, cudaMemcpyDeviceToHost, st));
   LG_TRY(cudaStreamSynchronize(st));
   g->n_items = tot[0];
   g->n_multi = tot[1];
+  g->heavy_prefix = 0;
+  g->mid_prefix = g->relabel == 1 ? first.mid : 0;
+  g->top_arcs = first.top;
   if (g->n_items == 0) return LG_OK;
   LG_TRY(pool_alloc((void**)&g->items, g->n_items * sizeof(HeavyItem), st));
   if (g->n_multi) LG_TRY(pool_alloc((void**)&g->multi, g->n_multi * sizeof(uint32_t), st));
@@ -575,7 +596,11 @@ static lg_status build_schedule(lg_graph* g, cudaStream_t st) {
     LG_TRY(ops->plan_carry(v, p, st));
     LG_TRY(plan_carry_scan(g->items, g->multi, g->n_multi, p.segsum, st));
   }
+  HeavyItem last;
+  if (g->relabel == 1)  // degrees descend: every vertex up to the last item's is heavy
+    LG_TRY(cudaMemcpyAsync(&last, g->items + g->n_items - 1, sizeof(last), cudaMemcpyDeviceToHost, st));
   LG_TRY(cudaStreamSynchronize(st));
+  if (g->relabel == 1) g->heavy_prefix = (uint64_t)last.v + 1;
   return LG_OK;
 }
 
@@ -903,10 +928,13 @@ extern "C" lg_status lg_pagerank(const lg_graph* g, float damping, uint32_t iter
       personal = personal_orig;
     }
   }
-  Tmp ca(st), cb(st), tpart(st);
+  const PrPlan plan = pr_plan(g);
+  Tmp ca(st), cb(st), tpart(st), tsync(st), taux(st);
   LG_TRY(ca.alloc(n * sizeof(float)));
   LG_TRY(cb.alloc(n * sizeof(float)));
-  if (g->n_multi) LG_TRY(tpart.alloc(g->n_items * sizeof(float)));
+  if (plan.part_floats) LG_TRY(tpart.alloc(plan.part_floats * sizeof(float)));
+  LG_TRY(tsync.alloc(plan.sync_words * sizeof(uint32_t)));
+  if (plan.aux_words) LG_TRY(taux.alloc(plan.aux_words * sizeof(uint64_t)));
   const GView v = make_view(g);
   const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
   PrArgs a;
@@ -919,6 +947,13 @@ extern "C" lg_status lg_pagerank(const lg_graph* g, float damping, uint32_t iter
   a.ranks_out = ranks;
   a.contrib_out = ca.as<float>();
   a.hot = hot_rows(g, sizeof(float));
+  a.tile_a = plan.tile_a;
+  a.tile_b = plan.tile_b;
+  a.tile_nv = plan.tile_nv;
+  a.tabn = plan.tabn;
+  a.sync = tsync.as<uint32_t>();
+  a.nsync = plan.sync_words;
+  a.aux = taux.as<uint64_t>();
   LG_TRY(ops->pr_init(v, a, st));
   float* cur = ca.as<float>();
   float* nxt = cb.as<float>();
@@ -926,8 +961,8 @@ extern "C" lg_status lg_pagerank(const lg_graph* g, float damping, uint32_t iter
     a.contrib_in = cur;
     a.contrib_out = nxt;
     a.last = (t + 1 == iters);
+    a.turn = t & 1;
     LG_TRY(ops->pr_pull(v, a, st));
-    LG_TRY(pr_finish_multi(v, a, st));
     float* tt = cur; cur = nxt; nxt = tt;
   }
   return LG_OK;

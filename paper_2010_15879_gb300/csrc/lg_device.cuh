@@ -70,6 +70,7 @@ struct GView {
   uint32_t s, H, omega, r, w_O, ef_l, sample_log2;
   uint32_t heavy_min;         // degrees above this are in the schedule
   uint32_t heavy_seg;         // max fields per schedule item
+  uint64_t heavy_prefix;      // the vertices below this label are all in the schedule (DM order; else 0)
 };
 
 __device__ __forceinline__ uint32_t bits_u32(uint32_t x) { return 32u - __clz(x); }
@@ -137,6 +138,12 @@ __device__ __forceinline__ void ldg256_stream(const uint32_t* p, uint64_t pol, u
 __device__ __forceinline__ float ldg_gather(const float* p, uint64_t pol) {
   float v;
   asm("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+  return v;
+}
+// past the L1
+__device__ __forceinline__ float ldcg_gather(const float* p, uint64_t pol) {
+  float v;
+  asm("ld.global.cg.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
   return v;
 }
 // one 32-bit word with an L2 cache policy

@@ -27,6 +27,9 @@ struct lg_graph {
   lg::HeavyItem *items; uint64_t n_items;
   uint32_t *multi;      uint64_t n_multi;
   uint32_t heavy_min, heavy_seg;
+  uint64_t heavy_prefix;  // DM order: the vertices below this label are all in the schedule (else 0)
+  uint64_t top_arcs;      // sum of the degrees of the first PW_TOP labels
+  uint64_t mid_prefix;    // DM order: the vertices below this label have more than 32 arcs (else 0)
 };
 
 namespace lg {
@@ -118,6 +121,8 @@ struct PlanArgs {
   HeavyItem* items;
   uint32_t* multi;
   uint32_t* segsum;          // per item: sum of its (gap) values
+  unsigned long long* top;   // sum of the degrees of the first PW_TOP labels
+  uint32_t* mid;             // largest v + 1 over the vertices of more than 32 arcs
 };
 
 struct PrArgs {
@@ -132,6 +137,22 @@ struct PrArgs {
   float* part;               // per heavy item partial sums (split vertices)
   uint32_t hot;              // gathers of contributions u < hot keep their L2 lines (evict-last), the
                              // others are evict-first (DM order puts the most gathered vertices first)
+  uint64_t tile_a, tile_b;   // vertices [tile_a, tile_b) in warp tiles of tile_nv, the others of 128 (PrPlan)
+  uint32_t tile_nv;
+  uint32_t tabn;             // contributions u < tabn are gathered from shared memory (PrPlan)
+  uint32_t turn;             // which of the two ticket counters this iteration uses
+  uint32_t* sync;            // [0..1] ticket counters, [2 + first item] arrived parts of a split vertex
+  uint64_t nsync;            // words of sync
+  uint64_t* aux;             // Elias-Fano: where each warp tile starts in the high vector
+};
+
+// How a PageRank call runs on a graph: chosen from its sizes by pr_plan.
+struct PrPlan {
+  uint64_t tile_a, tile_b;
+  uint32_t tile_nv, tabn;
+  uint64_t part_floats;      // PrArgs::part
+  uint64_t sync_words;       // PrArgs::sync
+  uint64_t aux_words;        // PrArgs::aux
 };
 
 struct BfsArgs {
@@ -215,7 +236,6 @@ struct TravOps {
 };
 
 // finishing kernels for vertices split into several heavy items (lg_api.cu)
-cudaError_t pr_finish_multi(const GView& g, const PrArgs& a, cudaStream_t st);
 cudaError_t bfs_finish_multi(const GView& g, const BfsArgs& a, int mask_bytes, cudaStream_t st);
 cudaError_t ppr_finish_multi(const GView& g, const PprArgs& a, cudaStream_t st);
 cudaError_t plan_carry_scan(HeavyItem* items, const uint32_t* multi, uint64_t n_multi, const uint32_t* segsum,
@@ -238,6 +258,8 @@ uint32_t hot_rows(const lg_graph* g, uint32_t elem_bytes);
 // ranks = r_0 (1/n, or the indicator of personal_orig >= 0): PageRank after zero
 // iterations (lg_api.cu)
 cudaError_t pr_fill0(float* ranks, uint64_t n, int64_t personal_orig, cudaStream_t st);
+
+PrPlan pr_plan(const lg_graph* g);
 
 // BFS helpers (lg_api.cu); vmajor: depth[v * S + s] instead of depth[s * n + v]
 cudaError_t bfs_seed(void* vis, void* front, uint32_t* depth, uint64_t n, const uint32_t* sources_stored,

@@ -18,7 +18,10 @@ namespace {
 
 constexpr uint64_t kMaxVertices = 1ull << 20;  // graphs up to 1,048,576 vertices
 constexpr uint64_t kMaxItems = 1ull << 18;     // heavy-schedule items with partial sums
-constexpr uint64_t kScratchFloats = 2 * kMaxVertices + kMaxItems;  // 9 MiB
+constexpr uint64_t kSyncWords = kMaxItems / 2 + 64;  // ticket counters, split vertices (two items each at least)
+constexpr uint64_t kAuxWords = kMaxVertices / 16 + kMaxVertices / 128 + 64;  // u64: starts of the warp tiles
+                                                                            // (pr_plan: >= 16 vertices from 2^16 on)
+constexpr uint64_t kScratchFloats = 2 * kMaxVertices + kMaxItems + kSyncWords + 2 * kAuxWords;  // 10.1 MiB
 
 __device__ __align__(256) float g_pr_scratch[kScratchFloats];
 
@@ -116,11 +119,13 @@ extern "C" lg_status lg_pagerank_noalloc(const lg_graph* g, float damping, uint3
     personal = ps;
   }
   if (e == cudaSuccess) {
-    // scratch layout: contributions A [n], contributions B [n], item partial sums;
-    // every element is written before it is read, so nothing needs clearing
+    // scratch layout: contributions A [n], contributions B [n], item partial
+    // sums, counters, tile starts; every element is written before it is read,
+    // so nothing needs clearing
     float* ca = scratch;
     float* cb = scratch + kMaxVertices;
     float* part = scratch + 2 * kMaxVertices;
+    const PrPlan plan = pr_plan(g);
     const GView v = make_view(g);
     const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
     PrArgs a;
@@ -133,6 +138,13 @@ extern "C" lg_status lg_pagerank_noalloc(const lg_graph* g, float damping, uint3
     a.hot = hot_rows(g, sizeof(float));
     a.ranks_out = ranks;
     a.contrib_out = ca;
+    a.tile_a = plan.tile_a;
+    a.tile_b = plan.tile_b;
+    a.tile_nv = plan.tile_nv;
+    a.tabn = plan.tabn;
+    a.sync = reinterpret_cast<uint32_t*>(part + kMaxItems);
+    a.nsync = plan.sync_words;
+    a.aux = reinterpret_cast<uint64_t*>(part + kMaxItems + kSyncWords);
     e = ops->pr_init(v, a, st);
     float* cur = ca;
     float* nxt = cb;
@@ -140,8 +152,8 @@ extern "C" lg_status lg_pagerank_noalloc(const lg_graph* g, float damping, uint3
       a.contrib_in = cur;
       a.contrib_out = nxt;
       a.last = (t + 1 == iters);
+      a.turn = t & 1;
       e = ops->pr_pull(v, a, st);
-      if (e == cudaSuccess) e = pr_finish_multi(v, a, st);
       float* tt = cur; cur = nxt; nxt = tt;
     }
   }

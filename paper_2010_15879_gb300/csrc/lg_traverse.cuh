@@ -1,7 +1,8 @@
 // Graph kernels with the Log(Graph) decoder fused in (Sections 3.7.2-3.7.3 for
 // the access path, Section 7.1.2 for BFS and PageRank).
 //
-// Pull sweeps (PageRank, bottom-up BFS) are one launch with two kinds of CTA:
+// PageRank sweeps are in lg_pull.cuh.  The other pull sweeps (bottom-up BFS,
+// batched personalized PageRank) are one launch with two kinds of CTA:
 //   * heavy CTAs walk the heavy-vertex schedule built at encode time: vertices
 //     of degree > heavy_min split into items of <= heavy_seg fields, one warp per
 //     item, lane i decoding field i of each 32-field chunk with 4 chunks in
@@ -21,6 +22,8 @@
 // Vertices split into several items are finished by a small second kernel.
 // Push steps and neighbor queries decode one random vertex per warp.
 #pragma once
+
+#include <algorithm>
 
 #include "lg_internal.h"
 
@@ -283,6 +286,12 @@ __device__ __forceinline__ void warp_ids(const GView& g, uint64_t start, uint32_
 
 constexpr int HEAVY_U = 4;  // chunks of 32 fields in flight per warp
 
+}  // namespace lg
+
+#include "lg_pull.cuh"
+
+namespace lg {
+
 // ---------------------------------------------------------------------------
 // tile phases shared by the pull kernels
 // ---------------------------------------------------------------------------
@@ -357,168 +366,45 @@ __host__ __device__ inline unsigned heavy_blocks(uint64_t n_items) {
 }
 
 // ===========================================================================
-// PageRank
+// PageRank: r_0 (the sweeps are in lg_pull.cuh).  Also zeroes the ticket and
+// part counters of the sweeps and, with Elias-Fano offsets, notes where each
+// warp tile's first one is in the high vector (`aux`), so that a sweep's tiles
+// need no select whatever the sample rate.
 // ===========================================================================
 template <int IDM, int OFF>
-__global__ void __launch_bounds__(TNT) k_pr_init(GView g, PrArgs a) {
-  __shared__ TileSmem sm;
-  const uint64_t v0 = (uint64_t)blockIdx.x * TV;
+__global__ void __launch_bounds__(TNT) k_pr_init(GView g, PrArgs a, uint32_t tile0) {
+  __shared__ uint64_t xs[TV + 1];
+  __shared__ TileScratch ts;
+  const uint64_t gt = (uint64_t)blockIdx.x * TNT + threadIdx.x, gs = (uint64_t)gridDim.x * TNT;
+  for (uint64_t i = gt; i < a.nsync; i += gs) a.sync[i] = 0;
+  // vertices of tiles that hold none but heavy ones
+  for (uint64_t i = gt; i < g.n_items && tile0; i += gs) {
+    const HeavyItem h = g.items[i];
+    if (h.f0 == 0) a.contrib_out[h.v] = (a.personal < 0 ? a.r0_all : ((int64_t)h.v == a.personal ? 1.0f : 0.0f)) / (float)h.deg;
+  }
+  const uint64_t v0 = ((uint64_t)blockIdx.x + tile0) * TV;
+  if (v0 >= g.n) return;
   const int cnt = (int)min((uint64_t)TV, g.n - v0);
-  tile_offsets<OFF>(g, v0, cnt, sm.xs, sm.ts);
+  tile_offsets<OFF>(g, v0, cnt, xs, ts);
   __syncthreads();
   for (int i = threadIdx.x; i < cnt; i += TNT) {
     uint64_t start; uint32_t d, w;
-    vgeo<IDM>(g, sm.xs[i], sm.xs[i + 1], start, d, w);
+    vgeo<IDM>(g, xs[i], xs[i + 1], start, d, w);
     const uint64_t v = v0 + i;
     const float r0 = a.personal < 0 ? a.r0_all : ((int64_t)v == a.personal ? 1.0f : 0.0f);
     a.contrib_out[v] = d ? r0 / (float)d : 0.0f;
-  }
-}
-
-__device__ __forceinline__ void pr_finish(const GView& g, const PrArgs& a, uint64_t v, uint32_t d, float sum) {
-  const float base = a.personal < 0 ? a.base_all : ((int64_t)v == a.personal ? a.base_all : 0.0f);
-  const float r = base + a.damp * sum;
-  __stcs(a.contrib_out + v, d ? r / (float)d : 0.0f);  // streamed: read again only next iteration
-  if (a.last) __stcs(a.ranks_out + (g.inv_perm ? (uint64_t)g.inv_perm[v] : v), r);
-}
-
-// One launch = one iteration.  Blocks [0, HB) take the heavy schedule (a warp
-// per item); the other blocks take one tile of 512 vertices each.
-template <int IDM, int OFF>
-__global__ void __launch_bounds__(TNT, (IDM == ID_LOCAL || IDM == ID_CSR32) ? 5 : 6) k_pr_pull(GView g, PrArgs a) {
-  __shared__ TileSmem sm;
-  const float* __restrict__ c = a.contrib_in;
-  const unsigned hb = heavy_blocks(g.n_items);
-  const int lane = threadIdx.x & 31;
-  const uint64_t pstream = policy_stream(), pkeep = policy_keep();
-  if (blockIdx.x < hb) {
-    const uint64_t it = (uint64_t)blockIdx.x * (TNT / 32) + (threadIdx.x >> 5);
-    if (it >= g.n_items) return;
-    const HeavyItem h = g.items[it];
-    const uint32_t f1 = h.f0 + h.nf;
-    uint32_t carry = h.carry;
-    float acc = 0.f, comp = 0.f;
-    for (uint32_t base = h.f0; base < f1; base += 32 * HEAVY_U) {
-      uint32_t id[HEAVY_U];
-      warp_ids<IDM, HEAVY_U>(g, h.bit, h.w, base, f1, carry, id);
-      float x[HEAVY_U];
-#pragma unroll
-      for (int u = 0; u < HEAVY_U; u++) x[u] = (base + 32u * u + lane < f1) ? ldg_gather(c + id[u], id[u] < a.hot ? pkeep : pstream) : 0.f;
-#pragma unroll
-      for (int u = 0; u < HEAVY_U; u++) {  // compensated (Kahan) lane sums
-        const float y = x[u] - comp;
-        const float t = acc + y;
-        comp = (t - acc) - y;
-        acc = t;
-      }
+    if (OFF == OFF_EF && v >= a.tile_a) {
+      const bool small = v < a.tile_b;
+      const uint64_t k = small ? v - a.tile_a : v - a.tile_b, nv = small ? a.tile_nv : PW_TV;
+      if (k % nv == 0) a.aux[k / nv + (small ? 0 : (a.tile_b - a.tile_a) / a.tile_nv)] = (xs[i] >> g.ef_l) + v;
     }
-    acc = warp_sum<float>(acc);
-    if (lane == 0) {
-      if (h.nitems == 1) pr_finish(g, a, h.v, h.deg, acc);
-      else a.part[it] = acc;
-    }
-    return;
-  }
-  const uint64_t v0 = (uint64_t)(blockIdx.x - hb) * TV;
-  const int cnt = (int)min((uint64_t)TV, g.n - v0);
-  tile_offsets<OFF>(g, v0, cnt, sm.xs, sm.ts);
-  __syncthreads();
-  tile_classify<IDM>(g, sm, cnt, [](int) { return true; });
-
-  // zero-degree vertices keep the teleport term only
-  for (int i = threadIdx.x; i < cnt; i += TNT)
-    if (sm.deg[i] == 0) pr_finish(g, a, v0 + i, 0, 0.0f);
-
-  if (IDM == ID_LOCAL_GAP) {
-    // gap-coded IDs cannot start mid-neighborhood: runs of whole vertices,
-    // sequential decode, 4 gathers in flight
-    uint32_t jb, je;
-    light_range(sm, jb, je);
-    for (uint32_t j = jb; j < je; j++) {
-      const int i = sm.clist[j];
-      const uint32_t d = sm.deg[i];
-      SeqDec<IDM> dec;
-      dec.init(g, sm.st[i], sm.wid[i], pstream);
-      float s0 = 0.f, s1 = 0.f;
-      uint32_t k = 0;
-      for (; k + 4 <= d; k += 4) {
-        const uint32_t u0 = dec.next(), u1 = dec.next(), u2 = dec.next(), u3 = dec.next();
-        const float f0 = ldg_gather(c + u0, u0 < a.hot ? pkeep : pstream), f1 = ldg_gather(c + u1, u1 < a.hot ? pkeep : pstream);
-        const float f2 = ldg_gather(c + u2, u2 < a.hot ? pkeep : pstream), f3 = ldg_gather(c + u3, u3 < a.hot ? pkeep : pstream);
-        s0 += f0 + f1;
-        s1 += f2 + f3;
-      }
-      for (; k < d; k++) {
-        const uint32_t u = dec.next();
-        s0 += ldg_gather(c + u, u < a.hot ? pkeep : pstream);
-      }
-      pr_finish(g, a, v0 + i, d, s0 + s1);
-    }
-    return;
-  }
-  // Fields-balanced light phase (as in k_ppr_pull): thread t decodes fields
-  // [F*t/TNT, F*(t+1)/TNT) of the tile's light fields, entering its first
-  // vertex mid-neighborhood if need be; per-vertex sums go to vsum, the
-  // partial sum of a vertex entered mid-way to carry[t]; a uniform phase adds
-  // them per vertex in thread order and finishes the vertex.
-  __shared__ float vsum[TV];
-  __shared__ float carry[TNT];
-  float* ps = nullptr;
-  const uint32_t F = sm.nfields, nl = sm.nlight;
-  const uint32_t flo = (uint32_t)((uint64_t)F * threadIdx.x / TNT);
-  const uint32_t fhi = (uint32_t)((uint64_t)F * (threadIdx.x + 1) / TNT);
-  carry[threadIdx.x] = 0.f;
-  if (flo < fhi) {
-    uint32_t lo = 0, hi = nl - 1;  // the vertex holding field flo: last j with fpre[j] <= flo
-    while (lo < hi) {
-      const uint32_t m = (lo + hi + 1) >> 1;
-      if (sm.fpre[m] <= flo) lo = m; else hi = m - 1;
-    }
-    uint32_t j = lo, f = flo;
-    ps = sm.fpre[j] < flo ? &carry[threadIdx.x] : &vsum[j];
-    while (f < fhi) {
-      const int i = sm.clist[j];
-      const uint32_t vend = min(sm.fpre[j + 1], fhi);
-      const uint32_t fw = IDM == ID_GLOBAL ? g.r : (IDM == ID_CSR32 ? 32u : (uint32_t)sm.wid[i]);
-      SeqDec<IDM> dec;
-      dec.init(g, sm.st[i] + (uint64_t)(f - sm.fpre[j]) * fw, sm.wid[i], pstream);
-      const uint32_t d = vend - f;
-      float s0 = 0.f, s1 = 0.f;
-      uint32_t k = 0;
-      for (; k + 4 <= d; k += 4) {  // four gathers in flight
-        const uint32_t u0 = dec.next(), u1 = dec.next(), u2 = dec.next(), u3 = dec.next();
-        const float f0 = ldg_gather(c + u0, u0 < a.hot ? pkeep : pstream), f1 = ldg_gather(c + u1, u1 < a.hot ? pkeep : pstream);
-        const float f2 = ldg_gather(c + u2, u2 < a.hot ? pkeep : pstream), f3 = ldg_gather(c + u3, u3 < a.hot ? pkeep : pstream);
-        s0 += f0 + f1;
-        s1 += f2 + f3;
-      }
-      for (; k < d; k++) {
-        const uint32_t u = dec.next();
-        s0 += ldg_gather(c + u, u < a.hot ? pkeep : pstream);
-      }
-      *ps = s0 + s1;
-      f = vend;
-      j++;
-      ps = &vsum[j];
-    }
-  }
-  __syncthreads();
-  for (uint32_t j = threadIdx.x; j < nl; j += TNT) {
-    const uint32_t fs = sm.fpre[j], fe = sm.fpre[j + 1];
-    float sum = vsum[j];
-    uint32_t q = (uint32_t)((uint64_t)fs * TNT / (F ? F : 1));  // the thread holding the first field
-    while (q + 1 < TNT && (uint32_t)((uint64_t)F * (q + 1) / TNT) <= fs) q++;
-    while (q > 0 && (uint32_t)((uint64_t)F * q / TNT) > fs) q--;
-    for (q = q + 1; q < TNT && (uint32_t)((uint64_t)F * q / TNT) < fe; q++) sum += carry[q];
-    const int i = sm.clist[j];
-    pr_finish(g, a, v0 + i, sm.deg[i], sum);
   }
 }
 
 // ===========================================================================
 // Personalized PageRank, PPR_K requests per sweep (serving engine).  Slot k
 // iterates r_t[v] = (1-d_k)[v == s_k] + d_k * sum_{u in N_v} r_{t-1}[u] / d_u;
-// the same tile / heavy-item structure as k_pr_pull, with PPR_K sums per
+// tile CTAs and heavy items as described at the top, with PPR_K sums per
 // vertex and one 32-byte gather per arc for all slots.
 // ===========================================================================
 __device__ __forceinline__ void ppr_finish(const PprArgs& a, uint64_t v, uint32_t d, const float (&sum)[PPR_K]) {
@@ -855,7 +741,7 @@ __global__ void __launch_bounds__(TNT, IDM == ID_LOCAL_GAP ? 6 : 5) k_bfs_pull(G
       bfs_finish<M>(g, a, v0 + i, need, acc, qbuf, &qn, &newpairs);
     }
   } else {
-    // fields-balanced (as in k_pr_pull): partial ORs of a vertex split over
+    // fields-balanced (as in k_ppr_pull): partial ORs of a vertex split over
     // threads are combined exactly in a uniform phase
     __shared__ M vor[TV];
     __shared__ M carry[TNT];
@@ -1523,13 +1409,20 @@ __global__ void __launch_bounds__(TNT) k_plan_count(GView g, PlanArgs p) {
   const int cnt = (int)min((uint64_t)TV, g.n - v0);
   tile_offsets<OFF>(g, v0, cnt, sm.xs, sm.ts);
   __syncthreads();
-  uint64_t mine = 0;
+  uint64_t mine = 0, top = 0;
+  uint32_t mid = 0;
   for (int i = threadIdx.x; i < cnt; i += TNT) {
     uint64_t start; uint32_t d, w;
     vgeo<IDM>(g, sm.xs[i], sm.xs[i + 1], start, d, w);
     const uint32_t k = items_of(g, d);
     mine += ((uint64_t)k << 32) | (k > 1 ? 1u : 0u);
+    if (d > 32) mid = (uint32_t)(v0 + i) + 1u;
+    if (v0 + i < PW_TOP) top += d;
   }
+  mid = __reduce_max_sync(LG_FULL_MASK, mid);
+  top = warp_sum<uint64_t>(top);
+  if ((threadIdx.x & 31) == 0 && mid) atomicMax(p.mid, mid);
+  if ((threadIdx.x & 31) == 0 && top) atomicAdd(p.top, (unsigned long long)top);
   uint64_t total;
   block_excl_scan<uint64_t, TNT>(mine, total, sm.red64);
   if (threadIdx.x == 0) {
@@ -1608,13 +1501,22 @@ inline unsigned tiles_of(uint64_t n) { return (unsigned)((n + TV - 1) / TV); }
 
 template <int IDM, int OFF>
 cudaError_t launch_pr_init(const GView& g, const PrArgs& a, cudaStream_t st) {
-  k_pr_init<IDM, OFF><<<tiles_of(g.n), TNT, 0, st>>>(g, a);
+  const cudaError_t e = a.tabn ? cudaFuncSetAttribute(k_pr_pull<IDM, OFF, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PW_SMEM)
+                               : cudaFuncSetAttribute(k_pr_pull<IDM, OFF, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PW_SMEM);
+  if (e != cudaSuccess) return e;
+  const uint32_t tile0 = (uint32_t)(g.heavy_prefix / TV);
+  k_pr_init<IDM, OFF><<<std::max(1u, tiles_of(g.n) - tile0), TNT, 0, st>>>(g, a, tile0);
   count_launch();
   return cudaGetLastError();
 }
 template <int IDM, int OFF>
 cudaError_t launch_pr_pull(const GView& g, const PrArgs& a, cudaStream_t st) {
-  k_pr_pull<IDM, OFF><<<heavy_blocks(g.n_items) + tiles_of(g.n), TNT, 0, st>>>(g, a);
+  const uint64_t units = g.n_items + (g.n - a.tile_a) / a.tile_nv + 1;
+  // the shared memory beside the table is the warps' (PrWarp)
+  const unsigned grid = (unsigned)std::min<uint64_t>(units, PW_SMS);
+  const size_t smem = PW_WARPS * sizeof(PrWarp) + (size_t)a.tabn * 4;
+  if (a.tabn) k_pr_pull<IDM, OFF, true><<<grid, PW_NT, smem, st>>>(g, a);
+  else k_pr_pull<IDM, OFF, false><<<grid, PW_NT, smem, st>>>(g, a);
   count_launch();
   return cudaGetLastError();
 }
