@@ -320,7 +320,9 @@ typedef struct lg_batch lg_batch; /* opaque; owns its device memory, not the inp
 typedef struct {
     uint32_t autotune;      /* 1: time the candidate decode schedules at creation      */
     uint32_t lanes;         /* 0: default/autotuned; else lanes per vertex for every
-                               graph, one of 1, 4, 8, 32 (disables autotune)          */
+                               graph, one of 1, 4, 8, 32 (disables autotune); graphs
+                               of at most 65,536 vertices take windows of 256 fields
+                               per warp whatever it is                                */
     uint64_t tile_arcs;     /* arcs per CTA before a graph gets a team of CTAs;
                                0: 2^19, or autotuned among 2^18 .. 2^21               */
     uint32_t wait_limit_us; /* time limit of a team barrier; 0 means 2 s              */

@@ -19,9 +19,11 @@
 // between sweeps or levels (contributions, depths, queues) is read with
 // L2-coherent loads (ld.global.cg).
 //
-// Each graph decodes its neighborhoods with T lanes per vertex (T = 1, 4, 8
-// or 32); T per average-degree class and the team tile are chosen by a timing
-// autotuner when the batch is created.
+// Graphs of up to 65,536 vertices keep their per-vertex state in the CTA's
+// shared memory (the second half of this file's kernels); the others decode
+// their neighborhoods with T lanes per vertex (T = 1, 4, 8 or 32).  T per
+// average-degree class and the team tile are chosen by a timing autotuner when
+// the batch is created.
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -29,6 +31,7 @@
 #include <mutex>
 
 #include "lg_internal.h"
+#include "lg_window.cuh"
 
 namespace lg {
 
@@ -49,7 +52,7 @@ struct BatchItem {
   uint32_t g, member;
 };
 
-constexpr int BNT = 256;  // threads per batch CTA
+constexpr int BNT = 768;  // threads per batch CTA, one CTA per SM (80 registers: no spills)
 constexpr uint32_t PH_ENCODE = 1, PH_BFS = 2, PH_PR = 4;
 constexpr uint32_t BERR_TIMEOUT = 1;
 constexpr uint32_t SYNC_WORDS = 4;  // per graph: barrier count + 3 rotating queue counters
@@ -222,6 +225,326 @@ __device__ __forceinline__ void pack_words(uint64_t* out, uint64_t k0, uint64_t 
   }
 }
 
+// ===========================================================================
+// Graphs of at most 2^16 vertices (IDs of at most 16 bits).
+//
+// A run reads every arc once per PageRank sweep, and what it does per arc
+// bounds it.  Reading contributions, depths and frontiers through L1 and L2
+// costs one line look-up per arc (274-297 G/s over the chip at best); shared
+// memory answers 1,515 G/s.  So a CTA holds the contributions of its graph (the
+// first BS_TAB vertices of it) and its visited and frontier bitmaps there, one
+// large CTA per SM instead of eight small ones.  Sweeps decode windows of 256
+// fields as the whole-graph sweeps do (lg_window.cuh); BFS turns bottom-up,
+// with early exit, while the frontier is large; packing assembles words from
+// windows of 256 records read coalesced.
+// Measured: 1,000 R-MAT graphs of 2^8 .. 2^16 vertices (438 M arcs), one run
+// (encode, BFS, 10 sweeps): 43.0 ms with T lanes per vertex through L1, 10.9 ms
+// here.
+// ===========================================================================
+constexpr uint32_t BS_MAX = 1u << 16;       // vertices
+constexpr int BS_WARPS = BNT / 32;
+constexpr uint32_t BS_TV = 64;              // vertices of a warp tile: v0 + lane and v0 + 32 + lane
+constexpr uint32_t BS_STAGE = 136;          // words of 256 fields of <= 16 bits, from a 16-byte boundary
+constexpr uint32_t BS_WORDS = BS_MAX / 32;  // words of a bitmap
+
+struct BWarp {
+  __align__(16) uint32_t stage[2][BS_STAGE];  // two windows of the stream; when packing, 256 records
+  uint32_t heads[2][PW_G];                    // bit f: field f of the window is the first of its vertex
+  float vsum[BS_TV];                          // sums of the tile's vertices that have arcs, in order
+};
+static_assert(2 * BS_STAGE >= PW_WF, "a window of records to pack fits the stages");
+// 194 KB of shared memory: a carve-out of 196 KB keeps the L1's full gather
+// rate, one of 228 KB halves it (measured)
+constexpr size_t BS_SMEM = 194 * 1024;
+constexpr uint32_t BS_TAB = (uint32_t)((BS_SMEM - BS_WARPS * sizeof(BWarp)) / sizeof(float)) & ~3u;
+static_assert(BS_TAB >= 3 * BS_WORDS, "the bitmaps share the table's memory");
+
+// Windows [i0, i1) of 256 records of w <= 32 bits: rec(j) is record j < nrec.
+// Lane l reads records l, l + 32, .., all in flight; then a lane assembles
+// whole 32-bit words.  The last window fills up its 64-bit word with zeros.
+template <typename Rec>
+__device__ __forceinline__ void pack_windows(uint32_t* out, uint64_t i0, uint64_t i1, uint64_t nrec, uint32_t w,
+                                             BWarp& W, Rec rec) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t* st = W.stage[0];
+  const uint32_t inv = ((1u << 20) + w - 1) / w;  // x / w = x * inv >> 20 for x < 2^13
+  for (uint64_t i = i0 + (threadIdx.x >> 5); i < i1; i += BS_WARPS) {
+    const uint64_t j0 = i * PW_WF;
+    const uint32_t cnt = (uint32_t)min((uint64_t)PW_WF, nrec - j0);
+    uint32_t r[PW_G];
+#pragma unroll
+    for (int u = 0; u < PW_G; u++) r[u] = 32u * u + lane < cnt ? rec(j0 + 32u * u + lane) : 0u;
+#pragma unroll
+    for (int u = 0; u < PW_G; u++) st[32 * u + lane] = r[u];
+    __syncwarp();
+    const uint32_t nw = 2 * ((cnt * w + 63) / 64);
+    uint32_t* o = out + i * PW_G * w;
+    for (uint32_t q = lane; q < nw; q += 32) {
+      uint32_t acc = 0;
+      for (uint32_t j = (uint32_t)(((uint64_t)(32u * q) * inv) >> 20); j < cnt && j * w < 32u * q + 32u; j++) {
+        const int at = (int)(j * w) - (int)(32u * q);
+        acc |= at >= 0 ? st[j] << at : st[j] >> -at;
+      }
+      o[q] = acc;
+    }
+    __syncwarp();
+  }
+}
+
+// One sweep of tile `tile`: r = base + d * sum over neighbors of cin, cin(id)
+// from the table below tabn, from global memory beyond.
+__device__ __forceinline__ void small_sweep_tile(const BatchArgs& a, const BatchGraph& G, uint32_t tile,
+                                                 const float* tab, uint32_t tabn, const float* cin, float* cout,
+                                                 bool last, uint64_t pol, BWarp& W) {
+  const uint32_t lane = threadIdx.x & 31u, lt = lane_lt_mask(), k0 = PW_E * lane;
+  const uint32_t* A32 = reinterpret_cast<const uint32_t*>(a.A + G.a_word);
+  const uint64_t* O = a.O + G.o_word;
+  const uint32_t v0 = tile * BS_TV, s = G.s, mask = mask_lo(s);
+  const uint32_t x0 = sfield(O, (uint64_t)min(v0 + lane, G.n) * G.w_O, G.w_O);
+  const uint32_t x1 = sfield(O, (uint64_t)min(v0 + 32 + lane, G.n) * G.w_O, G.w_O);
+  const uint32_t xe = sfield(O, (uint64_t)min(v0 + BS_TV, G.n) * G.w_O, G.w_O);
+  const uint32_t xb = __shfl_sync(LG_FULL_MASK, x0, 0), xm = __shfl_sync(LG_FULL_MASK, x1, 0);
+  uint32_t n0 = __shfl_down_sync(LG_FULL_MASK, x0, 1), n1 = __shfl_down_sync(LG_FULL_MASK, x1, 1);
+  if (lane == 31) { n0 = xm; n1 = xe; }
+  const uint32_t d0 = n0 - x0, d1 = n1 - x1;  // degrees
+  const uint32_t F = xe - xb;
+  auto open_window = [&](uint32_t f0, uint32_t b) {
+    const uint32_t nf = min(PW_WF, F - f0);
+    if (lane < PW_G) W.heads[b][lane] = 0;
+    __syncwarp();
+    const uint32_t h0 = x0 - xb - f0, h1 = x1 - xb - f0;
+    if (d0 && h0 < nf) atomicOr(&W.heads[b][h0 >> 5], 1u << (h0 & 31u));
+    if (d1 && h1 < nf) atomicOr(&W.heads[b][h1 >> 5], 1u << (h1 & 31u));
+    const uint64_t b0 = (uint64_t)(xb + f0) * s, w0 = (b0 >> 5) & ~3ull;
+    stage_issue<2>(W.stage[b], A32, w0, (uint32_t)(((b0 + nf * s + 31) >> 5) + 1 - w0), pol);
+  };
+  int jb = -1;
+  float open = 0.f;
+  if (F) open_window(0, 0);
+  uint32_t b = 0;
+  for (uint32_t f0 = 0; f0 < F; f0 += PW_WF, b ^= 1u) {
+    const uint32_t nf = min(PW_WF, F - f0);
+    if (f0 + PW_WF < F) {
+      open_window(f0 + PW_WF, b ^ 1u);
+      stage_wait<1>();
+    } else {
+      stage_wait<0>();
+    }
+    const uint32_t hb = (W.heads[b][lane >> 2] >> (8u * (lane & 3u))) & 255u;
+    const int c = (int)__popc(hb), ci = warp_incl_scan<int>(c), je = jb + ci - c;
+    jb += __shfl_sync(LG_FULL_MASK, ci, 31);
+    uint32_t p = sh_bit0(W.stage[b]) + ((uint32_t)((uint64_t)(xb + f0) * s) & 127u) + min(k0, nf) * s;
+    float val[PW_E];
+#pragma unroll
+    for (int e = 0; e < PW_E; e++, p += s) {
+      const uint32_t id = sh_bits(p) & mask;
+      val[e] = 0.f;
+      if (k0 + e < nf) val[e] = id < tabn ? tab[id] : __ldcg(cin + id);
+    }
+    open = join_window(val, hb, je, open, W.vsum);
+    __syncwarp();  // the stage and the heads may be overwritten
+  }
+  if (lane == 0 && jb >= 0) W.vsum[jb] = open;
+  __syncwarp();
+  const float base = (1.0f - a.damp) / (float)G.n;
+  const uint32_t m0 = __ballot_sync(LG_FULL_MASK, d0 != 0), m1 = __ballot_sync(LG_FULL_MASK, d1 != 0);
+  const float s0 = d0 ? W.vsum[__popc(m0 & lt)] : 0.f, s1 = d1 ? W.vsum[__popc(m0) + __popc(m1 & lt)] : 0.f;
+  const float r0 = base + a.damp * s0, r1 = base + a.damp * s1;
+  if (v0 + lane < G.n) {
+    cout[v0 + lane] = d0 ? r0 / (float)d0 : 0.f;
+    if (last) a.ranks[G.vbase + v0 + lane] = r0;
+  }
+  if (v0 + 32 + lane < G.n) {
+    cout[v0 + 32 + lane] = d1 ? r1 / (float)d1 : 0.f;
+    if (last) a.ranks[G.vbase + v0 + 32 + lane] = r1;
+  }
+  __syncwarp();
+}
+
+// Top-down step over the frontier words i = first, first + step, ..: a warp
+// per vertex marks the unvisited neighbors in nx.
+__device__ __forceinline__ void small_push(const BatchArgs& a, const BatchGraph& G, const uint32_t* fr,
+                                           const uint32_t* vis, uint32_t* nx, uint32_t first, uint32_t step) {
+  const uint64_t* A = a.A + G.a_word;
+  const uint64_t* O = a.O + G.o_word;
+  const uint32_t lane = threadIdx.x & 31u, nwd = (G.n + 31) / 32, s = G.s;
+  for (uint32_t i = first; i < nwd; i += step) {
+    for (uint32_t m = fr[i]; m; m &= m - 1) {
+      const uint32_t v = 32 * i + (uint32_t)__ffs((int)m) - 1u;
+      const uint32_t x1 = sfield(O, (uint64_t)(v + 1) * G.w_O, G.w_O);
+      for (uint32_t j = sfield(O, (uint64_t)v * G.w_O, G.w_O) + lane; j < x1; j += 128) {
+        uint32_t u[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) u[k] = j + 32u * k < x1 ? sfield(A, (uint64_t)(j + 32u * k) * s, s) : 0xffffffffu;
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+          if (u[k] != 0xffffffffu && !((vis[u[k] >> 5] >> (u[k] & 31u)) & 1u)) atomicOr(&nx[u[k] >> 5], 1u << (u[k] & 31u));
+      }
+    }
+  }
+}
+
+// Bottom-up step over the vertices of bitmap words [w0, w1): 8 lanes per
+// unvisited vertex look for a frontier neighbor.
+__device__ __forceinline__ void small_pull(const BatchArgs& a, const BatchGraph& G, const uint32_t* fr,
+                                           const uint32_t* vis, uint32_t* nx, uint32_t w0, uint32_t w1) {
+  const uint64_t* A = a.A + G.a_word;
+  const uint64_t* O = a.O + G.o_word;
+  const uint32_t lane = threadIdx.x & 31u, grp = lane >> 3, s = G.s;
+  for (uint32_t i = w0 + (threadIdx.x >> 5); i < w1; i += BS_WARPS) {
+    uint32_t found = 0;
+    for (uint32_t m = ~vis[i]; m;) {
+      uint32_t bit = 0;  // this group's vertex: one of the four lowest unvisited ones
+#pragma unroll
+      for (uint32_t k = 0; k < 4; k++) {
+        if (grp == k) bit = m & (0u - m);
+        m &= m - 1;
+      }
+      const uint32_t v = 32 * i + (uint32_t)__ffs((int)bit) - 1u;
+      uint32_t j = 0, x1 = 0;
+      if (bit) {
+        j = sfield(O, (uint64_t)v * G.w_O, G.w_O) + (lane & 7u);
+        x1 = sfield(O, (uint64_t)(v + 1) * G.w_O, G.w_O);
+      }
+      bool hit = false, any = false;
+      while (__any_sync(LG_FULL_MASK, !any && j < x1)) {
+        if (!any && j < x1) {
+          const uint32_t u0 = sfield(A, (uint64_t)j * s, s);
+          hit = (fr[u0 >> 5] >> (u0 & 31u)) & 1u;
+          if (j + 8 < x1) {
+            const uint32_t u1 = sfield(A, (uint64_t)(j + 8) * s, s);
+            hit = hit || ((fr[u1 >> 5] >> (u1 & 31u)) & 1u);
+          }
+        }
+        j += 16;
+        any = (__ballot_sync(LG_FULL_MASK, hit) >> (8 * grp)) & 255u;
+      }
+      found |= __reduce_or_sync(LG_FULL_MASK, any ? bit : 0u);
+    }
+    if (lane == 0) nx[i] = found;
+  }
+}
+
+__device__ void process_small(const BatchArgs& a, uint32_t gi, uint32_t m) {
+  __shared__ uint32_t ticket, count;
+  const BatchGraph G = a.graphs[gi];
+  const uint32_t p = G.team, n = G.n, wid = threadIdx.x >> 5;
+  uint32_t* bar = a.sync + (uint64_t)gi * SYNC_WORDS;
+  uint32_t round = 0;
+  BWarp& W = reinterpret_cast<BWarp*>(dyn_smem)[wid];
+  float* tab = reinterpret_cast<float*>(dyn_smem + BS_WARPS * sizeof(BWarp));
+  const uint64_t pol = policy_stream();
+  const uint32_t tiles = (n + BS_TV - 1) / BS_TV, nwd = (n + 31) / 32;
+  const uint32_t t0 = (uint32_t)((uint64_t)tiles * m / p), t1 = (uint32_t)((uint64_t)tiles * (m + 1) / p);
+  const uint32_t v0 = t0 * BS_TV, v1 = min(n, t1 * BS_TV);  // this member's vertices
+  const uint32_t w0 = t0 * (BS_TV / 32), w1 = min(nwd, t1 * (BS_TV / 32));
+
+  if (a.phases & PH_ENCODE) {
+    const uint32_t* col = a.col + G.abase;
+    const uint64_t* rp = a.row_ptr + G.vbase;
+    const uint64_t ab = G.abase, na = ((uint64_t)G.arcs + PW_WF - 1) / PW_WF, no = ((uint64_t)n + PW_WF) / PW_WF;
+    pack_windows(reinterpret_cast<uint32_t*>(a.A + G.a_word), na * m / p, na * (m + 1) / p, G.arcs, G.s, W,
+                 [&](uint64_t j) { return __ldcs(col + j); });
+    pack_windows(reinterpret_cast<uint32_t*>(a.O + G.o_word), no * m / p, no * (m + 1) / p, (uint64_t)n + 1, G.w_O, W,
+                 [&](uint64_t j) { return (uint32_t)(__ldg(rp + j) - ab); });
+    if (!team_sync(a, bar, p, ++round)) return;
+  }
+
+  if (a.phases & PH_BFS) {
+    uint32_t* depth = a.depth + G.vbase;
+    uint32_t* vis = reinterpret_cast<uint32_t*>(tab);
+    uint32_t *fr = vis + BS_WORDS, *nx = fr + BS_WORDS;
+    // a team shares each level's new bitmap through one of three global ones:
+    // written in a level, read after its barrier, cleared after the next one
+    uint32_t* shared_nx[3] = {a.q0 + G.vbase, a.q1 + G.vbase, reinterpret_cast<uint32_t*>(a.c0 + G.vbase)};
+    for (uint32_t i = threadIdx.x; i < nwd; i += BNT) {
+      vis[i] = (i == nwd - 1 && (n & 31u) ? ~0u << (n & 31u) : 0u) | (i == 0 ? 1u : 0u);
+      fr[i] = i == 0 ? 1u : 0u;
+      nx[i] = 0;
+    }
+    if (p > 1)
+      for (uint32_t i = w0 + threadIdx.x; i < w1; i += BNT)
+        for (int k = 0; k < 3; k++) shared_nx[k][i] = 0;
+    for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT) depth[v] = v == 0 ? 0u : INF32;
+    if (!team_sync(a, bar, p, ++round)) return;
+    uint32_t frontier = 1;
+    for (uint32_t level = 0; frontier > 0 && level < n; level++) {
+      const bool push = frontier < n / 32 + 1;  // a large frontier is found from the unvisited side, with early exit
+      if (push) small_push(a, G, fr, vis, nx, m + p * wid, p * BS_WARPS);
+      else small_pull(a, G, fr, vis, nx, w0, w1);
+      if (threadIdx.x == 0) count = 0;
+      __syncthreads();
+      if (p > 1) {
+        uint32_t* g = shared_nx[level % 3];
+        if (push) {
+          for (uint32_t i = threadIdx.x; i < nwd; i += BNT)
+            if (nx[i]) atomicOr(g + i, nx[i]);
+        } else {
+          for (uint32_t i = w0 + threadIdx.x; i < w1; i += BNT) __stcg(g + i, nx[i]);
+        }
+        if (!team_sync(a, bar, p, ++round)) return;
+        for (uint32_t i = threadIdx.x; i < nwd; i += BNT) nx[i] = __ldcg(g + i);
+        if (level > 0)
+          for (uint32_t i = w0 + threadIdx.x; i < w1; i += BNT) shared_nx[(level - 1) % 3][i] = 0;
+        __syncthreads();
+      }
+      uint32_t c = 0;
+      for (uint32_t i = threadIdx.x; i < nwd; i += BNT) {
+        const uint32_t x = nx[i];
+        fr[i] = x;
+        vis[i] |= x;
+        nx[i] = 0;
+        c += __popc(x);
+      }
+      c = __reduce_add_sync(LG_FULL_MASK, c);
+      if ((threadIdx.x & 31u) == 0 && c) atomicAdd(&count, c);
+      __syncthreads();
+      frontier = count;
+      for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT)
+        if ((fr[v >> 5] >> (v & 31u)) & 1u) depth[v] = level + 1;
+      __syncthreads();  // count is reset in the next level
+    }
+    __syncthreads();
+  }
+
+  if ((a.phases & PH_PR) && a.iters > 0) {
+    const uint64_t* O = a.O + G.o_word;
+    float* ci = a.c0 + G.vbase;
+    float* co = a.c1 + G.vbase;
+    // a graph of one CTA that fits twice stays in shared memory between sweeps
+    const uint32_t half = (n + 3) & ~3u;
+    const bool inside = p == 1 && 2 * half <= BS_TAB;
+    const uint32_t tabn = min(n, BS_TAB);
+    const float r0 = 1.0f / (float)n;
+    // team members finish their last BFS level before c0 is overwritten
+    if (!team_sync(a, bar, p, ++round)) return;
+    for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT) {
+      const uint32_t d = sfield(O, (uint64_t)(v + 1) * G.w_O, G.w_O) - sfield(O, (uint64_t)v * G.w_O, G.w_O);
+      (inside ? tab : ci)[v] = d ? r0 / (float)d : 0.f;
+    }
+    float *tin = tab, *tout = tab + half;
+    for (uint32_t t = 0; t < a.iters; t++) {
+      if (!team_sync(a, bar, p, ++round)) return;
+      if (!inside)
+        for (uint32_t i = threadIdx.x; i < tabn; i += BNT) tab[i] = __ldcg(ci + i);
+      if (threadIdx.x == 0) ticket = t0;
+      __syncthreads();
+      for (;;) {
+        uint32_t tile = 0;
+        if ((threadIdx.x & 31u) == 0) tile = atomicAdd(&ticket, 1u);
+        tile = __shfl_sync(LG_FULL_MASK, tile, 0);
+        if (tile >= t1) break;
+        small_sweep_tile(a, G, tile, tin, tabn, ci, inside ? tout : co, t + 1 == a.iters, pol, W);
+      }
+      float* x = ci;
+      ci = co;
+      co = x;
+      if (inside) { x = tin; tin = tout; tout = x; }
+    }
+    __syncthreads();
+  }
+}
+
 __device__ void process_item(const BatchArgs& a, uint32_t gi, uint32_t m) {
   const BatchGraph G = a.graphs[gi];
   const uint32_t p = G.team;
@@ -305,7 +628,7 @@ __device__ void process_item(const BatchArgs& a, uint32_t gi, uint32_t m) {
   }
 }
 
-__global__ void __launch_bounds__(BNT, 8) k_batch(BatchArgs a) {
+__global__ void __launch_bounds__(BNT, 1) k_batch(BatchArgs a) {
   __shared__ unsigned int slot_s;
   for (;;) {
     if (threadIdx.x == 0) slot_s = atomicAdd(a.next, 1u);
@@ -315,7 +638,8 @@ __global__ void __launch_bounds__(BNT, 8) k_batch(BatchArgs a) {
     if (slot >= a.n_items) return;
     const BatchItem it = a.items[slot];
     if (a.graphs[it.g].n == 0) continue;
-    process_item(a, it.g, it.member);
+    if (a.graphs[it.g].n <= BS_MAX) process_small(a, it.g, it.member);
+    else process_item(a, it.g, it.member);
   }
 }
 
@@ -405,7 +729,7 @@ void plan_queue(lg_batch* b, uint64_t tile) {
     uint64_t p = tile ? (x.arcs + tile - 1) / tile : 1;
     p = std::max<uint64_t>(p, 1);
     p = std::min<uint64_t>(p, max_team);
-    p = std::min<uint64_t>(p, std::max<uint32_t>(1, x.n / BNT));
+    p = std::min<uint64_t>(p, std::max<uint32_t>(1, x.n / 256));
     x.team = (uint32_t)p;
   }
   std::vector<uint32_t> order(b->count);
@@ -467,7 +791,7 @@ void enqueue_run(lg_batch* b, const BatchArgs& a, cudaStream_t st) {
   cudaMemsetAsync(b->next, 0, sizeof(unsigned int), st);
   cudaMemsetAsync(b->sync, 0, (size_t)b->count * SYNC_WORDS * 4, st);
   cudaMemsetAsync(b->err, 0, 4, st);
-  k_batch<<<b->grid, BNT, 0, st>>>(a);
+  k_batch<<<b->grid, BNT, BS_SMEM, st>>>(a);
 }
 
 lg_status time_run(lg_batch* b, const BatchArgs& a, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int reps,
@@ -506,8 +830,10 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
   BTRY(cudaMalloc((void**)&dlist, max_items * sizeof(BatchItem) + 16));
   lg_status s = LG_OK;
   for (auto& bin : bins) {
-    if (bin.empty()) continue;
-    std::vector<uint32_t> sample(bin);
+    std::vector<uint32_t> sample;
+    for (uint32_t g : bin)
+      if (b->host[g].n > BS_MAX) sample.push_back(g);
+    if (sample.empty()) continue;  // T plays no part for graphs on the shared-memory path
     std::sort(sample.begin(), sample.end(),
               [&](uint32_t x, uint32_t y) { return b->host[x].arcs > b->host[y].arcs; });
     if (sample.size() > 64) sample.resize(64);
@@ -615,7 +941,8 @@ lg_status batch_create_impl(lg_batch* b, const uint64_t* graph_vptr, cudaStream_
   b->words_A = aw + 4;  // + zero guard
   b->words_O = ow + 4;
   int per_sm = 0, sms = 0;
-  BTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, BNT, 0));
+  BTRY(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
+  BTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, BNT, BS_SMEM));
   BTRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
   b->grid = std::max(1, per_sm) * std::max(1, sms);
   b->tile_arcs = b->opts.tile_arcs ? b->opts.tile_arcs : (1ull << 19);

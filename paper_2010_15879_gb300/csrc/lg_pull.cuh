@@ -25,6 +25,7 @@
 #pragma once
 
 #include "lg_internal.h"
+#include "lg_window.cuh"
 
 namespace lg {
 
@@ -33,10 +34,7 @@ constexpr int PW_WARPS = PW_NT / 32;
 constexpr int PW_SMS = 152;
 constexpr int PW_VPL = 4;                 // vertices per lane of a warp tile
 constexpr uint32_t PW_TV = 32 * PW_VPL;   // vertices of a warp tile, at most
-constexpr int PW_G = 8;                   // groups of 32 fields per window
-constexpr uint32_t PW_WF = 32 * PW_G;     // fields per window
 constexpr uint32_t PW_STAGE = 344;        // stream words a window may need (see window_fields)
-constexpr int PW_E = 8;                   // consecutive fields of a window per lane
 constexpr uint32_t PW_POS_BITS = 26;      // bit positions inside a run of light fields
 constexpr uint32_t PW_POSM = (1u << PW_POS_BITS) - 1u;
 constexpr uint32_t PW_HEAVY_MAX = 4096;   // largest light degree (128 * 4096 fields of <= 38 bits < 2^26 bits)
@@ -64,42 +62,6 @@ struct PrWarp {
   uint32_t info[PW_TV];
   float vsum[PW_TV];
 };
-
-// Asynchronous copy of words [w0, w0 + nw) of the stream into a stage (w0 a
-// multiple of 4, nw <= PW_STAGE), as one group of this thread's copies; the
-// last 16 bytes may run into the stream's guard.  Copies pass the L1 by, whose
-// space the gathers in flight need.
-__device__ __forceinline__ void stage_issue(uint32_t* stage, const uint32_t* A, uint64_t w0, uint32_t nw,
-                                            uint64_t pol) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage) + 16u * lane;
-  const uint32_t* src = A + w0 + 4u * lane;
-#pragma unroll
-  for (int k = 0; k < 3; k++)
-    if (4u * lane + 128u * k < nw)
-      asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst + 512u * k),
-                   "l"(src + 128 * k), "l"(pol)
-                   : "memory");
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-// all but the newest N groups of the warp have landed and every lane sees them
-template <int N>
-__device__ __forceinline__ void stage_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-  __syncwarp();
-}
-
-extern __shared__ __align__(16) unsigned char pw_smem[];
-
-// The 32 bits from bit p on of the CTA's dynamic shared memory: two loads and
-// a funnel shift.
-__device__ __forceinline__ uint32_t sh_bits(uint32_t p) {
-  const uint32_t* a = reinterpret_cast<const uint32_t*>(pw_smem + ((p >> 3) & ~3u));
-  return __funnelshift_r(a[0], a[1], p);
-}
-__device__ __forceinline__ uint32_t sh_bit0(const void* p) {
-  return (uint32_t)(reinterpret_cast<const unsigned char*>(p) - pw_smem) * 8u;
-}
 
 // ---------------------------------------------------------------------------
 // offsets of a warp tile of nv vertices: x[q] = x_v for v = v0 + lane + 32 q,
@@ -196,7 +158,7 @@ __device__ __forceinline__ float pr_item(const GView& g, const HeavyItem& h, con
   };
   auto issue = [&](uint32_t base, uint32_t b) {
     const uint64_t w0 = first_word(base), b1 = origin + (uint64_t)(base + min(wf, f1 - base)) * w;
-    stage_issue(W.stage[b], g.A32, w0, (uint32_t)(((b1 + 31) >> 5) + 1 - w0), G.pstream);
+    stage_issue<3>(W.stage[b], g.A32, w0, (uint32_t)(((b1 + 31) >> 5) + 1 - w0), G.pstream);
   };
   uint32_t carry = h.carry, b = 0;
   float acc = 0.f, comp = 0.f;
@@ -351,7 +313,7 @@ __device__ __forceinline__ int open_window(const GView& g, const LightTile& T, W
     const uint64_t b0 = w.rbit + (uint64_t)(w.f0 - w.fcur) * rw;
     const uint64_t w0 = (b0 >> 5) & ~3ull;
     w.at = sh_bit0(W.stage[b]) + (uint32_t)(b0 - w0 * 32u);
-    stage_issue(W.stage[b], g.A32, w0, (uint32_t)(((b0 + w.nf * rw + 31) >> 5) + 1 - w0), pol);
+    stage_issue<3>(W.stage[b], g.A32, w0, (uint32_t)(((b0 + w.nf * rw + 31) >> 5) + 1 - w0), pol);
   } else {
     const uint64_t rb = w.rbit & ~127ull;
     w.ro = (uint32_t)(rb - T.tb);
@@ -363,7 +325,7 @@ __device__ __forceinline__ int open_window(const GView& g, const LightTile& T, W
     const uint32_t be = ((ib + (w.f0 + w.nf - 1) * wb - w.ro) & PW_POSM) + wb;
     const uint32_t w0 = (bs >> 5) & ~3u;
     w.at = sh_bit0(W.stage[b]) - w0 * 32u;
-    stage_issue(W.stage[b], g.A32, (rb >> 5) + w0, ((be + 31) >> 5) + 1 - w0, pol);
+    stage_issue<3>(W.stage[b], g.A32, (rb >> 5) + w0, ((be + 31) >> 5) + 1 - w0, pol);
   }
   return jn;
 }
@@ -468,39 +430,7 @@ __device__ __forceinline__ void pr_tile(const GView& g, const PrArgs& a, uint64_
 #pragma unroll
       for (int e = 0; e < PW_E; e++) val[e] = k0 + e < cur.nf ? val[e] : 0.f;
     }
-    // sums inside the lane: a vertex between two heads is complete, the part
-    // before the first head belongs to je
-    float run = 0.f, pre = 0.f;
-    if (!__any_sync(LG_FULL_MASK, c > 1)) {
-#pragma unroll
-      for (int e = 0; e < PW_E; e++) {
-        if (hb & ((2u << e) - 1u)) run += val[e];
-        else pre += val[e];
-      }
-      if (!hb) run = pre;
-    } else {
-      int j = je;
-#pragma unroll
-      for (int e = 0; e < PW_E; e++) {
-        const bool head = (hb >> e) & 1u, inner = head && (hb & ((1u << e) - 1u));
-        if (inner) W.vsum[j] = run;
-        pre = head && !inner ? run : pre;
-        j += head;
-        run = (head ? 0.f : run) + val[e];
-      }
-    }
-    const uint32_t before = __ballot_sync(LG_FULL_MASK, hb != 0) & (lt | (1u << lane));
-    const int seg = 31 - __clz((int)(before | 1u));
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const float z = __shfl_up_sync(LG_FULL_MASK, run, o);
-      if ((int)lane - o >= seg) run += z;
-    }
-    if (!before) run += open;
-    float in = __shfl_up_sync(LG_FULL_MASK, run, 1);
-    if (lane == 0) in = open;
-    if (hb && je >= 0) W.vsum[je] = in + pre;
-    open = __shfl_sync(LG_FULL_MASK, run, 31);
+    open = join_window(val, hb, je, open, W.vsum);
     __syncwarp();  // the stage and the heads may be overwritten
   }
   if (lane == 0 && jb >= 0) W.vsum[jb] = open;
@@ -524,8 +454,8 @@ __device__ __forceinline__ void pr_tile(const GView& g, const PrArgs& a, uint64_
 template <int IDM, int OFF, bool TAB>
 __global__ void __launch_bounds__(PW_NT, 1) k_pr_pull(GView g, PrArgs a) {
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  PrWarp& W = reinterpret_cast<PrWarp*>(pw_smem)[wid];
-  float* tab = reinterpret_cast<float*>(pw_smem + PW_WARPS * sizeof(PrWarp));
+  PrWarp& W = reinterpret_cast<PrWarp*>(dyn_smem)[wid];
+  float* tab = reinterpret_cast<float*>(dyn_smem + PW_WARPS * sizeof(PrWarp));
   if (blockIdx.x == 0 && threadIdx.x == 0) a.sync[a.turn ^ 1u] = 0;  // the next iteration's ticket counter
   if (TAB) {
     const float4* src = reinterpret_cast<const float4*>(a.contrib_in);

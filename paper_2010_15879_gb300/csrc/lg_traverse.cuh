@@ -26,6 +26,7 @@
 #include <algorithm>
 
 #include "lg_internal.h"
+#include "lg_window.cuh"
 
 namespace lg {
 
@@ -36,11 +37,6 @@ constexpr int TNT = 256;       // threads per tile CTA
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint64_t udiv_small(uint64_t a, uint32_t b) {
   return a < 0x100000000ull ? (uint64_t)((uint32_t)a / b) : a / b;
-}
-__device__ __forceinline__ uint32_t lane_lt_mask() {
-  uint32_t m;
-  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-  return m;
 }
 
 template <typename M> __device__ __forceinline__ M atomic_or_mask(M* p, M m);
