@@ -55,10 +55,9 @@ __global__ void __launch_bounds__(256) k_sssp_degrees(GView g, const uint32_t* n
                                                       uint64_t* start) {
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
   for (uint64_t q = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < len; q += warps) {
-    uint64_t x0, x1, st;
+    uint64_t st;
     uint32_t d, w;
-    offset_pair<OFF>(g, near[q], x0, x1);
-    vgeo<IDM>(g, x0, x1, st, d, w);
+    vertex_geo<IDM, OFF>(g, near[q], st, d, w);
     if ((threadIdx.x & 31) == 0) {
       eoff[q] = d;
       start[q] = st;

@@ -151,44 +151,58 @@ __device__ __forceinline__ void offset_pair<OFF_ROWPTR>(const GView& g, uint64_t
   x0 = __ldg(g.O + v);
   x1 = __ldg(g.O + v + 1);
 }
-// warp select of ones number v and v+1 (Section 4.1: O_v = select_O(v))
+// Warp select of ones number v and v+1 (Section 4.1: O_v = select_O(v)), from
+// the sample at or below v.  32 words hold the 512 ones of an ordinary sample
+// block; a hub among its vertices spreads it (degree >> l zeros), so later
+// steps take 128 words.
 template <>
 __device__ __forceinline__ void offset_pair<OFF_EF>(const GView& g, uint64_t v, uint64_t& x0, uint64_t& x1) {
-  const int lane = threadIdx.x & 31;
+  const uint32_t lane = threadIdx.x & 31u;
   const uint64_t k = v >> g.sample_log2;
   const uint64_t p0 = __ldg(g.ef_samples + k);
+  const uint64_t lo0 = g.ef_l ? ext64(g.ef_low, v * g.ef_l, g.ef_l) : 0;
+  const uint64_t lo1 = g.ef_l ? ext64(g.ef_low, (v + 1) * g.ef_l, g.ef_l) : 0;
   const uint64_t rem = v - (k << g.sample_log2);
-  uint64_t wbase = p0 >> 5;
   uint64_t carry = 0;
   uint64_t pos[2] = {0, 0};
   uint32_t found = 0;
-  bool first = true;
-  while (found != 3u && wbase < g.ef_high_words32) {
-    const uint64_t wi = wbase + lane;
-    uint32_t w = wi < g.ef_high_words32 ? __ldg(g.ef_high32 + wi) : 0u;
-    if (first && lane == 0) w &= (0xffffffffu << ((uint32_t)p0 & 31u));
-    const uint32_t c = __popc(w);
+  // a lane's words wi .. wi + 3 of the high vector
+  auto step = [&](const uint32_t (&w)[4], uint64_t wi) {
+    const uint32_t c = __popc(w[0]) + __popc(w[1]) + __popc(w[2]) + __popc(w[3]);
     const uint32_t incl = warp_incl_scan<uint32_t>(c);
-    const uint32_t excl = incl - c;
-    const uint32_t total = __shfl_sync(LG_FULL_MASK, incl, 31);
 #pragma unroll
     for (int t = 0; t < 2; t++) {
-      const uint64_t target = rem + t;
-      const bool here = !(found >> t & 1u) && carry + excl <= target && target < carry + incl;
+      const uint64_t at = carry + incl - c;
+      const bool here = !(found >> t & 1u) && at <= rem + t && rem + t < carry + incl;
       const uint32_t b = __ballot_sync(LG_FULL_MASK, here);
-      uint64_t p = here ? wi * 32u + select_in_u32(w, (uint32_t)(target - carry - excl)) : 0;
+      uint64_t p = 0;
+      if (here) {
+        uint32_t r = (uint32_t)(rem + t - at), q = 0, x = w[0];
+#pragma unroll
+        for (int z = 1; z < 4; z++)
+          if (r >= (uint32_t)__popc(x) && q == (uint32_t)(z - 1)) { r -= __popc(x); x = w[z]; q = z; }
+        p = (wi + q) * 32u + select_in_u32(x, r);
+      }
       if (b) {
-        p = __shfl_sync(LG_FULL_MASK, p, __ffs(b) - 1);
-        pos[t] = p;
+        pos[t] = __shfl_sync(LG_FULL_MASK, p, __ffs((int)b) - 1);
         found |= 1u << t;
       }
     }
-    carry += total;
-    wbase += 32;
-    first = false;
+    carry += __shfl_sync(LG_FULL_MASK, incl, 31);
+  };
+  uint64_t wbase = (p0 >> 5) & ~3ull;
+  {
+    const uint64_t wi = wbase + lane;
+    uint32_t w[4] = {wi < g.ef_high_words32 && wi >= (p0 >> 5) ? __ldg(g.ef_high32 + wi) : 0u, 0u, 0u, 0u};
+    if (wi == (p0 >> 5)) w[0] &= 0xffffffffu << ((uint32_t)p0 & 31u);
+    step(w, wi);
   }
-  const uint64_t lo0 = g.ef_l ? ext64(g.ef_low, v * g.ef_l, g.ef_l) : 0;
-  const uint64_t lo1 = g.ef_l ? ext64(g.ef_low, (v + 1) * g.ef_l, g.ef_l) : 0;
+  for (wbase += 32; found != 3u && wbase < g.ef_high_words32; wbase += 128) {
+    const uint64_t wi = wbase + 4u * lane;  // the array is padded to 16 bytes with zeros
+    const uint4 y = wi < g.ef_high_words32 ? ldg128(g.ef_high32 + wi) : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+    step(w, wi);
+  }
   x0 = ((pos[0] - v) << g.ef_l) | lo0;
   x1 = ((pos[1] - (v + 1)) << g.ef_l) | lo1;
 }
@@ -215,6 +229,38 @@ __device__ __forceinline__ void vgeo(const GView& g, uint64_t x0, uint64_t x1, u
     deg = len == g.H ? 0u : (w == 0 ? 1u : 1u + (uint32_t)udiv_small(len - g.H - g.s, w));
     start = x0 + g.H;
   }
+}
+
+// First schedule item of heavy vertex v (a warp; the items are in vertex order).
+__device__ __forceinline__ uint64_t first_item(const GView& g, uint64_t v) {
+  uint64_t lo = 0, hi = g.n_items;  // the first item whose vertex is not below v
+  while (lo < hi) {
+    const uint64_t step = (hi - lo + 31) / 32, at = lo + (threadIdx.x & 31u) * step;
+    const uint32_t c = __popc(__ballot_sync(LG_FULL_MASK, at < hi && (uint64_t)g.items[at].v < v));
+    const uint64_t next = c ? lo + (uint64_t)(c - 1) * step + 1 : lo;
+    hi = min(hi, lo + (uint64_t)c * step);
+    lo = next;
+  }
+  return lo;
+}
+
+// Geometry of one random vertex, by a warp.  In DM order the leading vertices'
+// Elias-Fano blocks are long (their first 512 vertices hold a tenth or more of
+// the arcs, thousands of words to scan: 24 us on R-MAT 2^20), so those are
+// looked up in the schedule, which lists them in order (four steps of 32
+// probes at most).
+template <int IDM, int OFF>
+__device__ __forceinline__ void vertex_geo(const GView& g, uint64_t v, uint64_t& start, uint32_t& d, uint32_t& w) {
+  if (OFF == OFF_EF && v < g.heavy_prefix) {
+    const HeavyItem* h = g.items + first_item(g, v);
+    start = h->bit;
+    d = h->deg;
+    w = h->w;
+    return;
+  }
+  uint64_t x0, x1;
+  offset_pair<OFF>(g, v, x0, x1);
+  vgeo<IDM>(g, x0, x1, start, d, w);
 }
 
 // sequential decoder for one neighborhood (light path)
@@ -527,6 +573,7 @@ __global__ void __launch_bounds__(TNT, 4) k_ppr_pull(GView g, PprArgs a) {
   }
   const uint64_t v0 = (uint64_t)(blockIdx.x - hb) * TV;
   const int cnt = (int)min((uint64_t)TV, g.n - v0);
+  if (v0 + cnt <= g.heavy_prefix) return;  // all in the schedule
   tile_offsets<OFF>(g, v0, cnt, sm.xs, sm.ts);
   __syncthreads();
   tile_classify<IDM>(g, sm, cnt, [](int) { return true; });
@@ -628,10 +675,9 @@ __global__ void __launch_bounds__(TNT, 4) k_ppr_pull(GView g, PprArgs a) {
 // whole sweep, or the array is fresh); r_0 = e_src gives cin[src] = 1 / d_src
 template <int IDM, int OFF>
 __global__ void __launch_bounds__(32) k_ppr_join(GView g, float* cin, uint32_t slot, uint32_t src) {
-  uint64_t x0, x1, start;
+  uint64_t start;
   uint32_t d, w;
-  offset_pair<OFF>(g, src, x0, x1);
-  vgeo<IDM>(g, x0, x1, start, d, w);
+  vertex_geo<IDM, OFF>(g, src, start, d, w);
   if (threadIdx.x == 0) cin[(uint64_t)src * PPR_K + slot] = d ? 1.0f / (float)d : 0.0f;
 }
 
@@ -703,6 +749,7 @@ __global__ void __launch_bounds__(TNT, IDM == ID_LOCAL_GAP ? 6 : 5) k_bfs_pull(G
   if (threadIdx.x == 0) { qn = 0; newpairs = 0; }
   const uint64_t v0 = (uint64_t)(blockIdx.x - hb) * TV;
   const int cnt = (int)min((uint64_t)TV, g.n - v0);
+  if (v0 + cnt <= g.heavy_prefix) return;  // all in the schedule
   for (int i = threadIdx.x; i < cnt; i += TNT) need_sm[i] = (M)(all & (M)~vis[v0 + i]);
   tile_offsets<OFF>(g, v0, cnt, sm.xs, sm.ts);
   __syncthreads();
@@ -865,6 +912,7 @@ __global__ void __launch_bounds__(256) k_bfs_push(GView g, BfsArgs a, unsigned h
     for (uint64_t q = (uint64_t)(blockIdx.x - hb) * (blockDim.x >> 5) + (threadIdx.x >> 5); q < a.queue_in_len;
          q += warps) {
       const uint32_t v = a.queue_in[q];
+      if (v < g.heavy_prefix) continue;  // in the heavy schedule
       const M m = fin[v];
       uint64_t x0, x1, start;
       uint32_t d, w;
@@ -892,10 +940,9 @@ __global__ void __launch_bounds__(256) k_nbr_degrees(GView g, NbrArgs a) {
       continue;
     }
     const uint64_t v = g.perm ? (uint64_t)g.perm[vo] : vo;
-    uint64_t x0, x1, start;
+    uint64_t start;
     uint32_t d, w;
-    offset_pair<OFF>(g, v, x0, x1);
-    vgeo<IDM>(g, x0, x1, start, d, w);
+    vertex_geo<IDM, OFF>(g, v, start, d, w);
     if (lane == 0) a.out_offsets[q] = d;
   }
 }
@@ -908,10 +955,9 @@ __global__ void __launch_bounds__(256) k_nbr_decode(GView g, NbrArgs a) {
     const uint32_t vo = a.vertices[q];
     if (vo >= g.n) continue;
     const uint64_t v = g.perm ? (uint64_t)g.perm[vo] : vo;
-    uint64_t x0, x1, start;
+    uint64_t start;
     uint32_t d, w;
-    offset_pair<OFF>(g, v, x0, x1);
-    vgeo<IDM>(g, x0, x1, start, d, w);
+    vertex_geo<IDM, OFF>(g, v, start, d, w);
     const uint64_t o = a.out_offsets[q];
     uint32_t carry = 0;
     for (uint32_t base = 0; base < d; base += 64) {
