@@ -545,9 +545,11 @@ extern "C" lg_status lg_arrays_get(const lg_graph* g, lg_arrays* out) {
   return LG_OK;
 }
 
-// Heavy-vertex schedule, derived from the encoded arrays: every vertex of
-// degree > heavy_min becomes ceil(d / HEAVY_SEG) items, listed in vertex order.
-static lg_status build_schedule(lg_graph* g, cudaStream_t st) {
+// Heavy-vertex schedule, derived from the encoded A and the plain offsets x_0 ..
+// x_n (decoding them again cost 1.5 ms at R-MAT 2^26: the hubs' Elias-Fano
+// block is 200,000 words long): every vertex of degree > heavy_min becomes
+// ceil(d / HEAVY_SEG) items, listed in vertex order.
+static lg_status build_schedule(lg_graph* g, const uint64_t* x, cudaStream_t st) {
   g->heavy_min = heavy_min_env();
   g->heavy_seg = heavy_seg_env();
   const uint64_t ntiles = (g->n + LG_TILE_V - 1) / LG_TILE_V;
@@ -569,6 +571,7 @@ static lg_status build_schedule(lg_graph* g, cudaStream_t st) {
   p.top = t_mid.as<unsigned long long>();
   p.mid = reinterpret_cast<uint32_t*>(p.top + 1);
   GView v = make_view(g);
+  v.O = x;
   const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
   LG_TRY(ops->plan_count(v, p, st));
   LG_TRY(scan_excl_u32(p.tile_count, ntiles, t_off.as<uint64_t>(), t_stmp.as<uint64_t>(), st));
@@ -672,8 +675,7 @@ static lg_status encode_impl(lg_graph* g, const uint64_t* row_ptr, const uint32_
       if (arcs) LG_TRY(cudaMemcpyAsync(g->W, wt, arcs * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st));
     }
     g->off_mode = OFF_ROWPTR;
-    LG_TRY(cudaStreamSynchronize(st));
-    return build_schedule(g, st);
+    return build_schedule(g, rp, st);
   }
 
   // ---- A stream
@@ -691,7 +693,15 @@ static lg_status encode_impl(lg_graph* g, const uint64_t* row_ptr, const uint32_
     LG_TRY(t_len.alloc(n * sizeof(uint64_t)));
     LG_TRY(t_x.alloc((n + 1) * sizeof(uint64_t)));
     LG_TRY(t_stmp.alloc(scan_tmp_words(n) * sizeof(uint64_t)));
-    LG_TRY(enc_local_lengths(rp, cl, n, gap, g->s, g->H, t_wid.as<uint8_t>(), t_len.as<uint64_t>(), st));
+    Tmp t_long(st);
+    LongRows rows, *L = nullptr;
+    if (g->max_degree > LONG_ROW) {
+      LG_TRY(t_long.alloc(long_rows_bytes(arcs)));
+      rows = long_rows(t_long.p, arcs);
+      L = &rows;
+      LG_TRY(enc_long_rows(rp, n, gap, rows, st));
+    }
+    LG_TRY(enc_local_lengths(rp, cl, n, gap, g->s, g->H, t_wid.as<uint8_t>(), t_len.as<uint64_t>(), L, st));
     LG_TRY(scan_excl_u64(t_len.as<uint64_t>(), n, t_x.as<uint64_t>(), t_stmp.as<uint64_t>(), st));
     LG_TRY(cudaMemcpyAsync(&U, t_x.as<uint64_t>() + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     LG_TRY(cudaStreamSynchronize(st));
@@ -699,7 +709,7 @@ static lg_status encode_impl(lg_graph* g, const uint64_t* row_ptr, const uint32_
     g->words_A = padded_words(g->bits_A);
     LG_TRY(alloc_words(&g->A, g->words_A, st));
     LG_TRY(enc_pack_local(rp, cl, t_x.as<uint64_t>(), t_wid.as<uint8_t>(), n, gap, g->s, g->H, g->A,
-                          (g->bits_A + 63) / 64, st));
+                          (g->bits_A + 63) / 64, L, st));
     xsrc = t_x.as<uint64_t>();
   }
 
@@ -729,8 +739,7 @@ static lg_status encode_impl(lg_graph* g, const uint64_t* row_ptr, const uint32_
     LG_TRY(enc_ef_samples(xsrc, N, g->ef_l, g->sample, g->ef_samples, g->n_samples, st));
     g->bits_O = g->ef_low_bits + g->ef_high_bits + 64 * g->n_samples;
   }
-  LG_TRY(cudaStreamSynchronize(st));
-  return build_schedule(g, st);
+  return build_schedule(g, xsrc, st);
 }
 
 extern "C" lg_status lg_encode(const uint64_t* row_ptr, const uint32_t* col, const uint32_t* weights, uint64_t n,

@@ -242,8 +242,76 @@ cudaError_t enc_check_symmetric(const uint64_t* rp, const uint32_t* col, uint64_
 // a row's width is that of its last (largest) ID.  Gaps: when the 32 rows hold
 // at most LL_STAGE arcs (contiguous in col) the warp copies them to shared
 // memory with coalesced loads and each lane scans its own row there; warps
-// with a longer row (near the hubs) reduce row by row over the warp.
+// with a longer row reduce row by row over the warp.
+//
+// Rows of more than LONG_ROW arcs would leave a hub, or 32 rows of hundreds of
+// arcs, to one warp, so they are listed in windows of LONG_WINDOW fields first
+// and a warp takes a window, here and in the packing below (community graph of
+// 1.5 M vertices: this pass 83 us, the packing 135; 486 and 904 with every
+// row left to its warp, 157 and 248 with only rows above 1,024 listed).
 constexpr int LL_STAGE = 1024;
+
+// fields of a row that windows count: gaps, or IDs
+__device__ __forceinline__ uint64_t row_fields(uint64_t d, int gap) { return gap ? d - 1 : d; }
+
+__global__ void __launch_bounds__(256) k_long_list(const uint64_t* __restrict__ rp, uint64_t n, int gap, LongRows L) {
+  for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t d = rp[v + 1] - rp[v];
+    if (d <= LONG_ROW) continue;
+    const uint32_t nw = (uint32_t)((row_fields(d, gap) + LONG_WINDOW - 1) / LONG_WINDOW);
+    const uint32_t slot = atomicAdd(L.counts + 1, 1u), at = atomicAdd(L.counts, nw);
+    L.rows[slot] = (uint32_t)v;
+    L.gmax[slot] = 0;
+    for (uint32_t k = 0; k < nw; k++) L.windows[at + k] = make_uint2(slot, k);
+  }
+}
+
+// largest gap of each window
+__global__ void __launch_bounds__(256) k_long_gaps(const uint64_t* __restrict__ rp, const uint32_t* __restrict__ col,
+                                                   LongRows L) {
+  const uint32_t lane = threadIdx.x & 31u, nw = L.counts[0];
+  for (uint32_t i = blockIdx.x * 8 + (threadIdx.x >> 5); i < nw; i += gridDim.x * 8) {
+    const uint2 e = L.windows[i];
+    const uint32_t v = L.rows[e.x];
+    const uint64_t lo = rp[v] + (uint64_t)e.y * LONG_WINDOW;
+    const uint32_t cnt = (uint32_t)min((uint64_t)LONG_WINDOW, rp[v + 1] - 1 - lo);
+    uint32_t mg = 0;
+#pragma unroll 8
+    for (uint32_t q = lane; q < cnt; q += 32) mg = max(mg, col[lo + q + 1] - col[lo + q]);
+    mg = __reduce_max_sync(LG_FULL_MASK, mg);
+    if (lane == 0) atomicMax(L.gmax + e.x, mg);
+  }
+}
+__global__ void k_long_lengths(const uint64_t* __restrict__ rp, uint32_t s, uint32_t H, uint8_t* __restrict__ wid,
+                               uint64_t* __restrict__ len, LongRows L) {
+  const uint32_t ns = L.counts[1];
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < ns; i += gridDim.x * blockDim.x) {
+    const uint32_t v = L.rows[i], w = max(1u, bits_u32(L.gmax[i]));
+    wid[v] = (uint8_t)w;
+    len[v] = (uint64_t)H + s + (rp[v + 1] - rp[v] - 1) * (uint64_t)w;
+  }
+}
+
+uint64_t long_rows_bytes(uint64_t arcs) {  // counts, rows and gmax per row, windows
+  const uint64_t rows = arcs / LONG_ROW + 1;
+  return 32 + rows * 8 + (rows + arcs / LONG_WINDOW + 1) * sizeof(uint2);
+}
+LongRows long_rows(void* mem, uint64_t arcs) {
+  const uint64_t rows = arcs / LONG_ROW + 1;  // a listed row has more than LONG_ROW arcs
+  LongRows L;
+  L.counts = reinterpret_cast<uint32_t*>(mem);
+  L.windows = reinterpret_cast<uint2*>(L.counts + 4);
+  L.rows = reinterpret_cast<uint32_t*>(L.windows + rows + arcs / LONG_WINDOW + 1);
+  L.gmax = L.rows + rows;
+  return L;
+}
+cudaError_t enc_long_rows(const uint64_t* rp, uint64_t n, int gap, const LongRows& L, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(L.counts, 0, 16, st);
+  if (e != cudaSuccess) return e;
+  k_long_list<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(rp, n, gap, L);
+  count_launch();
+  return cudaGetLastError();
+}
 __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restrict__ rp,
                                                        const uint32_t* __restrict__ col, uint64_t n, int gap,
                                                        uint32_t s, uint32_t H, uint8_t* __restrict__ wid,
@@ -281,7 +349,7 @@ __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restric
       } else {
         for (int r = 0; r < rows; r++) {
           const uint64_t lo = __shfl_sync(LG_FULL_MASK, mlo, r), hi = __shfl_sync(LG_FULL_MASK, mhi, r);
-          if (hi - lo < 2) continue;
+          if (hi - lo < 2 || hi - lo > LONG_ROW) continue;  // long rows: k_long_gaps
           uint32_t mg = 0;
           for (uint64_t j = lo + 1 + lane; j < hi; j += 32) mg = max(mg, col[j] - col[j - 1]);
           mg = __reduce_max_sync(LG_FULL_MASK, mg);
@@ -289,7 +357,7 @@ __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restric
         }
       }
     }
-    if (lane < rows) {
+    if (lane < rows && !(gap && mhi - mlo > LONG_ROW)) {
       const uint64_t d = mhi - mlo;
       wid[mv] = (uint8_t)mw;
       len[mv] = gap ? (uint64_t)H + (d >= 1 ? s : 0) + (d >= 2 ? (d - 1) * (uint64_t)mw : 0)
@@ -299,9 +367,15 @@ __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restric
 }
 
 cudaError_t enc_local_lengths(const uint64_t* rp, const uint32_t* col, uint64_t n, int gap, uint32_t s, uint32_t H,
-                              uint8_t* wid, uint64_t* len, cudaStream_t st) {
+                              uint8_t* wid, uint64_t* len, const LongRows* L, cudaStream_t st) {
   k_local_lengths<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(rp, col, n, gap, s, H, wid, len);
   count_launch();
+  if (gap && L) {
+    k_long_gaps<<<152 * 8, 256, 0, st>>>(rp, col, *L);
+    count_launch();
+    k_long_lengths<<<152, 256, 0, st>>>(rp, s, H, wid, len, *L);
+    count_launch();
+  }
   return cudaGetLastError();
 }
 
@@ -402,8 +476,9 @@ cudaError_t enc_pack_u64(const uint64_t* vals, uint64_t count, uint32_t w, uint6
 // most PK_ARCS arcs, their arcs are staged in shared memory with coalesced
 // loads and each lane emits its row's record into a shared copy of the
 // group's bit range (shared atomicOr, as neighbouring records share words).
-// Otherwise the warp packs the rows one at a time, in windows of up to
-// PK_ARCS fields, a lane per field.  Either way the warp then writes the bit
+// Otherwise the warp packs the rows one at a time, a lane per field; rows of
+// more than LONG_ROW arcs are left to k_pack_long, a warp per window of
+// LONG_WINDOW fields.  Either way the warp then writes the bit
 // range out coalesced: its inner 64-bit words are its own, its first and last
 // word may be shared with the neighbouring range and are OR-ed into A (zeroed
 // at allocation).
@@ -413,6 +488,7 @@ constexpr int PK_ARCS = 1024;
 constexpr int PK_STAGE = PK_ARCS + 8;  // a window's fields, plus the ID before them (gaps)
 constexpr int PK_W32 = 1104;           // >= 2 * ceil((PK_ARCS * 32 + PK_ROWS * 64 + 63) / 64), even
 constexpr int PK_WARPS = 4;
+static_assert(LONG_WINDOW == (uint32_t)PK_ARCS && LONG_ROW <= (uint32_t)PK_ARCS, "a window of a long row is one packing window");
 
 __device__ __forceinline__ void pk_emit(uint32_t* ob, uint64_t p, uint32_t w, uint32_t val) {
   if (w == 0) return;
@@ -437,6 +513,37 @@ __device__ __forceinline__ void pk_flush(const uint32_t* ob, uint64_t b0, uint64
 __device__ __forceinline__ void pk_clear(uint32_t* ob, uint64_t b0, uint64_t b1, int lane) {
   const uint32_t n32 = 2 * (uint32_t)((b1 - (b0 & ~63ull) + 63) >> 6);
   for (uint32_t q = lane; q < n32; q += 32) ob[q] = 0;
+}
+
+// Window of up to PK_ARCS data fields from field k0 on (gaps, or IDs) of the row
+// at col[lo .. lo + d), whose record is bits [rb, re) of out; the window of field
+// 0 has the header (and the first ID) too.
+template <bool GAP>
+__device__ __forceinline__ void pk_window(const uint32_t* __restrict__ col, uint64_t lo, uint64_t d, uint64_t rb,
+                                          uint64_t re, uint32_t w, uint64_t k0, uint32_t s, uint32_t H, uint32_t* stg,
+                                          uint32_t* ob, uint64_t* __restrict__ out, int lane) {
+  const uint64_t f0 = rb + H + (GAP && d >= 1 ? s : 0);  // bit of data field 0
+  const uint64_t nf = GAP ? (d >= 1 ? d - 1 : 0) : d;    // data fields
+  const uint32_t kn = (uint32_t)min((uint64_t)PK_ARCS, nf - min(nf, k0));
+  const uint64_t b0 = k0 == 0 ? rb : f0 + k0 * w;
+  const uint64_t b1 = k0 + kn >= nf ? re : f0 + (k0 + kn) * w;
+  const uint64_t base = b0 & ~63ull;
+  // staged IDs: the window's fields, plus the ID before the first gap
+  const uint32_t ns = GAP ? (d >= 1 ? kn + 1u : 0u) : kn;
+  for (uint32_t q = lane; q < ns; q += 32) stg[q] = col[lo + k0 + q];
+  pk_clear(ob, b0, b1, lane);
+  __syncwarp();
+  if (k0 == 0 && lane == 0) {
+    pk_emit(ob, rb - base, H, w);
+    if (GAP && d >= 1) pk_emit(ob, rb + H - base, s, stg[0]);
+  }
+  for (uint32_t q = lane; q < kn; q += 32) {
+    const uint32_t val = GAP ? stg[q + 1] - stg[q] : stg[q];
+    pk_emit(ob, f0 + (k0 + q) * w - base, w, val);
+  }
+  __syncwarp();
+  pk_flush(ob, b0, b1, out, lane);
+  __syncwarp();
 }
 
 template <bool GAP>
@@ -504,48 +611,46 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pack_local(const uint64_t* __
       __syncwarp();
       continue;
     }
-    // long rows present: one row at a time, windows of up to PK_ARCS fields
+    // more arcs than a window holds: one row at a time
     for (int r = 0; r < rows; r++) {
       const uint64_t lo = __shfl_sync(LG_FULL_MASK, mlo, r), hi = __shfl_sync(LG_FULL_MASK, mhi, r);
       const uint64_t rb = __shfl_sync(LG_FULL_MASK, xb, r), re = __shfl_sync(LG_FULL_MASK, xe, r);
       const uint32_t w = __shfl_sync(LG_FULL_MASK, wv, r);
-      const uint64_t d = hi - lo;
-      const uint64_t f0 = rb + H + (GAP && d >= 1 ? s : 0);  // bit of data field 0
-      const uint64_t nf = GAP ? (d >= 1 ? d - 1 : 0) : d;    // data fields
-      // data field k: gaps col[lo+k+1] - col[lo+k], or IDs col[lo+k]
-      for (uint64_t k0 = 0; k0 == 0 || k0 < nf; k0 += PK_ARCS) {
-        const uint32_t kn = (uint32_t)min((uint64_t)PK_ARCS, nf - min(nf, k0));
-        const uint64_t b0 = k0 == 0 ? rb : f0 + k0 * w;
-        const uint64_t b1 = k0 + kn >= nf ? re : f0 + (k0 + kn) * w;
-        const uint64_t base = b0 & ~63ull;
-        // staged IDs: the window's fields, plus the ID before the first gap
-        const uint32_t ns = GAP ? (d >= 1 ? kn + 1u : 0u) : kn;
-        for (uint32_t q = lane; q < ns; q += 32) stg[q] = col[lo + k0 + q];
-        pk_clear(ob, b0, b1, lane);
-        __syncwarp();
-        if (k0 == 0 && lane == 0) {
-          pk_emit(ob, rb - base, H, w);
-          if (GAP && d >= 1) pk_emit(ob, rb + H - base, s, stg[0]);
-        }
-        for (uint32_t q = lane; q < kn; q += 32) {
-          const uint32_t val = GAP ? stg[q + 1] - stg[q] : stg[q];
-          pk_emit(ob, f0 + (k0 + q) * w - base, w, val);
-        }
-        __syncwarp();
-        pk_flush(ob, b0, b1, out, lane);
-        __syncwarp();
-      }
+      if (hi - lo <= LONG_ROW) pk_window<GAP>(col, lo, hi - lo, rb, re, w, 0, s, H, stg, ob, out, lane);
     }
   }
 }
 
+template <bool GAP>
+__global__ void __launch_bounds__(PK_WARPS * 32) k_pack_long(const uint64_t* __restrict__ rp,
+                                                            const uint32_t* __restrict__ col,
+                                                            const uint64_t* __restrict__ x,
+                                                            const uint8_t* __restrict__ wid, uint32_t s, uint32_t H,
+                                                            uint64_t* __restrict__ out, LongRows L) {
+  __shared__ uint32_t stg_all[PK_WARPS][PK_STAGE];
+  __shared__ uint32_t ob_all[PK_WARPS][PK_W32];
+  const uint32_t nw = L.counts[0];
+  for (uint32_t i = blockIdx.x * PK_WARPS + (threadIdx.x >> 5); i < nw; i += gridDim.x * PK_WARPS) {
+    const uint2 e = L.windows[i];
+    const uint32_t v = L.rows[e.x];
+    pk_window<GAP>(col, rp[v], rp[v + 1] - rp[v], x[v], x[v + 1], wid[v], (uint64_t)e.y * LONG_WINDOW, s, H,
+                   stg_all[threadIdx.x >> 5], ob_all[threadIdx.x >> 5], out, threadIdx.x & 31);
+  }
+}
+
 cudaError_t enc_pack_local(const uint64_t* rp, const uint32_t* col, const uint64_t* x, const uint8_t* wid, uint64_t n,
-                           int gap, uint32_t s, uint32_t H, uint64_t* out, uint64_t data_words, cudaStream_t st) {
+                           int gap, uint32_t s, uint32_t H, uint64_t* out, uint64_t data_words, const LongRows* L,
+                           cudaStream_t st) {
   if (data_words == 0 || n == 0) return cudaSuccess;
   const unsigned grid = grid_for((n + PK_ROWS - 1) / PK_ROWS, PK_WARPS, 152 * 16);
   if (gap) k_pack_local<true><<<grid, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, n, s, H, out);
   else k_pack_local<false><<<grid, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, n, s, H, out);
   count_launch();
+  if (L) {
+    if (gap) k_pack_long<true><<<152 * 6, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, s, H, out, *L);
+    else k_pack_long<false><<<152 * 6, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, s, H, out, *L);
+    count_launch();
+  }
   return cudaGetLastError();
 }
 

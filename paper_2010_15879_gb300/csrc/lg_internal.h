@@ -99,13 +99,27 @@ cudaError_t enc_check_symmetric(const uint64_t* rp, const uint32_t* col, uint64_
 cudaError_t enc_dm_relabel(const uint64_t* rp, const uint32_t* col, const uint32_t* w, uint64_t n,
                            uint64_t arcs, uint64_t max_deg, uint32_t mode, uint32_t* perm, uint32_t* inv_perm,
                            uint64_t* nrp, uint32_t* ncol, uint32_t* nw, cudaStream_t st);
+// Rows of more than LONG_ROW arcs, listed for the local widths and packing in
+// windows of LONG_WINDOW fields (one long_rows_bytes(arcs) block; only needed if
+// such rows exist).
+constexpr uint32_t LONG_ROW = 256, LONG_WINDOW = 1024;
+struct LongRows {
+  uint32_t* counts;  // [0] windows, [1] rows
+  uint2* windows;    // (index in rows, window of the row)
+  uint32_t* rows;    // vertices
+  uint32_t* gmax;    // largest gap per row
+};
+uint64_t long_rows_bytes(uint64_t arcs);
+LongRows long_rows(void* mem, uint64_t arcs);
+cudaError_t enc_long_rows(const uint64_t* rp, uint64_t n, int gap, const LongRows& L, cudaStream_t st);
+// L: the listed rows, or null if no row is that long
 cudaError_t enc_local_lengths(const uint64_t* rp, const uint32_t* col, uint64_t n, int gap, uint32_t s,
-                              uint32_t H, uint8_t* wid, uint64_t* len, cudaStream_t st);
+                              uint32_t H, uint8_t* wid, uint64_t* len, const LongRows* L, cudaStream_t st);
 cudaError_t enc_pack_global(const uint32_t* col, const uint32_t* w, uint64_t arcs, uint32_t s,
                             uint32_t omega, uint64_t* out, uint64_t data_words, cudaStream_t st);
 cudaError_t enc_pack_local(const uint64_t* rp, const uint32_t* col, const uint64_t* x, const uint8_t* wid,
                            uint64_t n, int gap, uint32_t s, uint32_t H, uint64_t* out, uint64_t data_words,
-                           cudaStream_t st);
+                           const LongRows* L, cudaStream_t st);
 cudaError_t enc_pack_u64(const uint64_t* vals, uint64_t count, uint32_t w, uint64_t* out,
                          uint64_t data_words, cudaStream_t st);
 cudaError_t enc_ef_high(const uint64_t* x, uint64_t N, uint32_t l, uint64_t* out, cudaStream_t st);

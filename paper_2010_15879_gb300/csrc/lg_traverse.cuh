@@ -1650,7 +1650,8 @@ const TravOps* make_ops() {
   static const TravOps ops = {
       &launch_pr_init<IDM, OFF>,    &launch_pr_pull<IDM, OFF>,     &launch_bfs_pull<IDM, OFF>,
       &launch_bfs_push<IDM, OFF>,   &launch_nbr_degrees<IDM, OFF>, &launch_nbr_decode<IDM, OFF>,
-      &launch_plan_count<IDM, OFF>, &launch_plan_fill<IDM, OFF>,   &launch_plan_carry<IDM, OFF>,
+      // the schedule is built while the offsets are still at hand in plain form (GView::O)
+      &launch_plan_count<IDM, OFF_ROWPTR>, &launch_plan_fill<IDM, OFF_ROWPTR>, &launch_plan_carry<IDM, OFF>,
       &launch_ppr_pull<IDM, OFF>,   &launch_ppr_join<IDM, OFF>,   &launch_dec_all<IDM, OFF>,
   };
   return &ops;
