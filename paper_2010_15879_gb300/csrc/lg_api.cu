@@ -184,6 +184,7 @@ GView make_view(const lg_graph* g) {
   v.heavy_min = g->heavy_min;
   v.heavy_seg = g->heavy_seg;
   v.heavy_prefix = g->heavy_prefix;
+  v.mid_prefix = g->mid_prefix;
   return v;
 }
 
@@ -206,30 +207,6 @@ cudaError_t ppr_finish_multi(const GView& g, const PprArgs& a, cudaStream_t st) 
   if (g.n_multi == 0) return cudaSuccess;
   k_ppr_finish_multi<<<grid_for(g.n_multi, 256, 4096), 256, 0, st>>>(g, a);
   count_launch();
-  return cudaGetLastError();
-}
-
-template <typename M>
-__global__ void k_bfs_finish_multi(GView g, BfsArgs a) {
-  M* hacc = reinterpret_cast<M*>(a.hacc);
-  const M* vis = reinterpret_cast<const M*>(a.vis);
-  M* fout = reinterpret_cast<M*>(a.front_out);
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < g.n_multi; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t v = g.items[g.multi[i]].v;
-    const M need = (M)((M)a.all_mask & (M)~vis[v]);
-    const M acc = hacc[i];
-    hacc[i] = 0;
-    if (need == 0) fout[v] = 0;
-    else bfs_finish<M>(g, a, v, need, acc, nullptr, nullptr, nullptr);
-  }
-}
-
-cudaError_t bfs_finish_multi(const GView& g, const BfsArgs& a, int mb, cudaStream_t st) {
-  if (g.n_multi == 0) return cudaSuccess;
-  const unsigned grid = grid_for(g.n_multi, 256, 4096);
-  if (mb == 2) { k_bfs_finish_multi<uint16_t><<<grid, 256, 0, st>>>(g, a); count_launch(); }
-  else if (mb == 4) { k_bfs_finish_multi<uint32_t><<<grid, 256, 0, st>>>(g, a); count_launch(); }
-  else { k_bfs_finish_multi<uint64_t><<<grid, 256, 0, st>>>(g, a); count_launch(); }
   return cudaGetLastError();
 }
 
@@ -262,30 +239,25 @@ const TravOps* trav_ops(int id_mode, int off_mode) {
 }
 
 // ---------------------------------------------------------------- small kernels
-// Sources are few (<= 64 per sweep): one thread seeds them in order, so
-// duplicates merge into one frontier entry.
+// Start of a sweep: a thread per source (at most 64) checks and maps it, sets
+// its bit in the masks and queues its vertex once.  Nothing but scratch is
+// written, so a bad source leaves the caller's arrays as they were.
 template <typename M>
-__global__ void k_bfs_seed(M* vis, M* front, uint32_t* depth, uint64_t n, const uint32_t* src, uint32_t S,
-                           uint32_t vmajor, uint32_t* queue, uint32_t* counters) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  uint32_t q = 0;
-  for (uint32_t i = 0; i < S; i++) {
-    const uint32_t v = src[i];
-    const M bit = (M)((M)1 << i);
-    if (front[v] == 0) queue[q++] = v;
-    front[v] = (M)(front[v] | bit);
-    vis[v] = (M)(vis[v] | bit);
-    depth[vmajor ? (uint64_t)v * S + i : (uint64_t)i * n + v] = 0;
-  }
-  counters[0] = q;
+__global__ void __launch_bounds__(64) k_bfs_start(M* vis, M* front, uint64_t n, const uint32_t* src,
+                                                  const uint32_t* perm, uint32_t S, uint32_t* stored, uint32_t* queue,
+                                                  uint32_t* count, int* err) {
+  const uint32_t i = threadIdx.x;
+  if (i >= S) return;
+  if (src[i] >= n) { set_err(err, DERR_QUERY); return; }
+  const uint32_t v = perm ? perm[src[i]] : src[i];
+  const M bit = (M)((M)1 << i);
+  stored[i] = v;
+  atomic_or_mask<M>(vis + v, bit);
+  if (atomic_or_mask<M>(front + v, bit) == 0) queue[atomicAdd(count, 1u)] = v;
 }
-
-cudaError_t bfs_seed(void* vis, void* front, uint32_t* depth, uint64_t n, const uint32_t* src, uint32_t S,
-                     uint32_t vmajor, int mb, uint32_t* queue, uint32_t* counters, cudaStream_t st) {
-  if (mb == 2) { k_bfs_seed<uint16_t><<<1, 32, 0, st>>>((uint16_t*)vis, (uint16_t*)front, depth, n, src, S, vmajor, queue, counters); count_launch(); }
-  else if (mb == 4) { k_bfs_seed<uint32_t><<<1, 32, 0, st>>>((uint32_t*)vis, (uint32_t*)front, depth, n, src, S, vmajor, queue, counters); count_launch(); }
-  else { k_bfs_seed<uint64_t><<<1, 32, 0, st>>>((uint64_t*)vis, (uint64_t*)front, depth, n, src, S, vmajor, queue, counters); count_launch(); }
-  return cudaGetLastError();
+__global__ void k_bfs_depth0(uint32_t* depth, uint64_t n, const uint32_t* stored, uint32_t S, uint32_t vmajor) {
+  const uint32_t i = threadIdx.x;
+  if (i < S) depth[vmajor ? (uint64_t)stored[i] * S + i : (uint64_t)i * n + stored[i]] = 0;
 }
 
 // zero the mask entries listed in a queue (the nonzeros of a frontier)
@@ -828,25 +800,33 @@ extern "C" lg_status lg_bfs(const lg_graph* g, const uint32_t* sources, uint32_t
   const uint64_t n = g->n;
   const uint32_t maxb = S >= 64 ? 64 : S;
   const int mb = maxb <= 16 ? 2 : (maxb <= 32 ? 4 : 8);
-  Tmp t_src(st), t_vis(st), t_fa(st), t_fb(st), t_qa(st), t_qb(st), t_small(st), t_depth(st), t_hacc(st);
-  LG_TRY(t_src.alloc(S * sizeof(uint32_t)));
+  constexpr uint32_t RING = 64;  // levels whose counters are zeroed together
+  Tmp t_vis(st), t_fa(st), t_fb(st), t_qa(st), t_qb(st), t_small(st), t_depth(st), t_hacc(st);
   LG_TRY(t_vis.alloc(n * mb + 16));
   LG_TRY(t_fa.alloc(n * mb + 16));
   LG_TRY(t_fb.alloc(n * mb + 16));
   LG_TRY(t_qa.alloc(n * sizeof(uint32_t)));
   LG_TRY(t_qb.alloc(n * sizeof(uint32_t)));
-  LG_TRY(t_small.alloc(64));
+  // error and start count, stored sources, counters of RING levels
+  const size_t small_bytes = 16 + 64 * sizeof(uint32_t) + RING * 8;
+  LG_TRY(t_small.alloc(small_bytes));
   if (g->relabel) LG_TRY(t_depth.alloc((uint64_t)maxb * n * sizeof(uint32_t)));
-  LG_TRY(t_hacc.alloc(g->n_multi * mb + 16));
-  LG_TRY(cudaMemsetAsync(t_hacc.p, 0, g->n_multi * mb + 16, st));
+  const size_t hacc_bytes = (g->n_multi * mb + 15) / 16 * 16;
+  LG_TRY(t_hacc.alloc(hacc_bytes + g->n_multi * sizeof(uint32_t)));
+  LG_TRY(cudaMemsetAsync(t_hacc.p, 0, hacc_bytes + g->n_multi * sizeof(uint32_t), st));
   int* d_err = t_small.as<int>();
-  uint32_t* counters = reinterpret_cast<uint32_t*>(t_small.as<char>() + 16);
-  LG_TRY(cudaMemsetAsync(t_small.p, 0, 64, st));
-  LG_TRY(map_ids(sources, t_src.as<uint32_t>(), g->perm, S, n, d_err, st));
-  int herr = 0;
-  LG_TRY(cudaMemcpyAsync(&herr, d_err, 4, cudaMemcpyDeviceToHost, st));
-  LG_TRY(cudaStreamSynchronize(st));
-  if (herr) return describe_dev_err(herr);
+  uint32_t* stored = t_small.as<uint32_t>() + 4;
+  uint32_t* ring = stored + 64;
+  if (S > 64) {  // every source is checked before the first sweep writes its depths
+    Tmp t_src(st);
+    LG_TRY(t_src.alloc(S * sizeof(uint32_t)));
+    LG_TRY(cudaMemsetAsync(t_small.p, 0, 16, st));
+    LG_TRY(map_ids(sources, t_src.as<uint32_t>(), g->perm, S, n, d_err, st));
+    int herr = 0;
+    LG_TRY(cudaMemcpyAsync(&herr, d_err, 4, cudaMemcpyDeviceToHost, st));
+    LG_TRY(cudaStreamSynchronize(st));
+    if (herr) return describe_dev_err(herr);
+  }
 
   const GView v = make_view(g);
   const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
@@ -854,20 +834,27 @@ extern "C" lg_status lg_bfs(const lg_graph* g, const uint32_t* sources, uint32_t
   for (uint32_t b0 = 0; b0 < S; b0 += 64) {
     const uint32_t Sb = (S - b0) < 64 ? (S - b0) : 64;
     uint32_t* depth_b = g->relabel ? t_depth.as<uint32_t>() : depths + (uint64_t)b0 * n;
-    LG_TRY(cudaMemsetAsync(depth_b, 0xff, (uint64_t)Sb * n * sizeof(uint32_t), st));
-    LG_TRY(cudaMemsetAsync(t_vis.p, 0, n * mb, st));
-    LG_TRY(cudaMemsetAsync(t_fa.p, 0, n * mb, st));
-    LG_TRY(cudaMemsetAsync(t_fb.p, 0, n * mb, st));
-    LG_TRY(cudaMemsetAsync(counters, 0, 16, st));
-    LG_TRY(bfs_seed(t_vis.p, t_fa.p, depth_b, n, t_src.as<uint32_t>() + b0, Sb, g->relabel ? 1u : 0u, mb,
-                    t_qa.as<uint32_t>(), counters, st));
-    uint32_t hc[2] = {0, 0};
-    LG_TRY(cudaMemcpyAsync(hc, counters, 8, cudaMemcpyDeviceToHost, st));
+    LG_TRY(cudaMemsetAsync(t_vis.p, 0, n * mb + 16, st));
+    LG_TRY(cudaMemsetAsync(t_fa.p, 0, n * mb + 16, st));
+    LG_TRY(cudaMemsetAsync(t_small.p, 0, small_bytes, st));
+    uint32_t* qa = t_qa.as<uint32_t>();
+    if (mb == 2) k_bfs_start<uint16_t><<<1, 64, 0, st>>>(t_vis.as<uint16_t>(), t_fa.as<uint16_t>(), n, sources + b0, g->perm, Sb, stored, qa, stored - 3, d_err);
+    else if (mb == 4) k_bfs_start<uint32_t><<<1, 64, 0, st>>>(t_vis.as<uint32_t>(), t_fa.as<uint32_t>(), n, sources + b0, g->perm, Sb, stored, qa, stored - 3, d_err);
+    else k_bfs_start<uint64_t><<<1, 64, 0, st>>>(t_vis.as<uint64_t>(), t_fa.as<uint64_t>(), n, sources + b0, g->perm, Sb, stored, qa, stored - 3, d_err);
+    count_launch();
+    LG_TRY(cudaGetLastError());
+    uint32_t hc[2] = {0, 0};  // error, frontier
+    LG_TRY(cudaMemcpyAsync(hc, d_err, 8, cudaMemcpyDeviceToHost, st));
     LG_TRY(cudaStreamSynchronize(st));
-    uint32_t nq = hc[0];
+    if (hc[0]) return describe_dev_err((int)hc[0]);
+    LG_TRY(cudaMemsetAsync(depth_b, 0xff, (uint64_t)Sb * n * sizeof(uint32_t), st));
+    k_bfs_depth0<<<1, 64, 0, st>>>(depth_b, n, stored, Sb, g->relabel ? 1u : 0u);
+    count_launch();
+    LG_TRY(cudaGetLastError());
+    uint32_t nq = hc[1], prev = 0;  // lengths of this level's frontier and of the one before
     void* cur = t_fa.p;
     void* nxt = t_fb.p;
-    uint32_t* qcur = t_qa.as<uint32_t>();
+    uint32_t* qcur = qa;
     uint32_t* qnxt = t_qb.as<uint32_t>();
     BfsArgs a;
     memset(&a, 0, sizeof(a));
@@ -876,32 +863,34 @@ extern "C" lg_status lg_bfs(const lg_graph* g, const uint32_t* sources, uint32_t
     a.all_mask = Sb == 64 ? ~0ull : ((1ull << Sb) - 1ull);
     a.S = Sb;
     a.vmajor = g->relabel ? 1u : 0u;  // relabeled depths are permuted afterwards
-    a.counters = counters;
     a.hacc = t_hacc.p;
+    a.hcnt = reinterpret_cast<uint32_t*>(t_hacc.as<char>() + hacc_bytes);
     a.err = d_err;
     a.hot = hot_rows(g, mb);
     for (uint32_t level = 0; nq > 0; level++) {
-      LG_TRY(cudaMemsetAsync(counters, 0, 8, st));
+      if (level && level % RING == 0) LG_TRY(cudaMemsetAsync(ring, 0, RING * 8, st));
+      a.counters = ring + 2 * (level % RING);
       a.front_in = cur; a.front_out = nxt; a.level = level;
       a.queue_in = qcur; a.queue_in_len = nq; a.queue_out = qnxt;
       if ((uint64_t)nq > pull_threshold) {
         LG_TRY(ops->bfs_pull(v, a, mb, st));
-        LG_TRY(bfs_finish_multi(v, a, mb, st));
       } else {
+        // A push level adds to zeroed masks (a pull level writes them all): the
+        // output masks hold the frontier of the level before, listed in qnxt.
+        if (level == 0 || (uint64_t)prev * 16 >= n) {
+          LG_TRY(cudaMemsetAsync(nxt, 0, n * mb, st));
+        } else {
+          k_clear_queue<<<grid_for(prev, 256, 4096), 256, 0, st>>>(reinterpret_cast<uint8_t*>(nxt), mb, qnxt, prev);
+          count_launch();
+          LG_TRY(cudaGetLastError());
+        }
         LG_TRY(ops->bfs_push(v, a, mb, st));
       }
-      LG_TRY(cudaMemcpyAsync(hc, counters, 8, cudaMemcpyDeviceToHost, st));
-      // the frontier just consumed becomes the next output buffer: clear it
-      if ((uint64_t)nq * 16 < n) {
-        k_clear_queue<<<grid_for(nq, 256, 4096), 256, 0, st>>>(reinterpret_cast<uint8_t*>(cur), mb, qcur, nq);
-        count_launch();
-        LG_TRY(cudaGetLastError());
-      } else {
-        LG_TRY(cudaMemsetAsync(cur, 0, n * mb, st));
-      }
+      LG_TRY(cudaMemcpyAsync(hc, a.counters, 8, cudaMemcpyDeviceToHost, st));
       LG_TRY(cudaStreamSynchronize(st));
       void* t = cur; cur = nxt; nxt = t;
       uint32_t* tq = qcur; qcur = qnxt; qnxt = tq;
+      prev = nq;
       nq = hc[0];
     }
     if (g->relabel) LG_TRY(bfs_permute_depths(depth_b, depths + (uint64_t)b0 * n, g->perm, n, Sb, st));

@@ -71,6 +71,16 @@ struct GView {
   uint32_t heavy_min;         // degrees above this are in the schedule
   uint32_t heavy_seg;         // max fields per schedule item
   uint64_t heavy_prefix;      // the vertices below this label are all in the schedule (DM order; else 0)
+  uint64_t mid_prefix;        // the vertices below this label have more than 32 arcs (DM order; else 0)
+};
+
+// Work of a pull sweep's CTAs: heavy-schedule items, then tiles of `ta` vertices
+// from label a to b, then tiles of `tb` vertices to the end.
+struct TileMap {
+  uint64_t a, b;
+  uint32_t ta, tb;
+  uint32_t hb, na;  // CTAs of the items, of the tiles from a to b
+  uint32_t shared;  // 1: a CTA per item, 0: a warp per item
 };
 
 __device__ __forceinline__ uint32_t bits_u32(uint32_t x) { return 32u - __clz(x); }

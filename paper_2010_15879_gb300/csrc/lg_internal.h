@@ -185,7 +185,8 @@ struct BfsArgs {
   uint32_t queue_in_len;
   uint32_t* queue_out;       // vertices of the next frontier
   uint32_t* counters;        // [0] next queue length, [1] new (vertex, source) pairs
-  void* hacc;                // per split vertex: OR of its items' frontier masks
+  void* hacc;                // per split vertex: OR of its items' frontier masks (zero between levels)
+  uint32_t* hcnt;            // per split vertex: items that have arrived (zero between levels)
   int* err;
   uint32_t hot;              // pull gathers of masks u < hot are evict-last in L2, the others evict-first
 };
@@ -250,7 +251,6 @@ struct TravOps {
 };
 
 // finishing kernels for vertices split into several heavy items (lg_api.cu)
-cudaError_t bfs_finish_multi(const GView& g, const BfsArgs& a, int mask_bytes, cudaStream_t st);
 cudaError_t ppr_finish_multi(const GView& g, const PprArgs& a, cudaStream_t st);
 cudaError_t plan_carry_scan(HeavyItem* items, const uint32_t* multi, uint64_t n_multi, const uint32_t* segsum,
                             cudaStream_t st);
@@ -276,9 +276,6 @@ cudaError_t pr_fill0(float* ranks, uint64_t n, int64_t personal_orig, cudaStream
 PrPlan pr_plan(const lg_graph* g);
 
 // BFS helpers (lg_api.cu); vmajor: depth[v * S + s] instead of depth[s * n + v]
-cudaError_t bfs_seed(void* vis, void* front, uint32_t* depth, uint64_t n, const uint32_t* sources_stored,
-                     uint32_t S, uint32_t vmajor, int mask_bytes, uint32_t* queue, uint32_t* counters,
-                     cudaStream_t st);
 cudaError_t bfs_permute_depths(const uint32_t* tmp, uint32_t* out, const uint32_t* perm, uint64_t n,
                                uint32_t S, cudaStream_t st);
 cudaError_t map_ids(const uint32_t* in, uint32_t* out, const uint32_t* perm, uint64_t k, uint64_t n,

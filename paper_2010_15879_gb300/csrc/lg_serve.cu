@@ -285,7 +285,7 @@ struct Engine {
 // ------------------------------------------------------------------ BFS
 struct BfsEngine : Engine {
   uint64_t n;
-  uint64_t *vis = nullptr, *fa = nullptr, *fb = nullptr, *hacc = nullptr;
+  uint64_t *vis = nullptr, *fa = nullptr, *fb = nullptr, *hacc = nullptr;  // hacc: masks, then arrival counts
   uint32_t *qa = nullptr, *qb = nullptr, *counters = nullptr;
   unsigned long long* alive = nullptr;
   uint32_t** rows_dev = nullptr;
@@ -320,7 +320,7 @@ struct BfsEngine : Engine {
     A((void**)&vis, n * 8 + 16);
     A((void**)&fa, n * 8 + 16);
     A((void**)&fb, n * 8 + 16);
-    A((void**)&hacc, g->n_multi * 8 + 16);
+    A((void**)&hacc, g->n_multi * 12 + 16);
     A((void**)&qa, n * 4 + 16);
     A((void**)&qb, n * 4 + 16);
     A((void**)&counters, 64);
@@ -336,7 +336,7 @@ struct BfsEngine : Engine {
     if (e == cudaSuccess) e = cudaMemsetAsync(vis, 0, n * 8, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(fa, 0, n * 8, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(fb, 0, n * 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(hacc, 0, g->n_multi * 8 + 16, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(hacc, 0, g->n_multi * 12 + 16, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 16, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -432,11 +432,11 @@ struct BfsEngine : Engine {
     a.queue_out = qnxt;
     a.counters = counters;
     a.hacc = hacc;
+    a.hcnt = reinterpret_cast<uint32_t*>(hacc + g->n_multi);
     a.err = err;
     a.hot = hot_rows(g, 8);
     if ((uint64_t)nq > n / 64) {
       ECHK(ops->bfs_pull(view, a, 8, st));
-      ECHK(bfs_finish_multi(view, a, 8, st));
     } else {
       ECHK(ops->bfs_push(view, a, 8, st));
     }
