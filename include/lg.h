@@ -213,7 +213,7 @@ lg_status lg_bfs(const lg_graph *g, const uint32_t *sources, uint32_t S, uint32_
  * stepping) on a weighted graph (weights stored after each ID, Section 3.3),
  * neighborhoods and weights decoded inside the relaxation kernel.
  *   source  original ID (< n)
- *   delta   bucket width (0 = 32); any value gives the same distances
+ *   delta   bucket width (0 = 128); any value gives the same distances
  *   dist    device, n u64 indexed by original ID: the minimum over paths from
  *           source of the sum of arc weights, UINT64_MAX if unreachable
  * Needs a weighted graph in LG_ID_GLOBAL or LG_ID_CSR32 (else
