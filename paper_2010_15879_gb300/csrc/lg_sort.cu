@@ -4,6 +4,8 @@
 // CSR rows (the relabeled neighborhoods must be sorted again, Section 2.3).
 #include "lg_internal.h"
 
+#include <algorithm>
+
 namespace lg {
 
 // =========================================================================
@@ -19,6 +21,12 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
   return m;
 }
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <typename K>
 __global__ void __launch_bounds__(RS_NT) k_rs_hist(const K* __restrict__ keys, uint64_t n, uint32_t shift,
@@ -165,7 +173,8 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, u
 // segmented sort of CSR rows
 // =========================================================================
 constexpr uint32_t SEG_SMALL = 32;    // one thread per row, sorting network in registers
-constexpr uint32_t SEG_MEDIUM = NBR_SORT; // 4,096: 16 keys per lane, 4 lanes .. 8 warps per row
+constexpr uint32_t SEG_MEDIUM = NBR_SORT;  // 4,096: what the lookups' row kernel sorts itself
+constexpr uint32_t SEG_LARGE = 16384;      // what one CTA sorts
 constexpr int SROW = 33;              // shared slot stride of a small row (conflict-free lanes)
 
 // compare-exchange into ascending order, without branches
@@ -307,15 +316,21 @@ __global__ void __launch_bounds__(256) k_seg_small(uint32_t* __restrict__ keys, 
   }
 }
 
+// the rows of one size class: listed, or `count` consecutive ones from `first`
+struct SegRows {
+  const uint32_t* list;
+  uint32_t first, count;
+  __device__ __forceinline__ uint64_t row(uint32_t i) const { return list ? list[i] : first + i; }
+};
+
 // ---------------------------------------------------------------------------
-// Rows of 32 < d <= 4096 keys from a size-class list, P = 16 G W >= d keys per
-// row (padded with UINT32_MAX): G lanes per row in a warp (G <= 32), or W
-// warps per row (G = 32).  Lane g of warp w holds keys 16 (32 w + g) + e,
-// e < 16, so a bitonic compare-exchange at distance j is a register pair for
-// j < 16, a shuffle with lane g ^ (j / 16) for 16 <= j < 512 and an exchange
-// through shared memory with warp w ^ (j / 512) beyond.  The first four
-// levels are unrolled; the rest run as a loop (an unrolled network of this
-// size would outgrow the instruction cache).
+// Rows of 33..128 keys of a size class, P = 16 G >= d keys per row (padded
+// with UINT32_MAX), G lanes per row.  Lane g holds keys 16 g + e, e < 16, so a
+// bitonic compare-exchange at distance j is a register pair for j < 16 and a
+// shuffle with lane g ^ (j / 16) beyond.  The first four levels are unrolled;
+// the rest run as a loop (an unrolled network of this size would outgrow the
+// instruction cache).  From 129 keys on the network's log2(d) (log2(d) + 1) / 2
+// stages cost more than a radix sort's passes (169 keys: 35 G keys/s).
 // ---------------------------------------------------------------------------
 template <int J, bool VALS>
 __device__ __forceinline__ void blk_pairs(uint32_t (&x)[16], uint32_t (&y)[16], uint32_t base16, uint32_t k) {
@@ -354,26 +369,19 @@ __device__ __forceinline__ void blk_shfl(uint32_t (&x)[16], uint32_t (&y)[16], u
   }
 }
 
-template <int G, int W, bool VALS>
+template <int G, bool VALS>
 __global__ void __launch_bounds__(256) k_seg_blk(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                 const uint64_t* __restrict__ off, const uint32_t* __restrict__ list,
-                                                 uint32_t nlist) {
-  constexpr uint32_t P = 16u * G * W;
-  constexpr int RPB = 256 / (G * W);  // rows per block pass
-  extern __shared__ uint32_t bsm[];   // W > 1: RPB rows x P keys, then values
-  const int lane = threadIdx.x & 31;
-  const int g = lane % G;
-  const int wv = W > 1 ? (threadIdx.x >> 5) % W : 0;
-  const int grp = threadIdx.x / (G * W);
-  const uint32_t base16 = 16u * (32u * wv + g);
-  uint32_t* gk = bsm + grp * P;
-  uint32_t* gv = bsm + RPB * P + grp * P;
-  for (uint64_t base = (uint64_t)blockIdx.x * RPB; base < nlist; base += (uint64_t)gridDim.x * RPB) {
-    const uint64_t li = base + grp;
+                                                 const uint64_t* __restrict__ off, SegRows rows) {
+  constexpr uint32_t P = 16u * G;
+  constexpr int RPB = 256 / G;  // rows per block pass
+  const int g = threadIdx.x % G;
+  const uint32_t base16 = 16u * g;
+  for (uint64_t base = (uint64_t)blockIdx.x * RPB; base < rows.count; base += (uint64_t)gridDim.x * RPB) {
+    const uint64_t li = base + threadIdx.x / G;
     uint64_t lo = 0;
     uint32_t d = 0;
-    if (li < nlist) {
-      const uint64_t r = list[li];
+    if (li < rows.count) {
+      const uint64_t r = rows.row((uint32_t)li);
       lo = off[r];
       d = (uint32_t)(off[r + 1] - lo);
     }
@@ -397,28 +405,8 @@ __global__ void __launch_bounds__(256) k_seg_blk(uint32_t* __restrict__ keys, ui
       const bool up = (base16 & k) == 0;
 #pragma unroll 1
       for (uint32_t j = k >> 1; j >= 16; j >>= 1) {
-        if (W > 1 && j >= 512) {  // partner warp wv ^ (j / 512), same lane and register
-          const int jw = (int)(j >> 9);
-          __syncthreads();
-#pragma unroll
-          for (int e = 0; e < 16; e++) {
-            gk[wv * 512 + e * 32 + lane] = x[e];
-            if (VALS) gv[wv * 512 + e * 32 + lane] = y[e];
-          }
-          __syncthreads();
-          const bool keep_min = (((wv & jw) == 0) == up);
-#pragma unroll
-          for (int e = 0; e < 16; e++) {
-            const int at = (wv ^ jw) * 512 + e * 32 + lane;
-            const uint32_t ok = gk[at];
-            const bool take = keep_min ? (ok < x[e]) : (ok > x[e]);
-            if (VALS) y[e] = take ? gv[at] : y[e];
-            x[e] = take ? ok : x[e];
-          }
-        } else {
-          const uint32_t m = j >> 4;
-          blk_shfl<VALS>(x, y, m, ((g & m) == 0) == up);
-        }
+        const uint32_t m = j >> 4;
+        blk_shfl<VALS>(x, y, m, ((g & m) == 0) == up);
       }
       blk_tail<VALS>(x, y, up);
     }
@@ -433,17 +421,16 @@ __global__ void __launch_bounds__(256) k_seg_blk(uint32_t* __restrict__ keys, ui
   }
 }
 
-// size class of a row: 0 = warp path (d <= 32), 1..7 = P = 64..4096, 9 = radix
+// size class of a row: 0 for d <= 32, k = 1..9 for 2^(4+k) < d <= 2^(5+k),
+// SEG_BIG above
+constexpr int SEG_BIG = 10;
+constexpr int SEG_NCLASS = 11;
+
 __device__ __forceinline__ int seg_class(uint64_t d) {
   if (d <= SEG_SMALL) return 0;
-  if (d > SEG_MEDIUM) return 9;
-  int c = 1;
-  uint64_t P = 64;
-  while (P < d) { P <<= 1; c++; }
-  return c;
+  if (d > SEG_LARGE) return SEG_BIG;
+  return 27 - __clz((uint32_t)d - 1);
 }
-
-constexpr int SEG_NCLASS = 10;
 
 __global__ void k_seg_count(const uint64_t* __restrict__ off, uint64_t rows, uint32_t* __restrict__ cnt) {
   __shared__ uint32_t c[SEG_NCLASS];
@@ -507,106 +494,102 @@ __global__ void k_seg_big_sizes(const uint64_t* __restrict__ off, const uint32_t
 }
 
 // -------------------------------------------------------------------------
-// One stable split of a tile of up to RS_TILE keys by a 9-bit digit, for the
-// segmented radix sorts.  Warp w holds the consecutive chunk of keys
-// [c0, c0 + 32 G) with c0 = 32 G w, key c0 + 32 g + lane in x[g]: the warp
-// counts its chunk's digits into its own row of `wc` (one match per 32 keys,
-// the lowest lane of each digit adds its group's count), one block scan turns
-// the (digit, warp) counts into positions, and the warp writes its chunk in
-// order.  Three block barriers per pass, whatever the tile's length.
+// One stable split of up to 512 NW keys by a 9-bit digit, for the segmented
+// radix sorts.  Warp w holds the consecutive chunk [c0, c0 + 32 G) with
+// c0 = 32 G w, key c0 + 32 g + lane in register g: one match per 32 keys gives
+// a key's rank among its equals, the warp's own 16-bit counts (two digits to a
+// word, so the block scan adds both at once) the rank among the groups before,
+// and the scan over (digit, warp) the position.  The rank is kept beside the
+// digit, so the chunk goes out without another pass over the counts.  Three
+// block barriers per pass, whatever the tile's length.
 // -------------------------------------------------------------------------
 constexpr int SPL_BITS = 9;
 constexpr uint32_t SPL_NB = 1u << SPL_BITS;  // digits per pass
-constexpr int SPL_G = RS_TILE / RS_NT;       // groups of 32 keys per warp, at most
+constexpr int SPL_G = 16;                    // groups of 32 keys per warp, at most
+static_assert(SPL_G * RS_NT == RS_TILE, "a tile is one split of 8 warps");
 
+template <int NW>
 struct SplitSmem {
-  uint32_t wc[RS_NW][SPL_NB];  // per warp: its count, then its next position, of each digit
-  uint32_t dstart[SPL_NB];     // first position of each digit in the tile
-  uint32_t red[RS_NW];
+  uint32_t wc[NW][SPL_NB / 2];  // per warp: the counts, then the first position, of digits 2 i and 2 i + 1
+  uint32_t red[NW];
+  // the first position of a digit in the tile
+  __device__ __forceinline__ uint32_t start(uint32_t d) const { return reinterpret_cast<const uint16_t*>(wc[0])[d]; }
 };
 
 __host__ __device__ constexpr uint32_t spl_passes(uint32_t key_bits) { return (key_bits + SPL_BITS - 1) / SPL_BITS; }
 
-template <bool VALS>
-__device__ __forceinline__ void split_pass(const uint32_t (&x)[SPL_G], const uint32_t (&y)[SPL_G], uint32_t c0,
-                                           uint32_t len, int G, uint32_t shift, uint32_t* __restrict__ dk,
-                                           uint32_t* __restrict__ dv, SplitSmem& sp) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t lt = lanemask_lt();
-  for (uint32_t b = lane; b < SPL_NB; b += 32) sp.wc[w][b] = 0;
+// digit(g): of the key in register g; put(g, pos): writes it
+template <int NW, typename Digit, typename Put>
+__device__ __forceinline__ void split_pass(uint32_t c0, uint32_t len, int G, SplitSmem<NW>& sp, Digit digit, Put put) {
+  const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, lt = lanemask_lt();
+  uint4* mine4 = reinterpret_cast<uint4*>(sp.wc[w]);
+#pragma unroll
+  for (uint32_t b = 0; b < SPL_NB / 8; b += 32) mine4[b + lane] = make_uint4(0, 0, 0, 0);
   __syncwarp();
-  uint32_t pm[SPL_G];
+  uint16_t* mine = reinterpret_cast<uint16_t*>(sp.wc[w]);
+  uint32_t dr[SPL_G];  // the lanes of equal digit, then digit | rank in the chunk << 16
+#pragma unroll
+  for (int g = 0; g < SPL_G; g++)
+    if (g < G) dr[g] = __match_any_sync(LG_FULL_MASK, c0 + 32u * g + lane < len ? digit(g) : SPL_NB);
 #pragma unroll
   for (int g = 0; g < SPL_G; g++) {
-    pm[g] = 0;
     if (g < G) {
       const bool ok = c0 + 32u * g + lane < len;
-      const uint32_t dig = ok ? (x[g] >> shift) & (SPL_NB - 1) : SPL_NB;
-      pm[g] = __match_any_sync(LG_FULL_MASK, dig);
-      if (ok && (pm[g] & lt) == 0) sp.wc[w][dig] += __popc(pm[g]);
+      const uint32_t dig = ok ? digit(g) : 0u, peers = dr[g];
+      const uint32_t rank = mine[dig] + __popc(peers & lt);
       __syncwarp();
+      if (ok && peers >> lane == 1u) mine[dig] = (uint16_t)(rank + 1);  // the last lane of the digit
+      __syncwarp();
+      dr[g] = dig | rank << 16;
     }
   }
   __syncthreads();
-  constexpr int DPT = SPL_NB / RS_NT;  // digits per thread, consecutive
-  uint32_t tot[DPT], sum = 0;
-#pragma unroll
-  for (int q = 0; q < DPT; q++) {
-    const uint32_t b = threadIdx.x * DPT + q;
+  constexpr int WPT = NW < 8 ? 8 / NW : 1;  // count words per thread, consecutive
+  const bool scans = NW <= 8 || threadIdx.x < SPL_NB / 2;
+  uint32_t sum = 0;
+#pragma unroll 2
+  for (int q = 0; q < WPT; q++) {
     uint32_t acc = 0;
+    if (scans) {
+#pragma unroll 8
+      for (int v = 0; v < NW; v++) acc += sp.wc[v][threadIdx.x * WPT + q];
+    }
+    sum += (acc & 0xffffu) + (acc >> 16);
+  }
+  uint32_t incl = sum;
 #pragma unroll
-    for (int v = 0; v < RS_NW; v++) {
-      const uint32_t c = sp.wc[v][b];
-      sp.wc[v][b] = acc;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(LG_FULL_MASK, incl, o);
+    if (lane >= (uint32_t)o) incl += y;
+  }
+  if (lane == 31) sp.red[w] = incl;
+  __syncthreads();
+  uint32_t pre = incl - sum;
+#pragma unroll
+  for (int v = 0; v < (NW < 8 ? NW : 8); v++) pre += (uint32_t)v < w ? sp.red[v] : 0u;
+#pragma unroll 2
+  for (int q = 0; q < WPT; q++) {
+    if (!scans) break;
+    uint32_t acc = 0;
+#pragma unroll 8
+    for (int v = 0; v < NW; v++) {
+      const uint32_t c = sp.wc[v][threadIdx.x * WPT + q];
+      sp.wc[v][threadIdx.x * WPT + q] = acc;
       acc += c;
     }
-    tot[q] = acc;
-    sum += acc;
-  }
-  uint32_t total;
-  uint32_t pre = block_excl_scan<uint32_t, RS_NT>(sum, total, sp.red);
-#pragma unroll
-  for (int q = 0; q < DPT; q++) {
-    const uint32_t b = threadIdx.x * DPT + q;
-    sp.dstart[b] = pre;
-#pragma unroll
-    for (int v = 0; v < RS_NW; v++) sp.wc[v][b] += pre;
-    pre += tot[q];
+    const uint32_t both = pre | (pre + (acc & 0xffffu)) << 16;
+#pragma unroll 8
+    for (int v = 0; v < NW; v++) sp.wc[v][threadIdx.x * WPT + q] += both;
+    pre += (acc & 0xffffu) + (acc >> 16);
   }
   __syncthreads();
 #pragma unroll
-  for (int g = 0; g < SPL_G; g++) {
-    if (g < G) {
-      const bool ok = c0 + 32u * g + lane < len;
-      const uint32_t dig = (x[g] >> shift) & (SPL_NB - 1);
-      if (ok) {
-        const uint32_t pos = sp.wc[w][dig] + __popc(pm[g] & lt);
-        dk[pos] = x[g];
-        if (VALS) dv[pos] = y[g];
-      }
-      __syncwarp();
-      if (ok && (pm[g] & lt) == 0) sp.wc[w][dig] += __popc(pm[g]);
-      __syncwarp();
-    }
-  }
+  for (int g = 0; g < SPL_G; g++)
+    if (g < G && c0 + 32u * g + lane < len) put(g, mine[dr[g] & 0xffffu] + (dr[g] >> 16));
   __syncthreads();
 }
 
-template <bool VALS>
-__device__ __forceinline__ void split_load(const uint32_t* __restrict__ k, const uint32_t* __restrict__ v,
-                                           uint32_t c0, uint32_t len, int G, uint32_t (&x)[SPL_G],
-                                           uint32_t (&y)[SPL_G]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int g = 0; g < SPL_G; g++) {
-    const uint32_t i = c0 + 32u * g + lane;
-    const bool ok = g < G && i < len;
-    x[g] = ok ? k[i] : 0u;
-    y[g] = (VALS && ok) ? v[i] : 0u;
-  }
-}
-
-// Rows above SEG_MEDIUM keys: a segmented LSD radix sort of the rows gathered
+// Rows above SEG_LARGE keys: a segmented LSD radix sort of the rows gathered
 // into one buffer.  Tiles of RS_TILE keys never straddle two rows; the
 // histogram cells are laid out row by row, digit-major within a row, so one
 // exclusive scan over all cells gives every (row, digit, tile) its output
@@ -618,7 +601,7 @@ struct SrsTile {
   uint32_t len;       // keys in the tile (<= RS_TILE)
   uint32_t stride;    // tiles in the row
   uint32_t tl;        // index of the tile within its row
-  uint32_t pad;
+  uint32_t row;       // the row
 };
 
 __global__ void k_srs_tile_count(const uint64_t* __restrict__ boff, uint32_t nbig, uint32_t* __restrict__ nt) {
@@ -637,7 +620,7 @@ __global__ void k_srs_tile_fill(const uint64_t* __restrict__ boff, const uint64_
       d.len = (uint32_t)min((uint64_t)RS_TILE, size - (uint64_t)tl * RS_TILE);
       d.stride = nt;
       d.tl = tl;
-      d.pad = 0;
+      d.row = b;
       tiles[t0 + tl] = d;
     }
   }
@@ -655,47 +638,67 @@ __global__ void __launch_bounds__(RS_NT) k_srs_hist(const uint32_t* __restrict__
 }
 
 struct SrsSmem {
-  uint32_t k[RS_TILE];
+  uint32_t k[RS_TILE];   // as they came
   uint32_t v[RS_TILE];
-  uint64_t glob[SPL_NB];  // first output position of each digit of this tile
-  SplitSmem sp;
+  uint16_t at[RS_TILE];  // the order by digit
+  uint64_t glob[SPL_NB];  // first output position of each digit of this tile, less its first position here
+  SplitSmem<RS_NW> sp;
 };
 
 // One pass: the tile is split by digit in shared memory, then each key goes to
 // its digit's run for this tile (runs of one digit are consecutive in kout).
 template <bool VALS>
-__global__ void __launch_bounds__(RS_NT) k_srs_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+__global__ void __launch_bounds__(RS_NT, 4) k_srs_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
                                                        uint32_t* __restrict__ kout, uint32_t* __restrict__ vout,
                                                        const SrsTile* __restrict__ tiles, uint32_t shift,
                                                        const uint64_t* __restrict__ off) {
   extern __shared__ __align__(16) unsigned char srs_raw[];
   SrsSmem& sm = *reinterpret_cast<SrsSmem*>(srs_raw);
   const SrsTile d = tiles[blockIdx.x];
-  for (uint32_t b = threadIdx.x; b < SPL_NB; b += RS_NT) sm.glob[b] = off[d.cellbase + (uint64_t)b * d.stride + d.tl];
-  const int G = (int)((d.len + RS_NT - 1) / RS_NT);
+  const int G = (int)((d.len + RS_NT - 1) / RS_NT), lane = threadIdx.x & 31;
   const uint32_t c0 = 32u * G * (threadIdx.x >> 5);
-  uint32_t x[SPL_G], y[SPL_G];
-  split_load<VALS>(kin + d.start, vin + (VALS ? d.start : 0), c0, d.len, G, x, y);
-  split_pass<VALS>(x, y, c0, d.len, G, shift, sm.k, sm.v, sm.sp);
+  if (VALS) {
+    for (uint32_t i = threadIdx.x; i < d.len; i += RS_NT) cp_async4(&sm.v[i], vin + d.start + i);
+  }
+  uint32_t x[SPL_G];
+#pragma unroll
+  for (int g = 0; g < SPL_G; g++) {
+    const uint32_t i = c0 + 32u * g + lane;
+    x[g] = g < G && i < d.len ? kin[d.start + i] : 0u;
+  }
+#pragma unroll
+  for (int g = 0; g < SPL_G; g++)
+    if (g < G && c0 + 32u * g + lane < d.len) sm.k[c0 + 32u * g + lane] = x[g];
+  split_pass<RS_NW>(
+      c0, d.len, G, sm.sp, [&](int g) { return (x[g] >> shift) & (SPL_NB - 1); },
+      [&](int g, uint32_t pos) { sm.at[pos] = (uint16_t)(c0 + 32u * g + lane); });
+  for (uint32_t b = threadIdx.x; b < SPL_NB; b += RS_NT)
+    sm.glob[b] = off[d.cellbase + (uint64_t)b * d.stride + d.tl] - sm.sp.start(b);
+  if (VALS) cp_async_wait_all();
+  __syncthreads();
   for (uint32_t i = threadIdx.x; i < d.len; i += RS_NT) {
-    const uint32_t key = sm.k[i];
-    const uint32_t dig = (key >> shift) & (SPL_NB - 1);
-    const uint64_t pos = sm.glob[dig] + (i - sm.sp.dstart[dig]);
+    const uint32_t at = sm.at[i], key = sm.k[at];
+    const uint64_t pos = sm.glob[(key >> shift) & (SPL_NB - 1)] + i;
     kout[pos] = key;
-    if (VALS) vout[pos] = sm.v[i];
+    if (VALS) vout[pos] = sm.v[at];
   }
 }
 
-// The segmented radix passes over rows held back to back in (ka, va), row b at
-// [boff[b], boff[b+1]) with boff on the device; kb, vb hold as much.  On
-// return *result_in_b says whether the sorted rows ended in (kb, vb).
-static cudaError_t srs_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, const uint64_t* boff,
-                            uint32_t nbig, uint32_t key_bits, bool* result_in_b, cudaStream_t st) {
-  uint64_t *tbase = nullptr, *stmp = nullptr, *coff = nullptr, *ctmp = nullptr;
-  uint32_t *nt = nullptr, *hist = nullptr;
+// The tiles of nbig rows held back to back, row b at [boff[b], boff[b+1]) with
+// boff on the device.
+struct SrsTiles {
   SrsTile* tiles = nullptr;
-  uint64_t ntiles = 0;
-  *result_in_b = false;
+  uint64_t count = 0;  // tiles
+  uint64_t head = 0;   // tiles of the first nhead rows
+  void release(cudaStream_t st) {
+    if (tiles) cudaFreeAsync(tiles, st);
+    tiles = nullptr;
+  }
+};
+
+static cudaError_t srs_tiles(const uint64_t* boff, uint32_t nbig, uint32_t nhead, SrsTiles* out, cudaStream_t st) {
+  uint64_t *tbase = nullptr, *stmp = nullptr;
+  uint32_t* nt = nullptr;
   cudaError_t e = lg::pool_alloc((void**)&tbase, (nbig + 1) * sizeof(uint64_t), st);
   if (e == cudaSuccess) e = lg::pool_alloc((void**)&nt, nbig * sizeof(uint32_t), st);
   if (e == cudaSuccess) e = lg::pool_alloc((void**)&stmp, scan_tmp_words(nbig) * sizeof(uint64_t), st);
@@ -704,43 +707,59 @@ static cudaError_t srs_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* 
     count_launch();
     e = scan_excl_u32(nt, nbig, tbase, stmp, st);
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&ntiles, tbase + nbig, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&out->count, tbase + nbig, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&out->head, tbase + nhead, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  const uint64_t cells = (uint64_t)SPL_NB * ntiles;
-  if (e == cudaSuccess) e = lg::pool_alloc((void**)&tiles, (ntiles ? ntiles : 1) * sizeof(SrsTile), st);
-  if (e == cudaSuccess) e = lg::pool_alloc((void**)&hist, (cells ? cells : 1) * sizeof(uint32_t), st);
+  if (e == cudaSuccess)
+    e = lg::pool_alloc((void**)&out->tiles, (out->count ? out->count : 1) * sizeof(SrsTile), st);
+  if (e == cudaSuccess) {
+    k_srs_tile_fill<<<grid_for(nbig, 1, 4096), 256, 0, st>>>(boff, tbase, nbig, out->tiles);
+    count_launch();
+    e = cudaGetLastError();
+  }
+  if (tbase) cudaFreeAsync(tbase, st);
+  if (nt) cudaFreeAsync(nt, st);
+  if (stmp) cudaFreeAsync(stmp, st);
+  return e;
+}
+
+// The segmented radix passes over the head tiles' rows in (ka, va); kb, vb hold
+// as much.  On return *result_in_b says whether the sorted rows ended in (kb, vb).
+static cudaError_t srs_sort(uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, const SrsTiles& T,
+                            uint32_t key_bits, bool* result_in_b, cudaStream_t st) {
+  uint64_t *coff = nullptr, *ctmp = nullptr;
+  uint32_t* hist = nullptr;
+  *result_in_b = false;
+  const uint64_t cells = (uint64_t)SPL_NB * T.head;
+  cudaError_t e = lg::pool_alloc((void**)&hist, (cells ? cells : 1) * sizeof(uint32_t), st);
   if (e == cudaSuccess) e = lg::pool_alloc((void**)&coff, (cells + 1) * sizeof(uint64_t), st);
   if (e == cudaSuccess) e = lg::pool_alloc((void**)&ctmp, scan_tmp_words(cells) * sizeof(uint64_t), st);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(va ? k_srs_scatter<true> : k_srs_scatter<false>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SrsSmem));
-  if (e == cudaSuccess) {
-    k_srs_tile_fill<<<grid_for(nbig, 1, 4096), 256, 0, st>>>(boff, tbase, nbig, tiles);
-    count_launch();
-    e = cudaGetLastError();
-  }
   const uint32_t passes = spl_passes(key_bits);
-  for (uint32_t p = 0; p < passes && e == cudaSuccess && ntiles; p++) {
+  for (uint32_t p = 0; p < passes && e == cudaSuccess && T.head; p++) {
     const uint32_t shift = SPL_BITS * p;
-    k_srs_hist<<<(unsigned)ntiles, RS_NT, 0, st>>>(ka, tiles, shift, hist);
+    k_srs_hist<<<(unsigned)T.head, RS_NT, 0, st>>>(ka, T.tiles, shift, hist);
     count_launch();
     e = scan_excl_u32(hist, cells, coff, ctmp, st);
     if (e != cudaSuccess) break;
     if (va)
-      k_srs_scatter<true><<<(unsigned)ntiles, RS_NT, sizeof(SrsSmem), st>>>(ka, va, kb, vb, tiles, shift, coff);
+      k_srs_scatter<true><<<(unsigned)T.head, RS_NT, sizeof(SrsSmem), st>>>(ka, va, kb, vb, T.tiles, shift, coff);
     else
-      k_srs_scatter<false><<<(unsigned)ntiles, RS_NT, sizeof(SrsSmem), st>>>(ka, va, kb, vb, tiles, shift, coff);
+      k_srs_scatter<false><<<(unsigned)T.head, RS_NT, sizeof(SrsSmem), st>>>(ka, va, kb, vb, T.tiles, shift, coff);
     count_launch();
     e = cudaGetLastError();
     uint32_t* t = ka; ka = kb; kb = t;
     t = va; va = vb; vb = t;
     *result_in_b = !*result_in_b;
   }
-  cudaFreeAsync(tbase, st); cudaFreeAsync(nt, st); cudaFreeAsync(stmp, st);
-  cudaFreeAsync(tiles, st); cudaFreeAsync(hist, st); cudaFreeAsync(coff, st); cudaFreeAsync(ctmp, st);
+  if (hist) cudaFreeAsync(hist, st);
+  if (coff) cudaFreeAsync(coff, st);
+  if (ctmp) cudaFreeAsync(ctmp, st);
   return e;
 }
 
-// Rows above SEG_MEDIUM keys listed in `big`: gathered back to back, sorted,
+// Rows above SEG_LARGE keys listed in `big`: gathered back to back, sorted,
 // scattered back.
 static cudaError_t seg_sort_big(uint32_t* keys, uint32_t* vals, const uint64_t* off, const uint32_t* big,
                                 uint32_t nbig, uint32_t key_bits, cudaStream_t st) {
@@ -767,7 +786,10 @@ static cudaError_t seg_sort_big(uint32_t* keys, uint32_t* vals, const uint64_t* 
     e = cudaGetLastError();
   }
   bool in_b = false;
-  if (e == cudaSuccess) e = srs_sort(ka, vals ? va : nullptr, kb, vals ? vb : nullptr, boff, nbig, key_bits, &in_b, st);
+  SrsTiles T;
+  if (e == cudaSuccess) e = srs_tiles(boff, nbig, nbig, &T, st);
+  if (e == cudaSuccess) e = srs_sort(ka, vals ? va : nullptr, kb, vals ? vb : nullptr, T, key_bits, &in_b, st);
+  T.release(st);
   if (e == cudaSuccess) {
     k_seg_big_scatter<<<grid_for(nbig, 1, 4096), 256, 0, st>>>(keys, vals, off, big, boff, nbig, in_b ? kb : ka,
                                                                 in_b ? vb : va);
@@ -779,107 +801,172 @@ static cudaError_t seg_sort_big(uint32_t* keys, uint32_t* vals, const uint64_t* 
   return e;
 }
 
-// The first nbig rows are the rows above SEG_MEDIUM keys (degree-descending
-// order) and lie back to back from off[0] = 0: sorted in place, with one
-// buffer of the same size beside them.
-static cudaError_t seg_sort_big_prefix(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint32_t nbig,
+// The head tiles' rows lie back to back from 0 (the rows above SEG_LARGE keys in
+// degree-descending order, `total` keys): sorted in place, with one buffer of
+// the same size beside them.
+static cudaError_t seg_sort_big_prefix(uint32_t* keys, uint32_t* vals, const SrsTiles& T, uint64_t total,
                                        uint32_t key_bits, cudaStream_t st) {
-  uint64_t nb_total = 0;
-  cudaError_t e = cudaMemcpyAsync(&nb_total, off + nbig, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   uint32_t *kb = nullptr, *vb = nullptr;
-  if (e == cudaSuccess) e = lg::pool_alloc((void**)&kb, nb_total * sizeof(uint32_t), st);
-  if (e == cudaSuccess && vals) e = lg::pool_alloc((void**)&vb, nb_total * sizeof(uint32_t), st);
+  cudaError_t e = lg::pool_alloc((void**)&kb, total * sizeof(uint32_t), st);
+  if (e == cudaSuccess && vals) e = lg::pool_alloc((void**)&vb, total * sizeof(uint32_t), st);
   bool in_b = false;
-  if (e == cudaSuccess) e = srs_sort(keys, vals, kb, vb, off, nbig, key_bits, &in_b, st);
+  if (e == cudaSuccess) e = srs_sort(keys, vals, kb, vb, T, key_bits, &in_b, st);
   if (e == cudaSuccess && in_b) {
-    e = cudaMemcpyAsync(keys, kb, nb_total * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess && vals) e = cudaMemcpyAsync(vals, vb, nb_total * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
+    e = cudaMemcpyAsync(keys, kb, total * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess && vals) e = cudaMemcpyAsync(vals, vb, total * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
   }
   if (kb) cudaFreeAsync(kb, st);
   if (vb) cudaFreeAsync(vb, st);
   return e;
 }
 
-// Rows of 513..4096 keys: a CTA per row, a stable LSD radix sort with 9-bit
-// digits (ceil(key_bits / 9) passes of split_pass) -- a few compare-free steps
-// per key and pass instead of a bitonic network's log2(d) (log2(d) + 1) / 2
-// stages.
-constexpr uint32_t SEG_RADIX_MAX = 4096;
-static_assert(SEG_RADIX_MAX <= (uint32_t)RS_TILE, "a row must fit one split tile");
+// -------------------------------------------------------------------------
+// Rows of 129..16384 keys: a CTA of NW warps per row of up to 512 NW keys, a
+// stable LSD radix sort with 9-bit digits in shared memory.  The passes move
+// the keys' indices only, keys and values stay where they were loaded until
+// the sorted row is written.
+//
+// Degree-mapped rows need two passes whatever the number of vertices: a row
+// arrives sorted by its old IDs, in which order the labels of one degree
+// ascend, so only the degrees have to be sorted.  The sort key is a coarse
+// label of 18 bits -- exact below 2^17, one of 2^13 steps per power of two
+// above --, and index and key fit one word.  Two labels of one step are out of
+// order only if a change of degree lies between them: neighbors are compared,
+// a few exchanges repair such rows, and a row that these do not mend goes
+// through all passes of the whole label (as does every row of another order).
+// R-MAT 2^26, weighted: rows of 513..4096 keys 20.3 ms with three passes of
+// keys and values and a second pass over the counts, 9.7 so; rows of 129..512
+// 9.1 ms as bitonic networks, 5.8; rows of 4097..16384, 490 M of the 780 M keys
+// that went through the tiles' passes in global memory (20.3 ms in all), 10.0
+// beside 7.7 for the rest.
+// -------------------------------------------------------------------------
+constexpr uint32_t SEG_IDX_BITS = 14;
+constexpr uint32_t COARSE_BITS = 2 * SPL_BITS;
+constexpr int COARSE_REPAIRS = 16;  // rounds of exchanges
+static_assert(SEG_LARGE <= 1u << SEG_IDX_BITS && SEG_IDX_BITS + COARSE_BITS <= 32, "index and key share a word");
 
-template <bool VALS>
+__device__ __forceinline__ uint32_t coarse_label(uint32_t x) {
+  if (x < 1u << 17) return x;
+  const uint32_t e = 31u - __clz(x);
+  return (1u << 17) + ((e - 17u) << 13) + ((x >> (e - 13u)) & 8191u);  // at most 2^17 + 15 2^13 - 1
+}
+
+template <int NW, bool VALS>
 struct SegRadixSmem {
-  uint32_t k[SEG_RADIX_MAX];
-  uint32_t v[VALS ? SEG_RADIX_MAX : 1];
-  SplitSmem sp;
+  uint32_t k[512 * NW];
+  uint32_t v[VALS ? 512 * NW : 4];
+  uint32_t at[512 * NW];  // the sorted order: the key's index in the low bits
+  SplitSmem<NW> sp;
 };
 
-// Rows of SEG_SMALL < d <= SEG_RADIX_MAX keys, one row per block: the keys
-// stay in registers (warp chunks), each pass splits them into shared memory
-// and reads them back; the last pass's order is written out coalesced.
-template <bool VALS>
-__global__ void __launch_bounds__(RS_NT) k_seg_radix(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                     const uint64_t* __restrict__ off,
-                                                     const uint32_t* __restrict__ list, uint32_t nlist,
-                                                     uint32_t passes) {
+template <int NW, bool VALS>
+__global__ void __launch_bounds__(32 * NW, NW == 1 ? 30 : 32 / NW) k_seg_radix(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
+                                                                const uint64_t* __restrict__ off, SegRows rows,
+                                                                uint32_t passes, bool coarse) {
+  constexpr uint32_t NT = 32 * NW, IM = (1u << SEG_IDX_BITS) - 1;
   extern __shared__ __align__(16) unsigned char sr_raw[];
-  SegRadixSmem<VALS>& sm = *reinterpret_cast<SegRadixSmem<VALS>*>(sr_raw);
-  for (uint32_t li = blockIdx.x; li < nlist; li += gridDim.x) {
-    const uint64_t lo = off[list[li]];
-    const uint32_t d = (uint32_t)(off[list[li] + 1] - lo);
-    const int G = (int)((d + RS_NT - 1) / RS_NT);
+  SegRadixSmem<NW, VALS>& sm = *reinterpret_cast<SegRadixSmem<NW, VALS>*>(sr_raw);
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t li = blockIdx.x; li < rows.count; li += gridDim.x) {
+    const uint64_t r = rows.row(li), lo = off[r];
+    const uint32_t d = (uint32_t)(off[r + 1] - lo);
+    const int G = (int)((d + NT - 1) / NT);
     const uint32_t c0 = 32u * G * (threadIdx.x >> 5);
-    uint32_t x[SPL_G], y[SPL_G];
-    split_load<VALS>(keys + lo, vals + (VALS ? lo : 0), c0, d, G, x, y);
-    for (uint32_t p = 0; p < passes; p++) {
-      if (p) split_load<VALS>(sm.k, sm.v, c0, d, G, x, y);
-      split_pass<VALS>(x, y, c0, d, G, SPL_BITS * p, sm.k, sm.v, sm.sp);
+    uint32_t x[SPL_G];
+    if (VALS) {
+      for (uint32_t i = threadIdx.x; i < d; i += NT) cp_async4(&sm.v[i], vals + lo + i);
     }
-    for (uint32_t i = threadIdx.x; i < d; i += RS_NT) {
-      keys[lo + i] = sm.k[i];
-      if (VALS) vals[lo + i] = sm.v[i];
+#pragma unroll
+    for (int g = 0; g < SPL_G; g++) {
+      const uint32_t i = c0 + 32u * g + lane;
+      x[g] = g < G && i < d ? keys[lo + i] : 0u;
+    }
+#pragma unroll
+    for (int g = 0; g < SPL_G; g++) {
+      const uint32_t i = c0 + 32u * g + lane;
+      if (g < G && i < d) sm.k[i] = x[g];
+      x[g] = i | (coarse ? coarse_label(x[g]) << SEG_IDX_BITS : 0u);
+    }
+    // keys are written before they are read by index: a warp reads its own
+    // chunk's in the first pass, the passes' barriers come before the others
+    __syncwarp();
+    for (bool part = coarse;;) {
+      const uint32_t np = part ? 2u : passes;
+#pragma unroll 1
+      for (uint32_t p = 0; p < np; p++) {
+        // the word of a key: its index, then the whole coarse label or this
+        // pass's digit of the label
+#pragma unroll
+        for (int g = 0; g < SPL_G; g++) {
+          if (g < G) {
+            const uint32_t i = min(c0 + 32u * g + lane, d - 1);
+            if (p) x[g] = sm.at[i];
+            if (!part) {
+              const uint32_t at = p ? x[g] & IM : i;
+              x[g] = at | ((sm.k[at] >> (SPL_BITS * p)) & (SPL_NB - 1)) << SEG_IDX_BITS;
+            }
+          }
+        }
+        const uint32_t shift = SEG_IDX_BITS + (part ? SPL_BITS * p : 0u);
+        split_pass<NW>(
+            c0, d, G, sm.sp, [&](int g) { return (x[g] >> shift) & (SPL_NB - 1); },
+            [&](int g, uint32_t pos) { sm.at[pos] = x[g]; });
+      }
+      if (!part) break;
+      bool bad = false;
+      for (uint32_t i = threadIdx.x; i + 1 < d; i += NT) bad |= sm.k[sm.at[i] & IM] > sm.k[sm.at[i + 1] & IM];
+      bool done = !__syncthreads_or(bad);
+      for (int round = 0; round < COARSE_REPAIRS && !done; round++) {
+        bad = false;
+        for (uint32_t odd = 0; odd < 2; odd++) {
+          for (uint32_t i = 2 * threadIdx.x + odd; i + 1 < d; i += 2 * NT) {
+            const uint32_t a = sm.at[i], b = sm.at[i + 1];
+            if (sm.k[a & IM] > sm.k[b & IM]) {
+              sm.at[i] = b;
+              sm.at[i + 1] = a;
+              bad = true;
+            }
+          }
+          __syncthreads();
+        }
+        done = !__syncthreads_or(bad);
+      }
+      if (done) break;
+      part = false;
+    }
+    if (VALS) {
+      cp_async_wait_all();
+      __syncthreads();
+    }
+    for (uint32_t i = threadIdx.x; i < d; i += NT) {
+      const uint32_t at = sm.at[i] & IM;
+      keys[lo + i] = sm.k[at];
+      if (VALS) vals[lo + i] = sm.v[at];
     }
     __syncthreads();
   }
 }
 
-template <bool VALS>
-static cudaError_t seg_radix_launch(uint32_t* keys, uint32_t* vals, const uint64_t* off, const uint32_t* list,
-                                    uint32_t nlist, uint32_t key_bits, cudaStream_t st) {
-  const size_t smem = sizeof(SegRadixSmem<VALS>);
-  cudaError_t e = cudaFuncSetAttribute(k_seg_radix<VALS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int NW, bool VALS>
+static cudaError_t seg_radix_launch(uint32_t* keys, uint32_t* vals, const uint64_t* off, SegRows rows,
+                                    uint32_t key_bits, bool coarse, cudaStream_t st) {
+  if (!rows.count) return cudaSuccess;
+  const size_t smem = sizeof(SegRadixSmem<NW, VALS>);
+  cudaError_t e = cudaFuncSetAttribute(k_seg_radix<NW, VALS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_seg_radix<VALS><<<grid_for(nlist, 1, 152 * 8), RS_NT, smem, st>>>(keys, vals, off, list, nlist,
-                                                                      spl_passes(key_bits));
+  const uint32_t passes = spl_passes(key_bits);
+  k_seg_radix<NW, VALS><<<grid_for(rows.count, 1, 152 * 256), 32 * NW, smem, st>>>(
+      keys, vals, off, rows, passes, coarse && passes > 2);
   count_launch();
   return cudaGetLastError();
 }
 
-template <int G, int W, bool VALS>
-static cudaError_t seg_blk_launch(uint32_t* keys, uint32_t* vals, const uint64_t* off, const uint32_t* list,
-                                  uint32_t nlist, cudaStream_t st) {
-  constexpr int RPB = 256 / (G * W);
-  const size_t smem = W > 1 ? (size_t)RPB * 16 * G * W * sizeof(uint32_t) * (VALS ? 2 : 1) : 0;
-  k_seg_blk<G, W, VALS><<<grid_for(nlist, RPB, 152 * 16), 256, smem, st>>>(keys, vals, off, list, nlist);
+template <int G, bool VALS>
+static cudaError_t seg_blk_launch(uint32_t* keys, uint32_t* vals, const uint64_t* off, SegRows rows, cudaStream_t st) {
+  if (!rows.count) return cudaSuccess;
+  k_seg_blk<G, VALS><<<grid_for(rows.count, 256 / G, 152 * 16), 256, 0, st>>>(keys, vals, off, rows);
   count_launch();
   return cudaGetLastError();
-}
-
-// size class k holds rows of 2^(4+k) < d <= 2^(5+k) keys
-template <bool VALS>
-static cudaError_t seg_blk_class(int k, uint32_t* keys, uint32_t* vals, const uint64_t* off, const uint32_t* list,
-                                 uint32_t nlist, cudaStream_t st) {
-  switch (k) {
-    case 1: return seg_blk_launch<4, 1, VALS>(keys, vals, off, list, nlist, st);
-    case 2: return seg_blk_launch<8, 1, VALS>(keys, vals, off, list, nlist, st);
-    case 3: return seg_blk_launch<16, 1, VALS>(keys, vals, off, list, nlist, st);
-    case 4: return seg_blk_launch<32, 1, VALS>(keys, vals, off, list, nlist, st);
-    case 5: return seg_blk_launch<32, 2, VALS>(keys, vals, off, list, nlist, st);
-    case 6: return seg_blk_launch<32, 4, VALS>(keys, vals, off, list, nlist, st);
-    case 7: return seg_blk_launch<32, 8, VALS>(keys, vals, off, list, nlist, st);
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 static cudaError_t seg_small_launch(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint64_t rows,
@@ -896,9 +983,29 @@ static cudaError_t seg_small_launch(uint32_t* keys, uint32_t* vals, const uint64
   return cudaGetLastError();
 }
 
+// classes k0..9, `rows` in each; `coarse`: rows in the order of degree-mapped labels
+template <bool VALS>
+static cudaError_t seg_sort_classes(uint32_t* keys, uint32_t* vals, const uint64_t* off, const SegRows (&rows)[SEG_NCLASS],
+                                    int k0, uint32_t key_bits, bool coarse, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  for (int k = k0; k < SEG_BIG && e == cudaSuccess; k++) {
+    switch (k) {
+      case 1: e = seg_blk_launch<4, VALS>(keys, vals, off, rows[k], st); break;
+      case 2: e = seg_blk_launch<8, VALS>(keys, vals, off, rows[k], st); break;
+      case 3:
+      case 4: e = seg_radix_launch<1, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
+      case 5: e = seg_radix_launch<2, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
+      case 6: e = seg_radix_launch<4, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
+      case 7: e = seg_radix_launch<8, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
+      case 8: e = seg_radix_launch<16, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
+      default: e = seg_radix_launch<32, VALS>(keys, vals, off, rows[k], key_bits, coarse, st);
+    }
+  }
+  return e;
+}
+
 cudaError_t segmented_sort(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint64_t rows, uint64_t total,
-                           uint64_t max_row, cudaStream_t st, bool small_done, uint32_t key_bits, bool big_prefix,
-                           bool big_only) {
+                           uint64_t max_row, cudaStream_t st, bool small_done, uint32_t key_bits, bool big_only) {
   if (rows == 0 || total == 0 || max_row <= (big_only ? SEG_MEDIUM : 1)) return cudaSuccess;
   cudaError_t e;
   if (!small_done && !big_only && (e = seg_small_launch(keys, vals, off, rows, st)) != cudaSuccess) return e;
@@ -922,17 +1029,13 @@ cudaError_t segmented_sort(uint32_t* keys, uint32_t* vals, const uint64_t* off, 
   cudaMemcpyAsync(meta + SEG_NCLASS, base, sizeof(base), cudaMemcpyHostToDevice, st);
   k_seg_fill<<<grid_for(rows, 256, 152 * 16), 256, 0, st>>>(off, rows, meta + SEG_NCLASS, meta + 2 * SEG_NCLASS, list);
   count_launch();
-  for (int k = 1; k <= 4 && e == cudaSuccess && !big_only; k++)
-    if (cnt[k]) e = vals ? seg_blk_class<true>(k, keys, vals, off, list + base[k], cnt[k], st)
-                         : seg_blk_class<false>(k, keys, vals, off, list + base[k], cnt[k], st);
-  // rows of 513..4096 keys: one radix sort per row in shared memory
-  const uint32_t mid = cnt[5] + cnt[6] + cnt[7];  // classes 5..7 are adjacent in `list`
-  if (e == cudaSuccess && mid && !big_only)
-    e = vals ? seg_radix_launch<true>(keys, vals, off, list + base[5], mid, key_bits, st)
-             : seg_radix_launch<false>(keys, vals, off, list + base[5], mid, key_bits, st);
-  if (e == cudaSuccess && cnt[9])
-    e = big_prefix ? seg_sort_big_prefix(keys, vals, off, cnt[9], key_bits, st)
-                   : seg_sort_big(keys, vals, off, list + base[9], cnt[9], key_bits, st);
+  SegRows rows_of[SEG_NCLASS];
+  for (int k = 0; k < SEG_NCLASS; k++) rows_of[k] = {list + base[k], 0, cnt[k]};
+  const int k0 = big_only ? 8 : 1;
+  e = vals ? seg_sort_classes<true>(keys, vals, off, rows_of, k0, key_bits, false, st)
+           : seg_sort_classes<false>(keys, vals, off, rows_of, k0, key_bits, false, st);
+  if (e == cudaSuccess && cnt[SEG_BIG])
+    e = seg_sort_big(keys, vals, off, list + base[SEG_BIG], cnt[SEG_BIG], key_bits, st);
   cudaFreeAsync(list, st);
   cudaFreeAsync(meta, st);
   return e == cudaSuccess ? cudaGetLastError() : e;
@@ -1043,75 +1146,149 @@ __global__ void __launch_bounds__(256) k_dm_rows(const uint64_t* __restrict__ rp
   }
 }
 
-// Rows of more than SEG_SMALL arcs in DM order.  Labels go by degree
-// descending, so these rows are the first K new rows and their arcs the prefix
-// [0, nrp[K]) of the new CSR: the prefix is cut into chunks of DM_CHUNK arcs
-// spread evenly over the grid (a hub no longer rests on one warp).  chunk_row[c]
-// is the row holding arc c * DM_CHUNK; a lane walks 8 arcs 32 apart, all their
-// loads and perm lookups in flight together.
-constexpr uint32_t DM_CHUNK = 256;
+// ---------------------------------------------------------------------------
+// Rows of more than SEG_SMALL arcs in DM order, copied with their IDs mapped.
+// What bounds it is the random gather of perm: once perm outgrows the L2, each
+// arc fetches 51 B from DRAM for its 4 (R-MAT 2^26: 116 GB read for 15.6 GB of
+// arcs).  So the rows are cut in P parts by position and all rows' part 0 goes
+// first, then all part 1, ..: a row is sorted by its old IDs, so the parts of
+// one phase gather from much the same n / P labels, which stay in the L2
+// (gridDim.y = P: blocks start in that order).  Labels go by degree
+// descending, so the rows of a size class are consecutive; a warp takes
+// 2^lg of them and walks their parts as one range of slots, 8 slots a lane in
+// flight.  Rows above SEG_MEDIUM arcs are cut in the radix sort's tiles, each
+// of which belongs to one phase.
+// R-MAT 2^26, weighted, 2.1 G arcs: 22.4 ms in one phase, 14.1 in 8.
+// ---------------------------------------------------------------------------
+constexpr uint64_t DM_PART_BYTES = 32ull << 20;  // labels a phase gathers from
+constexpr uint32_t DM_MAX_PARTS = 32;
+constexpr uint32_t DM_TILES = 16;                // tiles a block looks at
+constexpr uint32_t DM_WARP_ARCS = 2048;          // arcs a warp takes in one phase, about
+constexpr int DM_T = 8;
 
-// K = the number of rows of more than SEG_SMALL arcs (degrees are descending)
-__global__ void k_dm_count_big(const uint32_t* __restrict__ newdeg, uint64_t n, unsigned long long* __restrict__ K) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-    if (newdeg[i] > SEG_SMALL && (i + 1 == n || newdeg[i + 1] <= SEG_SMALL)) *K = i + 1;
-}
-__global__ void k_dm_chunk_rows(const uint64_t* __restrict__ nrp, uint64_t n, const unsigned long long* __restrict__ K,
-                                uint32_t* __restrict__ chunk_row) {
-  const uint64_t k = *K;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k && i < n;
-       i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t c0 = (nrp[i] + DM_CHUNK - 1) / DM_CHUNK, c1 = (nrp[i + 1] + DM_CHUNK - 1) / DM_CHUNK;
-    for (uint64_t c = c0; c < c1; c++) chunk_row[c] = (uint32_t)i;
-  }
-}
+struct DmClass {
+  uint32_t first, rows;  // the class's rows
+  uint32_t lg;           // 2^lg rows per warp
+  uint32_t warp0;        // first warp
+};
+struct DmWork {
+  DmClass cls[8];
+  uint32_t ncls, warps;
+  const SrsTile* tiles;
+  uint64_t ntiles;
+  uint32_t tile_blocks;
+};
+
 template <bool VALS>
 __global__ void __launch_bounds__(256) k_dm_big(const uint64_t* __restrict__ rp, const uint32_t* __restrict__ col,
                                                 const uint32_t* __restrict__ w, const uint32_t* __restrict__ inv,
                                                 const uint32_t* __restrict__ perm, const uint64_t* __restrict__ nrp,
-                                                const unsigned long long* __restrict__ K,
-                                                const uint32_t* __restrict__ chunk_row, uint32_t* __restrict__ ncol,
-                                                uint32_t* __restrict__ nw) {
-  constexpr int T = DM_CHUNK / 32;
-  const int lane = threadIdx.x & 31;
-  const uint64_t E = nrp[*K];
-  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  const uint64_t pstream = policy_stream(), pkeep = policy_keep();
-  for (uint64_t c = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c * DM_CHUNK < E; c += warps) {
-    uint32_t i = chunk_row[c];
-    uint64_t rs = nrp[i], re = nrp[i + 1], old = rp[inv[i]];
-    uint32_t cc[T], wv[T];
+                                                DmWork a, uint32_t* __restrict__ ncol, uint32_t* __restrict__ nw) {
+  const uint32_t lane = threadIdx.x & 31u, part = blockIdx.y, parts = gridDim.y;
+  const uint64_t pstream = policy_stream();
+  if (blockIdx.x < a.tile_blocks) {
+    const uint64_t t0 = (uint64_t)blockIdx.x * DM_TILES, t1 = min(t0 + DM_TILES, a.ntiles);
+    for (uint64_t t = t0; t < t1; t++) {
+      const SrsTile d = a.tiles[t];
+      if ((uint32_t)((uint64_t)d.tl * parts / d.stride) != part) continue;
+      const uint64_t old = rp[inv[d.row]] + (uint64_t)d.tl * RS_TILE;
+      for (uint32_t i0 = threadIdx.x; i0 < d.len; i0 += 256 * DM_T) {
+        uint32_t c[DM_T], x[DM_T];
 #pragma unroll
-    for (int t = 0; t < T; t++) {
-      const uint64_t p = c * DM_CHUNK + lane + 32u * t;
-      cc[t] = 0;
-      wv[t] = 0;
-      if (p < E) {
-        while (re <= p) {  // next row (each holds more than SEG_SMALL arcs)
-          i++;
-          rs = re;
-          re = nrp[i + 1];
-          old = rp[inv[i]];
+        for (int j = 0; j < DM_T; j++) {
+          const uint32_t i = i0 + 256u * j;
+          c[j] = i < d.len ? ldg_hint(col + old + i, pstream) : 0u;
+          x[j] = VALS && i < d.len ? ldg_hint(w + old + i, pstream) : 0u;
         }
-        cc[t] = ldg_hint(col + old + (p - rs), pstream);
-        if (VALS) wv[t] = ldg_hint(w + old + (p - rs), pstream);
+#pragma unroll
+        for (int j = 0; j < DM_T; j++) c[j] = i0 + 256u * j < d.len ? __ldg(perm + c[j]) : 0u;
+#pragma unroll
+        for (int j = 0; j < DM_T; j++) {
+          const uint32_t i = i0 + 256u * j;
+          if (i < d.len) {
+            __stcs(ncol + d.start + i, c[j]);
+            if (VALS) __stcs(nw + d.start + i, x[j]);
+          }
+        }
       }
     }
-    uint32_t pv[T];
+    return;
+  }
+  const uint32_t gw = (blockIdx.x - a.tile_blocks) * 8 + (threadIdx.x >> 5);
+  if (gw >= a.warps) return;
+  uint32_t k = 0;
+  while (k + 1 < a.ncls && gw >= a.cls[k + 1].warp0) k++;
+  const uint32_t lg = a.cls[k].lg, r = ((gw - a.cls[k].warp0) << lg) + lane;
+  uint64_t src = 0, dst = 0;
+  uint32_t len = 0;
+  if (lane < (1u << lg) && r < a.cls[k].rows) {
+    const uint32_t i = a.cls[k].first + r;
+    const uint64_t lo = nrp[i], d = nrp[i + 1] - lo;
+    // the cuts lie on 64-byte boundaries of the output
+    const uint64_t c0 = part == 0 ? lo : max(lo, (lo + d * part / parts) & ~(uint64_t)15);
+    const uint64_t c1 = part + 1 == parts ? lo + d : max(lo, (lo + d * (part + 1) / parts) & ~(uint64_t)15);
+    src = rp[inv[i]] + (c0 - lo);
+    dst = c0;
+    len = (uint32_t)(c1 - c0);
+  }
+  uint32_t incl = len;
 #pragma unroll
-    for (int t = 0; t < T; t++) {
-      const uint64_t p = c * DM_CHUNK + lane + 32u * t;
-      pv[t] = p < E ? ldg_hint(perm + cc[t], pkeep) : 0u;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(LG_FULL_MASK, incl, o);
+    if (lane >= (uint32_t)o) incl += y;
+  }
+  const uint32_t total = __shfl_sync(LG_FULL_MASK, incl, 31);
+  src -= incl - len;  // slot s of the range lies at src + s, dst + s
+  dst -= incl - len;
+  for (uint32_t s0 = 0; s0 < total; s0 += 32 * DM_T) {
+    uint32_t c[DM_T], x[DM_T];
+    uint64_t to[DM_T];
+#pragma unroll
+    for (int j = 0; j < DM_T; j++) {
+      const uint32_t s = s0 + 32u * j + lane;
+      int o = 0;  // the slot's row: lanes with incl <= s come before it
+#pragma unroll
+      for (int step = 16; step; step >>= 1)
+        if (__shfl_sync(LG_FULL_MASK, incl, o + step - 1) <= s) o += step;
+      const uint64_t from = __shfl_sync(LG_FULL_MASK, src, o) + s;
+      to[j] = __shfl_sync(LG_FULL_MASK, dst, o) + s;
+      c[j] = s < total ? ldg_hint(col + from, pstream) : 0u;
+      x[j] = VALS && s < total ? ldg_hint(w + from, pstream) : 0u;
     }
 #pragma unroll
-    for (int t = 0; t < T; t++) {
-      const uint64_t p = c * DM_CHUNK + lane + 32u * t;
-      if (p < E) {
-        __stcs(ncol + p, pv[t]);
-        if (VALS) __stcs(nw + p, wv[t]);
+    for (int j = 0; j < DM_T; j++) c[j] = s0 + 32u * j + lane < total ? __ldg(perm + c[j]) : 0u;
+#pragma unroll
+    for (int j = 0; j < DM_T; j++) {
+      if (s0 + 32u * j + lane < total) {
+        __stcs(ncol + to[j], c[j]);
+        if (VALS) __stcs(nw + to[j], x[j]);
       }
     }
   }
+}
+
+// Maps the rows of classes [k0, k1] (and the tiles, if any) in `parts` phases.
+static cudaError_t dm_big(const uint64_t* rp, const uint32_t* col, const uint32_t* w, const uint32_t* inv,
+                          const uint32_t* perm, const uint64_t* nrp, const SegRows (&rows)[SEG_NCLASS], int k0, int k1,
+                          const SrsTiles& T, uint32_t parts, uint32_t* ncol, uint32_t* nw, cudaStream_t st) {
+  DmWork a{};
+  for (int k = k1; k >= k0; k--) {
+    if (!rows[k].count) continue;
+    uint32_t lg = 0;
+    while (lg < 5 && (2ull << lg) << (5 + k) <= (uint64_t)DM_WARP_ARCS * parts) lg++;
+    a.cls[a.ncls++] = {rows[k].first, rows[k].count, lg, a.warps};
+    a.warps += (uint32_t)(((uint64_t)rows[k].count + (1u << lg) - 1) >> lg);
+  }
+  a.tiles = T.tiles;
+  a.ntiles = T.count;
+  a.tile_blocks = (uint32_t)((T.count + DM_TILES - 1) / DM_TILES);
+  const uint64_t blocks = a.tile_blocks + (uint64_t)(a.warps + 7) / 8;
+  if (!blocks) return cudaSuccess;
+  const dim3 grid((unsigned)blocks, parts);
+  if (w) k_dm_big<true><<<grid, 256, 0, st>>>(rp, col, w, inv, perm, nrp, a, ncol, nw);
+  else k_dm_big<false><<<grid, 256, 0, st>>>(rp, col, w, inv, perm, nrp, a, ncol, nw);
+  count_launch();
+  return cudaGetLastError();
 }
 
 // =========================================================================
@@ -1154,6 +1331,51 @@ __global__ void __launch_bounds__(256) k_gr_first(const uint64_t* __restrict__ r
       if ((unsigned long long)(p + k) < first[u]) atomicMin(first + u, (unsigned long long)(p + k));
     }
   }
+}
+
+// The rows of more than SEG_SMALL arcs in DM order: mapped, then sorted.
+static cudaError_t dm_big_rows(const uint64_t* rp, const uint32_t* col, const uint32_t* w, uint64_t n,
+                               const uint32_t* perm, const uint32_t* inv_perm, const uint64_t* nrp, uint32_t* ncol,
+                               uint32_t* nw, cudaStream_t st) {
+  uint32_t* meta = nullptr;
+  uint32_t cnt[SEG_NCLASS];
+  uint64_t big_arcs = 0;
+  cudaError_t e = lg::pool_alloc((void**)&meta, sizeof(cnt), st);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(meta, 0, sizeof(cnt), st);
+  if (e == cudaSuccess) {
+    k_seg_count<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(nrp, n, meta);
+    count_launch();
+    e = cudaMemcpyAsync(cnt, meta, sizeof(cnt), cudaMemcpyDeviceToHost, st);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  cudaFreeAsync(meta, st);
+  if (e != cudaSuccess) return e;
+  SegRows rows[SEG_NCLASS] = {};
+  uint32_t at = 0;
+  for (int k = SEG_BIG; k >= 1; k--) {
+    rows[k] = {nullptr, at, cnt[k]};
+    at += cnt[k];
+  }
+  SrsTiles T;
+  const uint32_t tiled = rows[7].first;  // rows above SEG_MEDIUM arcs
+  if (tiled) {
+    e = cudaMemcpyAsync(&big_arcs, nrp + cnt[SEG_BIG], sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = srs_tiles(nrp, tiled, cnt[SEG_BIG], &T, st);  // waits
+  }
+  const uint32_t parts = (uint32_t)std::min<uint64_t>((n * sizeof(uint32_t) + DM_PART_BYTES - 1) / DM_PART_BYTES, DM_MAX_PARTS);
+  // a part below 16 arcs costs more in torn sectors than its gathers gain:
+  // rows of up to 128 arcs go in one phase
+  const int kp = parts > 1 ? 3 : 1;
+  if (e == cudaSuccess) e = dm_big(rp, col, w, inv_perm, perm, nrp, rows, kp, 7, T, parts, ncol, nw, st);
+  if (e == cudaSuccess && kp > 1) e = dm_big(rp, col, w, inv_perm, perm, nrp, rows, 1, kp - 1, SrsTiles{}, 1, ncol, nw, st);
+  if (e == cudaSuccess)
+    e = w ? seg_sort_classes<true>(ncol, nw, nrp, rows, 1, host_bits(n - 1), true, st)
+          : seg_sort_classes<false>(ncol, nullptr, nrp, rows, 1, host_bits(n - 1), true, st);
+  if (e == cudaSuccess && cnt[SEG_BIG])
+    e = seg_sort_big_prefix(ncol, w ? nw : nullptr, T, big_arcs, host_bits(n - 1), st);
+  T.release(st);
+  return e;
 }
 
 cudaError_t enc_dm_relabel(const uint64_t* rp, const uint32_t* col, const uint32_t* w, uint64_t n, uint64_t arcs,
@@ -1211,24 +1433,10 @@ cudaError_t enc_dm_relabel(const uint64_t* rp, const uint32_t* col, const uint32
     count_launch();
     e = scan_excl_u32(newdeg, n, nrp, stmp, st);
   }
-  // DM order (degree descending): the rows of more than SEG_SMALL arcs form a
-  // prefix and go to k_dm_big; the greedy order mixes sizes, so k_dm_rows
-  // copies its big rows itself
+  // DM order (degree descending): the rows of each size class are consecutive,
+  // the largest first, and go to k_dm_big; the greedy order mixes sizes, so
+  // k_dm_rows copies its big rows itself
   const int split_big = mode != 2;
-  unsigned long long* dK = nullptr;
-  uint32_t* chunk_row = nullptr;
-  if (e == cudaSuccess && split_big) {
-    e = lg::pool_alloc((void**)&dK, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) e = lg::pool_alloc((void**)&chunk_row, (arcs / DM_CHUNK + 2) * sizeof(uint32_t), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dK, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) {
-      k_dm_count_big<<<grid_for(n, 256, 152 * 32), 256, 0, st>>>(newdeg, n, dK);
-      count_launch();
-      k_dm_chunk_rows<<<grid_for(n, 256, 152 * 32), 256, 0, st>>>(nrp, n, dK, chunk_row);
-      count_launch();
-      e = cudaGetLastError();
-    }
-  }
   if (e == cudaSuccess) {
     const size_t smem = (size_t)8 * 32 * SROW * sizeof(uint32_t) * (w ? 2 : 1);
     if (w) {
@@ -1243,18 +1451,11 @@ cudaError_t enc_dm_relabel(const uint64_t* rp, const uint32_t* col, const uint32
     count_launch();
     if (e == cudaSuccess) e = cudaGetLastError();
   }
-  if (e == cudaSuccess && split_big) {
-    if (w) k_dm_big<true><<<152 * 8, 256, 0, st>>>(rp, col, w, inv_perm, perm, nrp, dK, chunk_row, ncol, nw);
-    else k_dm_big<false><<<152 * 8, 256, 0, st>>>(rp, col, w, inv_perm, perm, nrp, dK, chunk_row, ncol, nw);
-    count_launch();
-    e = cudaGetLastError();
-  }
-  if (dK) cudaFreeAsync(dK, st);
-  if (chunk_row) cudaFreeAsync(chunk_row, st);
   // rows of <= 32 arcs left k_dm_rows sorted
-  // DM order is degree-descending, so its rows above SEG_MEDIUM keys are the first rows
-  if (e == cudaSuccess)
-    e = segmented_sort(ncol, w ? nw : nullptr, nrp, n, arcs, max_deg, st, true, host_bits(n - 1), split_big != 0);
+  if (e == cudaSuccess && split_big && max_deg > SEG_SMALL)
+    e = dm_big_rows(rp, col, w, n, perm, inv_perm, nrp, ncol, nw, st);
+  else if (e == cudaSuccess && !split_big)
+    e = segmented_sort(ncol, w ? nw : nullptr, nrp, n, arcs, max_deg, st, true, host_bits(n - 1));
   cudaFreeAsync(keys, st); cudaFreeAsync(k2, st); cudaFreeAsync(v2, st); cudaFreeAsync(newdeg, st);
   cudaFreeAsync(stmp, st); cudaFreeAsync(rtmp, st);
   return e;
