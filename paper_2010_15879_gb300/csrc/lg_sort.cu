@@ -496,8 +496,8 @@ __global__ void k_seg_big_sizes(const uint64_t* __restrict__ off, const uint32_t
 // -------------------------------------------------------------------------
 // One stable split of up to 512 NW keys by a 9-bit digit, for the segmented
 // radix sorts.  Warp w holds the consecutive chunk [c0, c0 + 32 G) with
-// c0 = 32 G w, key c0 + 32 g + lane in register g: one match per 32 keys gives
-// a key's rank among its equals, the warp's own 16-bit counts (two digits to a
+// c0 = 32 G w, key c0 + 32 g + lane in register g: a vote per bit of the digit
+// gives a key's rank among its equals, the warp's own 16-bit counts (two digits to a
 // word, so the block scan adds both at once) the rank among the groups before,
 // and the scan over (digit, warp) the position.  The rank is kept beside the
 // digit, so the chunk goes out without another pass over the counts.  Three
@@ -518,30 +518,37 @@ struct SplitSmem {
 
 __host__ __device__ constexpr uint32_t spl_passes(uint32_t key_bits) { return (key_bits + SPL_BITS - 1) / SPL_BITS; }
 
-// digit(g): of the key in register g; put(g, pos): writes it
+// digit(g): of the key in register g; put(g, pos): writes it.  All 32 G NW
+// keys take part: the caller fills up with keys of the last digit, which stay
+// behind the others.
 template <int NW, typename Digit, typename Put>
-__device__ __forceinline__ void split_pass(uint32_t c0, uint32_t len, int G, SplitSmem<NW>& sp, Digit digit, Put put) {
+__device__ __forceinline__ void split_pass(int G, SplitSmem<NW>& sp, Digit digit, Put put) {
   const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, lt = lanemask_lt();
   uint4* mine4 = reinterpret_cast<uint4*>(sp.wc[w]);
 #pragma unroll
   for (uint32_t b = 0; b < SPL_NB / 8; b += 32) mine4[b + lane] = make_uint4(0, 0, 0, 0);
   __syncwarp();
   uint16_t* mine = reinterpret_cast<uint16_t*>(sp.wc[w]);
-  uint32_t dr[SPL_G];  // the lanes of equal digit, then digit | rank in the chunk << 16
-#pragma unroll
-  for (int g = 0; g < SPL_G; g++)
-    if (g < G) dr[g] = __match_any_sync(LG_FULL_MASK, c0 + 32u * g + lane < len ? digit(g) : SPL_NB);
+  uint32_t dr[SPL_G];  // digit | rank in the chunk << 16
 #pragma unroll
   for (int g = 0; g < SPL_G; g++) {
-    if (g < G) {
-      const bool ok = c0 + 32u * g + lane < len;
-      const uint32_t dig = ok ? digit(g) : 0u, peers = dr[g];
-      const uint32_t rank = mine[dig] + __popc(peers & lt);
-      __syncwarp();
-      if (ok && peers >> lane == 1u) mine[dig] = (uint16_t)(rank + 1);  // the last lane of the digit
-      __syncwarp();
-      dr[g] = dig | rank << 16;
+    if (g >= G) continue;
+    // The lanes of equal digit, by votes: a match takes longer the more digits
+    // differ.  R-MAT 2^26, rows of one to 32 warps: 5.2, 4.3, 6.2 ms (4 warps),
+    // 6.7 (16) and 3.3 (32) by match, 5.1, 3.8, 4.2, 4.6 and 2.1 by votes.
+    const uint32_t dig = digit(g);
+    uint32_t peers = LG_FULL_MASK;
+#pragma unroll
+    for (int b = 0; b < SPL_BITS; b++) {
+      const bool bit = dig >> b & 1u;
+      const uint32_t v = __ballot_sync(LG_FULL_MASK, bit);
+      peers &= bit ? v : ~v;
     }
+    const uint32_t rank = mine[dig] + __popc(peers & lt);
+    __syncwarp();
+    if (peers >> lane == 1u) mine[dig] = (uint16_t)(rank + 1);  // the last lane of the digit
+    __syncwarp();
+    dr[g] = dig | rank << 16;
   }
   __syncthreads();
   constexpr int WPT = NW < 8 ? 8 / NW : 1;  // count words per thread, consecutive
@@ -585,7 +592,7 @@ __device__ __forceinline__ void split_pass(uint32_t c0, uint32_t len, int G, Spl
   __syncthreads();
 #pragma unroll
   for (int g = 0; g < SPL_G; g++)
-    if (g < G && c0 + 32u * g + lane < len) put(g, mine[dr[g] & 0xffffu] + (dr[g] >> 16));
+    if (g < G) put(g, mine[dr[g] & 0xffffu] + (dr[g] >> 16));
   __syncthreads();
 }
 
@@ -670,7 +677,7 @@ __global__ void __launch_bounds__(RS_NT, 4) k_srs_scatter(const uint32_t* __rest
   for (int g = 0; g < SPL_G; g++)
     if (g < G && c0 + 32u * g + lane < d.len) sm.k[c0 + 32u * g + lane] = x[g];
   split_pass<RS_NW>(
-      c0, d.len, G, sm.sp, [&](int g) { return (x[g] >> shift) & (SPL_NB - 1); },
+      G, sm.sp, [&](int g) { return c0 + 32u * g + lane < d.len ? (x[g] >> shift) & (SPL_NB - 1) : SPL_NB - 1; },
       [&](int g, uint32_t pos) { sm.at[pos] = (uint16_t)(c0 + 32u * g + lane); });
   for (uint32_t b = threadIdx.x; b < SPL_NB; b += RS_NT)
     sm.glob[b] = off[d.cellbase + (uint64_t)b * d.stride + d.tl] - sm.sp.start(b);
@@ -830,19 +837,21 @@ static cudaError_t seg_sort_big_prefix(uint32_t* keys, uint32_t* vals, const Srs
 // arrives sorted by its old IDs, in which order the labels of one degree
 // ascend, so only the degrees have to be sorted.  The sort key is a coarse
 // label of 18 bits -- exact below 2^17, one of 2^13 steps per power of two
-// above --, and index and key fit one word.  Two labels of one step are out of
-// order only if a change of degree lies between them: neighbors are compared,
-// a few exchanges repair such rows, and a row that these do not mend goes
-// through all passes of the whole label (as does every row of another order).
-// R-MAT 2^26, weighted: rows of 513..4096 keys 20.3 ms with three passes of
-// keys and values and a second pass over the counts, 9.7 so; rows of 129..512
-// 9.1 ms as bitonic networks, 5.8; rows of 4097..16384, 490 M of the 780 M keys
-// that went through the tiles' passes in global memory (20.3 ms in all), 10.0
-// beside 7.7 for the rest.
+// above --, and index and key fit one word.  Labels of one step come out in
+// the order they had, which is wrong only where a change of degree lies between
+// them: the few such runs are sorted by insertion, and a row with a run of more
+// than RUN_MAX goes through all passes of the whole label (as do rows in
+// another order than the DM's).
+// What bounds it is instructions and shared-memory latency.  R-MAT 2^26,
+// weighted: rows of 513..4096 keys 20.3 ms with three passes of keys and values
+// and a second pass over the counts, 8.0 so; rows of 129..512 9.1 ms as bitonic
+// networks, 5.1; rows of 4097..16384, 490 M of the 780 M keys that went through
+// the tiles' passes in global memory (20.3 ms in all), 6.7 beside 7.0 for the
+// rest.
 // -------------------------------------------------------------------------
 constexpr uint32_t SEG_IDX_BITS = 14;
 constexpr uint32_t COARSE_BITS = 2 * SPL_BITS;
-constexpr int COARSE_REPAIRS = 16;  // rounds of exchanges
+constexpr uint32_t RUN_MAX = 64;
 static_assert(SEG_LARGE <= 1u << SEG_IDX_BITS && SEG_IDX_BITS + COARSE_BITS <= 32, "index and key share a word");
 
 __device__ __forceinline__ uint32_t coarse_label(uint32_t x) {
@@ -885,10 +894,11 @@ __global__ void __launch_bounds__(32 * NW, NW == 1 ? 30 : 32 / NW) k_seg_radix(u
     for (int g = 0; g < SPL_G; g++) {
       const uint32_t i = c0 + 32u * g + lane;
       if (g < G && i < d) sm.k[i] = x[g];
-      x[g] = i | (coarse ? coarse_label(x[g]) << SEG_IDX_BITS : 0u);
+      // no coarse label reaches 2^18 - 1: the padding's word comes last
+      x[g] = i < d ? i | (coarse ? coarse_label(x[g]) << SEG_IDX_BITS : 0u) : ~0u;
     }
-    // keys are written before they are read by index: a warp reads its own
-    // chunk's in the first pass, the passes' barriers come before the others
+    // a warp reads its own chunk's keys in the first pass; the passes'
+    // barriers come before the others
     __syncwarp();
     for (bool part = coarse;;) {
       const uint32_t np = part ? 2u : passes;
@@ -899,40 +909,46 @@ __global__ void __launch_bounds__(32 * NW, NW == 1 ? 30 : 32 / NW) k_seg_radix(u
 #pragma unroll
         for (int g = 0; g < SPL_G; g++) {
           if (g < G) {
-            const uint32_t i = min(c0 + 32u * g + lane, d - 1);
-            if (p) x[g] = sm.at[i];
-            if (!part) {
-              const uint32_t at = p ? x[g] & IM : i;
+            if (p) x[g] = sm.at[c0 + 32u * g + lane];
+            if (!part && x[g] != ~0u) {
+              const uint32_t at = x[g] & IM;
               x[g] = at | ((sm.k[at] >> (SPL_BITS * p)) & (SPL_NB - 1)) << SEG_IDX_BITS;
             }
           }
         }
         const uint32_t shift = SEG_IDX_BITS + (part ? SPL_BITS * p : 0u);
         split_pass<NW>(
-            c0, d, G, sm.sp, [&](int g) { return (x[g] >> shift) & (SPL_NB - 1); },
+            G, sm.sp, [&](int g) { return (x[g] >> shift) & (SPL_NB - 1); },
             [&](int g, uint32_t pos) { sm.at[pos] = x[g]; });
       }
       if (!part) break;
+      // a run's first key sorts it; others read only what the run's keys share
       bool bad = false;
-      for (uint32_t i = threadIdx.x; i + 1 < d; i += NT) bad |= sm.k[sm.at[i] & IM] > sm.k[sm.at[i + 1] & IM];
-      bool done = !__syncthreads_or(bad);
-      for (int round = 0; round < COARSE_REPAIRS && !done; round++) {
-        bad = false;
-        for (uint32_t odd = 0; odd < 2; odd++) {
-          for (uint32_t i = 2 * threadIdx.x + odd; i + 1 < d; i += 2 * NT) {
-            const uint32_t a = sm.at[i], b = sm.at[i + 1];
-            if (sm.k[a & IM] > sm.k[b & IM]) {
-              sm.at[i] = b;
-              sm.at[i + 1] = a;
-              bad = true;
-            }
+      for (uint32_t i = threadIdx.x; i + 1 < d; i += NT) {
+        const uint32_t first = sm.at[i];
+        if ((first ^ sm.at[i + 1]) > IM) continue;
+        if (i && (first ^ sm.at[i - 1]) <= IM) continue;
+        for (uint32_t e = i + 1; e < d; e++) {
+          const uint32_t next = sm.at[e];
+          if ((next ^ first) > IM) break;
+          if (e - i == RUN_MAX) {
+            bad = true;
+            break;
           }
-          __syncthreads();
+          const uint32_t key = sm.k[next & IM];
+          uint32_t j = e;
+          for (; j > i; j--) {
+            const uint32_t prev = sm.at[j - 1];
+            if (sm.k[prev & IM] <= key) break;
+            sm.at[j] = prev;
+          }
+          if (j < e) sm.at[j] = next;
         }
-        done = !__syncthreads_or(bad);
       }
-      if (done) break;
+      if (!__syncthreads_or(bad)) break;
       part = false;
+#pragma unroll
+      for (int g = 0; g < SPL_G; g++) x[g] = c0 + 32u * g + lane < d ? c0 + 32u * g + lane : ~0u;
     }
     if (VALS) {
       cp_async_wait_all();
@@ -1071,13 +1087,20 @@ __global__ void k_dm_perm(const uint32_t* __restrict__ inv, uint64_t n, uint32_t
 // randomly gathered perm array stays resident (evict-last).
 constexpr int DM_INFLIGHT = 8;  // rows whose loads and perm lookups are in flight together
 
-template <bool VALS>
+// The weights of short rows: none, moved with the keys, or fetched by the old
+// position that the low 5 bits of the sorted word hold (labels below 2^27: half
+// the shared memory and a network on one word; R-MAT 2^26 6.4 ms moved, 4.3
+// indexed).
+enum { DM_PLAIN, DM_MOVED, DM_INDEXED };
+
+template <int MODE>
 __global__ void __launch_bounds__(256) k_dm_rows(const uint64_t* __restrict__ rp, const uint32_t* __restrict__ col,
                                                  const uint32_t* __restrict__ w, const uint32_t* __restrict__ inv,
                                                  const uint32_t* __restrict__ perm, const uint64_t* __restrict__ nrp,
                                                  uint32_t* __restrict__ ncol, uint32_t* __restrict__ nw, uint64_t n,
                                                  int skip_big) {
-  extern __shared__ uint32_t dsm[];  // 8 warps x 32 slots of keys, then of weights
+  constexpr bool VALS = MODE != DM_PLAIN, MOVED = MODE == DM_MOVED, IDX = MODE == DM_INDEXED;
+  extern __shared__ uint32_t dsm[];  // 8 warps x 32 slots of keys, then of weights if they are moved
   const int lane = threadIdx.x & 31;
   uint32_t* sk = dsm + (threadIdx.x >> 5) * 32 * SROW;
   uint32_t* sv = dsm + 8 * 32 * SROW + (threadIdx.x >> 5) * 32 * SROW;
@@ -1112,22 +1135,45 @@ __global__ void __launch_bounds__(256) k_dm_rows(const uint64_t* __restrict__ rp
         const uint32_t dq = __shfl_sync(LG_FULL_MASK, d, q[z]);
         on[z] = on[z] && (uint32_t)lane < dq;
         c[z] = on[z] ? ldg_hint(col + lq + lane, pstream) : 0u;
-        if (VALS && on[z]) sv[q[z] * SROW + lane] = ldg_hint(w + lq + lane, pstream);
+        if (MOVED && on[z]) sv[q[z] * SROW + lane] = ldg_hint(w + lq + lane, pstream);
       }
 #pragma unroll
       for (int z = 0; z < DM_INFLIGHT; z++) {
-        if (on[z]) sk[q[z] * SROW + lane] = ldg_hint(perm + c[z], pkeep);
+        if (on[z]) {
+          const uint32_t x = ldg_hint(perm + c[z], pkeep);
+          sk[q[z] * SROW + lane] = IDX ? x << 5 | (uint32_t)lane : x;
+        }
       }
     }
     __syncwarp();
-    warp_sort_slots<VALS>(sk, sv, d, small, lane);
-    for (uint32_t t = todo; t; t &= t - 1) {
-      const int q = __ffs(t) - 1;
-      const uint64_t oq = __shfl_sync(LG_FULL_MASK, o, q);
-      const uint32_t dq = __shfl_sync(LG_FULL_MASK, d, q);
-      if ((uint32_t)lane < dq) {
-        __stcs(ncol + oq + lane, sk[q * SROW + lane]);
-        if (VALS) __stcs(nw + oq + lane, sv[q * SROW + lane]);
+    warp_sort_slots<MOVED>(sk, sv, d, small, lane);
+    for (uint32_t t = todo; t;) {
+      int q[DM_INFLIGHT];
+      uint32_t x[DM_INFLIGHT], y[DM_INFLIGHT];
+#pragma unroll
+      for (int z = 0; z < DM_INFLIGHT; z++) {
+        q[z] = t ? __ffs(t) - 1 : -1;
+        if (t) t &= t - 1;
+      }
+#pragma unroll
+      for (int z = 0; z < DM_INFLIGHT; z++) {
+        const uint64_t lq = IDX ? __shfl_sync(LG_FULL_MASK, lo, max(q[z], 0)) : 0;
+        const uint32_t dq = __shfl_sync(LG_FULL_MASK, d, max(q[z], 0));
+        if (q[z] < 0 || (uint32_t)lane >= dq) q[z] = -1 - max(q[z], 0);  // nothing here
+        x[z] = q[z] >= 0 ? sk[q[z] * SROW + lane] : 0u;
+        y[z] = MOVED && q[z] >= 0 ? sv[q[z] * SROW + lane] : 0u;
+        if (IDX) {
+          if (q[z] >= 0) y[z] = ldg_hint(w + lq + (x[z] & 31u), pstream);
+          x[z] >>= 5;
+        }
+      }
+#pragma unroll
+      for (int z = 0; z < DM_INFLIGHT; z++) {
+        const uint64_t oq = __shfl_sync(LG_FULL_MASK, o, q[z] >= 0 ? q[z] : -1 - q[z]);
+        if (q[z] >= 0) {
+          __stcs(ncol + oq + lane, x[z]);
+          if (VALS) __stcs(nw + oq + lane, y[z]);
+        }
       }
     }
     __syncwarp();
@@ -1155,16 +1201,17 @@ __global__ void __launch_bounds__(256) k_dm_rows(const uint64_t* __restrict__ rp
 // one phase gather from much the same n / P labels, which stay in the L2
 // (gridDim.y = P: blocks start in that order).  Labels go by degree
 // descending, so the rows of a size class are consecutive; a warp takes
-// 2^lg of them and walks their parts as one range of slots, 8 slots a lane in
-// flight.  Rows above SEG_MEDIUM arcs are cut in the radix sort's tiles, each
+// 2^lg of them and walks their parts as one range of slots, 4 slots a lane in
+// flight (8 take more registers: 2 % slower).  Rows above SEG_MEDIUM arcs are cut in the radix sort's tiles, each
 // of which belongs to one phase.
-// R-MAT 2^26, weighted, 2.1 G arcs: 22.4 ms in one phase, 14.1 in 8.
+// R-MAT 2^26, weighted, 2.1 G arcs: 22.4 ms in one phase, 14.0 in 8 (the L2's
+// sectors for the gathers and the arcs' 16 bytes: 7 TB/s).
 // ---------------------------------------------------------------------------
 constexpr uint64_t DM_PART_BYTES = 32ull << 20;  // labels a phase gathers from
 constexpr uint32_t DM_MAX_PARTS = 32;
 constexpr uint32_t DM_TILES = 16;                // tiles a block looks at
 constexpr uint32_t DM_WARP_ARCS = 2048;          // arcs a warp takes in one phase, about
-constexpr int DM_T = 8;
+constexpr int DM_T = 4;
 
 struct DmClass {
   uint32_t first, rows;  // the class's rows
@@ -1438,16 +1485,12 @@ cudaError_t enc_dm_relabel(const uint64_t* rp, const uint32_t* col, const uint32
   // k_dm_rows copies its big rows itself
   const int split_big = mode != 2;
   if (e == cudaSuccess) {
-    const size_t smem = (size_t)8 * 32 * SROW * sizeof(uint32_t) * (w ? 2 : 1);
-    if (w) {
-      e = cudaFuncSetAttribute(k_dm_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e == cudaSuccess)
-        k_dm_rows<true><<<grid_for(n, 256, 152 * 16), 256, smem, st>>>(rp, col, w, inv_perm, perm, nrp, ncol, nw, n,
-                                                                       split_big);
-    } else {
-      k_dm_rows<false><<<grid_for(n, 256, 152 * 16), 256, smem, st>>>(rp, col, w, inv_perm, perm, nrp, ncol, nw, n,
-                                                                      split_big);
-    }
+    const bool moved = w && host_bits(n - 1) > 27;
+    const size_t smem = (size_t)8 * 32 * SROW * sizeof(uint32_t) * (moved ? 2 : 1);
+    const auto rows = !w ? k_dm_rows<DM_PLAIN> : moved ? k_dm_rows<DM_MOVED> : k_dm_rows<DM_INDEXED>;
+    if (moved) e = cudaFuncSetAttribute(rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+      rows<<<grid_for(n, 256, 152 * 16), 256, smem, st>>>(rp, col, w, inv_perm, perm, nrp, ncol, nw, n, split_big);
     count_launch();
     if (e == cudaSuccess) e = cudaGetLastError();
   }
