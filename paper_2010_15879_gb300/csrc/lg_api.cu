@@ -424,7 +424,8 @@ extern "C" lg_status lg_decode(const lg_graph* g, uint64_t* row_ptr, uint32_t* c
   }
   // local IDs: one launch (row offsets by a single-pass look-back over the
   // tiles, then the rows); its small state is zeroed first
-  const uint64_t ntiles = (n + LG_TILE_V - 1) / LG_TILE_V;
+  dec_tiles(n, v.mid_prefix, a);
+  const uint64_t ntiles = a.tiles;
   Tmp t_state(st);
   const size_t bytes = ntiles * (sizeof(unsigned long long) + sizeof(uint32_t)) + 16;
   LG_TRY(t_state.alloc(bytes));

@@ -244,7 +244,31 @@ struct DecArgs {
   uint32_t* ticket;          // next block to start (blocks take tiles in start order)
   int* err;                  // DERR_INTERNAL if a wait for another block ran out
   uint64_t wait_ns;          // limit of each such wait
+  uint64_t tiles_a, tiles;   // tiles of nv_a vertices per warp, which come first; all tiles
+  uint32_t nv_a, nv;         // vertices per warp of these and of the others
 };
+constexpr uint32_t DEC_WARPS = 8;
+__host__ __device__ constexpr uint32_t dec_tile(uint32_t nv) { return DEC_WARPS * nv; }
+// Vertices per warp of the local-ID decode: a lane's four, fewer on graphs that
+// would leave SMs idle, and fewer for the vertices of more than 32 arcs, which
+// come first in DM order, a thousand arcs and more each: in tiles like the
+// others' those blocks were still busy when the rest had ended.  lg_decode,
+// community graphs in DM order, us:
+//   vertices        0.3 M  0.6 M    1 M    2 M    4 M
+//   all 128           223    235    259    290    383
+//   32 first          120    143    165    238    373   (then 64, 64, 128, ..)
+//   16 first          121    146    175    250    402
+//   8 first           116    150    183    264    446
+//   16, then 32       133    170    221    352    608
+//   16, then 64       121    144    184    279    464
+inline void dec_tiles(uint64_t n, uint64_t mid_prefix, DecArgs& a) {
+  const bool large = n >= 4 * 152 * dec_tile(128);  // four blocks for every SM
+  a.nv_a = large ? 32u : 8u;
+  a.nv = large ? 128u : n >= 2 * 152 * dec_tile(64) ? 64u : 32u;
+  a.tiles_a = (mid_prefix + dec_tile(a.nv_a) - 1) / dec_tile(a.nv_a);
+  const uint64_t v = a.tiles_a * dec_tile(a.nv_a);
+  a.tiles = a.tiles_a + (n > v ? (n - v + dec_tile(a.nv) - 1) / dec_tile(a.nv) : 0);
+}
 
 struct TravOps {
   cudaError_t (*pr_init)(const GView&, const PrArgs&, cudaStream_t);

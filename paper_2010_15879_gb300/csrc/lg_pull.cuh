@@ -21,7 +21,7 @@
 // reader; heavy items by warp) and now: R-MAT 2^16 60 -> 17 us, R-MAT 2^18 in
 // DM order 376 -> 40 us, 2^22 597 -> 355 us, 2^24 1.75 -> 1.61 ms (not
 // relabeled 3.63 -> 2.10), 2^26 8.95 -> 7.08 ms (297 G arcs/s); community 2^24
-// in local-gap IDs 1.99 -> 1.93 ms, in global IDs 1.93 -> 1.55 ms.
+// in local-gap IDs 1.99 -> 1.90 ms, in global IDs 1.93 -> 1.55 ms.
 #pragma once
 
 #include "lg_internal.h"
@@ -221,21 +221,23 @@ struct LightTile {
 // info of a light vertex (local modes): width << 26 | base, its field f of the
 // tile is at bit (base + f * width) mod 2^26; gap mode: the fields after the
 // first, which holds s bits and begins s - width bits before that formula
-template <int IDM, int OFF>
-__device__ __forceinline__ void light_tile(const GView& g, uint64_t v0, uint32_t nv, uint64_t p0, PrWarp& W,
-                                           LightTile& T) {
+//
+// x: the offsets of the owned vertices, xe of ve.  seen(q, d, h): owned vertex
+// q has degree d, h its number among the tile's heavy vertices (or ~0).
+template <int IDM, class Seen>
+__device__ __forceinline__ void light_geometry(const GView& g, uint64_t v0, uint64_t ve, const uint64_t (&x)[PW_VPL],
+                                               uint64_t xe, PrWarp& W, LightTile& T, Seen seen) {
   const uint32_t lane = threadIdx.x & 31u, lt = lane_lt_mask();
   constexpr bool FLAT = IDM == ID_GLOBAL || IDM == ID_CSR32;
   const uint32_t rw = FLAT ? (IDM == ID_GLOBAL ? g.r : 32u) : 1u;  // stream bits per unit of an offset
-  const uint64_t ve = min(g.n, v0 + nv);
-  uint64_t x[PW_VPL], xe;
-  warp_offsets<OFF>(g, v0, nv, p0, W.stage[0], x, xe);
   const uint64_t first = __shfl_sync(LG_FULL_MASK, x[0], 0) * rw;
   T.tb = first & ~127ull;
   T.first = (uint32_t)(first - T.tb);
   T.F = 0;
   T.NH = 0;
-  uint32_t NL = 0;
+  uint32_t NL = 0, head[PW_VPL];  // the headers' loads go out together
+#pragma unroll
+  for (int q = 0; q < PW_VPL; q++) head[q] = v0 + lane + 32u * q < ve ? vhead<IDM>(g, x[q]) : 0u;
 #pragma unroll
   for (int q = 0; q < PW_VPL; q++) {
     uint64_t x1 = __shfl_down_sync(LG_FULL_MASK, x[q], 1);
@@ -243,7 +245,7 @@ __device__ __forceinline__ void light_tile(const GView& g, uint64_t v0, uint32_t
     if (lane == 31) x1 = nx;
     uint64_t start = 0;
     uint32_t d = 0, w = 0;
-    if (v0 + lane + 32u * q < ve) vgeo<IDM>(g, x[q], x1, start, d, w);
+    if (v0 + lane + 32u * q < ve) vgeo<IDM>(g, x[q], x1, head[q], start, d, w);
     const bool heavy = d > g.heavy_min, light = d > 0 && !heavy;
     const uint32_t lf = heavy ? 0u : d;
     const uint32_t incl = warp_incl_scan<uint32_t>(lf);
@@ -265,9 +267,18 @@ __device__ __forceinline__ void light_tile(const GView& g, uint64_t v0, uint32_t
       W.info[h] = ((uint32_t)(after >> 32) << 19) | fp;
       W.vsum[h] = __uint_as_float((uint32_t)after);
     }
+    seen(q, d, heavy ? T.NH + __popc(hm & lt) : ~0u);
     T.NH += __popc(hm);
   }
   __syncwarp();
+}
+
+template <int IDM, int OFF>
+__device__ __forceinline__ void light_tile(const GView& g, uint64_t v0, uint32_t nv, uint64_t p0, PrWarp& W,
+                                           LightTile& T) {
+  uint64_t x[PW_VPL], xe;
+  warp_offsets<OFF>(g, v0, nv, p0, W.stage[0], x, xe);
+  light_geometry<IDM>(g, v0, min(g.n, v0 + nv), x, xe, W, T, [](int, uint32_t, uint32_t) {});
 }
 
 // A window: fields [f0, f0 + nf) of the tile, inside one run of light fields
@@ -343,24 +354,20 @@ __device__ __forceinline__ void decode_window(const GView& g, const Window& wd, 
     for (int e = 0; e < PW_E; e++, p += rw) id[e] = sh_bits(p) & mask;
     return;
   }
-  const uint32_t s = g.s;
-  uint32_t v = 0, p = 0, w = 0, mask = 0;
-  auto enter = [&](uint32_t e, uint32_t f) {
-    w = e >> PW_POS_BITS;
-    p = ((e + f * w - wd.ro) & PW_POSM) + wd.at;
-    mask = mask_lo(w);
-  };
-  const uint32_t n8 = k0 < wd.nf ? min(wd.nf - k0, (uint32_t)PW_E) : 0u;
-  if (n8 && !(hb & 1u)) enter(W.info[je], wd.f0 + k0);
-  int j = je;
+  // A field's place comes from its vertex's info alone, so that no lane waits
+  // for one that enters a vertex there (a step per entered vertex: 4 % more
+  // instructions in a whole-graph decode).
+  const uint32_t n8 = k0 < wd.nf ? wd.nf - k0 : 0u, rel = wd.ro;
+  uint32_t v = 0;
+  int j = je;  // -1 only before the tile's first field
 #pragma unroll
   for (int e = 0; e < PW_E; e++) {
     const bool head = (hb >> e) & 1u;
-    if (head) enter(W.info[++j], wd.f0 + k0 + e);
-    const bool wide = IDM == ID_LOCAL_GAP && head;  // an absolute ID of s bits
-    uint32_t x = 0;
-    if (e < n8) x = sh_bits(wide ? p - (s - w) : p) & (wide ? mask_lo(s) : mask);
-    p += w;
+    j += head;
+    const uint32_t i = e < n8 ? W.info[j] : 0u, w = i >> PW_POS_BITS;
+    const uint32_t bits = IDM == ID_LOCAL_GAP && head ? g.s : w;  // a first field is an absolute ID of s bits
+    const uint32_t p = (i + (wd.f0 + k0 + e) * w - rel) & PW_POSM;
+    const uint32_t x = e < n8 ? sh_bits(p + wd.at - (bits - w)) & mask_lo(bits) : 0u;
     v = IDM == ID_LOCAL_GAP && !head ? v + x : x;
     id[e] = v;
   }

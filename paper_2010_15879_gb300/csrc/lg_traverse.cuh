@@ -84,8 +84,6 @@ __device__ __forceinline__ void write_depths(const BfsArgs& a, uint64_t n, uint6
 // offsets of a tile: xs[i] = x_{v0+i}, i = 0..cnt (cnt+1 values)
 // ---------------------------------------------------------------------------
 struct TileScratch {
-  uint32_t cum[TNT];
-  uint32_t w[TNT];
   uint32_t red[TNT / 32];
 };
 
@@ -105,7 +103,9 @@ __device__ __forceinline__ void tile_offsets<OFF_ROWPTR>(const GView& g, uint64_
 }
 
 // Elias-Fano block decode (Section 4.3): ones number v0 .. v0+cnt of the high
-// vector, starting from the sample at or below v0.
+// vector, starting from the sample at or below v0.  A thread lists the ones of
+// its word: some twelve, while a search of the words' ranks for every one took
+// a hundred instructions each.
 template <>
 __device__ __forceinline__ void tile_offsets<OFF_EF>(const GView& g, uint64_t v0, int cnt, uint64_t* xs,
                                                      TileScratch& ts) {
@@ -113,38 +113,36 @@ __device__ __forceinline__ void tile_offsets<OFF_EF>(const GView& g, uint64_t v0
   const uint64_t p0 = __ldg(g.ef_samples + k);
   const uint64_t skip = v0 - (k << g.sample_log2);
   const uint64_t need_end = skip + (uint64_t)cnt + 1;
-  uint64_t wbase = p0 >> 5;
-  uint64_t carry = 0;
-  bool first = true;
-  while (carry < need_end && wbase < g.ef_high_words32) {
+  uint64_t wbase = (p0 >> 5) & ~3ull, carry = 0;
+  auto list = [&](uint32_t w, uint64_t wi, int64_t i) {  // the word's first one is that of vertex v0 + i
+    for (; w && i <= cnt; i++, w &= w - 1u)
+      if (i >= 0) xs[i] = wi * 32u + (uint32_t)__ffs((int)w) - 1u;
+  };
+  uint32_t total;
+  {
     const uint64_t wi = wbase + threadIdx.x;
-    uint32_t w = wi < g.ef_high_words32 ? __ldg(g.ef_high32 + wi) : 0u;
-    if (first && threadIdx.x == 0) w &= (0xffffffffu << ((uint32_t)p0 & 31u));
-    uint32_t total;
+    uint32_t w = wi < g.ef_high_words32 && wi >= (p0 >> 5) ? __ldg(g.ef_high32 + wi) : 0u;
+    if (wi == (p0 >> 5)) w &= 0xffffffffu << ((uint32_t)p0 & 31u);
     const uint32_t pre = block_excl_scan<uint32_t, TNT>((uint32_t)__popc(w), total, ts.red);
-    ts.cum[threadIdx.x] = pre;
-    ts.w[threadIdx.x] = w;
-    __syncthreads();
-    const uint64_t r_lo = carry > skip ? carry : skip;
-    const uint64_t r_hi = (carry + total) < need_end ? (carry + total) : need_end;
-    for (uint64_t r = r_lo + threadIdx.x; r < r_hi; r += TNT) {
-      const uint32_t local = (uint32_t)(r - carry);
-      int lo = 0, hi = TNT - 1;
-      while (lo < hi) {
-        const int m = (lo + hi + 1) >> 1;
-        if (ts.cum[m] <= local) lo = m; else hi = m - 1;
-      }
-      const uint64_t pos = (wbase + (uint64_t)lo) * 32u + select_in_u32(ts.w[lo], local - ts.cum[lo]);
-      const uint64_t i = r - skip;
-      xs[i] = (pos - (v0 + i)) << g.ef_l;
-    }
-    carry += total;
-    wbase += TNT;
-    first = false;
-    __syncthreads();
+    list(w, wi, (int64_t)pre - (int64_t)skip);
   }
-  if (g.ef_l)
-    for (int i = threadIdx.x; i <= cnt; i += TNT) xs[i] |= ext64(g.ef_low, (v0 + i) * g.ef_l, g.ef_l);
+  // hubs spread a tile over thousands of words: four per thread from here on
+  for (carry = total, wbase += TNT; carry < need_end && wbase < g.ef_high_words32; carry += total, wbase += 4 * TNT) {
+    const uint64_t wi = wbase + 4u * threadIdx.x;  // the array is padded to 16 bytes with zeros
+    const uint4 y = wi < g.ef_high_words32 ? ldg128(g.ef_high32 + wi) : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t c0 = __popc(y.x), c1 = c0 + __popc(y.y), c2 = c1 + __popc(y.z);
+    const uint32_t pre = block_excl_scan<uint32_t, TNT>(c2 + __popc(y.w), total, ts.red);
+    const int64_t i = (int64_t)(carry + pre) - (int64_t)skip;
+    list(y.x, wi, i);
+    list(y.y, wi + 1, i + c0);
+    list(y.z, wi + 2, i + c1);
+    list(y.w, wi + 3, i + c2);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i <= cnt; i += TNT) {
+    const uint64_t lo = g.ef_l ? ext64(g.ef_low, (v0 + i) * g.ef_l, g.ef_l) : 0u;
+    xs[i] = ((xs[i] - (v0 + i)) << g.ef_l) | lo;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -225,22 +223,31 @@ __device__ __forceinline__ void offset_pair<OFF_EF>(const GView& g, uint64_t v, 
 //   start: bit of the first field; w: field width (IDs, or gaps for LOCAL_GAP)
 // ---------------------------------------------------------------------------
 template <int IDM>
-__device__ __forceinline__ void vgeo(const GView& g, uint64_t x0, uint64_t x1, uint64_t& start, uint32_t& deg,
-                                     uint32_t& w) {
+__device__ __forceinline__ uint32_t vhead(const GView& g, uint64_t x0) {  // the header of a neighborhood, if it has one
+  return IDM == ID_LOCAL || IDM == ID_LOCAL_GAP ? ext32(g.A32, x0, g.H) : 0u;
+}
+template <int IDM>
+__device__ __forceinline__ void vgeo(const GView& g, uint64_t x0, uint64_t x1, uint32_t head, uint64_t& start,
+                                     uint32_t& deg, uint32_t& w) {
   if (IDM == ID_GLOBAL) {
     start = x0 * g.r; deg = (uint32_t)(x1 - x0); w = g.s;
   } else if (IDM == ID_CSR32) {
     start = x0 * 32u; deg = (uint32_t)(x1 - x0); w = 32;
   } else if (IDM == ID_LOCAL) {
-    w = ext32(g.A32, x0, g.H);
+    w = head;
     deg = w ? (uint32_t)udiv_small(x1 - x0 - g.H, w) : 0u;
     start = x0 + g.H;
   } else {
-    w = ext32(g.A32, x0, g.H);
+    w = head;
     const uint64_t len = x1 - x0;
     deg = len == g.H ? 0u : (w == 0 ? 1u : 1u + (uint32_t)udiv_small(len - g.H - g.s, w));
     start = x0 + g.H;
   }
+}
+template <int IDM>
+__device__ __forceinline__ void vgeo(const GView& g, uint64_t x0, uint64_t x1, uint64_t& start, uint32_t& deg,
+                                     uint32_t& w) {
+  vgeo<IDM>(g, x0, x1, vhead<IDM>(g, x0), start, deg, w);
 }
 
 // First schedule item of heavy vertex v (a warp; the items are in vertex order).
@@ -1222,17 +1229,6 @@ __global__ void __launch_bounds__(256) k_nbr_rows(GView g, NbrArgs a) {
 // consecutive threads on consecutive records (coalesced stream reads and
 // coalesced writes, no vertex lookup).  Local IDs: one
 // kernel, described above k_dec_local.
-//
-// Local IDs: a degree pass and a scan give the row offsets, then tiles of TV
-// vertices decode their offsets once and split the tile's light fields into
-// rounds of DEC_C fields.  In a round every thread decodes a contiguous run of
-// fields sequentially (bit reader, one shift and mask per field, a running sum
-// for gaps), entering its first neighborhood mid-way if need be, into a
-// shared-memory stage; the stage is then written out coalesced.  A run that
-// starts inside a gap-coded neighborhood sums its gaps from 0; a segmented
-// scan over the threads' last values (absolute once the neighborhood's first
-// field has been read) supplies the missing prefix.  Heavy vertices come from
-// the heavy schedule, a warp per item, a lane per field.
 // ===========================================================================
 template <int IDM, int U>
 __device__ __forceinline__ void dec_fields(const GView& g, const DecArgs& a, uint64_t start, uint32_t w, uint32_t f0,
@@ -1315,45 +1311,42 @@ __global__ void __launch_bounds__(256) k_dec_flat(GView g, DecArgs a, uint64_t p
 // Local-ID decode: one launch writes row_ptr and every row.
 //
 // Blocks take a ticket when they start: tickets below the tile count are tile
-// CTAs (tiles in start order), the rest are heavy-schedule CTAs.  A tile CTA
-// decodes its offsets and geometry, publishes its arc count, and finds the
-// arcs of all earlier tiles by a decoupled look-back over their published
-// counts (a tile waits only on tiles that started before it).  It writes its
-// row offsets, flags them ready (heavy items read their row start there), and
-// then decodes its light vertices window by window: a window is up to DEC_C
-// light fields of one run of light vertices with no heavy vertex between them,
-// so its stream bits are contiguous; they are staged in shared memory with
-// 16-byte loads, every thread decodes DEC_C / TNT consecutive fields from
-// there (a shift and a mask per field, a running sum for gaps), a segmented
-// scan over the threads supplies the prefix of gap runs entered mid-way, and
-// the window is written out coalesced.
+// CTAs (tiles in start order), the rest are heavy-schedule CTAs, a warp per
+// item.  A tile CTA decodes its offsets together; then each warp has its own
+// vertices (see dec_tiles) as in the pull sweep: geometry, and the arcs counted.  The
+// CTA publishes its arc count, finds the arcs of all earlier tiles by a
+// decoupled look-back over their published counts (a tile waits only on tiles
+// that started before it) while its warps' first windows are on their way, and
+// writes its row offsets, flagged ready for the heavy items.  The warps then
+// decode window by window -- 256 fields, 8 consecutive ones per lane, the next
+// window's words in flight -- and write a window's IDs coalesced by way of
+// shared memory.
+//
+// What bounds it is instructions and the blocks' start: 2.6 warp instructions
+// a field, 3.3 with a serial reader per lane and vertex.  4 M vertices, 94 M arcs in
+// local-gap IDs: 438 us before, 307 now, of which the offsets, the geometry and
+// the look-back take half (18 us a block, overlapped by the SM's other three).
 // ---------------------------------------------------------------------------
-constexpr int DEC_P = 9;                   // light fields per lane and window (odd: the lanes' stage
-                                           // stores fall in distinct banks)
-constexpr int DEC_WF = 32 * DEC_P;         // light fields per warp window
-constexpr int DEC_WCAP = 400;              // stream words a warp window may stage (longer windows shrink)
 constexpr uint64_t DEC_AGG = 1ull << 62, DEC_INCL = 2ull << 62, DEC_VAL = (1ull << 62) - 1;
-
-struct DecWarp {
-  __align__(16) uint32_t words[DEC_WCAP + 8];  // stream words of the warp's current window
-  uint32_t stage[DEC_WF];                      // decoded IDs of the warp's current window
-};
+static_assert(DEC_WARPS == TNT / 32, "a warp tile per warp");
 
 struct DecSmem {
-  TileSmem t;                  // offsets (xs, reused for the all-degree prefix), geometry, light list
-  DecWarp w[TNT / 32];
-  uint64_t rdelta[TV];         // per run of light vertices: output index - light field index
-  uint16_t rfirst[TV + 1];     // per run: its first light index
-  uint64_t base;               // arcs of all earlier tiles
-  uint64_t scan2[2 * (TNT / 32)];
-  uint32_t nruns, ticket, ok;
+  PrWarp w[DEC_WARPS];
+  uint32_t hdeg[DEC_WARPS][PW_TV];  // degrees of the warp tile's heavy vertices
+  union {
+    uint64_t xs[DEC_WARPS * PW_TV + 1];               // the tile's offsets, until the geometry is known
+    __align__(16) uint32_t out[DEC_WARPS][PW_WF];     // a window's IDs
+  };
+  TileScratch ts;
+  uint64_t sums[DEC_WARPS];  // arcs of each warp tile, then of those before it
+  uint64_t base;             // arcs of all earlier tiles
+  uint32_t ticket, ok;
 };
 
-static_assert(sizeof(DecSmem) <= 44 * 1024, "five decode CTAs per SM");
-
-__device__ __forceinline__ uint64_t ld_acquire_u64(const unsigned long long* p) {
+// flag and count of a tile are one word: nothing else is read on its account
+__device__ __forceinline__ uint64_t ld_relaxed_u64(const unsigned long long* p) {
   uint64_t v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_release_u64(unsigned long long* p, uint64_t v) {
@@ -1373,22 +1366,6 @@ __device__ __forceinline__ uint64_t dec_clock_ns() {
   return t;
 }
 
-// bit of light field k of a vertex starting at bit st with field width w
-template <int IDM>
-__device__ __forceinline__ uint64_t dec_pos(uint64_t st, uint32_t k, uint32_t w, uint32_t s) {
-  if (IDM == ID_LOCAL_GAP) return k == 0 ? st : st + s + (uint64_t)(k - 1) * w;
-  return st + (uint64_t)k * w;
-}
-template <int IDM>
-__device__ __forceinline__ uint32_t dec_width(uint32_t k, uint32_t w, uint32_t s) {
-  return (IDM == ID_LOCAL_GAP && k == 0) ? s : w;
-}
-
-// segmented combine of (absolute?, value) pairs: x = e then x
-__device__ __forceinline__ void seg_after(uint32_t& xf, uint32_t& xv, uint32_t ef, uint32_t ev) {
-  if (!xf) { xv += ev; xf = ef; }
-}
-
 // Arcs of all tiles before tile b (warp 0 of the tile CTA; the result in lane 0).
 // Returns false if a wait ran out.
 __device__ __forceinline__ bool dec_lookback(const DecArgs& a, uint64_t b, uint64_t& base) {
@@ -1398,7 +1375,7 @@ __device__ __forceinline__ bool dec_lookback(const DecArgs& a, uint64_t b, uint6
   const uint64_t t0 = dec_clock_ns();
   uint64_t spins = 0;
   while (true) {
-    const uint64_t v = p >= 0 ? ld_acquire_u64(a.tile_status + p) : DEC_INCL;  // nothing before tile 0
+    const uint64_t v = p >= 0 ? ld_relaxed_u64(a.tile_status + p) : DEC_INCL;  // nothing before tile 0
     const uint64_t flag = v >> 62;
     const uint32_t incl = __ballot_sync(LG_FULL_MASK, flag == 2);
     const uint32_t stop = incl ? (uint32_t)(__ffs(incl) - 1) : 31u;  // nearest inclusive prefix
@@ -1415,11 +1392,9 @@ __device__ __forceinline__ bool dec_lookback(const DecArgs& a, uint64_t b, uint6
 }
 
 template <int IDM, int OFF>
-__global__ void __launch_bounds__(TNT, 5) k_dec_local(GView g, DecArgs a) {
-  extern __shared__ __align__(16) unsigned char dec_smem_raw[];
-  DecSmem& sm = *reinterpret_cast<DecSmem*>(dec_smem_raw);
-  TileSmem& ts = sm.t;
-  const uint64_t ntiles = (g.n + TV - 1) / TV;
+__global__ void __launch_bounds__(TNT, 4) k_dec_local(GView g, DecArgs a) {
+  DecSmem& sm = *reinterpret_cast<DecSmem*>(dyn_smem);
+  const uint64_t ntiles = a.tiles, va = a.tiles_a * dec_tile(a.nv_a);  // from vertex va on tiles of a.nv per warp
   if (threadIdx.x == 0) sm.ticket = atomicAdd(a.ticket, 1u);
   __syncthreads();
   const uint64_t b = sm.ticket;
@@ -1432,9 +1407,11 @@ __global__ void __launch_bounds__(TNT, 5) k_dec_local(GView g, DecArgs a) {
     uint64_t o = 0;
     bool ok = true;
     if (lane == 0) {
+      const uint32_t* ready =
+          a.tile_ready + (h.v < va ? h.v / dec_tile(a.nv_a) : a.tiles_a + (h.v - va) / dec_tile(a.nv));
       const uint64_t t0 = dec_clock_ns();
       uint64_t spins = 0;
-      while (ld_acquire_u32(a.tile_ready + h.v / TV) == 0) {
+      while (ld_acquire_u32(ready) == 0) {
         if (++spins > (a.wait_ns >> 5) + 1024 || ((spins & 63u) == 0 && dec_clock_ns() - t0 > a.wait_ns)) {
           ok = false;
           break;
@@ -1449,223 +1426,112 @@ __global__ void __launch_bounds__(TNT, 5) k_dec_local(GView g, DecArgs a) {
     dec_fields<IDM, HEAVY_U>(g, a, h.bit, h.w, h.f0, h.f0 + h.nf, h.carry, o);
     return;
   }
-  // ---- tile: offsets and geometry
-  const uint64_t v0 = b * TV;
-  const int cnt = (int)min((uint64_t)TV, g.n - v0);
-  tile_offsets<OFF>(g, v0, cnt, ts.xs, ts.ts);
+  // ---- the tile's offsets, then each warp's own vertices
+  const uint32_t nv = b < a.tiles_a ? a.nv_a : a.nv;
+  const uint64_t v0 = b < a.tiles_a ? b * dec_tile(a.nv_a) : va + (b - a.tiles_a) * dec_tile(a.nv);
+  const uint32_t cnt = (uint32_t)min((uint64_t)dec_tile(nv), g.n - v0);
+  tile_offsets<OFF>(g, v0, (int)cnt, sm.xs, sm.ts);
   __syncthreads();
-  uint32_t lc = 0, lf = 0, hc = 0;
-  uint64_t all = 0;
-  bool light[TV / TNT];
-  uint32_t dq[TV / TNT];
-#pragma unroll
-  for (int q = 0; q < TV / TNT; q++) {
-    const int i = threadIdx.x * (TV / TNT) + q;
-    light[q] = false;
-    dq[q] = 0;
-    if (i < cnt) {
-      uint64_t start; uint32_t d, w;
-      vgeo<IDM>(g, ts.xs[i], ts.xs[i + 1], start, d, w);
-      ts.st[i] = start; ts.deg[i] = d; ts.wid[i] = (uint8_t)w;
-      dq[q] = d;
-      all += d;
-      if (d > 0 && d <= g.heavy_min) { light[q] = true; lc++; lf += d; }
-      hc += d > g.heavy_min;
-    }
-  }
-  // one pass over the block: (heavy count, light count, light fields) packed
-  // into 16 / 16 / 32 bits, and the sum of all degrees
-  uint64_t lpre, apre, ltot, atot;
-  block_excl_scan2<uint64_t, TNT>(((uint64_t)hc << 48) | ((uint64_t)lc << 32) | lf, all, lpre, apre, ltot, atot,
-                                  sm.scan2);  // xs reads are done
-  const bool no_heavy = (ltot >> 48) == 0;
-  ltot &= (1ull << 48) - 1;
-  lpre &= (1ull << 48) - 1;
-  uint64_t* pre_all = ts.xs;  // reused: in-tile exclusive prefix of all degrees
+  PrWarp& W = sm.w[wid];
+  const uint32_t i0 = min(cnt, wid * nv), i1 = min(cnt, i0 + nv);
+  uint64_t ap[PW_VPL], total = 0;  // arcs of the warp tile before each owned vertex, and in all
+  LightTile T;
   {
-    uint32_t ci = (uint32_t)(lpre >> 32), cf = (uint32_t)lpre;
-    uint64_t ca = apre;
+    uint64_t x[PW_VPL];
+    uint32_t deg[PW_VPL];
 #pragma unroll
-    for (int q = 0; q < TV / TNT; q++) {
-      const int i = threadIdx.x * (TV / TNT) + q;
-      if (i < cnt) pre_all[i] = ca;
-      ca += dq[q];
-      if (light[q]) {
-        ts.clist[ci] = (uint16_t)i;
-        ts.fpre[ci] = cf;
-        ci++;
-        cf += dq[q];
-      }
+    for (int q = 0; q < PW_VPL; q++) x[q] = sm.xs[min(i1, i0 + lane + 32u * q)];
+    light_geometry<IDM>(g, v0 + i0, v0 + i1, x, sm.xs[i1], W, T, [&](int q, uint32_t d, uint32_t h) {
+      deg[q] = d;
+      if (h != ~0u) sm.hdeg[wid][h] = d;
+    });
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < PW_VPL; q++) {
+      const uint64_t incl = T.NH ? warp_incl_scan<uint64_t>(deg[q]) : warp_incl_scan<uint32_t>(deg[q]);
+      ap[q] = total + incl - deg[q];
+      total += __shfl_sync(LG_FULL_MASK, incl, 31);
     }
   }
-  if (threadIdx.x == 0) {
-    ts.nlight = (uint32_t)(ltot >> 32);
-    ts.nfields = (uint32_t)ltot;
-    ts.fpre[ts.nlight] = (uint32_t)ltot;
-    sm.ok = 1;
-  }
-  // ---- arcs before this tile (decoupled look-back), then the row offsets
+  if (lane == 0) sm.sums[wid] = total;
+  // ---- the first window is on its way while the CTA finds the arcs before its tile
+  const uint64_t pol = policy_stream();
+  int jb = -1, ja = -1;  // the light vertices open before and after the window
+  Window cur, nxt;
+  nxt.f0 = nxt.nf = nxt.fcur = 0;
+  nxt.h = 0;
+  nxt.fend = T.NH ? W.info[PW_TV - 1] & ((1u << 19) - 1u) : T.F;
+  nxt.rbit = T.tb + T.first;
+  nxt.at = nxt.ro = 0;
+  uint32_t gcarry = 0, buf = 0, hseen = 0;
+  bool more = next_window(T, W, PW_WF, nxt);
+  if (more) ja = open_window<IDM>(g, T, nxt, 0, -1, pol, W);
+  __syncthreads();
   if (wid == 0) {
+    const uint64_t mine = lane < DEC_WARPS ? sm.sums[lane] : 0;
+    const uint64_t incl = warp_incl_scan<uint64_t>(mine), all = __shfl_sync(LG_FULL_MASK, incl, 31);
+    if (lane < DEC_WARPS) sm.sums[lane] = incl - mine;
+    if (lane == 0) st_release_u64(a.tile_status + b, (b == 0 ? DEC_INCL : DEC_AGG) | all);
+    uint64_t before = 0;
+    const bool ok = b == 0 || dec_lookback(a, b, before);
     if (lane == 0) {
-      if (b == 0) st_release_u64(a.tile_status, DEC_INCL | atot);
-      else st_release_u64(a.tile_status + b, DEC_AGG | atot);
-    }
-    uint64_t base = 0;
-    bool ok = true;
-    if (b > 0) ok = dec_lookback(a, b, base);
-    if (lane == 0) {
-      if (!ok) { atomicOr(a.err, DERR_INTERNAL); sm.ok = 0; }
-      if (b > 0) st_release_u64(a.tile_status + b, DEC_INCL | (base + atot));
-      sm.base = base;
+      if (!ok) atomicOr(a.err, DERR_INTERNAL);
+      if (b > 0) st_release_u64(a.tile_status + b, DEC_INCL | (before + all));
+      sm.base = before;
+      sm.ok = ok;
+      if (v0 + cnt == g.n) a.row_out[g.n] = before + all;
     }
   }
   __syncthreads();
-  if (!sm.ok) return;
-  const uint64_t base = sm.base;
-  for (int i = threadIdx.x; i < cnt; i += TNT) a.row_out[v0 + i] = base + pre_all[i];
-  if (v0 + (uint64_t)cnt == g.n && threadIdx.x == 0) a.row_out[g.n] = base + atot;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    st_release_u32(a.tile_ready + b, 1u);
+  if (!sm.ok) {
+    stage_wait<0>();
+    return;
   }
-  const uint32_t nl = ts.nlight;
-  if (nl == 0) return;
-  // ---- runs of light vertices with contiguous output rows (a heavy vertex breaks a run)
-  if (no_heavy) {  // one run
+  uint64_t base = sm.base + sm.sums[wid];  // arcs before the warp tile; later also its heavy ones passed
+#pragma unroll
+  for (int q = 0; q < PW_VPL; q++)
+    if (i0 + lane + 32u * q < i1) a.row_out[v0 + i0 + lane + 32u * q] = base + ap[q];
+  if (g.n_items) {  // heavy items read their row's start
+    __syncthreads();
     if (threadIdx.x == 0) {
-      sm.nruns = 1;
-      sm.rfirst[0] = 0;
-      sm.rfirst[1] = (uint16_t)nl;
-      sm.rdelta[0] = base + pre_all[ts.clist[0]];
+      __threadfence();
+      st_release_u32(a.tile_ready + b, 1u);
     }
-  } else {
-    uint32_t fl[TV / TNT], c = 0;
-    uint64_t dl[TV / TNT];
-#pragma unroll
-    for (int q = 0; q < TV / TNT; q++) {
-      const uint32_t j = threadIdx.x * (TV / TNT) + q;
-      fl[q] = 0;
-      dl[q] = 0;
-      if (j < nl) {
-        // output index of light field f is row_ptr[v] + (f - fpre[j]): constant offset
-        // along light vertices with only zero-degree vertices between them
-        dl[q] = base + pre_all[ts.clist[j]] - (uint64_t)ts.fpre[j];
-        fl[q] = j == 0 || dl[q] != base + pre_all[ts.clist[j - 1]] - (uint64_t)ts.fpre[j - 1];
-        c += fl[q];
-      }
-    }
-    uint32_t total;
-    uint32_t pos = block_excl_scan<uint32_t, TNT>(c, total, ts.ts.red);
-#pragma unroll
-    for (int q = 0; q < TV / TNT; q++) {
-      const uint32_t j = threadIdx.x * (TV / TNT) + q;
-      if (fl[q]) { sm.rfirst[pos] = (uint16_t)j; sm.rdelta[pos] = dl[q]; pos++; }
-    }
-    if (threadIdx.x == 0) { sm.nruns = total; sm.rfirst[total] = (uint16_t)nl; }
   }
-  __syncthreads();
-  // ---- warps: ranges of whole light vertices balanced by fields, decoded in
-  // windows of up to DEC_WF fields that never cross a run (contiguous stream
-  // bits, one output offset); lanes decode DEC_P consecutive fields each
-  {
-    const uint32_t s = g.s, F = ts.nfields;
-    const uint32_t* fpre = ts.fpre;
-    DecWarp& W = sm.w[wid];
-    // warp range: from the first light vertex starting at or after F * wid / 8
-    // to the one starting at or after F * (wid + 1) / 8
-    auto first_at_or_after = [&](uint32_t target) {
-      uint32_t lo = 0, hi = nl;
-      while (lo < hi) { const uint32_t m = (lo + hi) >> 1; if (fpre[m] < target) lo = m + 1; else hi = m; }
-      return lo;
-    };
-    const uint32_t jr0 = first_at_or_after((uint32_t)((uint64_t)F * wid / (TNT / 32)));
-    const uint32_t jr1 = wid + 1 == TNT / 32 ? nl : first_at_or_after((uint32_t)((uint64_t)F * (wid + 1) / (TNT / 32)));
-    const uint32_t Rend = fpre[jr1];
-    // the last light vertex holding field f, searched in [lo, hi]
-    auto vertex_of = [&](uint32_t f, uint32_t lo, uint32_t hi) {
-      while (lo < hi) { const uint32_t m = (lo + hi + 1) >> 1; if (fpre[m] <= f) lo = m; else hi = m - 1; }
-      return lo;
-    };
-    uint32_t q = 0;           // run holding W0
-    uint32_t wcarry = 0;      // absolute ID of the field before W0 (gap mode, W0 inside a vertex)
-    for (uint32_t W0 = fpre[jr0]; W0 < Rend;) {
-      while (q + 1 < sm.nruns && fpre[sm.rfirst[q + 1]] <= W0) q++;
-      const uint32_t RE = min(Rend, fpre[sm.rfirst[q + 1]]);
-      uint32_t Fw = min((uint32_t)DEC_WF, RE - W0);
-      const uint32_t ja = vertex_of(W0, jr0, jr1 - 1);
-      const int ia = ts.clist[ja];
-      const uint64_t bA = dec_pos<IDM>(ts.st[ia], W0 - fpre[ja], ts.wid[ia], s);
-      const uint64_t wA = (bA >> 5) & ~3ull;
-      uint32_t jb, nw;
-      while (true) {  // shrink the window until its stream words fit
-        jb = vertex_of(W0 + Fw - 1, ja, jr1 - 1);
-        const int ib = ts.clist[jb];
-        const uint32_t kb = W0 + Fw - 1 - fpre[jb];
-        const uint64_t bB = dec_pos<IDM>(ts.st[ib], kb, ts.wid[ib], s) + dec_width<IDM>(kb, ts.wid[ib], s);
-        nw = (uint32_t)(((bB + 31) >> 5) + 1 - wA);
-        if (nw <= DEC_WCAP || Fw == 1) break;
-        Fw = (Fw + 1) >> 1;
-      }
-      const uint4* src = reinterpret_cast<const uint4*>(g.A32 + wA);
-      uint4* dst = reinterpret_cast<uint4*>(W.words);
-      for (uint32_t x = lane; x * 4 < nw; x += 32) dst[x] = __ldcs(src + x);
-      __syncwarp();
-      const uint32_t fa = W0 + Fw * lane / 32, fb = W0 + Fw * (lane + 1) / 32;
-      uint32_t lastf = 0, lastv = 0, pend = fa;
-      if (fa < fb) {
-        uint32_t j = vertex_of(fa, ja, jb), f = fa, k = fa - fpre[j];
-        pend = k ? min(fb, fpre[j + 1]) : fa;  // fields of a neighborhood entered mid-way
-        const uint64_t wbase = wA * 32;
-        while (f < fb) {
-          const int i = ts.clist[j];
-          const uint32_t w = ts.wid[i], mw = mask_lo(w);
-          uint32_t m = min(ts.deg[i] - k, fb - f);
-          uint32_t* out = W.stage + (f - W0);
-          f += m;
-          uint32_t p = (uint32_t)(dec_pos<IDM>(ts.st[i], k, w, s) - wbase);
-          uint32_t run = 0;
-          if (IDM == ID_LOCAL_GAP && k == 0) {
-            run = __funnelshift_r(W.words[p >> 5], W.words[(p >> 5) + 1], p & 31u) & mask_lo(s);
-            *out++ = run;
-            p += s;
-            m--;
-          }
-          for (; m; m--) {
-            const uint32_t x = __funnelshift_r(W.words[p >> 5], W.words[(p >> 5) + 1], p & 31u) & mw;
-            p += w;
-            if (IDM == ID_LOCAL_GAP) { run += x; *out++ = run; }
-            else *out++ = x;
-          }
-          lastf = k == 0;
-          lastv = run;
-          j++;
-          k = 0;
-        }
-      }
-      if (IDM == ID_LOCAL_GAP) {
-        // inclusive segmented scan of (lastf, lastv) over the lanes, after the
-        // window's carry (the absolute ID of field W0 - 1 when W0 is inside a vertex)
-        const uint32_t cf = fpre[ja] < W0 ? 1u : 0u, cv = cf ? wcarry : 0u;
-        uint32_t xf = lastf, xv = lastv;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t ef = __shfl_up_sync(LG_FULL_MASK, xf, o), ev = __shfl_up_sync(LG_FULL_MASK, xv, o);
-          if (lane >= (uint32_t)o) seg_after(xf, xv, ef, ev);
-        }
-        uint32_t lf = __shfl_up_sync(LG_FULL_MASK, xf, 1), lv = __shfl_up_sync(LG_FULL_MASK, xv, 1);
-        if (lane == 0) { lf = 0; lv = 0; }
-        seg_after(lf, lv, cf, cv);
-        for (uint32_t f = fa; f < pend; f++) W.stage[f - W0] += lv;
-        seg_after(xf, xv, cf, cv);
-        wcarry = __shfl_sync(LG_FULL_MASK, xv, 31);  // the absolute ID of the window's last field
-      }
-      __syncwarp();
-      const uint64_t dst0 = sm.rdelta[q] + W0;
-      for (uint32_t x = lane; x < Fw; x += 32) __stcs(a.ids + dst0 + x, W.stage[x]);
-      __syncwarp();
-      W0 += Fw;
+  // ---- windows
+  const uint32_t k0 = PW_E * lane;
+  uint32_t* out = sm.out[wid];
+  auto rows_to = [&](const Window& w) {  // light field f of the tile goes to base + f
+    for (; hseen < w.h; hseen++) base += sm.hdeg[wid][hseen];
+    return base + w.f0;
+  };
+  uint64_t dst = 0, dst_next = more ? rows_to(nxt) : 0;
+  for (; more; buf ^= 1u) {
+    cur = nxt;
+    dst = dst_next;
+    const int jc = ja;
+    more = next_window(T, W, PW_WF, nxt);
+    if (more) {
+      dst_next = rows_to(nxt);
+      ja = open_window<IDM>(g, T, nxt, buf ^ 1u, jc, pol, W);
+      stage_wait<1>();
+    } else {
+      stage_wait<0>();
     }
+    const uint32_t hb = (W.heads[buf][lane >> 2] >> (8u * (lane & 3u))) & 255u;
+    const int c = (int)__popc(hb);
+    const int je = jb + warp_incl_scan<int>(c) - c;
+    jb = jc;
+    uint32_t id[PW_E];
+    decode_window<IDM>(g, cur, hb, je, W, gcarry, id);
+    uint4* o4 = reinterpret_cast<uint4*>(out + k0);
+    o4[0] = make_uint4(id[0], id[1], id[2], id[3]);
+    o4[1] = make_uint4(id[4], id[5], id[6], id[7]);
+    __syncwarp();
+#pragma unroll
+    for (uint32_t u = 0; u < PW_G; u++)
+      if (lane + 32u * u < cur.nf) __stcs(a.ids + dst + lane + 32u * u, out[lane + 32u * u]);
+    __syncwarp();  // the stage, the heads and the IDs may be overwritten
   }
 }
 
@@ -1874,7 +1740,7 @@ cudaError_t launch_dec_all(const GView& g, const DecArgs& a, cudaStream_t st) {
     const cudaError_t e = cudaFuncSetAttribute(k_dec_local<IDM, OFF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)sizeof(DecSmem));
     if (e != cudaSuccess) return e;
-    k_dec_local<IDM, OFF><<<tiles_of(g.n) + heavy_blocks(g.n_items), TNT, sizeof(DecSmem), st>>>(g, a);
+    k_dec_local<IDM, OFF><<<(unsigned)a.tiles + heavy_blocks(g.n_items), TNT, sizeof(DecSmem), st>>>(g, a);
   }
   count_launch();
   return cudaGetLastError();
