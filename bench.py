@@ -170,9 +170,12 @@ def kernel_source_hash(workload="community"):
     """Hash of the sources of the kernel the roofline reports (k_pr_pull, or
     k_batch for the batch workload)."""
     files = ("lg_batch.cu",) if workload == "batch" else ("lg_traverse.cuh", "lg_device.cuh")
+    csrc = os.path.join(ROOT, "paper_2010_15879_gb300", "csrc")
     h = hashlib.sha256()
-    for f in files:
-        h.update(open(os.path.join(ROOT, "paper_2010_15879_gb300", "csrc", f), "rb").read())
+    for f in files + ("lg_pull.cuh", "lg_window.cuh"):  # the sweep itself, and the windows both share
+        path = os.path.join(csrc, f)
+        if f in files or os.path.exists(path):
+            h.update(open(path, "rb").read())
     return h.hexdigest()[:16]
 
 
