@@ -52,13 +52,13 @@ __global__ void __launch_bounds__(TNT) k_sssp_offsets(GView g, uint64_t* x, uint
   if (tile0)
     for (uint64_t i = (uint64_t)blockIdx.x * TNT + threadIdx.x; i < g.n_items; i += (uint64_t)gridDim.x * TNT)
       if (g.items[i].f0 == 0) x[g.items[i].v] = g.items[i].bit / r;
+  if (blockIdx.x == 0 && threadIdx.x == 0) x[g.n] = g.arcs;  // here: every tile may come from the schedule
   const uint64_t v0 = ((uint64_t)blockIdx.x + tile0) * TV;
   if (v0 >= g.n) return;
   const int cnt = (int)min((uint64_t)TV, g.n - v0);
   tile_offsets<OFF>(g, v0, cnt, xs, ts);
   __syncthreads();
   for (int i = threadIdx.x; i < cnt; i += TNT) x[v0 + i] = xs[i];
-  if (v0 + cnt == g.n && threadIdx.x == 0) x[g.n] = xs[cnt];
 }
 
 // Exclusive sums of the near vertices' degrees, the round's arcs at eoff[len]:
