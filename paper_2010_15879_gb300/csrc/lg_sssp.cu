@@ -318,7 +318,7 @@ __global__ void k_sssp_unpermute(const unsigned long long* dist, const uint32_t*
 template <int IDM, int OFF>
 cudaError_t launch_sssp_offsets(const GView& g, uint64_t* x, cudaStream_t st) {
   const uint32_t tile0 = (uint32_t)(g.heavy_prefix / TV);
-  k_sssp_offsets<IDM, OFF><<<std::max(1u, tiles_of(g.n) - tile0), TNT, 0, st>>>(g, x, tile0);
+  k_sssp_offsets<IDM, OFF><<<schedule_tiles_grid(g, tile0), TNT, 0, st>>>(g, x, tile0);
   count_launch();
   return cudaGetLastError();
 }

@@ -1639,13 +1639,22 @@ __global__ void __launch_bounds__(256) k_plan_carry(GView g, PlanArgs p) {
 // ===========================================================================
 inline unsigned tiles_of(uint64_t n) { return (unsigned)((n + TV - 1) / TV); }
 
+// Grid of the kernels whose tiles start at tile0 and whose threads fill the
+// labels before them from the schedule: a block per tile, and enough of them
+// for the items.  (400,000 vertices of degree 300 in degree order leave one
+// tile, whose block then walked 400,000 items alone: 740 us.)
+inline unsigned schedule_tiles_grid(const GView& g, uint32_t tile0) {
+  const unsigned items = tile0 ? grid_for(g.n_items, TNT, 152 * 8) : 1u;
+  return std::max(items, tiles_of(g.n) - tile0);
+}
+
 template <int IDM, int OFF>
 cudaError_t launch_pr_init(const GView& g, const PrArgs& a, cudaStream_t st) {
   const cudaError_t e = a.tabn ? cudaFuncSetAttribute(k_pr_pull<IDM, OFF, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PW_SMEM)
                                : cudaFuncSetAttribute(k_pr_pull<IDM, OFF, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PW_SMEM);
   if (e != cudaSuccess) return e;
   const uint32_t tile0 = (uint32_t)(g.heavy_prefix / TV);
-  k_pr_init<IDM, OFF><<<std::max(1u, tiles_of(g.n) - tile0), TNT, 0, st>>>(g, a, tile0);
+  k_pr_init<IDM, OFF><<<schedule_tiles_grid(g, tile0), TNT, 0, st>>>(g, a, tile0);
   count_launch();
   return cudaGetLastError();
 }

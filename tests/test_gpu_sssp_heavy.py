@@ -34,3 +34,16 @@ def test_distances(heavy, light, off_mode):
     for s in (0, n // 2, n - 1):
         want = oracle.sssp(n, h.row_ptr, h.col, h.weights, s)
         assert np.array_equal(lg.lg_sssp(g, s).cpu().numpy().view(np.uint64), want), s
+
+
+@pytest.mark.parametrize("id_mode", [lg.LG_ID_GLOBAL, lg.LG_ID_LOCAL, lg.LG_ID_LOCAL_GAP])
+@pytest.mark.parametrize("heavy, light", [(512, 0), (1024, 0), (1024, 700), (1500, 1)])
+def test_ranks(heavy, light, id_mode):
+    """PageRank's first contributions come from the schedule in the same way,
+    by more blocks than there are tiles left."""
+    lg.load(auto_build=True)
+    h = graph(heavy, light)
+    g = lg.lg_encode(h.row_ptr, h.col, id_mode=id_mode, off_mode=lg.LG_OFF_EF, relabel=lg.LG_RELABEL_DM)
+    want = oracle.pagerank(heavy + light, h.row_ptr, h.col, 0.85, 5)
+    got = lg.lg_pagerank(g, 0.85, 5).cpu().numpy()
+    assert np.max(np.abs(got - want) / want) <= 1e-4
