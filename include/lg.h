@@ -324,7 +324,9 @@ typedef struct {
                                of at most 65,536 vertices take windows of 256 fields
                                per warp whatever it is                                */
     uint64_t tile_arcs;     /* arcs per CTA before a graph gets a team of CTAs;
-                               0: 2^19, or autotuned among 2^18 .. 2^21               */
+                               0: 2^19, or autotuned among 2^18 .. 2^21; graphs of
+                               more than 65,536 vertices: from 2^15 on, by their
+                               arcs in all, or autotuned among 2^15 .. 2^21           */
     uint32_t wait_limit_us; /* time limit of a team barrier; 0 means 2 s              */
     uint32_t flags;         /* LG_BATCH_FLAG_* bits                                    */
 } lg_batch_opts;
@@ -351,8 +353,10 @@ typedef struct {
     uint64_t words_O;
     const lg_batch_graph *graphs;  /* device, count entries                        */
     uint32_t n_items;              /* work items (graph, team member) per run     */
-    uint32_t grid, threads;        /* persistent launch shape                     */
-    uint64_t tile_arcs;            /* tile in use                                 */
+    uint32_t grid, threads;        /* persistent launch shape: that of the graphs of up
+                                      to 65,536 vertices if there are any, else of the
+                                      larger ones, which have a kernel of their own */
+    uint64_t tile_arcs;            /* tile in use (of the same graphs)            */
     uint32_t teams, max_team;      /* graphs with more than one CTA; largest team */
     uint64_t bits_total;           /* sum over graphs of arcs*s + (n+1)*w_O       */
     uint64_t launches;             /* batch kernel launches so far (one per run)  */

@@ -1,11 +1,12 @@
-// Batches of independent graphs in one persistent launch.
+// Batches of independent graphs in one persistent launch (two if graphs of more
+// than 65,536 vertices are among others).
 //
 // Every graph g of the batch is encoded with its own widths -- vertex IDs at
 // s_g = bits(n_g - 1) (Section 3.2.1, 0-based IDs) and offsets packed at
 // w_O = bits(arcs_g) (Section 3.4, "ptrLogn") -- then searched breadth-first
 // from its vertex 0 and ranked by pull PageRank (Section 7.1.2), reading only
-// the stream it just wrote.  The whole batch is ONE kernel launch, captured
-// once as a CUDA graph and replayed.
+// the stream it just wrote.  The whole batch is one launch of a CUDA graph,
+// captured once and replayed.
 //
 // Work queue.  Items are (graph, member) pairs in a size-ordered queue
 // (largest per-member work first).  A graph larger than the tile gets a team
@@ -20,8 +21,19 @@
 // L2-coherent loads (ld.global.cg).
 //
 // Graphs of up to 65,536 vertices keep their per-vertex state in the CTA's
-// shared memory (the second half of this file's kernels); the others decode
-// their neighborhoods with T lanes per vertex (T = 1, 4, 8 or 32).  T per
+// shared memory (k_batch, one large CTA per SM).  The others decode their
+// neighborhoods with T lanes per vertex (T = 1, 4, 8 or 32; k_batch_lanes):
+// their gathers miss the SM, so they want the threads and the L1 that the first
+// kernel gives up.  Measured, autotuned, ms: with one CTA per SM beside 194 KB
+// of shared memory, 8 CTAs of 256 threads, 4 of 512, 2 of 768 (taken), 2 of
+// 1,024: 64 graphs of 2^17 .. 2^18 vertices 32.0, 26.2, 24.2, 22.5, 22.4; one
+// of 2^22 43.9, 36.8, 36.0, 34.7, 36.8; 200 of 100,000 21.6, 23.7, 14.1, 14.7,
+// 15.0; 16 of 70,000 in 48 items 5.1, 15.7, 13.1, 6.8, 7.0.  Where the items
+// are no more than the SMs, one CTA per SM with twice the registers is quicker
+// still.  Each kernel has its own queue and takes the whole chip, one after the
+// other, so that no team waits for a CTA that another kernel's team keeps off
+// the SMs; a batch without graphs of one kind does not launch that kind's
+// kernel.  T per
 // average-degree class and the team tile are chosen by a timing autotuner when
 // the batch is created.
 #include <cstdio>
@@ -52,7 +64,8 @@ struct BatchItem {
   uint32_t g, member;
 };
 
-constexpr int BNT = 768;  // threads per batch CTA, one CTA per SM (80 registers: no spills)
+constexpr int BNT = 768;  // threads per CTA of k_batch, one CTA per SM (80 registers: no spills)
+constexpr int LNT = 768;  // threads per CTA of k_batch_lanes, two CTAs per SM (one if the items are few)
 constexpr uint32_t PH_ENCODE = 1, PH_BFS = 2, PH_PR = 4;
 constexpr uint32_t BERR_TIMEOUT = 1;
 constexpr uint32_t SYNC_WORDS = 4;  // per graph: barrier count + 3 rotating queue counters
@@ -60,9 +73,9 @@ constexpr uint32_t INF32 = 0xffffffffu;
 
 struct BatchArgs {
   const BatchGraph* graphs;
-  const BatchItem* items;
-  uint32_t n_items;
-  unsigned int* next;       // queue head
+  const BatchItem* items;   // those of the shared-memory path, then those of the lanes path
+  uint32_t n_small, n_items;
+  unsigned int* next;       // queue heads of the two paths
   uint32_t* sync;           // SYNC_WORDS per graph
   uint32_t* err;
   const uint64_t* row_ptr;  // input CSR (global arc offsets)
@@ -152,7 +165,7 @@ __device__ void pr_sweep(const BatchArgs& a, const BatchGraph& G, uint32_t v0, u
                          float* cout, bool last) {
   const uint64_t* A = a.A + G.a_word;
   const uint64_t* O = a.O + G.o_word;
-  constexpr uint32_t groups = BNT / T;
+  constexpr uint32_t groups = LNT / T;
   const uint32_t gid = threadIdx.x / T, lane = threadIdx.x % T;
   const float base = (1.0f - a.damp) / (float)G.n;
   const uint32_t s = G.s;
@@ -193,7 +206,7 @@ __device__ void bfs_level(const BatchArgs& a, const BatchGraph& G, uint32_t memb
   const uint64_t* A = a.A + G.a_word;
   const uint64_t* O = a.O + G.o_word;
   uint32_t* depth = a.depth + G.vbase;
-  constexpr uint32_t groups = BNT / T;
+  constexpr uint32_t groups = LNT / T;
   const uint32_t gid = threadIdx.x / T, lane = threadIdx.x % T;
   for (uint32_t q = member * groups + gid; q < qlen; q += p * groups) {
     const uint32_t v = __ldcg(qin + q);
@@ -211,7 +224,7 @@ __device__ void bfs_level(const BatchArgs& a, const BatchGraph& G, uint32_t memb
 template <typename Rec>
 __device__ __forceinline__ void pack_words(uint64_t* out, uint64_t k0, uint64_t k1, uint64_t nrec, uint32_t w,
                                            Rec rec) {
-  for (uint64_t k = k0 + threadIdx.x; k < k1; k += BNT) {
+  for (uint64_t k = k0 + threadIdx.x; k < k1; k += LNT) {
     const uint64_t b0 = k * 64, j0 = b0 / w;
     uint64_t j1 = (b0 + 63) / w;
     if (j1 >= nrec) j1 = nrec - 1;
@@ -570,7 +583,7 @@ __device__ void process_item(const BatchArgs& a, uint32_t gi, uint32_t m) {
 
   if (a.phases & PH_BFS) {
     uint32_t* depth = a.depth + G.vbase;
-    for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT) depth[v] = INF32;
+    for (uint32_t v = v0 + threadIdx.x; v < v1; v += LNT) depth[v] = INF32;
     __syncthreads();
     uint32_t* qa = a.q0 + G.vbase;
     uint32_t* qb = a.q1 + G.vbase;
@@ -602,7 +615,7 @@ __device__ void process_item(const BatchArgs& a, uint32_t gi, uint32_t m) {
     float* ci = a.c0 + G.vbase;
     float* co = a.c1 + G.vbase;
     const float r0 = 1.0f / (float)G.n;
-    for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT) {
+    for (uint32_t v = v0 + threadIdx.x; v < v1; v += LNT) {
       const uint32_t d = sfield(O, (uint64_t)(v + 1) * G.w_O, G.w_O) - sfield(O, (uint64_t)v * G.w_O, G.w_O);
       ci[v] = d ? r0 / (float)d : 0.f;
     }
@@ -628,29 +641,45 @@ __device__ void process_item(const BatchArgs& a, uint32_t gi, uint32_t m) {
   }
 }
 
+// next item of a queue, the same for the whole CTA
+__device__ __forceinline__ unsigned int take_item(unsigned int* next) {
+  __shared__ unsigned int slot;
+  if (threadIdx.x == 0) slot = atomicAdd(next, 1u);
+  __syncthreads();
+  const unsigned int s = slot;
+  __syncthreads();
+  return s;
+}
+
 __global__ void __launch_bounds__(BNT, 1) k_batch(BatchArgs a) {
-  __shared__ unsigned int slot_s;
   for (;;) {
-    if (threadIdx.x == 0) slot_s = atomicAdd(a.next, 1u);
-    __syncthreads();
-    const unsigned int slot = slot_s;
-    __syncthreads();
-    if (slot >= a.n_items) return;
+    const unsigned int slot = take_item(a.next);
+    if (slot >= a.n_small) return;
     const BatchItem it = a.items[slot];
-    if (a.graphs[it.g].n == 0) continue;
-    if (a.graphs[it.g].n <= BS_MAX) process_small(a, it.g, it.member);
-    else process_item(a, it.g, it.member);
+    if (a.graphs[it.g].n) process_small(a, it.g, it.member);
   }
 }
 
+template <int PER_SM>
+__global__ void __launch_bounds__(LNT, PER_SM) k_batch_lanes(BatchArgs a) {
+  for (;;) {
+    const unsigned int slot = take_item(a.next + 1);
+    if (slot >= a.n_items - a.n_small) return;
+    const BatchItem it = a.items[a.n_small + slot];
+    process_item(a, it.g, it.member);
+  }
+}
+
+constexpr int VNT = 256;  // threads per validating CTA
+
 // every graph's rows: bounds monotone inside the graph's arc range, local IDs
 // < n_g, rows strictly increasing
-__global__ void __launch_bounds__(BNT) k_batch_validate(const BatchGraph* graphs, uint32_t count,
+__global__ void __launch_bounds__(VNT) k_batch_validate(const BatchGraph* graphs, uint32_t count,
                                                         const uint64_t* row_ptr, const uint32_t* col, int* err) {
   for (uint32_t g = blockIdx.x; g < count; g += gridDim.x) {
     const BatchGraph G = graphs[g];
     int flags = 0;
-    for (uint32_t v = threadIdx.x; v < G.n; v += BNT) {
+    for (uint32_t v = threadIdx.x; v < G.n; v += VNT) {
       const uint64_t lo = row_ptr[G.vbase + v], hi = row_ptr[G.vbase + v + 1];
       if (hi < lo || lo < G.abase || hi > G.abase + G.arcs) {
         flags |= DERR_ROWPTR;
@@ -685,8 +714,8 @@ struct lg_batch {
   std::vector<BatchItem> items_h;
   BatchGraph* graphs = nullptr;  // device descriptors
   BatchItem* items = nullptr;
-  uint32_t n_items = 0;
-  unsigned int* next = nullptr;  // queue head
+  uint32_t n_items = 0, n_small = 0;  // items; those of the shared-memory path, which come first
+  unsigned int* next = nullptr;  // queue heads
   uint32_t* sync = nullptr;      // SYNC_WORDS per graph
   uint32_t* err = nullptr;
   uint64_t* A = nullptr;
@@ -696,8 +725,9 @@ struct lg_batch {
   uint32_t* q1 = nullptr;
   float* c0 = nullptr;
   float* c1 = nullptr;
-  uint64_t tile_arcs = 0;
-  int grid = 1;
+  uint64_t tile_arcs = 0, tile_lanes = 0;  // of the shared-memory path, of the lanes path
+  int sms = 1;
+  int grid = 1, grid_lanes = 1;  // CTAs of k_batch, of k_batch_lanes
   uint64_t launches = 0;         // batch kernel launches (each graph replay counts one)
   std::mutex mu;                 // guards the cached executable graph
   cudaStream_t cap = nullptr;    // private stream used for capture
@@ -723,9 +753,10 @@ lg_status batch_fail(const char* what, cudaError_t e) {
 
 // Team sizes and the queue: by decreasing work per member, a team's members
 // on consecutive slots.
-void plan_queue(lg_batch* b, uint64_t tile) {
-  const uint32_t max_team = (uint32_t)std::max(1, b->grid / 2);
+void plan_queue(lg_batch* b) {
   for (auto& x : b->host) {
+    const uint64_t tile = x.n <= BS_MAX ? b->tile_arcs : b->tile_lanes;
+    const uint32_t max_team = (uint32_t)std::max(1, (x.n <= BS_MAX ? b->grid : b->grid_lanes) / 2);
     uint64_t p = tile ? (x.arcs + tile - 1) / tile : 1;
     p = std::max<uint64_t>(p, 1);
     p = std::min<uint64_t>(p, max_team);
@@ -737,8 +768,12 @@ void plan_queue(lg_batch* b, uint64_t tile) {
   auto work = [&](uint32_t g) { return ((uint64_t)b->host[g].arcs * 2 + b->host[g].n) / b->host[g].team; };
   std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return work(x) > work(y); });
   b->items_h.clear();
-  for (uint32_t g : order)
-    for (uint32_t m = 0; m < b->host[g].team; m++) b->items_h.push_back({g, m});
+  for (const bool small : {true, false}) {
+    for (uint32_t g : order)
+      if ((b->host[g].n <= BS_MAX) == small)
+        for (uint32_t m = 0; m < b->host[g].team; m++) b->items_h.push_back({g, m});
+    if (small) b->n_small = (uint32_t)b->items_h.size();
+  }
   b->n_items = (uint32_t)b->items_h.size();
 }
 
@@ -759,11 +794,12 @@ lg_status upload_plan(lg_batch* b, cudaStream_t st) {
 }
 
 BatchArgs make_args(lg_batch* b, uint32_t* depth, float* ranks, float damp, uint32_t iters, uint32_t phases,
-                    const BatchItem* items, uint32_t n_items, int lanes) {
+                    const BatchItem* items, uint32_t n_small, uint32_t n_items, int lanes) {
   BatchArgs a;
   memset(&a, 0, sizeof(a));
   a.graphs = b->graphs;
   a.items = items;
+  a.n_small = n_small;
   a.n_items = n_items;
   a.next = b->next;
   a.sync = b->sync;
@@ -786,12 +822,20 @@ BatchArgs make_args(lg_batch* b, uint32_t* depth, float* ranks, float damp, uint
   return a;
 }
 
-// one run: reset the queue head, team counters and error word, then the persistent launch
+// one run: reset the queue heads, team counters and error word, then the persistent launches
 void enqueue_run(lg_batch* b, const BatchArgs& a, cudaStream_t st) {
-  cudaMemsetAsync(b->next, 0, sizeof(unsigned int), st);
+  cudaMemsetAsync(b->next, 0, 2 * sizeof(unsigned int), st);
   cudaMemsetAsync(b->sync, 0, (size_t)b->count * SYNC_WORDS * 4, st);
   cudaMemsetAsync(b->err, 0, 4, st);
-  k_batch<<<b->grid, BNT, BS_SMEM, st>>>(a);
+  const uint32_t lanes = a.n_items - a.n_small;
+  if (lanes > (uint32_t)b->sms) k_batch_lanes<2><<<b->grid_lanes, LNT, 0, st>>>(a);
+  else if (lanes) k_batch_lanes<1><<<lanes, LNT, 0, st>>>(a);
+  if (a.n_small) k_batch<<<b->grid, BNT, BS_SMEM, st>>>(a);
+}
+
+void count_kernels(const BatchArgs& a) {
+  if (a.n_small) count_launch();
+  if (a.n_items > a.n_small) count_launch();
 }
 
 lg_status time_run(lg_batch* b, const BatchArgs& a, cudaStream_t st, cudaEvent_t e0, cudaEvent_t e1, int reps,
@@ -801,7 +845,7 @@ lg_status time_run(lg_batch* b, const BatchArgs& a, cudaStream_t st, cudaEvent_t
     BTRY(cudaEventRecord(e0, st));
     enqueue_run(b, a, st);
     b->launches++;
-    count_launch();
+    count_kernels(a);
     BTRY(cudaGetLastError());
     BTRY(cudaEventRecord(e1, st));
     BTRY(cudaEventSynchronize(e1));
@@ -814,8 +858,8 @@ lg_status time_run(lg_batch* b, const BatchArgs& a, cudaStream_t st, cudaEvent_t
 
 // Timing autotuner.  (1) T per average-degree class: the class's 64 largest
 // graphs run alone (encode + 2 PageRank sweeps) with T = 1, 4, 8 and 32.
-// (2) The team tile, if not fixed: the whole batch (encode + BFS + 2 sweeps)
-// with tiles of 2^18 .. 2^21 arcs.
+// (2) The team tiles, if not fixed: each path's graphs (encode + BFS + 2
+// sweeps) with tiles of 2^18 .. 2^21 arcs, the lanes path's from 2^15 on.
 lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStream_t st, cudaEvent_t e0,
                    cudaEvent_t e1) {
   const int cand_t[4] = {1, 4, 8, 32};
@@ -825,7 +869,7 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
     const double avg = x.n ? (double)x.arcs / x.n : 0.0;
     bins[avg <= 8 ? 0 : avg <= 16 ? 1 : avg <= 32 ? 2 : avg <= 64 ? 3 : 4].push_back(g);
   }
-  const size_t max_items = 64 * (size_t)std::max(1, b->grid / 2);
+  const size_t max_items = 64 * (size_t)std::max(1, b->grid_lanes / 2);
   BatchItem* dlist = nullptr;
   BTRY(cudaMalloc((void**)&dlist, max_items * sizeof(BatchItem) + 16));
   lg_status s = LG_OK;
@@ -848,7 +892,7 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
     float best = 1e30f;
     int best_t = 8;
     for (int c = 0; c < 4 && s == LG_OK; c++) {
-      BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_PR, dlist, (uint32_t)its.size(),
+      BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_PR, dlist, 0, (uint32_t)its.size(),
                               cand_t[c]);
       float ms = 0;
       s = time_run(b, a, st, e0, e1, 2, &ms);
@@ -862,22 +906,29 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
   cudaFree(dlist);
   if (s != LG_OK) return s;
   if (b->opts.tile_arcs == 0) {
-    const uint64_t cand_k[4] = {1ull << 18, 1ull << 19, 1ull << 20, 1ull << 21};
-    float best = 1e30f;
-    uint64_t best_k = b->tile_arcs;
-    for (uint64_t k : cand_k) {
-      plan_queue(b, k);
-      if ((s = upload_plan(b, st)) != LG_OK) return s;
-      BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_BFS | PH_PR, b->items, b->n_items, 0);
-      float ms = 0;
-      if ((s = time_run(b, a, st, e0, e1, 2, &ms)) != LG_OK) return s;
-      if (ms < best) {
-        best = ms;
-        best_k = k;
+    for (const bool small : {true, false}) {
+      uint64_t& tile = small ? b->tile_arcs : b->tile_lanes;
+      float best = 1e30f;
+      uint64_t best_k = tile;
+      for (uint64_t k : {1ull << 15, 1ull << 17, 1ull << 18, 1ull << 19, 1ull << 20, 1ull << 21}) {
+        if (small && k < 1ull << 18) continue;
+        tile = k;
+        plan_queue(b);
+        const uint32_t n = small ? b->n_small : b->n_items - b->n_small;
+        if (n == 0) break;
+        if ((s = upload_plan(b, st)) != LG_OK) return s;
+        BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_BFS | PH_PR,
+                                b->items + (small ? 0 : b->n_small), small ? n : 0, n, 0);
+        float ms = 0;
+        if ((s = time_run(b, a, st, e0, e1, 2, &ms)) != LG_OK) return s;
+        if (ms < best) {
+          best = ms;
+          best_k = k;
+        }
       }
+      tile = best_k;
     }
-    b->tile_arcs = best_k;
-    plan_queue(b, best_k);
+    plan_queue(b);
   }
   if ((s = upload_plan(b, st)) != LG_OK) return s;
   uint32_t herr = 0;
@@ -944,9 +995,26 @@ lg_status batch_create_impl(lg_batch* b, const uint64_t* graph_vptr, cudaStream_
   BTRY(cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS_SMEM));
   BTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, BNT, BS_SMEM));
   BTRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device));
-  b->grid = std::max(1, per_sm) * std::max(1, sms);
-  b->tile_arcs = b->opts.tile_arcs ? b->opts.tile_arcs : (1ull << 19);
-  plan_queue(b, b->tile_arcs);
+  b->sms = std::max(1, sms);
+  b->grid = std::max(1, per_sm) * b->sms;
+  BTRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_lanes<2>, LNT, 0));
+  b->grid_lanes = std::max(1, per_sm) * b->sms;
+  b->tile_arcs = b->tile_lanes = b->opts.tile_arcs ? b->opts.tile_arcs : (1ull << 19);
+  if (!b->opts.tile_arcs) {
+    // few large graphs are split until there is a member for every SM, and no
+    // further: each adds to a team's barriers (8 graphs of 2^18 vertices among
+    // 500 small ones: 18.0 ms in 264 items, 14.4 in 144)
+    uint64_t arcs = 0;
+    int large = 0;
+    for (const auto& x : b->host)
+      if (x.n > BS_MAX) {
+        arcs += x.arcs;
+        large++;
+      }
+    const uint64_t members = (uint64_t)std::max(b->sms - large, std::max(1, b->sms / 2));
+    b->tile_lanes = std::min(b->tile_lanes, std::max<uint64_t>(arcs / members, 1ull << 15));
+  }
+  plan_queue(b);
   BTRY(cudaMalloc((void**)&b->graphs, G * sizeof(BatchGraph) + 16));
   BTRY(cudaMalloc((void**)&b->next, 16));
   BTRY(cudaMalloc((void**)&b->sync, (size_t)G * SYNC_WORDS * 4 + 16));
@@ -965,7 +1033,7 @@ lg_status batch_create_impl(lg_batch* b, const uint64_t* graph_vptr, cudaStream_
   int* d_err = nullptr;
   BTRY(cudaMalloc((void**)&d_err, 4));
   BTRY(cudaMemsetAsync(d_err, 0, 4, st));
-  k_batch_validate<<<grid_for(G, 1, 152 * 16), BNT, 0, st>>>(b->graphs, G, b->row_ptr, b->col, d_err);
+  k_batch_validate<<<grid_for(G, 1, 152 * 16), VNT, 0, st>>>(b->graphs, G, b->row_ptr, b->col, d_err);
   count_launch();
   int herr = 0;
   ce = cudaMemcpyAsync(&herr, d_err, 4, cudaMemcpyDeviceToHost, st);
@@ -1004,6 +1072,7 @@ lg_status batch_create_impl(lg_batch* b, const uint64_t* graph_vptr, cudaStream_
       while (j + 1 < b->items_h.size() && b->items_h[j + 1].g == g) j++;
       b->items_h.erase(b->items_h.begin() + (long)j);
       b->n_items--;
+      if (j < b->n_small) b->n_small--;
       break;
     }
     if ((s = upload_plan(b, st)) != LG_OK) return s;
@@ -1090,7 +1159,7 @@ extern "C" lg_status lg_batch_run(lg_batch* b, float damping, uint32_t iters, ui
       b->exec = nullptr;
     }
     cudaGraph_t graph = nullptr;
-    BatchArgs a = make_args(b, depths, ranks, damping, iters, PH_ENCODE | PH_BFS | PH_PR, b->items, b->n_items, 0);
+    BatchArgs a = make_args(b, depths, ranks, damping, iters, PH_ENCODE | PH_BFS | PH_PR, b->items, b->n_small, b->n_items, 0);
     cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       enqueue_run(b, a, b->cap);
@@ -1111,7 +1180,7 @@ extern "C" lg_status lg_batch_run(lg_batch* b, float damping, uint32_t iters, ui
   if (status == LG_OK) {
     cudaError_t e = cudaGraphLaunch(b->exec, st);
     b->launches++;
-    count_launch();
+    count_kernels(make_args(b, depths, ranks, damping, iters, 0, b->items, b->n_small, b->n_items, 0));
     if (e != cudaSuccess) status = batch_fail("lg_batch_run: cudaGraphLaunch", e);
   }
   if (prev != b->device) cudaSetDevice(prev);
@@ -1151,9 +1220,10 @@ extern "C" lg_status lg_batch_info_get(const lg_batch* b, lg_batch_info* out) {
   out->words_O = b->words_O;
   out->graphs = reinterpret_cast<const lg_batch_graph*>(b->graphs);
   out->n_items = b->n_items;
-  out->grid = (uint32_t)b->grid;
+  out->grid = (uint32_t)(b->n_small ? b->grid : b->grid_lanes);
+  static_assert(BNT == LNT, "one number of threads to report");
   out->threads = BNT;
-  out->tile_arcs = b->tile_arcs;
+  out->tile_arcs = b->n_small ? b->tile_arcs : b->tile_lanes;
   uint64_t teams = 0, bits = 0, max_team = 0;
   for (const auto& x : b->host) {
     teams += x.team > 1;
