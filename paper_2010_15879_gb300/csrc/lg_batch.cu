@@ -21,7 +21,8 @@
 // L2-coherent loads (ld.global.cg).
 //
 // Graphs of up to 65,536 vertices keep their per-vertex state in the CTA's
-// shared memory (k_batch, one large CTA per SM).  The others decode their
+// shared memory (k_batch, one large CTA per SM, whose warps split up for small
+// graphs).  The others decode their
 // neighborhoods with T lanes per vertex (T = 1, 4, 8 or 32; k_batch_lanes):
 // their gathers miss the SM, so they want the threads and the L1 that the first
 // kernel gives up.  Measured, autotuned, ms: with one CTA per SM beside 194 KB
@@ -73,9 +74,11 @@ constexpr uint32_t INF32 = 0xffffffffu;
 
 struct BatchArgs {
   const BatchGraph* graphs;
-  const BatchItem* items;   // those of the shared-memory path, then those of the lanes path
-  uint32_t n_small, n_items;
-  unsigned int* next;       // queue heads of the two paths
+  // those of the shared-memory path (graphs for a CTA, for 8 warps, for a warp),
+  // then those of the lanes path
+  const BatchItem* items;
+  uint32_t n_cta, n_eight, n_small, n_items;  // ends of the four parts
+  unsigned int* next;       // queue heads of the lanes path, of CTAs, of 8 warps, of warps
   uint32_t* sync;           // SYNC_WORDS per graph
   uint32_t* err;
   const uint64_t* row_ptr;  // input CSR (global arc offsets)
@@ -272,16 +275,46 @@ constexpr size_t BS_SMEM = 194 * 1024;
 constexpr uint32_t BS_TAB = (uint32_t)((BS_SMEM - BS_WARPS * sizeof(BWarp)) / sizeof(float)) & ~3u;
 static_assert(BS_TAB >= 3 * BS_WORDS, "the bitmaps share the table's memory");
 
+// A graph of a few tiles leaves most of a CTA's warps idle, and each of its
+// steps waits for all of them: 20,000 graphs of 256 vertices took 6.5 ms a run,
+// 2,000 of 64 vertices 1.13.  So once a CTA's queue is empty, its warps go on
+// as three groups of 8, then as single warps, each with a graph and a part of
+// the table of its own: 1.37 and 0.15 ms.  GW: warps of a group.
+template <int GW>
+struct BGroup {
+  static constexpr uint32_t NT = 32 * GW;
+  static constexpr uint32_t TAB8 = (BS_TAB / (BS_WARPS / 8)) & ~3u;
+  static constexpr uint32_t TAB = GW == BS_WARPS ? BS_TAB : GW == 8 ? TAB8 : (TAB8 / 8) & ~3u;  // floats of its table
+  // most vertices of a graph for a part of a CTA: contributions twice
+  static constexpr uint32_t MAX_N = (TAB / 2) & ~3u;
+  static __device__ __forceinline__ uint32_t tid() { return threadIdx.x % NT; }
+  static __device__ __forceinline__ uint32_t wid() { return (threadIdx.x >> 5) % GW; }
+  static __device__ __forceinline__ uint32_t index() { return (threadIdx.x >> 5) / GW * GW; }  // its first warp
+  static __device__ __forceinline__ float* table() {
+    float* t = reinterpret_cast<float*>(dyn_smem + BS_WARPS * sizeof(BWarp));
+    if (GW == BS_WARPS) return t;
+    const uint32_t w = threadIdx.x >> 5;
+    return t + (w / 8) * TAB8 + (GW == 1 ? (w % 8) * TAB : 0u);
+  }
+  static __device__ __forceinline__ void sync() {
+    if (GW == BS_WARPS) __syncthreads();
+    else if (GW == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1u + (threadIdx.x >> 5) / GW), "n"(32 * GW) : "memory");
+  }
+};
+static_assert(BS_WARPS % 8 == 0 && 3 * (BGroup<8>::MAX_N / 32 + 1) <= BGroup<8>::TAB &&
+                  3 * (BGroup<1>::MAX_N / 32 + 1) <= BGroup<1>::TAB, "groups");
+
 // Windows [i0, i1) of 256 records of w <= 32 bits: rec(j) is record j < nrec.
 // Lane l reads records l, l + 32, .., all in flight; then a lane assembles
 // whole 32-bit words.  The last window fills up its 64-bit word with zeros.
-template <typename Rec>
+template <int GW, typename Rec>
 __device__ __forceinline__ void pack_windows(uint32_t* out, uint64_t i0, uint64_t i1, uint64_t nrec, uint32_t w,
                                              BWarp& W, Rec rec) {
   const uint32_t lane = threadIdx.x & 31u;
   uint32_t* st = W.stage[0];
   const uint32_t inv = ((1u << 20) + w - 1) / w;  // x / w = x * inv >> 20 for x < 2^13
-  for (uint64_t i = i0 + (threadIdx.x >> 5); i < i1; i += BS_WARPS) {
+  for (uint64_t i = i0 + BGroup<GW>::wid(); i < i1; i += GW) {
     const uint64_t j0 = i * PW_WF;
     const uint32_t cnt = (uint32_t)min((uint64_t)PW_WF, nrec - j0);
     uint32_t r[PW_G];
@@ -399,12 +432,13 @@ __device__ __forceinline__ void small_push(const BatchArgs& a, const BatchGraph&
 
 // Bottom-up step over the vertices of bitmap words [w0, w1): 8 lanes per
 // unvisited vertex look for a frontier neighbor.
+template <int GW>
 __device__ __forceinline__ void small_pull(const BatchArgs& a, const BatchGraph& G, const uint32_t* fr,
                                            const uint32_t* vis, uint32_t* nx, uint32_t w0, uint32_t w1) {
   const uint64_t* A = a.A + G.a_word;
   const uint64_t* O = a.O + G.o_word;
   const uint32_t lane = threadIdx.x & 31u, grp = lane >> 3, s = G.s;
-  for (uint32_t i = w0 + (threadIdx.x >> 5); i < w1; i += BS_WARPS) {
+  for (uint32_t i = w0 + BGroup<GW>::wid(); i < w1; i += GW) {
     uint32_t found = 0;
     for (uint32_t m = ~vis[i]; m;) {
       uint32_t bit = 0;  // this group's vertex: one of the four lowest unvisited ones
@@ -438,14 +472,25 @@ __device__ __forceinline__ void small_pull(const BatchArgs& a, const BatchGraph&
   }
 }
 
+// the group's steps end in a barrier of its own, or of the team (whole CTAs)
+template <int GW>
+__device__ __forceinline__ bool small_sync(const BatchArgs& a, uint32_t* bar, uint32_t p, uint32_t round) {
+  if (GW == BS_WARPS) return team_sync(a, bar, p, round);
+  BGroup<GW>::sync();
+  return true;
+}
+
+template <int GW>
 __device__ void process_small(const BatchArgs& a, uint32_t gi, uint32_t m) {
-  __shared__ uint32_t ticket, count;
+  using Grp = BGroup<GW>;
+  __shared__ uint32_t tickets[BS_WARPS], counts[BS_WARPS];
+  uint32_t &ticket = tickets[Grp::index()], &count = counts[Grp::index()];
   const BatchGraph G = a.graphs[gi];
-  const uint32_t p = G.team, n = G.n, wid = threadIdx.x >> 5;
+  const uint32_t p = GW == BS_WARPS ? G.team : 1u, n = G.n, wid = Grp::wid(), tid = Grp::tid();
   uint32_t* bar = a.sync + (uint64_t)gi * SYNC_WORDS;
   uint32_t round = 0;
-  BWarp& W = reinterpret_cast<BWarp*>(dyn_smem)[wid];
-  float* tab = reinterpret_cast<float*>(dyn_smem + BS_WARPS * sizeof(BWarp));
+  BWarp& W = reinterpret_cast<BWarp*>(dyn_smem)[threadIdx.x >> 5];
+  float* tab = Grp::table();
   const uint64_t pol = policy_stream();
   const uint32_t tiles = (n + BS_TV - 1) / BS_TV, nwd = (n + 31) / 32;
   const uint32_t t0 = (uint32_t)((uint64_t)tiles * m / p), t1 = (uint32_t)((uint64_t)tiles * (m + 1) / p);
@@ -456,53 +501,53 @@ __device__ void process_small(const BatchArgs& a, uint32_t gi, uint32_t m) {
     const uint32_t* col = a.col + G.abase;
     const uint64_t* rp = a.row_ptr + G.vbase;
     const uint64_t ab = G.abase, na = ((uint64_t)G.arcs + PW_WF - 1) / PW_WF, no = ((uint64_t)n + PW_WF) / PW_WF;
-    pack_windows(reinterpret_cast<uint32_t*>(a.A + G.a_word), na * m / p, na * (m + 1) / p, G.arcs, G.s, W,
+    pack_windows<GW>(reinterpret_cast<uint32_t*>(a.A + G.a_word), na * m / p, na * (m + 1) / p, G.arcs, G.s, W,
                  [&](uint64_t j) { return __ldcs(col + j); });
-    pack_windows(reinterpret_cast<uint32_t*>(a.O + G.o_word), no * m / p, no * (m + 1) / p, (uint64_t)n + 1, G.w_O, W,
+    pack_windows<GW>(reinterpret_cast<uint32_t*>(a.O + G.o_word), no * m / p, no * (m + 1) / p, (uint64_t)n + 1, G.w_O, W,
                  [&](uint64_t j) { return (uint32_t)(__ldg(rp + j) - ab); });
-    if (!team_sync(a, bar, p, ++round)) return;
+    if (!small_sync<GW>(a, bar, p, ++round)) return;
   }
 
   if (a.phases & PH_BFS) {
     uint32_t* depth = a.depth + G.vbase;
     uint32_t* vis = reinterpret_cast<uint32_t*>(tab);
-    uint32_t *fr = vis + BS_WORDS, *nx = fr + BS_WORDS;
+    uint32_t *fr = vis + nwd, *nx = fr + nwd;
     // a team shares each level's new bitmap through one of three global ones:
     // written in a level, read after its barrier, cleared after the next one
     uint32_t* shared_nx[3] = {a.q0 + G.vbase, a.q1 + G.vbase, reinterpret_cast<uint32_t*>(a.c0 + G.vbase)};
-    for (uint32_t i = threadIdx.x; i < nwd; i += BNT) {
+    for (uint32_t i = tid; i < nwd; i += Grp::NT) {
       vis[i] = (i == nwd - 1 && (n & 31u) ? ~0u << (n & 31u) : 0u) | (i == 0 ? 1u : 0u);
       fr[i] = i == 0 ? 1u : 0u;
       nx[i] = 0;
     }
     if (p > 1)
-      for (uint32_t i = w0 + threadIdx.x; i < w1; i += BNT)
+      for (uint32_t i = w0 + tid; i < w1; i += Grp::NT)
         for (int k = 0; k < 3; k++) shared_nx[k][i] = 0;
-    for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT) depth[v] = v == 0 ? 0u : INF32;
-    if (!team_sync(a, bar, p, ++round)) return;
+    for (uint32_t v = v0 + tid; v < v1; v += Grp::NT) depth[v] = v == 0 ? 0u : INF32;
+    if (!small_sync<GW>(a, bar, p, ++round)) return;
     uint32_t frontier = 1;
     for (uint32_t level = 0; frontier > 0 && level < n; level++) {
       const bool push = frontier < n / 32 + 1;  // a large frontier is found from the unvisited side, with early exit
-      if (push) small_push(a, G, fr, vis, nx, m + p * wid, p * BS_WARPS);
-      else small_pull(a, G, fr, vis, nx, w0, w1);
-      if (threadIdx.x == 0) count = 0;
-      __syncthreads();
+      if (push) small_push(a, G, fr, vis, nx, m + p * wid, p * GW);
+      else small_pull<GW>(a, G, fr, vis, nx, w0, w1);
+      if (tid == 0) count = 0;
+      Grp::sync();
       if (p > 1) {
         uint32_t* g = shared_nx[level % 3];
         if (push) {
-          for (uint32_t i = threadIdx.x; i < nwd; i += BNT)
+          for (uint32_t i = tid; i < nwd; i += Grp::NT)
             if (nx[i]) atomicOr(g + i, nx[i]);
         } else {
-          for (uint32_t i = w0 + threadIdx.x; i < w1; i += BNT) __stcg(g + i, nx[i]);
+          for (uint32_t i = w0 + tid; i < w1; i += Grp::NT) __stcg(g + i, nx[i]);
         }
-        if (!team_sync(a, bar, p, ++round)) return;
-        for (uint32_t i = threadIdx.x; i < nwd; i += BNT) nx[i] = __ldcg(g + i);
+        if (!small_sync<GW>(a, bar, p, ++round)) return;
+        for (uint32_t i = tid; i < nwd; i += Grp::NT) nx[i] = __ldcg(g + i);
         if (level > 0)
-          for (uint32_t i = w0 + threadIdx.x; i < w1; i += BNT) shared_nx[(level - 1) % 3][i] = 0;
-        __syncthreads();
+          for (uint32_t i = w0 + tid; i < w1; i += Grp::NT) shared_nx[(level - 1) % 3][i] = 0;
+        Grp::sync();
       }
       uint32_t c = 0;
-      for (uint32_t i = threadIdx.x; i < nwd; i += BNT) {
+      for (uint32_t i = tid; i < nwd; i += Grp::NT) {
         const uint32_t x = nx[i];
         fr[i] = x;
         vis[i] |= x;
@@ -511,13 +556,13 @@ __device__ void process_small(const BatchArgs& a, uint32_t gi, uint32_t m) {
       }
       c = __reduce_add_sync(LG_FULL_MASK, c);
       if ((threadIdx.x & 31u) == 0 && c) atomicAdd(&count, c);
-      __syncthreads();
+      Grp::sync();
       frontier = count;
-      for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT)
+      for (uint32_t v = v0 + tid; v < v1; v += Grp::NT)
         if ((fr[v >> 5] >> (v & 31u)) & 1u) depth[v] = level + 1;
-      __syncthreads();  // count is reset in the next level
+      Grp::sync();  // count is reset in the next level
     }
-    __syncthreads();
+    Grp::sync();
   }
 
   if ((a.phases & PH_PR) && a.iters > 0) {
@@ -526,22 +571,22 @@ __device__ void process_small(const BatchArgs& a, uint32_t gi, uint32_t m) {
     float* co = a.c1 + G.vbase;
     // a graph of one CTA that fits twice stays in shared memory between sweeps
     const uint32_t half = (n + 3) & ~3u;
-    const bool inside = p == 1 && 2 * half <= BS_TAB;
-    const uint32_t tabn = min(n, BS_TAB);
+    const bool inside = p == 1 && 2 * half <= Grp::TAB;
+    const uint32_t tabn = min(n, Grp::TAB);
     const float r0 = 1.0f / (float)n;
     // team members finish their last BFS level before c0 is overwritten
-    if (!team_sync(a, bar, p, ++round)) return;
-    for (uint32_t v = v0 + threadIdx.x; v < v1; v += BNT) {
+    if (!small_sync<GW>(a, bar, p, ++round)) return;
+    for (uint32_t v = v0 + tid; v < v1; v += Grp::NT) {
       const uint32_t d = sfield(O, (uint64_t)(v + 1) * G.w_O, G.w_O) - sfield(O, (uint64_t)v * G.w_O, G.w_O);
       (inside ? tab : ci)[v] = d ? r0 / (float)d : 0.f;
     }
     float *tin = tab, *tout = tab + half;
     for (uint32_t t = 0; t < a.iters; t++) {
-      if (!team_sync(a, bar, p, ++round)) return;
+      if (!small_sync<GW>(a, bar, p, ++round)) return;
       if (!inside)
-        for (uint32_t i = threadIdx.x; i < tabn; i += BNT) tab[i] = __ldcg(ci + i);
-      if (threadIdx.x == 0) ticket = t0;
-      __syncthreads();
+        for (uint32_t i = tid; i < tabn; i += Grp::NT) tab[i] = __ldcg(ci + i);
+      if (tid == 0) ticket = t0;
+      Grp::sync();
       for (;;) {
         uint32_t tile = 0;
         if ((threadIdx.x & 31u) == 0) tile = atomicAdd(&ticket, 1u);
@@ -554,7 +599,7 @@ __device__ void process_small(const BatchArgs& a, uint32_t gi, uint32_t m) {
       co = x;
       if (inside) { x = tin; tin = tout; tout = x; }
     }
-    __syncthreads();
+    Grp::sync();
   }
 }
 
@@ -641,31 +686,38 @@ __device__ void process_item(const BatchArgs& a, uint32_t gi, uint32_t m) {
   }
 }
 
-// next item of a queue, the same for the whole CTA
-__device__ __forceinline__ unsigned int take_item(unsigned int* next) {
-  __shared__ unsigned int slot;
-  if (threadIdx.x == 0) slot = atomicAdd(next, 1u);
-  __syncthreads();
-  const unsigned int s = slot;
-  __syncthreads();
-  return s;
+// the items [first, end) of a queue, taken by groups of GW warps
+template <int GW>
+__device__ __forceinline__ void small_queue(const BatchArgs& a, unsigned int* next, uint32_t first, uint32_t end) {
+  __shared__ unsigned int slots[BS_WARPS];
+  unsigned int& slot = slots[BGroup<GW>::index()];
+  while (first < end) {
+    if (BGroup<GW>::tid() == 0) slot = atomicAdd(next, 1u);
+    BGroup<GW>::sync();
+    const unsigned int at = first + slot;
+    BGroup<GW>::sync();
+    if (at >= end) return;
+    const BatchItem it = a.items[at];
+    if (a.graphs[it.g].n) process_small<GW>(a, it.g, it.member);
+  }
 }
 
 __global__ void __launch_bounds__(BNT, 1) k_batch(BatchArgs a) {
-  for (;;) {
-    const unsigned int slot = take_item(a.next);
-    if (slot >= a.n_small) return;
-    const BatchItem it = a.items[slot];
-    if (a.graphs[it.g].n) process_small(a, it.g, it.member);
-  }
+  small_queue<BS_WARPS>(a, a.next + 1, 0, a.n_cta);
+  small_queue<8>(a, a.next + 2, a.n_cta, a.n_eight);
+  small_queue<1>(a, a.next + 3, a.n_eight, a.n_small);
 }
 
 template <int PER_SM>
 __global__ void __launch_bounds__(LNT, PER_SM) k_batch_lanes(BatchArgs a) {
+  __shared__ unsigned int slot;
   for (;;) {
-    const unsigned int slot = take_item(a.next + 1);
-    if (slot >= a.n_items - a.n_small) return;
-    const BatchItem it = a.items[a.n_small + slot];
+    if (threadIdx.x == 0) slot = a.n_small + atomicAdd(a.next, 1u);
+    __syncthreads();
+    const unsigned int at = slot;
+    __syncthreads();
+    if (at >= a.n_items) return;
+    const BatchItem it = a.items[at];
     process_item(a, it.g, it.member);
   }
 }
@@ -714,7 +766,8 @@ struct lg_batch {
   std::vector<BatchItem> items_h;
   BatchGraph* graphs = nullptr;  // device descriptors
   BatchItem* items = nullptr;
-  uint32_t n_items = 0, n_small = 0;  // items; those of the shared-memory path, which come first
+  uint32_t n_items = 0, n_cta = 0, n_eight = 0, n_small = 0;  // items, ends of their parts (BatchArgs)
+  bool narrow = true;            // small graphs go to parts of a CTA
   unsigned int* next = nullptr;  // queue heads
   uint32_t* sync = nullptr;      // SYNC_WORDS per graph
   uint32_t* err = nullptr;
@@ -767,14 +820,30 @@ void plan_queue(lg_batch* b) {
   for (uint32_t g = 0; g < b->count; g++) order[g] = g;
   auto work = [&](uint32_t g) { return ((uint64_t)b->host[g].arcs * 2 + b->host[g].n) / b->host[g].team; };
   std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return work(x) > work(y); });
+  // A graph goes to 8 warps or to one if its time there, 3 or 24 times that of
+  // a CTA's, is no more than a CTA's share of the whole queue: the narrower
+  // groups waste less, but a batch of few graphs needs every warp of a CTA for
+  // each.  A graph's barriers count like GRAPH_WORK of work (30 us).
+  constexpr uint64_t GRAPH_WORK = 16384;
+  uint64_t share = 0;
+  for (uint32_t g : order)
+    if (b->host[g].n <= BS_MAX) share += work(g) * b->host[g].team + GRAPH_WORK;
+  share /= (uint64_t)b->grid;
+  auto part = [&](uint32_t g) {
+    const BatchGraph& x = b->host[g];
+    if (x.n > BS_MAX) return 3;
+    if (!b->narrow || x.team > 1) return 0;
+    if (x.n <= BGroup<1>::MAX_N && work(g) * BS_WARPS <= share) return 2;
+    return x.n <= BGroup<8>::MAX_N && work(g) * (BS_WARPS / 8) <= share ? 1 : 0;
+  };
   b->items_h.clear();
-  for (const bool small : {true, false}) {
+  uint32_t* const ends[4] = {&b->n_cta, &b->n_eight, &b->n_small, &b->n_items};
+  for (int k = 0; k < 4; k++) {
     for (uint32_t g : order)
-      if ((b->host[g].n <= BS_MAX) == small)
+      if (part(g) == k)
         for (uint32_t m = 0; m < b->host[g].team; m++) b->items_h.push_back({g, m});
-    if (small) b->n_small = (uint32_t)b->items_h.size();
+    *ends[k] = (uint32_t)b->items_h.size();
   }
-  b->n_items = (uint32_t)b->items_h.size();
 }
 
 lg_status upload_plan(lg_batch* b, cudaStream_t st) {
@@ -794,13 +863,15 @@ lg_status upload_plan(lg_batch* b, cudaStream_t st) {
 }
 
 BatchArgs make_args(lg_batch* b, uint32_t* depth, float* ranks, float damp, uint32_t iters, uint32_t phases,
-                    const BatchItem* items, uint32_t n_small, uint32_t n_items, int lanes) {
+                    int lanes) {
   BatchArgs a;
   memset(&a, 0, sizeof(a));
   a.graphs = b->graphs;
-  a.items = items;
-  a.n_small = n_small;
-  a.n_items = n_items;
+  a.items = b->items;
+  a.n_cta = b->n_cta;
+  a.n_eight = b->n_eight;
+  a.n_small = b->n_small;
+  a.n_items = b->n_items;
   a.next = b->next;
   a.sync = b->sync;
   a.err = b->err;
@@ -824,7 +895,7 @@ BatchArgs make_args(lg_batch* b, uint32_t* depth, float* ranks, float damp, uint
 
 // one run: reset the queue heads, team counters and error word, then the persistent launches
 void enqueue_run(lg_batch* b, const BatchArgs& a, cudaStream_t st) {
-  cudaMemsetAsync(b->next, 0, 2 * sizeof(unsigned int), st);
+  cudaMemsetAsync(b->next, 0, 4 * sizeof(unsigned int), st);
   cudaMemsetAsync(b->sync, 0, (size_t)b->count * SYNC_WORDS * 4, st);
   cudaMemsetAsync(b->err, 0, 4, st);
   const uint32_t lanes = a.n_items - a.n_small;
@@ -860,6 +931,7 @@ lg_status time_run(lg_batch* b, const BatchArgs& a, cudaStream_t st, cudaEvent_t
 // graphs run alone (encode + 2 PageRank sweeps) with T = 1, 4, 8 and 32.
 // (2) The team tiles, if not fixed: each path's graphs (encode + BFS + 2
 // sweeps) with tiles of 2^18 .. 2^21 arcs, the lanes path's from 2^15 on.
+// (3) Whether small graphs go to parts of a CTA.
 lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStream_t st, cudaEvent_t e0,
                    cudaEvent_t e1) {
   const int cand_t[4] = {1, 4, 8, 32};
@@ -892,8 +964,10 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
     float best = 1e30f;
     int best_t = 8;
     for (int c = 0; c < 4 && s == LG_OK; c++) {
-      BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_PR, dlist, 0, (uint32_t)its.size(),
-                              cand_t[c]);
+      BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_PR, cand_t[c]);
+      a.items = dlist;
+      a.n_cta = a.n_eight = a.n_small = 0;
+      a.n_items = (uint32_t)its.size();
       float ms = 0;
       s = time_run(b, a, st, e0, e1, 2, &ms);
       if (ms < best) {
@@ -905,22 +979,31 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
   }
   cudaFree(dlist);
   if (s != LG_OK) return s;
-  if (b->opts.tile_arcs == 0) {
-    for (const bool small : {true, false}) {
-      uint64_t& tile = small ? b->tile_arcs : b->tile_lanes;
-      float best = 1e30f;
-      uint64_t best_k = tile;
+  // the present plan's part of one path
+  auto time_path = [&](bool small, float* ms) {
+    plan_queue(b);
+    lg_status r = upload_plan(b, st);
+    if (r != LG_OK) return r;
+    BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_BFS | PH_PR, 0);
+    if (small) {
+      a.n_items = a.n_small;
+    } else {
+      a.items += a.n_small;
+      a.n_items -= a.n_small;
+      a.n_cta = a.n_eight = a.n_small = 0;
+    }
+    return time_run(b, a, st, e0, e1, 2, ms);
+  };
+  for (const bool small : {true, false}) {
+    if (small ? !b->n_small : b->n_items == b->n_small) continue;
+    uint64_t& tile = small ? b->tile_arcs : b->tile_lanes;
+    float best = 1e30f, ms = 0;
+    uint64_t best_k = tile;
+    if (b->opts.tile_arcs == 0) {
       for (uint64_t k : {1ull << 15, 1ull << 17, 1ull << 18, 1ull << 19, 1ull << 20, 1ull << 21}) {
         if (small && k < 1ull << 18) continue;
         tile = k;
-        plan_queue(b);
-        const uint32_t n = small ? b->n_small : b->n_items - b->n_small;
-        if (n == 0) break;
-        if ((s = upload_plan(b, st)) != LG_OK) return s;
-        BatchArgs a = make_args(b, depth_tmp, ranks_tmp, 0.85f, 2, PH_ENCODE | PH_BFS | PH_PR,
-                                b->items + (small ? 0 : b->n_small), small ? n : 0, n, 0);
-        float ms = 0;
-        if ((s = time_run(b, a, st, e0, e1, 2, &ms)) != LG_OK) return s;
+        if ((s = time_path(small, &ms)) != LG_OK) return s;
         if (ms < best) {
           best = ms;
           best_k = k;
@@ -928,8 +1011,14 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
       }
       tile = best_k;
     }
-    plan_queue(b);
+    if (small && b->n_small > b->n_cta) {
+      if (best == 1e30f && (s = time_path(true, &best)) != LG_OK) return s;
+      b->narrow = false;
+      if ((s = time_path(true, &ms)) != LG_OK) return s;
+      b->narrow = best <= ms;
+    }
   }
+  plan_queue(b);
   if ((s = upload_plan(b, st)) != LG_OK) return s;
   uint32_t herr = 0;
   BTRY(cudaMemcpy(&herr, b->err, 4, cudaMemcpyDeviceToHost));
@@ -1071,8 +1160,7 @@ lg_status batch_create_impl(lg_batch* b, const uint64_t* graph_vptr, cudaStream_
       size_t j = i;
       while (j + 1 < b->items_h.size() && b->items_h[j + 1].g == g) j++;
       b->items_h.erase(b->items_h.begin() + (long)j);
-      b->n_items--;
-      if (j < b->n_small) b->n_small--;
+      for (uint32_t* end : {&b->n_cta, &b->n_eight, &b->n_small, &b->n_items}) *end -= j < *end;
       break;
     }
     if ((s = upload_plan(b, st)) != LG_OK) return s;
@@ -1159,7 +1247,7 @@ extern "C" lg_status lg_batch_run(lg_batch* b, float damping, uint32_t iters, ui
       b->exec = nullptr;
     }
     cudaGraph_t graph = nullptr;
-    BatchArgs a = make_args(b, depths, ranks, damping, iters, PH_ENCODE | PH_BFS | PH_PR, b->items, b->n_small, b->n_items, 0);
+    BatchArgs a = make_args(b, depths, ranks, damping, iters, PH_ENCODE | PH_BFS | PH_PR, 0);
     cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       enqueue_run(b, a, b->cap);
@@ -1180,7 +1268,7 @@ extern "C" lg_status lg_batch_run(lg_batch* b, float damping, uint32_t iters, ui
   if (status == LG_OK) {
     cudaError_t e = cudaGraphLaunch(b->exec, st);
     b->launches++;
-    count_kernels(make_args(b, depths, ranks, damping, iters, 0, b->items, b->n_small, b->n_items, 0));
+    count_kernels(make_args(b, depths, ranks, damping, iters, 0, 0));
     if (e != cudaSuccess) status = batch_fail("lg_batch_run: cudaGraphLaunch", e);
   }
   if (prev != b->device) cudaSetDevice(prev);
