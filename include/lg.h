@@ -519,8 +519,9 @@ lg_status lg_server_stats_get(lg_server *s, lg_server_stats *out);
  * is submitted by a separate thread at arrival_ns[i] after the start (PPR
  * with the server's default iterations and damping 0.85).  The calling thread
  * collects every result: latency_ns[i] = completion - scheduled arrival; if
- * keep and keep[i] are not NULL the result bytes are copied there (the caller
- * sizes it: see lg_result.data); every result is released.  All requests are
+ * keep and keep[i] are not NULL the result bytes are copied there before the
+ * call returns (the caller sizes it: see lg_result.data; where buffers overlap,
+ * in completion order); every result is released.  All requests are
  * validated before the clock starts.  Returns LG_ECUDA if a request failed.
  */
 lg_status lg_server_replay(lg_server *s, uint64_t n, const uint32_t *kind, const uint32_t *graph,

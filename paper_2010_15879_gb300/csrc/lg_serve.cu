@@ -31,12 +31,13 @@
 #include <deque>
 #include <memory>
 #include <mutex>
-#include <system_error>
+#include <optional>
 #include <thread>
 #include <unordered_map>
 #include <vector>
 
 #include "lg_arena.h"
+#include "lg_copies.h"
 #include "lg_internal.h"
 
 namespace lg {
@@ -1203,37 +1204,9 @@ extern "C" lg_status lg_server_replay(lg_server* s, uint64_t n, const uint32_t* 
   // Kept results are copied by a few helper threads, so that a burst's depth
   // and rank rows do not queue behind one thread's memcpy (84 MB of them took
   // 9 ms, the GPU's work 4); a result is released once it is copied.
-  struct Copy {
-    void* to;
-    const void* from;
-    uint64_t bytes, ticket;
-  };
-  std::mutex copy_mu;
-  std::condition_variable copy_cv;
-  std::deque<Copy> copies;
-  bool copy_end = false;
-  std::vector<std::thread> copiers;
-  auto copier = [&] {
-    for (;;) {
-      Copy c;
-      {
-        std::unique_lock<std::mutex> l(copy_mu);
-        copy_cv.wait(l, [&] { return copy_end || !copies.empty(); });
-        if (copies.empty()) return;
-        c = copies.front();
-        copies.pop_front();
-      }
-      memcpy(c.to, c.from, c.bytes);
-      lg_server_release(s, c.ticket);
-    }
-  };
-  if (keep) {
-    try {
-      for (unsigned k = 0; k < std::min(4u, std::max(1u, std::thread::hardware_concurrency() / 4)); k++)
-        copiers.emplace_back(copier);
-    } catch (const std::system_error&) {  // no more threads: those there copy, or this one
-    }
-  }
+  std::optional<CopyQueue> copies;
+  if (keep) copies.emplace(std::min(4u, std::max(1u, std::thread::hardware_concurrency() / 4)),
+                           [s](uint64_t ticket) { lg_server_release(s, ticket); });
   uint64_t got_all = 0, failed = 0, t_last = t0;
   std::vector<lg_result> buf(256);
   while (got_all < n) {
@@ -1247,27 +1220,12 @@ extern "C" lg_status lg_server_replay(lg_server* s, uint64_t n, const uint32_t* 
       if (r.status != LG_OK) failed++;
       t_last = std::max(t_last, r.t_done_ns);
       got_all++;
-      if (i < n && keep && keep[i] && r.data && copiers.empty()) {
-        memcpy(keep[i], r.data, r.bytes);
-        lg_server_release(s, r.ticket);
-      } else if (i < n && keep && keep[i] && r.data) {
-        {
-          std::lock_guard<std::mutex> l(copy_mu);
-          copies.push_back(Copy{keep[i], r.data, r.bytes, r.ticket});
-        }
-        copy_cv.notify_one();
-      } else {
-        lg_server_release(s, r.ticket);
-      }
+      if (i < n && keep && keep[i] && r.data) copies->push(keep[i], r.data, r.bytes, r.ticket);
+      else lg_server_release(s, r.ticket);
     }
   }
   submitter.join();
-  {
-    std::lock_guard<std::mutex> l(copy_mu);
-    copy_end = true;
-  }
-  copy_cv.notify_all();
-  for (auto& t : copiers) t.join();
+  copies.reset();  // waits for them
   if (out) {
     memset(out, 0, sizeof(*out));
     out->completed = got_all;
