@@ -183,6 +183,7 @@ GView make_view(const lg_graph* g) {
   v.n_multi = g->n_multi;
   v.heavy_min = g->heavy_min;
   v.heavy_seg = g->heavy_seg;
+  v.light_max = (uint32_t)(g->max_degree < g->heavy_min ? g->max_degree : g->heavy_min);
   v.heavy_prefix = g->heavy_prefix;
   v.mid_prefix = g->mid_prefix;
   return v;

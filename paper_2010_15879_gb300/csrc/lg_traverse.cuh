@@ -430,13 +430,24 @@ __host__ __device__ inline unsigned heavy_blocks(uint64_t n_items) {
 // time: 130 us for a BFS level, 490 us for a personalized PageRank sweep, even
 // on a graph of 62,000 vertices (measured), and a warp per 4,096-field item 30
 // to 60 us.  On large graphs other CTAs fill that time; below 2^22 vertices
-// the DM-ordered vertices of more than 32 arcs go in tiles of 64, the others in
-// tiles small enough for about four CTAs per SM, and when items are few a whole
-// CTA takes one (gap-coded items cannot be entered mid-way).
+// the DM-ordered vertices of more than 32 arcs go in tiles of 64 to 512, as many
+// as keep a tile's fields (at most light_max a vertex) a small part of the
+// arcs: 1 / 450 where every degree is near the largest, down to 1 / 1800 where
+// few are and the large tiles all start first.  Small tiles spend their time on
+// offsets and scans, large ones end late; BFS from 16 sources at 64 / 128 / 256
+// / 512, us (taken: *): R-MAT 2^18 577* 696 821 1118, 2^20 1017* 1043 1191 1622,
+// 3 M vertices 1713 1705* 1942 2528; community 0.7 M 702* 757 866 1074; 400,000
+// vertices of degree 160 608 549 474* 513, 1.5 M of 40 1703 1355 1202 1165*,
+// 1 M of 250 1779 1483 1241 1239*.  The others go in tiles small enough for
+// about four CTAs per SM, and when items are few a whole CTA takes one
+// (gap-coded items cannot be entered mid-way).
 inline TileMap tile_map(const GView& g, bool gap) {
   TileMap m;
   const bool small = g.n < (1ull << 22);
+  const uint64_t mean = g.n ? g.arcs / g.n : 0, most = std::max(g.light_max, 1u);
+  const uint64_t fields = g.arcs / most * std::max(std::min(mean, most), most / 4) / 450;
   m.ta = 64;
+  while (m.ta < TV && 2ull * m.ta * most <= fields) m.ta *= 2;
   m.tb = TV;
   if (small)
     while (m.tb > 64 && g.n / m.tb < 4 * 152) m.tb /= 2;
