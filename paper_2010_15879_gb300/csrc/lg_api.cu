@@ -183,7 +183,7 @@ GView make_view(const lg_graph* g) {
   v.n_multi = g->n_multi;
   v.heavy_min = g->heavy_min;
   v.heavy_seg = g->heavy_seg;
-  v.light_max = (uint32_t)(g->max_degree < g->heavy_min ? g->max_degree : g->heavy_min);
+  v.max_degree = (uint32_t)g->max_degree;
   v.heavy_prefix = g->heavy_prefix;
   v.mid_prefix = g->mid_prefix;
   return v;
@@ -343,21 +343,42 @@ uint32_t hot_rows(const lg_graph* g, uint32_t elem_bytes) {
 // the tile's own cost against the longest unit; measured per sweep at 4 / 8 /
 // 16 / 32 vertices: R-MAT 2^12 in DM order 8 / 10 / 13 / 19 us, community 2^15
 // 25 / 26 / 34 / 54, community 2^18 in DM order 133 / 80 / 58 / 80, R-MAT 2^18
-// not relabeled 110 / 72 / 53 / 47, R-MAT 900,000 287 / 173 / 114 / 85.  The shared-memory table
-// of contributions pays when it answers some of the gathers of a sweep that is
-// long enough to fill it (R-MAT 2^24 in DM order, 28 % of the arcs on the
-// first 16,384 labels: 1.78 -> 1.61 ms a sweep; community 2^23, 9 %: 0.94 ->
-// 0.91; 2^24, 6 %: equal; R-MAT 2^18, 76 %: 41 -> 43 us).
+// not relabeled 110 / 72 / 53 / 47, R-MAT 900,000 287 / 173 / 114 / 85.  Where
+// no degree is above four times the mean, no unit is long for its size, and
+// tiles are as large as leaves one for every second warp: 5 M vertices of
+// degree 40 in DM order, local-gap IDs, 1.02 ms in tiles of 32, 0.90 in 128,
+// 300,000 of degree 40 86 and 76 us.  Such a graph's heavy items, short ones,
+// come after its tiles (1 M vertices of degree 250, 35 % of them heavy: 1.27 ms
+// with the items first, 1.12 so), several to a ticket.
+//
+// The shared-memory table of contributions pays when it answers some of the
+// gathers of a sweep that is long enough to fill it (R-MAT 2^24 in DM order,
+// 28 % of the arcs on the first 16,384 labels: 1.78 -> 1.61 ms a sweep;
+// community 2^23, 9 %: 0.94 -> 0.91; 2^24, 6 %: equal; R-MAT 2^18, 76 %: 41 ->
+// 43 us).  Without it the L1 answers some too, and on a small graph more, unless
+// its hubs take a third of the arcs and it is not that small: degree 1,600, 40,000 vertices 147 us with
+// the table, 83 without, 100,000 of 1,000 294 and 269, 200,000 of 500 348 and
+// 368; R-MAT 2^17 in DM order 46 and 49, not relabeled 75 and 69.
 PrPlan pr_plan(const lg_graph* g) {
   PrPlan p;
   const uint64_t warps = (uint64_t)PW_WARPS * PW_SMS;
   const bool small = g->n < 2 * warps * PW_TV;
-  p.tile_a = g->heavy_prefix & ~31ull;
-  p.tile_nv = g->n < (1u << 14) ? 4 : g->n < (1u << 16) ? 8 : g->n < (1u << 19) && g->relabel == 1 ? 16 : 32;
-  const uint64_t end = small ? g->n : g->mid_prefix > p.tile_a ? g->mid_prefix : p.tile_a;
+  const bool even = g->max_degree * g->n <= 4 * g->arcs;
+  p.tile_a = g->heavy_prefix & ~(uint64_t)(PW_TV - 1);
+  uint64_t end = small || even ? g->n : g->mid_prefix > p.tile_a ? g->mid_prefix : p.tile_a;
+  if (even) {
+    p.tile_nv = g->arcs > g->heavy_min * g->n ? 32 : 4;  // tiles of next to no light fields are not worth splitting
+    while (p.tile_nv < PW_TV && g->n / (2 * p.tile_nv) >= warps / 2) p.tile_nv *= 2;
+    p.items = 1;
+    while (g->n_items / (2 * p.items) >= 12 * warps) p.items *= 2;
+  } else {
+    p.tile_nv = g->n < (1u << 14) ? 4 : g->n < (1u << 16) ? 8 : g->n < (1u << 19) && g->relabel == 1 ? 16 : 32;
+    p.items = 1;
+  }
   p.tile_b = (end + PW_TV - 1) & ~(uint64_t)(PW_TV - 1);
   const uint64_t most = (PW_SMEM - PW_WARPS * sizeof(PrWarp)) / sizeof(float);
-  p.tabn = g->arcs >> 24 && 12 * g->top_arcs >= g->arcs ? (uint32_t)(g->n < most ? g->n : most) : 0;
+  const bool table = g->n >= 3u << 16 ? 12 * g->top_arcs >= g->arcs : g->n >= 1u << 17 && 3 * g->top_arcs >= g->arcs;
+  p.tabn = g->arcs >> 24 && table ? (uint32_t)(g->n < most ? g->n : most) : 0;
   p.part_floats = g->n_multi ? g->n_items : 0;
   p.sync_words = 2 + g->n_multi;
   p.aux_words = g->off_mode == OFF_EF ? (p.tile_b - p.tile_a) / p.tile_nv + g->n / PW_TV + 1 : 0;
@@ -955,6 +976,7 @@ extern "C" lg_status lg_pagerank(const lg_graph* g, float damping, uint32_t iter
   a.tile_a = plan.tile_a;
   a.tile_b = plan.tile_b;
   a.tile_nv = plan.tile_nv;
+  a.items = plan.items;
   a.tabn = plan.tabn;
   a.sync = tsync.as<uint32_t>();
   a.nsync = plan.sync_words;

@@ -70,7 +70,7 @@ struct GView {
   uint32_t s, H, omega, r, w_O, ef_l, sample_log2;
   uint32_t heavy_min;         // degrees above this are in the schedule
   uint32_t heavy_seg;         // max fields per schedule item
-  uint32_t light_max;         // no vertex outside the schedule has a larger degree
+  uint32_t max_degree;
   uint64_t heavy_prefix;      // the vertices below this label are all in the schedule (DM order; else 0)
   uint64_t mid_prefix;        // the vertices below this label have more than 32 arcs (DM order; else 0)
 };

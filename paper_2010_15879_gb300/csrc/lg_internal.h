@@ -152,9 +152,10 @@ struct PrArgs {
                              // others are evict-first (DM order puts the most gathered vertices first)
   uint64_t tile_a, tile_b;   // vertices [tile_a, tile_b) in warp tiles of tile_nv, the others of 128 (PrPlan)
   uint32_t tile_nv;
+  uint32_t items;            // heavy items per ticket (PrPlan)
   uint32_t tabn;             // contributions u < tabn are gathered from shared memory (PrPlan)
   uint32_t turn;             // which of the two ticket counters this iteration uses
-  uint32_t* sync;            // [0..1] ticket counters, [2 + first item] arrived parts of a split vertex
+  uint32_t* sync;            // [0..1] ticket counters, [2 + slot] arrived parts of a split vertex
   uint64_t nsync;            // words of sync
   uint64_t* aux;             // Elias-Fano: where each warp tile starts in the high vector
 };
@@ -162,7 +163,7 @@ struct PrArgs {
 // How a PageRank call runs on a graph: chosen from its sizes by pr_plan.
 struct PrPlan {
   uint64_t tile_a, tile_b;
-  uint32_t tile_nv, tabn;
+  uint32_t tile_nv, items, tabn;
   uint64_t part_floats;      // PrArgs::part
   uint64_t sync_words;       // PrArgs::sync
   uint64_t aux_words;        // PrArgs::aux

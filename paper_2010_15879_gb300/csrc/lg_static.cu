@@ -141,6 +141,7 @@ extern "C" lg_status lg_pagerank_noalloc(const lg_graph* g, float damping, uint3
     a.tile_a = plan.tile_a;
     a.tile_b = plan.tile_b;
     a.tile_nv = plan.tile_nv;
+    a.items = plan.items;
     a.tabn = plan.tabn;
     a.sync = reinterpret_cast<uint32_t*>(part + kMaxItems);
     a.nsync = plan.sync_words;

@@ -431,7 +431,7 @@ __host__ __device__ inline unsigned heavy_blocks(uint64_t n_items) {
 // on a graph of 62,000 vertices (measured), and a warp per 4,096-field item 30
 // to 60 us.  On large graphs other CTAs fill that time; below 2^22 vertices
 // the DM-ordered vertices of more than 32 arcs go in tiles of 64 to 512, as many
-// as keep a tile's fields (at most light_max a vertex) a small part of the
+// as keep a tile's fields (at most heavy_min a vertex) a small part of the
 // arcs: 1 / 450 where every degree is near the largest, down to 1 / 1800 where
 // few are and the large tiles all start first.  Small tiles spend their time on
 // offsets and scans, large ones end late; BFS from 16 sources at 64 / 128 / 256
@@ -444,10 +444,11 @@ __host__ __device__ inline unsigned heavy_blocks(uint64_t n_items) {
 inline TileMap tile_map(const GView& g, bool gap) {
   TileMap m;
   const bool small = g.n < (1ull << 22);
-  const uint64_t mean = g.n ? g.arcs / g.n : 0, most = std::max(g.light_max, 1u);
-  const uint64_t fields = g.arcs / most * std::max(std::min(mean, most), most / 4) / 450;
+  // 1 / 4 .. 1: mean degree over the largest
+  const double even = std::max(0.25, (double)g.arcs / ((double)g.n * std::max(g.max_degree, 1u)));
+  const double vertices = (double)g.arcs * even / 450.0 / std::max(std::min(g.max_degree, g.heavy_min), 1u);
   m.ta = 64;
-  while (m.ta < TV && 2ull * m.ta * most <= fields) m.ta *= 2;
+  while (m.ta < TV && 2.0 * m.ta <= vertices) m.ta *= 2;
   m.tb = TV;
   if (small)
     while (m.tb > 64 && g.n / m.tb < 4 * 152) m.tb /= 2;
