@@ -336,6 +336,9 @@ uint32_t hot_rows(const lg_graph* g, uint32_t elem_bytes) {
   return (uint32_t)(rows < all ? rows : all);
 }
 
+// no degree far above the mean
+bool even_degrees(const lg_graph* g) { return g->max_degree * g->n <= 4 * g->arcs; }
+
 // Warp tiles hold 128 vertices, but fewer where that would make a long unit: in
 // a small graph (fewer than two tiles of 128 per resident warp), and for the
 // DM-ordered vertices of more than 32 arcs (a warp walks 256 fields in about
@@ -363,7 +366,7 @@ PrPlan pr_plan(const lg_graph* g) {
   PrPlan p;
   const uint64_t warps = (uint64_t)PW_WARPS * PW_SMS;
   const bool small = g->n < 2 * warps * PW_TV;
-  const bool even = g->max_degree * g->n <= 4 * g->arcs;
+  const bool even = even_degrees(g);
   p.tile_a = g->heavy_prefix & ~(uint64_t)(PW_TV - 1);
   uint64_t end = small || even ? g->n : g->mid_prefix > p.tile_a ? g->mid_prefix : p.tile_a;
   if (even) {
@@ -446,7 +449,9 @@ extern "C" lg_status lg_decode(const lg_graph* g, uint64_t* row_ptr, uint32_t* c
   }
   // local IDs: one launch (row offsets by a single-pass look-back over the
   // tiles, then the rows); its small state is zeroed first
-  dec_tiles(n, v.mid_prefix, a);
+  const bool even = even_degrees(g);
+  dec_tiles(n, v.mid_prefix, even, a);
+  a.heavy_after = even && g->arcs > (uint64_t)g->heavy_min * n;
   const uint64_t ntiles = a.tiles;
   Tmp t_state(st);
   const size_t bytes = ntiles * (sizeof(unsigned long long) + sizeof(uint32_t)) + 16;
