@@ -324,13 +324,16 @@ struct SegRows {
 };
 
 // ---------------------------------------------------------------------------
-// Rows of 33..128 keys of a size class, P = 16 G >= d keys per row (padded
-// with UINT32_MAX), G lanes per row.  Lane g holds keys 16 g + e, e < 16, so a
+// Rows of 33..128 keys of a size class, and of up to 512 without values, P =
+// 16 G >= d keys per row (padded with UINT32_MAX), G lanes per row.  Lane g holds keys 16 g + e, e < 16, so a
 // bitonic compare-exchange at distance j is a register pair for j < 16 and a
 // shuffle with lane g ^ (j / 16) beyond.  The first four levels are unrolled;
 // the rest run as a loop (an unrolled network of this size would outgrow the
-// instruction cache).  From 129 keys on the network's log2(d) (log2(d) + 1) / 2
-// stages cost more than a radix sort's passes (169 keys: 35 G keys/s).
+// instruction cache).  Values double each stage's moves, so from 129 keys on
+// rows with values are quicker by radix, which moves indices (R-MAT 2^22, whole
+// encode, degree order: 3.80 ms, 4.54 with the network up to 512; 3 M vertices
+// of degree 200 15.2 and 20.4); rows of keys alone are not (2.99 and 2.94, 12.9
+// and 7.7; in greedy order 19.7 and 10.6).
 // ---------------------------------------------------------------------------
 template <int J, bool VALS>
 __device__ __forceinline__ void blk_pairs(uint32_t (&x)[16], uint32_t (&y)[16], uint32_t base16, uint32_t k) {
@@ -828,7 +831,7 @@ static cudaError_t seg_sort_big_prefix(uint32_t* keys, uint32_t* vals, const Srs
 }
 
 // -------------------------------------------------------------------------
-// Rows of 129..16384 keys: a CTA of NW warps per row of up to 512 NW keys, a
+// Rows of 129..16384 keys (513.. without values): a CTA of NW warps per row of up to 512 NW keys, a
 // stable LSD radix sort with 9-bit digits in shared memory.  The passes move
 // the keys' indices only, keys and values stay where they were loaded until
 // the sorted row is written.
@@ -1009,7 +1012,11 @@ static cudaError_t seg_sort_classes(uint32_t* keys, uint32_t* vals, const uint64
       case 1: e = seg_blk_launch<4, VALS>(keys, vals, off, rows[k], st); break;
       case 2: e = seg_blk_launch<8, VALS>(keys, vals, off, rows[k], st); break;
       case 3:
-      case 4: e = seg_radix_launch<1, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
+      case 4:
+        if (VALS) e = seg_radix_launch<1, VALS>(keys, vals, off, rows[k], key_bits, coarse, st);
+        else if (k == 3) e = seg_blk_launch<16, false>(keys, nullptr, off, rows[k], st);
+        else e = seg_blk_launch<32, false>(keys, nullptr, off, rows[k], st);
+        break;
       case 5: e = seg_radix_launch<2, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
       case 6: e = seg_radix_launch<4, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
       case 7: e = seg_radix_launch<8, VALS>(keys, vals, off, rows[k], key_bits, coarse, st); break;
