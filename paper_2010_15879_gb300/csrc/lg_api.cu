@@ -695,7 +695,8 @@ static lg_status encode_impl(lg_graph* g, const uint64_t* row_ptr, const uint32_
     LG_TRY(t_stmp.alloc(scan_tmp_words(n) * sizeof(uint64_t)));
     Tmp t_long(st);
     LongRows rows, *L = nullptr;
-    if (g->max_degree > LONG_ROW) {
+    const bool alike = even_degrees(g) && g->max_degree <= LONG_WINDOW && n >= 32ull * 152 * 16;
+    if (g->max_degree > LONG_ROW && !alike) {
       LG_TRY(t_long.alloc(long_rows_bytes(arcs)));
       rows = long_rows(t_long.p, arcs);
       L = &rows;

@@ -248,18 +248,33 @@ cudaError_t enc_check_symmetric(const uint64_t* rp, const uint32_t* col, uint64_
 // arcs, to one warp, so they are listed in windows of LONG_WINDOW fields first
 // and a warp takes a window, here and in the packing below (community graph of
 // 1.5 M vertices: this pass 83 us, the packing 135; 486 and 904 with every
-// row left to its warp, 157 and 248 with only rows above 1,024 listed).
+// row left to its warp, 157 and 248 with only rows above 1,024 listed).  Where
+// rows are all alike and no longer than a window nothing is listed (LongRows
+// null): the warps' shares are even anyhow (400,000 rows of 300 arcs, whole
+// encode: 960 us listed, 905 not).
 constexpr int LL_STAGE = 1024;
 
 // fields of a row that windows count: gaps, or IDs
 __device__ __forceinline__ uint64_t row_fields(uint64_t d, int gap) { return gap ? d - 1 : d; }
 
+// (A warp counts its rows and windows before it adds to the two counters: an add
+// per row took 206 us for 350,000 rows among 1 M.)
 __global__ void __launch_bounds__(256) k_long_list(const uint64_t* __restrict__ rp, uint64_t n, int gap, LongRows L) {
-  for (uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t d = rp[v + 1] - rp[v];
-    if (d <= LONG_ROW) continue;
-    const uint32_t nw = (uint32_t)((row_fields(d, gap) + LONG_WINDOW - 1) / LONG_WINDOW);
-    const uint32_t slot = atomicAdd(L.counts + 1, 1u), at = atomicAdd(L.counts, nw);
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < n; v0 += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t v = v0 + lane, d = v < n ? rp[v + 1] - rp[v] : 0;
+    const uint32_t nw = d > LONG_ROW ? (uint32_t)((row_fields(d, gap) + LONG_WINDOW - 1) / LONG_WINDOW) : 0u;
+    const uint32_t rows = __ballot_sync(LG_FULL_MASK, nw != 0);
+    if (!rows) continue;
+    const uint32_t incl = warp_incl_scan<uint32_t>(nw);
+    uint32_t slot = 0, at = 0;
+    if (lane == 31) {
+      slot = atomicAdd(L.counts + 1, (uint32_t)__popc(rows));
+      at = atomicAdd(L.counts, incl);
+    }
+    slot = __shfl_sync(LG_FULL_MASK, slot, 31) + __popc(rows & ((1u << lane) - 1u));
+    at = __shfl_sync(LG_FULL_MASK, at, 31) + incl - nw;
+    if (!nw) continue;
     L.rows[slot] = (uint32_t)v;
     L.gmax[slot] = 0;
     for (uint32_t k = 0; k < nw; k++) L.windows[at + k] = make_uint2(slot, k);
@@ -315,7 +330,7 @@ cudaError_t enc_long_rows(const uint64_t* rp, uint64_t n, int gap, const LongRow
 __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restrict__ rp,
                                                        const uint32_t* __restrict__ col, uint64_t n, int gap,
                                                        uint32_t s, uint32_t H, uint8_t* __restrict__ wid,
-                                                       uint64_t* __restrict__ len) {
+                                                       uint64_t* __restrict__ len, uint32_t long_row) {
   __shared__ uint32_t stage[8][LL_STAGE];
   const int lane = threadIdx.x & 31;
   uint32_t* sk = stage[threadIdx.x >> 5];
@@ -334,7 +349,7 @@ __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restric
         const uint32_t tot = (uint32_t)(r1 - r0);
         for (uint32_t q = lane; q < tot; q += 32) sk[q] = col[r0 + q];
         __syncwarp();
-        if (lane < rows && mhi - mlo >= 2) {
+        if (lane < rows && mhi - mlo >= 2 && mhi - mlo <= long_row) {
           const uint32_t* row = sk + (mlo - r0);
           const uint32_t d = (uint32_t)(mhi - mlo);
           uint32_t prev = row[0], mg = 0;
@@ -349,7 +364,7 @@ __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restric
       } else {
         for (int r = 0; r < rows; r++) {
           const uint64_t lo = __shfl_sync(LG_FULL_MASK, mlo, r), hi = __shfl_sync(LG_FULL_MASK, mhi, r);
-          if (hi - lo < 2 || hi - lo > LONG_ROW) continue;  // long rows: k_long_gaps
+          if (hi - lo < 2 || hi - lo > long_row) continue;  // long rows: k_long_gaps
           uint32_t mg = 0;
           for (uint64_t j = lo + 1 + lane; j < hi; j += 32) mg = max(mg, col[j] - col[j - 1]);
           mg = __reduce_max_sync(LG_FULL_MASK, mg);
@@ -357,7 +372,7 @@ __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restric
         }
       }
     }
-    if (lane < rows && !(gap && mhi - mlo > LONG_ROW)) {
+    if (lane < rows && !(gap && mhi - mlo > long_row)) {
       const uint64_t d = mhi - mlo;
       wid[mv] = (uint8_t)mw;
       len[mv] = gap ? (uint64_t)H + (d >= 1 ? s : 0) + (d >= 2 ? (d - 1) * (uint64_t)mw : 0)
@@ -368,7 +383,7 @@ __global__ void __launch_bounds__(256) k_local_lengths(const uint64_t* __restric
 
 cudaError_t enc_local_lengths(const uint64_t* rp, const uint32_t* col, uint64_t n, int gap, uint32_t s, uint32_t H,
                               uint8_t* wid, uint64_t* len, const LongRows* L, cudaStream_t st) {
-  k_local_lengths<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(rp, col, n, gap, s, H, wid, len);
+  k_local_lengths<<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(rp, col, n, gap, s, H, wid, len, L ? LONG_ROW : ~0u);
   count_launch();
   if (gap && L) {
     k_long_gaps<<<152 * 8, 256, 0, st>>>(rp, col, *L);
@@ -487,9 +502,9 @@ cudaError_t enc_pack_u64(const uint64_t* vals, uint64_t count, uint32_t w, uint6
 // most PK_ARCS arcs, their arcs are staged in shared memory with coalesced
 // loads and each lane emits its row's record into a shared copy of the
 // group's bit range (shared atomicOr, as neighbouring records share words).
-// Otherwise the warp packs the rows one at a time, a lane per field; rows of
-// more than LONG_ROW arcs are left to k_pack_long, a warp per window of
-// LONG_WINDOW fields.  Either way the warp then writes the bit
+// Otherwise the warp packs the rows one at a time, a lane per field.  In both
+// ways listed rows (of more than LONG_ROW arcs) are left to k_pack_long, a warp
+// per window of LONG_WINDOW fields, which runs afterwards.  Either way the warp then writes the bit
 // range out coalesced: its inner 64-bit words are its own, its first and last
 // word may be shared with the neighbouring range and are OR-ed into A (zeroed
 // at allocation).
@@ -562,7 +577,7 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pack_local(const uint64_t* __
                                                              const uint32_t* __restrict__ col,
                                                              const uint64_t* __restrict__ x,
                                                              const uint8_t* __restrict__ wid, uint64_t n, uint32_t s,
-                                                             uint32_t H, uint64_t* __restrict__ out) {
+                                                             uint32_t H, uint64_t* __restrict__ out, uint32_t long_row) {
   __shared__ uint32_t stg_all[PK_WARPS][PK_STAGE];
   __shared__ uint32_t ob_all[PK_WARPS][PK_W32];
   const int lane = threadIdx.x & 31;
@@ -592,7 +607,7 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pack_local(const uint64_t* __
       for (uint32_t q = lane; q < tot; q += 32) stg[q] = col[r0 + q];
       pk_clear(ob, B0, B1, lane);
       __syncwarp();
-      if (lane < rows) {
+      if (lane < rows && mhi - mlo <= long_row) {
         const uint32_t* row = stg + (mlo - r0);
         const uint32_t d = (uint32_t)(mhi - mlo);
         uint64_t p = xb - base;
@@ -627,7 +642,7 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pack_local(const uint64_t* __
       const uint64_t lo = __shfl_sync(LG_FULL_MASK, mlo, r), hi = __shfl_sync(LG_FULL_MASK, mhi, r);
       const uint64_t rb = __shfl_sync(LG_FULL_MASK, xb, r), re = __shfl_sync(LG_FULL_MASK, xe, r);
       const uint32_t w = __shfl_sync(LG_FULL_MASK, wv, r);
-      if (hi - lo <= LONG_ROW) pk_window<GAP>(col, lo, hi - lo, rb, re, w, 0, s, H, stg, ob, out, lane);
+      if (hi - lo <= long_row) pk_window<GAP>(col, lo, hi - lo, rb, re, w, 0, s, H, stg, ob, out, lane);
     }
   }
 }
@@ -654,8 +669,9 @@ cudaError_t enc_pack_local(const uint64_t* rp, const uint32_t* col, const uint64
                            cudaStream_t st) {
   if (data_words == 0 || n == 0) return cudaSuccess;
   const unsigned grid = grid_for((n + PK_ROWS - 1) / PK_ROWS, PK_WARPS, 152 * 16);
-  if (gap) k_pack_local<true><<<grid, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, n, s, H, out);
-  else k_pack_local<false><<<grid, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, n, s, H, out);
+  const uint32_t long_row = L ? LONG_ROW : LONG_WINDOW;  // no row is longer than a window without a list
+  if (gap) k_pack_local<true><<<grid, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, n, s, H, out, long_row);
+  else k_pack_local<false><<<grid, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, n, s, H, out, long_row);
   count_launch();
   if (L) {
     if (gap) k_pack_long<true><<<152 * 6, PK_WARPS * 32, 0, st>>>(rp, col, x, wid, s, H, out, *L);

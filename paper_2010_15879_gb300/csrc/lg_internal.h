@@ -99,8 +99,7 @@ cudaError_t enc_dm_relabel(const uint64_t* rp, const uint32_t* col, const uint32
                            uint64_t arcs, uint64_t max_deg, uint32_t mode, uint32_t* perm, uint32_t* inv_perm,
                            uint64_t* nrp, uint32_t* ncol, uint32_t* nw, cudaStream_t st);
 // Rows of more than LONG_ROW arcs, listed for the local widths and packing in
-// windows of LONG_WINDOW fields (one long_rows_bytes(arcs) block; only needed if
-// such rows exist).
+// windows of LONG_WINDOW fields (one long_rows_bytes(arcs) block).
 constexpr uint32_t LONG_ROW = 256, LONG_WINDOW = 1024;
 struct LongRows {
   uint32_t* counts;  // [0] windows, [1] rows
@@ -111,7 +110,7 @@ struct LongRows {
 uint64_t long_rows_bytes(uint64_t arcs);
 LongRows long_rows(void* mem, uint64_t arcs);
 cudaError_t enc_long_rows(const uint64_t* rp, uint64_t n, int gap, const LongRows& L, cudaStream_t st);
-// L: the listed rows, or null if no row is that long
+// L: the listed rows, or null if none is listed and every row stays with its warp
 cudaError_t enc_local_lengths(const uint64_t* rp, const uint32_t* col, uint64_t n, int gap, uint32_t s,
                               uint32_t H, uint8_t* wid, uint64_t* len, const LongRows* L, cudaStream_t st);
 cudaError_t enc_pack_global(const uint32_t* col, const uint32_t* w, uint64_t arcs, uint32_t s,
@@ -315,6 +314,9 @@ uint32_t hot_rows(const lg_graph* g, uint32_t elem_bytes);
 cudaError_t pr_fill0(float* ranks, uint64_t n, int64_t personal_orig, cudaStream_t st);
 
 PrPlan pr_plan(const lg_graph* g);
+
+// no degree far above the mean (lg_api.cu)
+bool even_degrees(const lg_graph* g);
 
 // BFS helpers (lg_api.cu); vmajor: depth[v * S + s] instead of depth[s * n + v]
 cudaError_t bfs_permute_depths(const uint32_t* tmp, uint32_t* out, const uint32_t* perm, uint64_t n,
