@@ -553,39 +553,34 @@ static lg_status build_schedule(lg_graph* g, const uint64_t* x, cudaStream_t st)
   g->heavy_min = heavy_min_env();
   g->heavy_seg = heavy_seg_env();
   const uint64_t ntiles = (g->n + LG_TILE_V - 1) / LG_TILE_V;
-  Tmp t_cnt(st), t_mcnt(st), t_off(st), t_moff(st), t_stmp(st), t_seg(st), t_mid(st);
-  struct { unsigned long long top; uint32_t mid, pad; } first = {};
-  LG_TRY(t_mid.alloc(sizeof(first)));
-  LG_TRY(cudaMemsetAsync(t_mid.p, 0, sizeof(first), st));
-  LG_TRY(t_cnt.alloc(ntiles * sizeof(uint32_t)));
-  LG_TRY(t_mcnt.alloc(ntiles * sizeof(uint32_t)));
-  LG_TRY(t_off.alloc((ntiles + 1) * sizeof(uint64_t)));
-  LG_TRY(t_moff.alloc((ntiles + 1) * sizeof(uint64_t)));
-  LG_TRY(t_stmp.alloc(scan_tmp_words(ntiles) * sizeof(uint64_t)));
+  // counts of items, then of split vertices, per tile, scanned together
+  Tmp t_cnt(st), t_off(st), t_stmp(st), t_seg(st);
+  struct { uint64_t end; unsigned long long top; uint32_t mid, pad; } sums;  // end: of the scan
+  LG_TRY(t_cnt.alloc(2 * ntiles * sizeof(uint32_t)));
+  LG_TRY(t_off.alloc(2 * ntiles * sizeof(uint64_t) + sizeof(sums)));
+  LG_TRY(t_stmp.alloc(scan_tmp_words(2 * ntiles) * sizeof(uint64_t)));
+  uint64_t* off = t_off.as<uint64_t>();
+  LG_TRY(cudaMemsetAsync(off + 2 * ntiles, 0, sizeof(sums), st));
   PlanArgs p;
   memset(&p, 0, sizeof(p));
   p.tile_count = t_cnt.as<uint32_t>();
-  p.multi_count = t_mcnt.as<uint32_t>();
-  p.tile_off = t_off.as<uint64_t>();
-  p.multi_off = t_moff.as<uint64_t>();
-  p.top = t_mid.as<unsigned long long>();
-  p.mid = reinterpret_cast<uint32_t*>(p.top + 1);
+  p.multi_count = p.tile_count + ntiles;
+  p.tile_off = off;
+  p.multi_off = off + ntiles;  // behind all items
+  p.top = reinterpret_cast<unsigned long long*>(off + 2 * ntiles + 1);
+  p.mid = g->relabel == 1 ? reinterpret_cast<uint32_t*>(p.top + 1) : nullptr;
   GView v = make_view(g);
   v.O = x;
   const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
   LG_TRY(ops->plan_count(v, p, st));
-  LG_TRY(scan_excl_u32(p.tile_count, ntiles, t_off.as<uint64_t>(), t_stmp.as<uint64_t>(), st));
-  LG_TRY(scan_excl_u32(p.multi_count, ntiles, t_moff.as<uint64_t>(), t_stmp.as<uint64_t>(), st));
-  uint64_t tot[2] = {0, 0};
-  LG_TRY(cudaMemcpyAsync(&first, t_mid.p, sizeof(first), cudaMemcpyDeviceToHost, st));
-  LG_TRY(cudaMemcpyAsync(&tot[0], t_off.as<uint64_t>() + ntiles, 8, cudaMemcpyDeviceToHost, st));
-  LG_TRY(cudaMemcpyAsync(&tot[1], t_moff.as<uint64_t>() + ntiles, 8, cudaMemcpyDeviceToHost, st));
+  LG_TRY(scan_excl_u32(p.tile_count, 2 * ntiles, off, t_stmp.as<uint64_t>(), st));
+  LG_TRY(cudaMemcpyAsync(&g->n_items, off + ntiles, sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
+  LG_TRY(cudaMemcpyAsync(&sums, off + 2 * ntiles, sizeof(sums), cudaMemcpyDeviceToHost, st));
   LG_TRY(cudaStreamSynchronize(st));
-  g->n_items = tot[0];
-  g->n_multi = tot[1];
+  g->n_multi = sums.end - g->n_items;
   g->heavy_prefix = 0;
-  g->mid_prefix = g->relabel == 1 ? first.mid : 0;
-  g->top_arcs = first.top;
+  g->mid_prefix = g->relabel == 1 ? sums.mid : 0;
+  g->top_arcs = sums.top;
   if (g->n_items == 0) return LG_OK;
   LG_TRY(pool_alloc((void**)&g->items, g->n_items * sizeof(HeavyItem), st));
   if (g->n_multi) LG_TRY(pool_alloc((void**)&g->multi, g->n_multi * sizeof(uint32_t), st));

@@ -128,13 +128,13 @@ cudaError_t enc_ef_samples(const uint64_t* x, uint64_t N, uint32_t l, uint32_t s
 struct PlanArgs {
   uint32_t* tile_count;      // items per tile (count pass) / multi vertices per tile
   const uint64_t* tile_off;  // exclusive prefix of tile_count (fill pass)
-  const uint64_t* multi_off; // exclusive prefix of multi vertices per tile
+  const uint64_t* multi_off; // exclusive prefix of multi vertices per tile, from [0] on
   uint32_t* multi_count;
   HeavyItem* items;
   uint32_t* multi;
   uint32_t* segsum;          // per item: sum of its (gap) values
   unsigned long long* top;   // sum of the degrees of the first PW_TOP labels
-  uint32_t* mid;             // largest v + 1 over the vertices of more than 32 arcs
+  uint32_t* mid;             // largest v + 1 over the vertices of more than 32 arcs (null: not wanted)
 };
 
 struct PrArgs {

@@ -1584,10 +1584,14 @@ __global__ void __launch_bounds__(TNT) k_plan_count(GView g, PlanArgs p) {
     if (d > 32) mid = (uint32_t)(v0 + i) + 1u;
     if (v0 + i < PW_TOP) top += d;
   }
-  mid = __reduce_max_sync(LG_FULL_MASK, mid);
-  top = warp_sum<uint64_t>(top);
-  if ((threadIdx.x & 31) == 0 && mid) atomicMax(p.mid, mid);
-  if ((threadIdx.x & 31) == 0 && top) atomicAdd(p.top, (unsigned long long)top);
+  if (p.mid) {
+    mid = __reduce_max_sync(LG_FULL_MASK, mid);
+    if ((threadIdx.x & 31) == 0 && mid) atomicMax(p.mid, mid);
+  }
+  if (v0 < PW_TOP) {
+    top = warp_sum<uint64_t>(top);
+    if ((threadIdx.x & 31) == 0 && top) atomicAdd(p.top, (unsigned long long)top);
+  }
   uint64_t total;
   block_excl_scan<uint64_t, TNT>(mine, total, sm.red64);
   if (threadIdx.x == 0) {
@@ -1617,7 +1621,7 @@ __global__ void __launch_bounds__(TNT) k_plan_fill(GView g, PlanArgs p) {
   uint64_t total;
   const uint64_t pre = block_excl_scan<uint64_t, TNT>(mine, total, sm.red64);
   uint64_t it = p.tile_off[blockIdx.x] + (pre >> 32);
-  uint64_t slot = p.multi_off[blockIdx.x] + (uint32_t)pre;
+  uint64_t slot = p.multi_off[blockIdx.x] - p.multi_off[0] + (uint32_t)pre;
 #pragma unroll
   for (int q = 0; q < TV / TNT; q++) {
     const uint32_t k = items_of(g, d_[q]);
