@@ -631,6 +631,7 @@ static lg_status encode_impl(lg_graph* g, const uint64_t* row_ptr, const uint32_
   g->H = host_bits(g->s);
   g->omega = 0;
   if (weights) {
+    g->max_weight = h.maxw;
     g->omega = o.weight_bits ? o.weight_bits : host_bits(h.maxw);
     if (g->omega < 1) g->omega = 1;
   }

@@ -16,6 +16,7 @@ struct lg_graph {
   uint64_t bits_A, bits_O;
   uint64_t ef_N, ef_U, ef_low_bits, ef_high_bits, n_samples;
   uint64_t max_degree;
+  uint32_t max_weight;
   uint64_t *A;          uint64_t words_A;
   uint64_t *O;          uint64_t words_O;  // packed offsets, or row_ptr for CSR32
   uint64_t *ef_low;     uint64_t words_ef_low;

@@ -15,6 +15,7 @@
 //     far list is split into that bucket's near queue and the rest.
 // Distances are integers (sums of stored weights), so the result is the exact
 // shortest-path distance whatever the order of relaxations.
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <utility>
@@ -372,6 +373,24 @@ lg_status fail(const char* what, cudaError_t e) {
     if (e_ != cudaSuccess) return fail(#call, e_); \
   } while (0)
 
+// Bucket width of a call that names none.  In wide buckets arcs are relaxed
+// again and again, more the more short arcs a vertex has; narrow ones are a
+// round and two reads each.  Measured for weights of 1 .. 255, the best width is
+// inverse to the mean degree, as the method's analysis has it (width of the
+// order of the largest weight over the degree); at 4096 / degree and its
+// neighbors, ms at a quarter / half / taken / twice / four times: R-MAT 2^20 (30)
+// 2.73 1.99 1.51 1.44 1.31, 2^22 and 2^24 best at 128 as taken; 2 M vertices of
+// degree 8 3.52 2.62 2.18 2.01 2.47, 1.5 M of 40 2.89 2.79 2.77 4.18 4.64,
+// 400,000 of 160 1.93 1.81 1.75 2.37 2.65, of 300 2.10 1.92 1.84 3.00 3.49.
+// Other weights scale it (16 bits on R-MAT 2^20: 36 ms in buckets of 128, 1.6 in
+// 2^15), but below 8 bits the rounds are so few that narrower ones do not pay
+// (4 bits: 0.73 ms in 128, 1.09 in 8).
+uint64_t default_delta(const lg_graph* g) {
+  const double w = std::max((double)g->max_weight + 1.0, 256.0);
+  const double width = 16.0 * w * (double)g->n / (double)std::max<uint64_t>(g->arcs, 1);
+  return (uint64_t)1 << (int)std::min(std::max(std::round(std::log2(width)), 0.0), 62.0);
+}
+
 }  // namespace
 
 extern "C" lg_status lg_sssp(const lg_graph* g, uint32_t source, uint64_t delta, uint64_t* dist, void* stream) {
@@ -392,10 +411,7 @@ extern "C" lg_status lg_sssp(const lg_graph* g, uint32_t source, uint64_t delta,
     set_error_message("lg_sssp: weights exist only in global-ID and CSR-32 graphs");
     return LG_EUNSUPPORTED;
   }
-  // R-MAT, weights 1 .. 255: 2^12 vertices 1.24 ms at 32, 0.65 at 128; 2^22
-  // 4.9 and 4.0; 2^24 15.2 and 13.3; 2^26 67 and 66 (wider is quicker still on
-  // the small ones, up to 10 % slower on the large)
-  if (delta == 0) delta = 128;
+  if (delta == 0) delta = default_delta(g);
   int prev = -1;
   cudaGetDevice(&prev);
   if (prev != g->device) cudaSetDevice(g->device);
