@@ -226,6 +226,7 @@ struct NbrArgs {
   uint32_t* out_weights;
   NbrStat* stat;             // degree pass
   int scan;                  // degree pass: 1 = it writes the offsets (k <= NBR_SCAN), 0 = the degrees
+  uint32_t per;              // row pass: queries per CTA (set by its launch)
   int sort;                  // row pass: put rows of up to NBR_SORT neighbors in ascending order
 };
 

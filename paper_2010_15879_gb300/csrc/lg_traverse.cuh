@@ -1086,14 +1086,119 @@ __device__ __forceinline__ uint32_t nbr_weight(const GView& g, uint64_t start, u
   return 0u;
 }
 
+// Ascending order of a warp's 32 R keys, key R lane + r in x[r], by a bitonic
+// network: compare-exchanges inside a lane's registers and by shuffles.  VALS:
+// y moves along.
+template <bool VALS>
+__device__ __forceinline__ void exchange(uint32_t& a, uint32_t& b, uint32_t& va, uint32_t& vb, bool up) {
+  if (VALS) {
+    const bool swap = up ? a > b : a < b;
+    const uint32_t ta = swap ? b : a, tb = swap ? a : b, sa = swap ? vb : va, sb = swap ? va : vb;
+    a = ta; b = tb; va = sa; vb = sb;
+  } else {
+    const uint32_t lo = min(a, b), hi = max(a, b);
+    a = up ? lo : hi;
+    b = up ? hi : lo;
+  }
+}
+template <int R, bool VALS>
+__device__ __forceinline__ void warp_sort(uint32_t (&x)[R], uint32_t (&y)[R]) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (int k = 2; k <= R; k *= 2) {
+#pragma unroll
+    for (int j = k / 2; j > 0; j /= 2) {
+#pragma unroll
+      for (int r = 0; r < R; r++)
+        if ((r & j) == 0) exchange<VALS>(x[r], x[r | j], y[r], y[r | j], k < R ? (r & k) == 0 : (lane & 1u) == 0);
+    }
+  }
+#pragma unroll 1
+  for (uint32_t k = 2; k <= 32; k *= 2) {  // runs of k lanes
+    const bool up = (lane & k) == 0;
+#pragma unroll 1
+    for (uint32_t m = k / 2; m > 0; m /= 2) {
+      const bool low = ((lane & m) == 0) == up;
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        const uint32_t o = __shfl_xor_sync(LG_FULL_MASK, x[r], m);
+        if (VALS) {
+          const uint32_t ov = __shfl_xor_sync(LG_FULL_MASK, y[r], m);
+          const bool take = low ? o < x[r] : o > x[r];
+          x[r] = take ? o : x[r];
+          y[r] = take ? ov : y[r];
+        } else {
+          x[r] = low ? min(x[r], o) : max(x[r], o);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = R / 2; j > 0; j /= 2) {
+#pragma unroll
+      for (int r = 0; r < R; r++)
+        if ((r & j) == 0) exchange<VALS>(x[r], x[r | j], y[r], y[r | j], up);
+    }
+  }
+}
+
 // Rows, decoded and (a.sort: on relabeled graphs) put in ascending order.  A
-// CTA takes 8 queries: a warp decodes a row of up to 256 neighbors into
-// registers and ranks each ID among the row's in shared memory; the CTA then
-// takes its longer rows together, sorting up to NBR_SORT of them with a bitonic
-// network in shared memory.  Longer rows are left unsorted (the caller sorts
-// them).  A hub's row no longer rests on one warp, and a batch needs one launch
-// where the decode and the size-class sort took eight and a wait.
+// CTA takes a.per queries, 8 at most and fewer where that leaves SMs idle: a
+// warp decodes a row of up to 256 neighbors into registers and sorts it there
+// (1, 2, 4 or 8 keys a lane); the CTA then takes its longer rows together,
+// sorting up to NBR_SORT of them with a bitonic network in shared memory.
+// Longer rows are left unsorted (the caller sorts them).  A hub's row does not
+// rest on one warp, and a batch needs one launch where the decode and the
+// size-class sort took eight and a wait.  All rows of 400,000 vertices of degree
+// 160: 1.34 ms with those, 2.25 with each ID ranked among its row's, 1.34 so.
 constexpr uint32_t NBR_WARP = 256;  // neighbors of a row that a warp takes
+
+// a row of up to 32 R neighbors, id[u] that of field 32 u + lane, to out
+template <int IDM, int R>
+__device__ __forceinline__ void nbr_row(const GView& g, const NbrArgs& a, const uint32_t (&id)[NBR_WARP / 32],
+                                        uint64_t start, uint32_t d, uint64_t o, uint32_t* mine) {
+  const uint32_t lane = threadIdx.x & 31u;
+  // with weights the field moves along: in the key's low 8 bits if the IDs leave them
+  const bool packed = a.sort && a.out_weights && g.n <= 1ull << 24, beside = a.sort && a.out_weights && !packed;
+  uint32_t x[R], y[R];
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    y[r] = 32u * r + lane;
+    x[r] = y[r] < d ? (packed ? id[r] << 8 | y[r] : id[r]) : 0xffffffffu;
+  }
+  if (a.sort) {
+    if (beside) warp_sort<R, true>(x, y);
+    else warp_sort<R, false>(x, y);
+    // sorted by lane; out in order
+#pragma unroll
+    for (int r = 0; r < R; r++) mine[R * lane + r] = x[r];
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; r++) x[r] = mine[32 * r + lane];
+    if (packed) {
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        y[r] = x[r] & 255u;
+        x[r] >>= 8;
+      }
+    }
+    if (beside) {
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < R; r++) mine[R * lane + r] = y[r];
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < R; r++) y[r] = mine[32 * r + lane];
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    if (32u * r + lane < d) {
+      a.out_ids[o + 32u * r + lane] = x[r];
+      if (a.out_weights) a.out_weights[o + 32u * r + lane] = nbr_weight<IDM>(g, start, y[r]);
+    }
+  }
+}
+
 template <int IDM, int OFF>
 __global__ void __launch_bounds__(256) k_nbr_rows(GView g, NbrArgs a) {
   __shared__ __align__(16) uint32_t sk[NBR_SORT];
@@ -1102,8 +1207,8 @@ __global__ void __launch_bounds__(256) k_nbr_rows(GView g, NbrArgs a) {
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   if (threadIdx.x == 0) nbig = 0;
   __syncthreads();
-  const uint64_t q0 = (uint64_t)blockIdx.x * 8;
-  if (q0 + wid < a.k) {
+  const uint64_t q0 = (uint64_t)blockIdx.x * a.per;
+  if (wid < a.per && q0 + wid < a.k) {
     const uint32_t vo = a.vertices[q0 + wid];
     uint64_t start;
     uint32_t d, w, carry = 0;
@@ -1113,46 +1218,24 @@ __global__ void __launch_bounds__(256) k_nbr_rows(GView g, NbrArgs a) {
     } else if (d) {
       constexpr int U = NBR_WARP / 32;
       const uint64_t o = a.out_offsets[q0 + wid];
-      const uint32_t nu = (d + 31) / 32;
       uint32_t id[U];
-      if (nu == 1) {
+      if (d <= 32) {
         uint32_t one[1];
         warp_ids<IDM, 1>(g, start, w, 0, d, carry, one);
         id[0] = one[0];
       } else {
         warp_ids<IDM, U>(g, start, w, 0, d, carry, id);
       }
-      uint32_t* mine = sk + wid * NBR_WARP;
       if (g.inv_perm) {
 #pragma unroll
         for (int u = 0; u < U; u++)
-          if (u < nu && 32u * u + lane < d) id[u] = g.inv_perm[id[u]];
+          if (32u * u + lane < d) id[u] = g.inv_perm[id[u]];
       }
-      uint32_t at[U];
-#pragma unroll
-      for (int u = 0; u < U; u++) at[u] = 32u * u + lane;
-      if (a.sort) {
-#pragma unroll
-        for (int u = 0; u < U; u++)
-          if (u < nu) mine[32 * u + lane] = 32u * u + lane < d ? id[u] : 0xffffffffu;
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < U; u++) at[u] = 0;
-        for (uint32_t j = 0; j < (d + 3) / 4; j++) {
-          const uint4 x = reinterpret_cast<const uint4*>(mine)[j];
-#pragma unroll
-          for (int u = 0; u < U; u++)
-            if (u < nu) at[u] += (x.x < id[u]) + (x.y < id[u]) + (x.z < id[u]) + (x.w < id[u]);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; u++) {
-        const uint32_t idx = 32u * u + lane;
-        if (u < nu && idx < d) {
-          a.out_ids[o + at[u]] = id[u];
-          if (a.out_weights) a.out_weights[o + at[u]] = nbr_weight<IDM>(g, start, idx);
-        }
-      }
+      uint32_t* mine = sk + wid * NBR_WARP;
+      if (d <= 32) nbr_row<IDM, 1>(g, a, id, start, d, o, mine);
+      else if (d <= 64) nbr_row<IDM, 2>(g, a, id, start, d, o, mine);
+      else if (d <= 128) nbr_row<IDM, 4>(g, a, id, start, d, o, mine);
+      else nbr_row<IDM, 8>(g, a, id, start, d, o, mine);
     }
   }
   __syncthreads();
@@ -1728,7 +1811,9 @@ cudaError_t launch_nbr_degrees(const GView& g, const NbrArgs& a, cudaStream_t st
 template <int IDM, int OFF>
 cudaError_t launch_nbr_rows(const GView& g, const NbrArgs& a, cudaStream_t st) {
   if (a.k == 0) return cudaSuccess;
-  k_nbr_rows<IDM, OFF><<<(unsigned)((a.k + 7) / 8), 256, 0, st>>>(g, a);
+  NbrArgs b = a;
+  b.per = (uint32_t)std::min<uint64_t>(8, (a.k + 152 * 4 - 1) / (152 * 4));  // four CTAs per SM before they share
+  k_nbr_rows<IDM, OFF><<<(unsigned)((a.k + b.per - 1) / b.per), 256, 0, st>>>(g, b);
   count_launch();
   return cudaGetLastError();
 }
