@@ -816,7 +816,7 @@ extern "C" lg_status lg_neighbors(const lg_graph* g, const uint32_t* vertices, u
   if (h.total && !out_ids) { set_errf("lg_neighbors: out_ids is NULL"); return LG_EINVAL; }
   if (h.total) LG_TRY(ops->nbr_rows(v, a, st));
   if (g->relabel)
-    LG_TRY(segmented_sort(out_ids, out_weights, out_offsets, k, h.total, h.max_degree, st, true, 32, true));
+    LG_TRY(segmented_sort(out_ids, out_weights, out_offsets, k, h.total, h.max_degree, st, 32, true));
   LG_TRY(cudaStreamSynchronize(st));
   return LG_OK;
 }

@@ -83,10 +83,10 @@ cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, uint32_t* keys_alt, u
 cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
                            uint64_t n, uint32_t key_bits, void* tmp, cudaStream_t st);
 // Sort each row [off[i], off[i+1]) of keys ascending, moving vals (nullable) along.
-// Rows of <= 32 keys are skipped when `small_done` (their producer sorted them).
+// Rows of <= 32 keys are left alone (their producer sorts them).
 // Every key is below 2^key_bits.  `big_only`: rows of up to 4,096 keys are left alone.
 cudaError_t segmented_sort(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint64_t rows,
-                           uint64_t total, uint64_t max_row, cudaStream_t st, bool small_done = false,
+                           uint64_t total, uint64_t max_row, cudaStream_t st,
                            uint32_t key_bits = 32, bool big_only = false);
 
 // ------------------------------------------------------------------ encoder

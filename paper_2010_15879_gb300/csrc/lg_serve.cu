@@ -843,7 +843,7 @@ struct NbrEngine : Engine {
         for (uint64_t i = 0; i < k; i++) most = std::max(most, hoff[i + 1] - hoff[i]);
         good = ops->nbr_rows(view, a, st) == cudaSuccess &&
                (!g->relabel ||
-                segmented_sort(a.out_ids, nullptr, doff, k, total, most, st, true, 32, true) == cudaSuccess) &&
+                segmented_sort(a.out_ids, nullptr, doff, k, total, most, st, 32, true) == cudaSuccess) &&
                cudaEventRecord(t1, st) == cudaSuccess &&
                cudaMemcpyAsync(hids, dids, total * 4, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
                cudaStreamSynchronize(st) == cudaSuccess;

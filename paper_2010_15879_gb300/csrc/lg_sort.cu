@@ -172,7 +172,7 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, u
 // =========================================================================
 // segmented sort of CSR rows
 // =========================================================================
-constexpr uint32_t SEG_SMALL = 32;    // one thread per row, sorting network in registers
+constexpr uint32_t SEG_SMALL = 32;    // what a row's producer sorts (a thread per row, a network in registers)
 constexpr uint32_t SEG_MEDIUM = NBR_SORT;  // 4,096: what the lookups' row kernel sorts itself
 constexpr uint32_t SEG_LARGE = 16384;      // what one CTA sorts
 constexpr int SROW = 33;              // shared slot stride of a small row (conflict-free lanes)
@@ -267,53 +267,6 @@ __device__ __forceinline__ void warp_sort_slots(uint32_t* sk, uint32_t* sv, uint
     else slot_sort<16, VALS>(k, v, d);
   }
   __syncwarp();
-}
-
-// rows of <= 32 keys, in place: a warp takes 32 consecutive rows, copies the
-// small ones into its shared slots (coalesced, a row per step), sorts a row
-// per lane and copies them back.
-template <bool VALS>
-__global__ void __launch_bounds__(256) k_seg_small(uint32_t* __restrict__ keys, uint32_t* __restrict__ vals,
-                                                   const uint64_t* __restrict__ off, uint64_t rows) {
-  extern __shared__ uint32_t ssm[];  // 8 warps x 32 slots of keys, then of values
-  const int lane = threadIdx.x & 31;
-  uint32_t* sk = ssm + (threadIdx.x >> 5) * 32 * SROW;
-  uint32_t* sv = ssm + 8 * 32 * SROW + (threadIdx.x >> 5) * 32 * SROW;
-  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  for (uint64_t r0 = ((uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; r0 < rows;
-       r0 += warps * 32) {
-    const uint64_t r = r0 + lane;
-    uint64_t lo = 0;
-    uint32_t d = 0;
-    if (r < rows) {
-      lo = off[r];
-      d = (uint32_t)(off[r + 1] - lo);
-    }
-    const bool small = d > 1 && d <= SEG_SMALL;
-    const uint32_t todo = __ballot_sync(LG_FULL_MASK, small);
-    if (!todo) continue;
-    for (uint32_t t = todo; t; t &= t - 1) {
-      const int q = __ffs(t) - 1;
-      const uint64_t lq = __shfl_sync(LG_FULL_MASK, lo, q);
-      const uint32_t dq = __shfl_sync(LG_FULL_MASK, d, q);
-      if ((uint32_t)lane < dq) {
-        sk[q * SROW + lane] = keys[lq + lane];
-        if (VALS) sv[q * SROW + lane] = vals[lq + lane];
-      }
-    }
-    __syncwarp();
-    warp_sort_slots<VALS>(sk, sv, d, small, lane);
-    for (uint32_t t = todo; t; t &= t - 1) {
-      const int q = __ffs(t) - 1;
-      const uint64_t lq = __shfl_sync(LG_FULL_MASK, lo, q);
-      const uint32_t dq = __shfl_sync(LG_FULL_MASK, d, q);
-      if ((uint32_t)lane < dq) {
-        keys[lq + lane] = sk[q * SROW + lane];
-        if (VALS) vals[lq + lane] = sv[q * SROW + lane];
-      }
-    }
-    __syncwarp();
-  }
 }
 
 // the rows of one size class: listed, or `count` consecutive ones from `first`
@@ -988,20 +941,6 @@ static cudaError_t seg_blk_launch(uint32_t* keys, uint32_t* vals, const uint64_t
   return cudaGetLastError();
 }
 
-static cudaError_t seg_small_launch(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint64_t rows,
-                                    cudaStream_t st) {
-  const size_t smem = (size_t)8 * 32 * SROW * sizeof(uint32_t) * (vals ? 2 : 1);
-  if (vals) {
-    const cudaError_t e = cudaFuncSetAttribute(k_seg_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  if (vals) k_seg_small<true><<<grid_for(rows, 256, 152 * 16), 256, smem, st>>>(keys, vals, off, rows);
-  else k_seg_small<false><<<grid_for(rows, 256, 152 * 16), 256, smem, st>>>(keys, vals, off, rows);
-  count_launch();
-  return cudaGetLastError();
-}
-
 // classes k0..9, `rows` in each; `coarse`: rows in the order of degree-mapped labels
 template <bool VALS>
 static cudaError_t seg_sort_classes(uint32_t* keys, uint32_t* vals, const uint64_t* off, const SegRows (&rows)[SEG_NCLASS],
@@ -1028,13 +967,11 @@ static cudaError_t seg_sort_classes(uint32_t* keys, uint32_t* vals, const uint64
 }
 
 cudaError_t segmented_sort(uint32_t* keys, uint32_t* vals, const uint64_t* off, uint64_t rows, uint64_t total,
-                           uint64_t max_row, cudaStream_t st, bool small_done, uint32_t key_bits, bool big_only) {
-  if (rows == 0 || total == 0 || max_row <= (big_only ? SEG_MEDIUM : 1)) return cudaSuccess;
+                           uint64_t max_row, cudaStream_t st, uint32_t key_bits, bool big_only) {
+  if (rows == 0 || total == 0 || max_row <= (big_only ? SEG_MEDIUM : SEG_SMALL)) return cudaSuccess;
   cudaError_t e;
-  if (!small_done && !big_only && (e = seg_small_launch(keys, vals, off, rows, st)) != cudaSuccess) return e;
-  if (max_row <= SEG_SMALL) return cudaSuccess;
   // rows by power-of-two size class
-  uint32_t* meta = nullptr;  // cnt[10], base[10], cursor[10]
+  uint32_t* meta = nullptr;  // SEG_NCLASS counts, first places in the list, cursors
   if ((e = lg::pool_alloc((void**)&meta, 3 * SEG_NCLASS * sizeof(uint32_t), st)) != cudaSuccess) return e;
   cudaMemsetAsync(meta, 0, 3 * SEG_NCLASS * sizeof(uint32_t), st);
   k_seg_count<<<grid_for(rows, 256, 152 * 16), 256, 0, st>>>(off, rows, meta);
@@ -1505,7 +1442,7 @@ cudaError_t enc_dm_relabel(const uint64_t* rp, const uint32_t* col, const uint32
   if (e == cudaSuccess && split_big && max_deg > SEG_SMALL)
     e = dm_big_rows(rp, col, w, n, perm, inv_perm, nrp, ncol, nw, st);
   else if (e == cudaSuccess && !split_big)
-    e = segmented_sort(ncol, w ? nw : nullptr, nrp, n, arcs, max_deg, st, true, host_bits(n - 1));
+    e = segmented_sort(ncol, w ? nw : nullptr, nrp, n, arcs, max_deg, st, host_bits(n - 1));
   cudaFreeAsync(keys, st); cudaFreeAsync(k2, st); cudaFreeAsync(v2, st); cudaFreeAsync(newdeg, st);
   cudaFreeAsync(stmp, st); cudaFreeAsync(rtmp, st);
   return e;
