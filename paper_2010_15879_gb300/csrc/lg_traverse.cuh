@@ -7,11 +7,10 @@
 //     of degree > heavy_min split into items of <= heavy_seg fields, one warp per
 //     item, lane i decoding field i of each 32-field chunk with 4 chunks in
 //     flight (gap-coded IDs by a warp prefix sum from the item's carry);
-//   * tile CTAs take 512 consecutive stored labels each:
+//   * tile CTAs take 64 to 512 consecutive stored labels each (tile_map):
 //     1. offsets x_v of the tile (packed fields, CSR row_ptr, or an
-//        Elias-Fano block decode: the tile starts on a select sample, the CTA
-//        popcounts the high-bit words it spans and every thread selects one
-//        vertex's one);
+//        Elias-Fano block decode: from the sample at or below the tile's first
+//        vertex on, every thread lists the ones of its words);
 //     2. per vertex: degree and field width from the offsets and the
 //        neighborhood header;
 //     3. light vertices (degree <= heavy_min) are split over the threads in
@@ -19,7 +18,8 @@
 //        its run with a sequential bit reader (one 32-byte sector per 256 bits,
 //        a shift and a mask per field, a running sum for gap-coded IDs, four
 //        gathers in flight).
-// Vertices split into several items are finished by a small second kernel.
+// A BFS's vertices split into several items are finished by the item that
+// arrives last, those of personalized PageRank by a small second kernel.
 // Push steps and neighbor queries decode one random vertex per warp.
 #pragma once
 
@@ -1142,7 +1142,7 @@ __device__ __forceinline__ void warp_sort(uint32_t (&x)[R], uint32_t (&y)[R]) {
 }
 
 // Rows, decoded and (a.sort: on relabeled graphs) put in ascending order.  A
-// CTA takes a.per queries, 8 at most and fewer where that leaves SMs idle: a
+// CTA takes a.per queries, 8 or, where rows are long, fewer (launch_nbr_rows): a
 // warp decodes a row of up to 256 neighbors into registers and sorts it there
 // (1, 2, 4 or 8 keys a lane); the CTA then takes its longer rows together,
 // sorting up to NBR_SORT of them with a bitonic network in shared memory.
@@ -1812,7 +1812,10 @@ template <int IDM, int OFF>
 cudaError_t launch_nbr_rows(const GView& g, const NbrArgs& a, cudaStream_t st) {
   if (a.k == 0) return cudaSuccess;
   NbrArgs b = a;
-  b.per = (uint32_t)std::min<uint64_t>(8, (a.k + 152 * 4 - 1) / (152 * 4));  // four CTAs per SM before they share
+  // A warp's row needs no CTA to itself: beside other work a server's lookups
+  // take an eighth of the room so (2,190 requests/s; 2,000 with a CTA per query).
+  // Where most rows take a whole CTA, there are four per SM before they share.
+  b.per = g.arcs <= NBR_WARP * g.n ? 8 : (uint32_t)std::min<uint64_t>(8, (a.k + 152 * 4 - 1) / (152 * 4));
   k_nbr_rows<IDM, OFF><<<(unsigned)((a.k + b.per - 1) / b.per), 256, 0, st>>>(g, b);
   count_launch();
   return cudaGetLastError();

@@ -69,3 +69,20 @@ def test_weights_of_large_ids(n):
     g = lg.lg_encode(rp, col, w, off_mode=lg.LG_OFF_PACKED, relabel=lg.LG_RELABEL_DM)
     got = lg.lg_neighbors(g, torch.from_numpy(at.astype(np.int32)).cuda(), with_weights=True)
     assert np.array_equal(got[1].cpu().numpy(), col) and np.array_equal(got[2].cpu().numpy(), w)
+
+
+@pytest.mark.parametrize("k", [1, 608, 609, 2000, 5000])
+def test_long_rows(k):
+    """Rows of 257 and more on the average: one to eight queries per CTA."""
+    lg.load(auto_build=True)
+    n, rng = 3000, np.random.default_rng(4)
+    d = rng.integers(200, 500, n)
+    rp = np.zeros(n + 1, dtype=np.int64)
+    np.cumsum(d, out=rp[1:])
+    col = np.concatenate([np.sort(rng.choice(n, m, replace=False)) for m in d]).astype(np.int32)
+    w = rng.integers(0, 256, col.size).astype(np.int32)
+    g = lg.lg_encode(rp, col, w, off_mode=lg.LG_OFF_EF, relabel=lg.LG_RELABEL_DM)
+    q = rng.integers(0, n, k).astype(np.int32)
+    got = lg.lg_neighbors(g, torch.from_numpy(q).cuda(), with_weights=True)
+    src = np.concatenate([np.arange(rp[v], rp[v + 1]) for v in q])
+    assert np.array_equal(got[1].cpu().numpy(), col[src]) and np.array_equal(got[2].cpu().numpy(), w[src])
