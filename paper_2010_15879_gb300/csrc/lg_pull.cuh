@@ -8,8 +8,8 @@
 // up one line per clock, so gathers that leave the SM cannot pass 274-297 G/s
 // on this GPU (152 SMs, measured with 32 distinct lines per request), while
 // shared memory answers 1,515 G/s.  The CTA therefore keeps the contributions
-// of the first `tabn` stored labels in shared memory: in DM order these are
-// the hubs, and a small graph fits whole.  The rest of the design serves the
+// of the first `tabn` stored labels in shared memory where that pays (pr_plan):
+// in DM order these are the hubs.  The rest of the design serves the
 // gathers: the stream comes in once, by 16-byte loads, a window of 256 fields
 // at a time, and every lane takes 8 fields of the window whatever vertices
 // they belong to, so its eight gathers are in flight together and no lane
@@ -351,8 +351,9 @@ __device__ __forceinline__ int open_window(const GView& g, const LightTile& T, W
 }
 
 // IDs of the lane's 8 consecutive fields of a window: hb their head bits, je
-// the light vertex that is open before them.
-template <int IDM>
+// the light vertex that is open before them.  RUNS: windows in which no lane
+// enters a second vertex are decoded in their own way.
+template <int IDM, bool RUNS>
 __device__ __forceinline__ void decode_window(const GView& g, const Window& wd, uint32_t hb, int je, const PrWarp& W,
                                               uint32_t& gcarry, uint32_t (&id)[PW_E]) {
   const uint32_t lane = threadIdx.x & 31u, k0 = PW_E * lane;
@@ -363,22 +364,46 @@ __device__ __forceinline__ void decode_window(const GView& g, const Window& wd, 
     for (int e = 0; e < PW_E; e++, p += rw) id[e] = sh_bits(p) & mask;
     return;
   }
-  // A field's place comes from its vertex's info alone, so that no lane waits
-  // for one that enters a vertex there (a step per entered vertex: 4 % more
-  // instructions in a whole-graph decode).
-  const uint32_t n8 = k0 < wd.nf ? wd.nf - k0 : 0u, rel = wd.ro;
+  const uint32_t rel = wd.ro;
   uint32_t v = 0;
-  int j = je;  // -1 only before the tile's first field
+  if (RUNS && wd.nf == PW_WF && !__any_sync(LG_FULL_MASK, (hb & (hb - 1u)) != 0)) {
+    // The fields before the lane's head h follow each other at one width, those
+    // from it on at another: one vertex's info each, and no multiplication per
+    // field.  Local-gap IDs in DM order, ms a sweep: 1.5 M vertices of degree 40
+    // 0.302 -> 0.291, community 2^24 1.92 -> 1.87, R-MAT 2^16 0.043 -> 0.039.
+    // Sweeps of graphs that are not relabeled, whose windows mix short and long
+    // vertices, lose 3 % to the two paths and keep the other.
+    const uint32_t h = hb ? (uint32_t)__ffs((int)hb) - 1u : (uint32_t)PW_E;
+    const uint32_t ia = W.info[max(je, 0)], ib = W.info[je + (hb != 0)];  // je is -1 only if the first field is a head
+    const uint32_t wa = ia >> PW_POS_BITS, wb = ib >> PW_POS_BITS, ma = mask_lo(wa), mb = mask_lo(wb);
+    const uint32_t ph = ((ib + (wd.f0 + k0 + h) * wb - rel) & PW_POSM) + wd.at;
+    uint32_t pa = ((ia + (wd.f0 + k0) * wa - rel) & PW_POSM) + wd.at, pb = ph - h * wb;
+    // a first field is an absolute ID of s bits
+    const uint32_t first = IDM == ID_LOCAL_GAP ? sh_bits(hb ? ph - (g.s - wb) : pa) & mask_lo(g.s) : 0u;
 #pragma unroll
-  for (int e = 0; e < PW_E; e++) {
-    const bool head = (hb >> e) & 1u;
-    j += head;
-    const uint32_t i = e < n8 ? W.info[j] : 0u, w = i >> PW_POS_BITS;
-    const uint32_t bits = IDM == ID_LOCAL_GAP && head ? g.s : w;  // a first field is an absolute ID of s bits
-    const uint32_t p = (i + (wd.f0 + k0 + e) * w - rel) & PW_POSM;
-    const uint32_t x = e < n8 ? sh_bits(p + wd.at - (bits - w)) & mask_lo(bits) : 0u;
-    v = IDM == ID_LOCAL_GAP && !head ? v + x : x;
-    id[e] = v;
+    for (int e = 0; e < PW_E; e++, pa += wa, pb += wb) {
+      const bool after = e >= h;
+      const uint32_t x = sh_bits(after ? pb : pa) & (after ? mb : ma);
+      v = IDM == ID_LOCAL_GAP ? (e == h ? first : v + x) : x;
+      id[e] = v;
+    }
+  } else {
+    // A field's place comes from its vertex's info alone, so that no lane waits
+    // for one that enters a vertex there (a step per entered vertex: 4 % more
+    // instructions in a whole-graph decode).
+    const uint32_t n8 = k0 < wd.nf ? wd.nf - k0 : 0u;
+    int j = je;  // -1 only before the tile's first field
+#pragma unroll
+    for (int e = 0; e < PW_E; e++) {
+      const bool head = (hb >> e) & 1u;
+      j += head;
+      const uint32_t i = e < n8 ? W.info[j] : 0u, w = i >> PW_POS_BITS;
+      const uint32_t bits = IDM == ID_LOCAL_GAP && head ? g.s : w;  // a first field is an absolute ID of s bits
+      const uint32_t p = (i + (wd.f0 + k0 + e) * w - rel) & PW_POSM;
+      const uint32_t x = e < n8 ? sh_bits(p + wd.at - (bits - w)) & mask_lo(bits) : 0u;
+      v = IDM == ID_LOCAL_GAP && !head ? v + x : x;
+      id[e] = v;
+    }
   }
   if (IDM == ID_LOCAL_GAP) {
     // fields before the lane's first head continue the neighborhood of the lane before
@@ -400,7 +425,7 @@ __device__ __forceinline__ void decode_window(const GView& g, const Window& wd, 
   }
 }
 
-template <int IDM, int OFF, class Gather>
+template <int IDM, int OFF, bool RUNS, class Gather>
 __device__ __forceinline__ void pr_tile(const GView& g, const PrArgs& a, uint64_t v0, uint32_t nv, uint64_t p0,
                                         const Gather& G, PrWarp& W) {
   const uint32_t lane = threadIdx.x & 31u, lt = lane_lt_mask(), k0 = PW_E * lane;
@@ -434,7 +459,7 @@ __device__ __forceinline__ void pr_tile(const GView& g, const PrArgs& a, uint64_
     const int je = jb + warp_incl_scan<int>(c) - c;
     jb = jc;
     uint32_t id[PW_E];
-    decode_window<IDM>(g, cur, hb, je, W, gcarry, id);
+    decode_window<IDM, RUNS>(g, cur, hb, je, W, gcarry, id);
     const bool whole = cur.nf == PW_WF;
     if (!whole) {
 #pragma unroll
@@ -479,7 +504,7 @@ __device__ __forceinline__ uint32_t first_unit(uint32_t ticket, uint32_t n1, uin
 __device__ __forceinline__ bool same_ticket(uint32_t t, uint32_t n1, uint32_t n2, uint32_t k) {
   return t - n1 + 1 < n2 && ((t - n1 + 1) & (k - 1)) != 0;
 }
-template <int IDM, int OFF, bool TAB>
+template <int IDM, int OFF, bool TAB, bool RUNS>
 __global__ void __launch_bounds__(PW_NT, 1) k_pr_pull(GView g, PrArgs a) {
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   PrWarp& W = reinterpret_cast<PrWarp*>(dyn_smem)[wid];
@@ -523,7 +548,7 @@ __global__ void __launch_bounds__(PW_NT, 1) k_pr_pull(GView g, PrArgs a) {
       const bool small = t < n1;
       const uint64_t v0 = small ? a.tile_a + (uint64_t)a.tile_nv * t : a.tile_b + (uint64_t)PW_TV * (t - n1 - n2);
       const uint64_t p0 = OFF == OFF_EF ? __ldg(a.aux + (small ? t : t - n2)) : 0;
-      pr_tile<IDM, OFF>(g, a, v0, small ? a.tile_nv : PW_TV, p0, G, W);
+      pr_tile<IDM, OFF, RUNS>(g, a, v0, small ? a.tile_nv : PW_TV, p0, G, W);
     }
     t = same_ticket(t, n1, n2, k) ? t + 1
                                   : first_unit(PW_WARPS * gridDim.x + __shfl_sync(LG_FULL_MASK, next, 0), n1, n2, k);

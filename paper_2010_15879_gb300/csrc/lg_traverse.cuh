@@ -1487,7 +1487,7 @@ __device__ __forceinline__ bool dec_lookback(const DecArgs& a, uint64_t b, uint6
   }
 }
 
-template <int IDM, int OFF>
+template <int IDM, int OFF, bool RUNS>
 __global__ void __launch_bounds__(TNT, 4) k_dec_local(GView g, DecArgs a) {
   DecSmem& sm = *reinterpret_cast<DecSmem*>(dyn_smem);
   const uint64_t ntiles = a.tiles, va = a.tiles_a * dec_tile(a.nv_a);  // from vertex va on tiles of a.nv per warp
@@ -1619,7 +1619,7 @@ __global__ void __launch_bounds__(TNT, 4) k_dec_local(GView g, DecArgs a) {
     const int je = jb + warp_incl_scan<int>(c) - c;
     jb = jc;
     uint32_t id[PW_E];
-    decode_window<IDM>(g, cur, hb, je, W, gcarry, id);
+    decode_window<IDM, RUNS>(g, cur, hb, je, W, gcarry, id);
     uint4* o4 = reinterpret_cast<uint4*>(out + k0);
     o4[0] = make_uint4(id[0], id[1], id[2], id[3]);
     o4[1] = make_uint4(id[4], id[5], id[6], id[7]);
@@ -1760,10 +1760,18 @@ inline unsigned schedule_tiles_grid(const GView& g, uint32_t tile0) {
   return std::max(items, tiles_of(g.n) - tile0);
 }
 
+// the sweep for a graph (see decode_window on relabeled ones) and plan
+template <int IDM, int OFF>
+auto pr_pull_kernel(const GView& g, const PrArgs& a) {
+  if constexpr (IDM == ID_LOCAL || IDM == ID_LOCAL_GAP) {
+    if (g.perm) return a.tabn ? k_pr_pull<IDM, OFF, true, true> : k_pr_pull<IDM, OFF, false, true>;
+  }
+  return a.tabn ? k_pr_pull<IDM, OFF, true, false> : k_pr_pull<IDM, OFF, false, false>;
+}
 template <int IDM, int OFF>
 cudaError_t launch_pr_init(const GView& g, const PrArgs& a, cudaStream_t st) {
-  const cudaError_t e = a.tabn ? cudaFuncSetAttribute(k_pr_pull<IDM, OFF, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PW_SMEM)
-                               : cudaFuncSetAttribute(k_pr_pull<IDM, OFF, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PW_SMEM);
+  const cudaError_t e = cudaFuncSetAttribute(pr_pull_kernel<IDM, OFF>(g, a),
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PW_SMEM);
   if (e != cudaSuccess) return e;
   const uint32_t tile0 = (uint32_t)(g.heavy_prefix / TV);
   k_pr_init<IDM, OFF><<<schedule_tiles_grid(g, tile0), TNT, 0, st>>>(g, a, tile0);
@@ -1776,8 +1784,7 @@ cudaError_t launch_pr_pull(const GView& g, const PrArgs& a, cudaStream_t st) {
   // the shared memory beside the table is the warps' (PrWarp)
   const unsigned grid = (unsigned)std::min<uint64_t>(units, PW_SMS);
   const size_t smem = PW_WARPS * sizeof(PrWarp) + (size_t)a.tabn * 4;
-  if (a.tabn) k_pr_pull<IDM, OFF, true><<<grid, PW_NT, smem, st>>>(g, a);
-  else k_pr_pull<IDM, OFF, false><<<grid, PW_NT, smem, st>>>(g, a);
+  pr_pull_kernel<IDM, OFF>(g, a)<<<grid, PW_NT, smem, st>>>(g, a);
   count_launch();
   return cudaGetLastError();
 }
@@ -1863,17 +1870,18 @@ cudaError_t launch_dec_all(const GView& g, const DecArgs& a, cudaStream_t st) {
     const uint64_t per_block = (g.arcs + tiles - 1) / tiles;
     k_dec_flat<IDM, OFF><<<(unsigned)tiles, 256, 0, st>>>(g, a, (per_block + unit - 1) / unit * unit);
   } else {
-    const cudaError_t e = cudaFuncSetAttribute(k_dec_local<IDM, OFF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const auto tiles_kernel = g.perm ? k_dec_local<IDM, OFF, true> : k_dec_local<IDM, OFF, false>;
+    const cudaError_t e = cudaFuncSetAttribute(tiles_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)sizeof(DecSmem));
     if (e != cudaSuccess) return e;
     if (a.heavy_after && g.n_items) {
       GView tiles = g;
       tiles.n_items = 0;
-      k_dec_local<IDM, OFF><<<(unsigned)a.tiles, TNT, sizeof(DecSmem), st>>>(tiles, a);
+      tiles_kernel<<<(unsigned)a.tiles, TNT, sizeof(DecSmem), st>>>(tiles, a);
       count_launch();
       k_dec_heavy<IDM><<<heavy_blocks(g.n_items), TNT, 0, st>>>(g, a);
     } else {
-      k_dec_local<IDM, OFF><<<(unsigned)a.tiles + heavy_blocks(g.n_items), TNT, sizeof(DecSmem), st>>>(g, a);
+      tiles_kernel<<<(unsigned)a.tiles + heavy_blocks(g.n_items), TNT, sizeof(DecSmem), st>>>(g, a);
     }
   }
   count_launch();
