@@ -213,9 +213,10 @@ lg_status lg_bfs(const lg_graph *g, const uint32_t *sources, uint32_t S, uint32_
  * stepping) on a weighted graph (weights stored after each ID, Section 3.3),
  * neighborhoods and weights decoded inside the relaxation kernel.
  *   source  original ID (< n)
- *   delta   bucket width; 0 = by the largest weight and the mean degree (the power
- *           of two nearest to 16 max(weight + 1, 256) n / arcs: 128 for weights
- *           of 8 bits on R-MAT of edge factor 16); any value gives the same distances
+ *   delta   bucket width; 0 = by the weights and degrees: with w = max(largest
+ *           weight + 1, 256) the power of two nearest to w / 2, or to 16 w n / arcs
+ *           where no degree is above four times the mean; any value gives the
+ *           same distances
  *   dist    device, n u64 indexed by original ID: the minimum over paths from
  *           source of the sum of arc weights, UINT64_MAX if unreachable
  * Needs a weighted graph in LG_ID_GLOBAL or LG_ID_CSR32 (else
