@@ -346,13 +346,17 @@ bool even_degrees(const lg_graph* g) { return g->max_degree * g->n <= 4 * g->arc
 // the tile's own cost against the longest unit; measured per sweep at 4 / 8 /
 // 16 / 32 vertices: R-MAT 2^12 in DM order 8 / 10 / 13 / 19 us, community 2^15
 // 25 / 26 / 34 / 54, community 2^18 in DM order 133 / 80 / 58 / 80, R-MAT 2^18
-// not relabeled 110 / 72 / 53 / 47, R-MAT 900,000 287 / 173 / 114 / 85.  Where
+// not relabeled 110 / 72 / 53 / 47, R-MAT 900,000 287 / 173 / 114 / 85; but
+// tiles of too few fields are all cost.  Where
 // no degree is above four times the mean, no unit is long for its size, and
 // tiles are as large as leaves one for every second warp: 5 M vertices of
 // degree 40 in DM order, local-gap IDs, 1.02 ms in tiles of 32, 0.90 in 128,
 // 300,000 of degree 40 86 and 76 us.  Such a graph's heavy items, short ones,
 // come after its tiles (1 M vertices of degree 250, 35 % of them heavy: 1.27 ms
-// with the items first, 1.12 so), several to a ticket.
+// with the items first, 1.12 so), several to a ticket.  Tiles start right after
+// the vertices that are all in the schedule: one that held a few hubs would have
+// a warp search their Elias-Fano block alone (ten hubs of 200,000 arcs among
+// 500,000 vertices: 156 us a sweep, 32 so).
 //
 // The shared-memory table of contributions pays when it answers some of the
 // gathers of a sweep that is long enough to fill it (R-MAT 2^24 in DM order,
@@ -367,18 +371,20 @@ PrPlan pr_plan(const lg_graph* g) {
   const uint64_t warps = (uint64_t)PW_WARPS * PW_SMS;
   const bool small = g->n < 2 * warps * PW_TV;
   const bool even = even_degrees(g);
-  p.tile_a = g->heavy_prefix & ~(uint64_t)(PW_TV - 1);
+  p.tile_a = g->heavy_prefix;
   uint64_t end = small || even ? g->n : g->mid_prefix > p.tile_a ? g->mid_prefix : p.tile_a;
   if (even) {
-    p.tile_nv = g->arcs > g->heavy_min * g->n ? 32 : 4;  // tiles of next to no light fields are not worth splitting
+    p.tile_nv = 2 * g->heavy_arcs > g->arcs ? 32 : 4;  // tiles of next to no light fields are not worth splitting
     while (p.tile_nv < PW_TV && g->n / (2 * p.tile_nv) >= warps / 2) p.tile_nv *= 2;
-    p.items = 1;
-    while (g->n_items / (2 * p.items) >= 12 * warps) p.items *= 2;
   } else {
     p.tile_nv = g->n < (1u << 14) ? 4 : g->n < (1u << 16) ? 8 : g->n < (1u << 19) && g->relabel == 1 ? 16 : 32;
-    p.items = 1;
+    // 512 light fields a tile on the average, if there are two tiles per warp
+    while (p.tile_nv < PW_TV && 2 * p.tile_nv * (g->arcs - g->heavy_arcs) <= 512 * g->n && g->n / (2 * p.tile_nv) >= 2 * warps)
+      p.tile_nv *= 2;
   }
-  p.tile_b = (end + PW_TV - 1) & ~(uint64_t)(PW_TV - 1);
+  p.tile_b = p.tile_a + ((end > p.tile_a ? end - p.tile_a : 0) + PW_TV - 1) / PW_TV * PW_TV;
+  p.items = 1;  // short ones share a ticket as long as there are eight for every warp
+  while (g->n_items / (2 * p.items) >= 8 * warps && (even || g->heavy_arcs <= 512 * g->n_items)) p.items *= 2;
   const uint64_t most = (PW_SMEM - PW_WARPS * sizeof(PrWarp)) / sizeof(float);
   const bool table = g->n >= 3u << 16 ? 12 * g->top_arcs >= g->arcs : g->n >= 1u << 17 && 3 * g->top_arcs >= g->arcs;
   p.tabn = g->arcs >> 24 && table ? (uint32_t)(g->n < most ? g->n : most) : 0;
@@ -451,7 +457,7 @@ extern "C" lg_status lg_decode(const lg_graph* g, uint64_t* row_ptr, uint32_t* c
   // tiles, then the rows); its small state is zeroed first
   const bool even = even_degrees(g);
   dec_tiles(n, v.mid_prefix, even, a);
-  a.heavy_after = even && g->arcs > (uint64_t)g->heavy_min * n;
+  a.heavy_after = 3 * g->heavy_arcs >= 2 * g->arcs;
   const uint64_t ntiles = a.tiles;
   Tmp t_state(st);
   const size_t bytes = ntiles * (sizeof(unsigned long long) + sizeof(uint32_t)) + 16;
@@ -555,7 +561,7 @@ static lg_status build_schedule(lg_graph* g, const uint64_t* x, cudaStream_t st)
   const uint64_t ntiles = (g->n + LG_TILE_V - 1) / LG_TILE_V;
   // counts of items, then of split vertices, per tile, scanned together
   Tmp t_cnt(st), t_off(st), t_stmp(st), t_seg(st);
-  struct { uint64_t end; unsigned long long top; uint32_t mid, pad; } sums;  // end: of the scan
+  struct { uint64_t end; unsigned long long top, heavy; uint32_t mid, pad; } sums;  // end: of the scan
   LG_TRY(t_cnt.alloc(2 * ntiles * sizeof(uint32_t)));
   LG_TRY(t_off.alloc(2 * ntiles * sizeof(uint64_t) + sizeof(sums)));
   LG_TRY(t_stmp.alloc(scan_tmp_words(2 * ntiles) * sizeof(uint64_t)));
@@ -568,7 +574,8 @@ static lg_status build_schedule(lg_graph* g, const uint64_t* x, cudaStream_t st)
   p.tile_off = off;
   p.multi_off = off + ntiles;  // behind all items
   p.top = reinterpret_cast<unsigned long long*>(off + 2 * ntiles + 1);
-  p.mid = g->relabel == 1 ? reinterpret_cast<uint32_t*>(p.top + 1) : nullptr;
+  p.heavy = p.top + 1;
+  p.mid = g->relabel == 1 ? reinterpret_cast<uint32_t*>(p.heavy + 1) : nullptr;
   GView v = make_view(g);
   v.O = x;
   const TravOps* ops = trav_ops((int)g->id_mode, (int)g->off_mode);
@@ -581,6 +588,7 @@ static lg_status build_schedule(lg_graph* g, const uint64_t* x, cudaStream_t st)
   g->heavy_prefix = 0;
   g->mid_prefix = g->relabel == 1 ? sums.mid : 0;
   g->top_arcs = sums.top;
+  g->heavy_arcs = sums.heavy;
   if (g->n_items == 0) return LG_OK;
   LG_TRY(pool_alloc((void**)&g->items, g->n_items * sizeof(HeavyItem), st));
   if (g->n_multi) LG_TRY(pool_alloc((void**)&g->multi, g->n_multi * sizeof(uint32_t), st));

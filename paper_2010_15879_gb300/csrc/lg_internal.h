@@ -30,6 +30,7 @@ struct lg_graph {
   uint32_t heavy_min, heavy_seg;
   uint64_t heavy_prefix;  // DM order: the vertices below this label are all in the schedule (else 0)
   uint64_t top_arcs;      // sum of the degrees of the first PW_TOP labels
+  uint64_t heavy_arcs;    // sum of the degrees of the vertices in the schedule
   uint64_t mid_prefix;    // DM order: the vertices below this label have more than 32 arcs (else 0)
 };
 
@@ -135,6 +136,7 @@ struct PlanArgs {
   uint32_t* multi;
   uint32_t* segsum;          // per item: sum of its (gap) values
   unsigned long long* top;   // sum of the degrees of the first PW_TOP labels
+  unsigned long long* heavy; // sum of the degrees of the vertices in the schedule
   uint32_t* mid;             // largest v + 1 over the vertices of more than 32 arcs (null: not wanted)
 };
 
@@ -248,7 +250,7 @@ struct DecArgs {
   uint64_t wait_ns;          // limit of each such wait
   uint64_t tiles_a, tiles;   // tiles of nv_a vertices per warp, which come first; all tiles
   uint32_t nv_a, nv;         // vertices per warp of these and of the others
-  int heavy_after;           // the heavy items go in a launch of their own, after the tiles
+  int heavy_after;           // the heavy items go in a launch of their own, after the tiles (two thirds of the arcs)
 };
 constexpr uint32_t DEC_WARPS = 8;
 __host__ __device__ constexpr uint32_t dec_tile(uint32_t nv) { return DEC_WARPS * nv; }

@@ -1404,7 +1404,7 @@ __global__ void __launch_bounds__(256) k_dec_flat(GView g, DecArgs a, uint64_t p
 
 // ---------------------------------------------------------------------------
 // Local-ID decode: one launch writes row_ptr and every row (a graph that is mostly
-// heavy and even has its heavy items in a second one, see k_dec_heavy).
+// heavy has its heavy items in a second one, see k_dec_heavy).
 //
 // Blocks take a ticket when they start: tickets below the tile count are tile
 // CTAs (tiles in start order), the rest are heavy-schedule CTAs, a warp per
@@ -1634,7 +1634,8 @@ __global__ void __launch_bounds__(TNT, 4) k_dec_local(GView g, DecArgs a) {
 // The heavy items of a graph that is mostly heavy (DecArgs::heavy_after), a warp
 // each, once the rows' offsets are written: they need none of the tiles' shared
 // memory, which leaves an SM 32 warps (400,000 vertices of degree 300, local IDs
-// in DM order: 539 us with the tiles, 346 so).
+// in DM order: 539 us with the tiles, 346 so; R-MAT 2^19 of degree 90 in local-gap
+// IDs 454 and 288).
 template <int IDM>
 __global__ void __launch_bounds__(TNT) k_dec_heavy(GView g, DecArgs a) {
   const uint64_t it = (uint64_t)blockIdx.x * (TNT / 32) + (threadIdx.x >> 5);
@@ -1657,7 +1658,7 @@ __global__ void __launch_bounds__(TNT) k_plan_count(GView g, PlanArgs p) {
   const int cnt = (int)min((uint64_t)TV, g.n - v0);
   tile_offsets<OFF>(g, v0, cnt, sm.xs, sm.ts);
   __syncthreads();
-  uint64_t mine = 0, top = 0;
+  uint64_t mine = 0, top = 0, heavy = 0;
   uint32_t mid = 0;
   for (int i = threadIdx.x; i < cnt; i += TNT) {
     uint64_t start; uint32_t d, w;
@@ -1666,6 +1667,7 @@ __global__ void __launch_bounds__(TNT) k_plan_count(GView g, PlanArgs p) {
     mine += ((uint64_t)k << 32) | (k > 1 ? 1u : 0u);
     if (d > 32) mid = (uint32_t)(v0 + i) + 1u;
     if (v0 + i < PW_TOP) top += d;
+    if (k) heavy += d;
   }
   if (p.mid) {
     mid = __reduce_max_sync(LG_FULL_MASK, mid);
@@ -1680,6 +1682,11 @@ __global__ void __launch_bounds__(TNT) k_plan_count(GView g, PlanArgs p) {
   if (threadIdx.x == 0) {
     p.tile_count[blockIdx.x] = (uint32_t)(total >> 32);
     p.multi_count[blockIdx.x] = (uint32_t)total;
+  }
+  if (total) {  // the same in every thread
+    uint64_t arcs;
+    block_excl_scan<uint64_t, TNT>(heavy, arcs, sm.red64);
+    if (threadIdx.x == 0) atomicAdd(p.heavy, (unsigned long long)arcs);
   }
 }
 

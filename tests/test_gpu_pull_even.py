@@ -50,3 +50,14 @@ def test_tickets(monkeypatch, heavy_min, seg, opts):
     monkeypatch.setenv("LG_HEAVY_MIN", heavy_min)
     monkeypatch.setenv("LG_HEAVY_SEG", seg)
     check(even(200003, 12), 200003, **opts)
+
+
+# tiles start right after the vertices that are all in the schedule
+@pytest.mark.parametrize("hubs", [1, 10, 127, 128, 129, 200])
+@pytest.mark.parametrize("opts", MODES + [dict(off_mode=lg.LG_OFF_EF, relabel=lg.LG_RELABEL_DM)])
+def test_hubs(hubs, opts):
+    lg.load(auto_build=True)
+    n, rng = 50001, np.random.default_rng(hubs)
+    e = [np.stack([np.full(3000, v), rng.integers(0, n, 3000)], 1) for v in range(hubs)]
+    h = gen.from_edges(n, np.concatenate(e + [rng.integers(0, n, (n, 2))]))
+    check(h, n, **opts)
