@@ -767,7 +767,6 @@ struct lg_batch {
   BatchGraph* graphs = nullptr;  // device descriptors
   BatchItem* items = nullptr;
   uint32_t n_items = 0, n_cta = 0, n_eight = 0, n_small = 0;  // items, ends of their parts (BatchArgs)
-  bool narrow = true;            // small graphs go to parts of a CTA
   unsigned int* next = nullptr;  // queue heads
   uint32_t* sync = nullptr;      // SYNC_WORDS per graph
   uint32_t* err = nullptr;
@@ -823,19 +822,32 @@ void plan_queue(lg_batch* b) {
   // A graph goes to 8 warps or to one if its time there, 3 or 24 times that of
   // a CTA's, is no more than a CTA's share of the whole queue: the narrower
   // groups waste less, but a batch of few graphs needs every warp of a CTA for
-  // each.  A graph's barriers count like GRAPH_WORK of work (30 us).
+  // each.  Beside graphs for whole CTAs, which go first, it may take a 32nd of
+  // the share, as it ends the run, and such graphs must be a fifth of the work to
+  // be worth it (1,000 graphs of 2^8 .. 2^16 vertices, 2 % of the work in those of
+  // up to 2^11: 10.84 ms whole, 11.35 and 11.05 with all of the share and a
+  // 32nd; 10,000 of 256 beside 4 of 30,000 3.27 ms whole, 1.23 so).  A graph's
+  // barriers count like GRAPH_WORK of work (30 us).
   constexpr uint64_t GRAPH_WORK = 16384;
-  uint64_t share = 0;
+  auto cost = [&](uint32_t g) { return work(g) * b->host[g].team + GRAPH_WORK; };
+  uint64_t total = 0;
   for (uint32_t g : order)
-    if (b->host[g].n <= BS_MAX) share += work(g) * b->host[g].team + GRAPH_WORK;
-  share /= (uint64_t)b->grid;
+    if (b->host[g].n <= BS_MAX) total += cost(g);
+  uint64_t share = total / (uint64_t)b->grid;
   auto part = [&](uint32_t g) {
     const BatchGraph& x = b->host[g];
     if (x.n > BS_MAX) return 3;
-    if (!b->narrow || x.team > 1) return 0;
+    if (x.team > 1) return 0;
     if (x.n <= BGroup<1>::MAX_N && work(g) * BS_WARPS <= share) return 2;
     return x.n <= BGroup<8>::MAX_N && work(g) * (BS_WARPS / 8) <= share ? 1 : 0;
   };
+  if (std::any_of(order.begin(), order.end(), [&](uint32_t g) { return part(g) == 0; })) {
+    share /= 32;
+    uint64_t narrow = 0;
+    for (uint32_t g : order)
+      if (part(g) == 1 || part(g) == 2) narrow += cost(g);
+    if (5 * narrow < total) share = 0;
+  }
   b->items_h.clear();
   uint32_t* const ends[4] = {&b->n_cta, &b->n_eight, &b->n_small, &b->n_items};
   for (int k = 0; k < 4; k++) {
@@ -931,7 +943,6 @@ lg_status time_run(lg_batch* b, const BatchArgs& a, cudaStream_t st, cudaEvent_t
 // graphs run alone (encode + 2 PageRank sweeps) with T = 1, 4, 8 and 32.
 // (2) The team tiles, if not fixed: each path's graphs (encode + BFS + 2
 // sweeps) with tiles of 2^18 .. 2^21 arcs, the lanes path's from 2^15 on.
-// (3) Whether small graphs go to parts of a CTA.
 lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStream_t st, cudaEvent_t e0,
                    cudaEvent_t e1) {
   const int cand_t[4] = {1, 4, 8, 32};
@@ -1010,12 +1021,6 @@ lg_status autotune(lg_batch* b, uint32_t* depth_tmp, float* ranks_tmp, cudaStrea
         }
       }
       tile = best_k;
-    }
-    if (small && b->n_small > b->n_cta) {
-      if (best == 1e30f && (s = time_path(true, &best)) != LG_OK) return s;
-      b->narrow = false;
-      if ((s = time_path(true, &ms)) != LG_OK) return s;
-      b->narrow = best <= ms;
     }
   }
   plan_queue(b);
