@@ -214,9 +214,9 @@ lg_status lg_bfs(const lg_graph *g, const uint32_t *sources, uint32_t S, uint32_
  * neighborhoods and weights decoded inside the relaxation kernel.
  *   source  original ID (< n)
  *   delta   bucket width; 0 = by the weights and degrees: with w = max(largest
- *           weight + 1, 256) the power of two nearest to w / 2, or to 16 w n / arcs
- *           where no degree is above four times the mean; any value gives the
- *           same distances
+ *           weight + 1, 256) the power of two nearest to w / 2, or where no degree is
+ *           above four times the mean to 16 w n / arcs (below 2^24 arcs: if that
+ *           is more); any value gives the same distances
  *   dist    device, n u64 indexed by original ID: the minimum over paths from
  *           source of the sum of arc weights, UINT64_MAX if unreachable
  * Needs a weighted graph in LG_ID_GLOBAL or LG_ID_CSR32 (else

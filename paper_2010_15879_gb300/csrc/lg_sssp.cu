@@ -382,13 +382,19 @@ lg_status fail(const char* what, cudaError_t e) {
 // degree 8 3.52 2.62 2.18 2.01 2.47, 1.5 M of 40 2.89 2.79 2.77 4.18 4.64,
 // 400,000 of 160 1.93 1.81 1.75 2.37 2.65, of 300 2.10 1.92 1.84 3.00 3.49.
 // Where few vertices have most arcs the mean says little (R-MAT 2^18, degree 104:
-// 2.14 1.50 1.12 ms in 32, 64, 128): half the largest weight there.
+// 2.14 1.50 1.12 ms in 32, 64, 128): half the largest weight there, and at least
+// that below 2^24 arcs, where the rounds take longer than their arcs (3,000
+// vertices of degree 2,400: 0.33 ms in 128, 0.41 in 2).
 // Other weights scale it (16 bits on R-MAT 2^20: 36 ms in buckets of 128, 1.6 in
 // 2^15), but below 8 bits the rounds are so few that narrower ones do not pay
 // (4 bits: 0.73 ms in 128, 1.09 in 8).
 uint64_t default_delta(const lg_graph* g) {
   const double w = std::max((double)g->max_weight + 1.0, 256.0);
-  const double width = even_degrees(g) ? 16.0 * w * (double)g->n / (double)std::max<uint64_t>(g->arcs, 1) : w / 2;
+  double width = w / 2;
+  if (even_degrees(g) && g->arcs) {
+    const double by_degree = 16.0 * w * (double)g->n / (double)g->arcs;
+    width = g->arcs >> 24 ? by_degree : std::max(by_degree, width);
+  }
   return (uint64_t)1 << (int)std::min(std::max(std::round(std::log2(width)), 0.0), 62.0);
 }
 
