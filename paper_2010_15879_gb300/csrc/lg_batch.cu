@@ -287,9 +287,9 @@ struct BGroup {
   static constexpr uint32_t TAB = GW == BS_WARPS ? BS_TAB : GW == 8 ? TAB8 : (TAB8 / 8) & ~3u;  // floats of its table
   // most vertices of a graph for a part of a CTA: contributions twice
   static constexpr uint32_t MAX_N = (TAB / 2) & ~3u;
-  static __device__ __forceinline__ uint32_t tid() { return threadIdx.x % NT; }
-  static __device__ __forceinline__ uint32_t wid() { return (threadIdx.x >> 5) % GW; }
-  static __device__ __forceinline__ uint32_t index() { return (threadIdx.x >> 5) / GW * GW; }  // its first warp
+  static __device__ __forceinline__ uint32_t tid() { return GW == BS_WARPS ? threadIdx.x : threadIdx.x % NT; }
+  static __device__ __forceinline__ uint32_t wid() { return tid() >> 5; }
+  static __device__ __forceinline__ uint32_t index() { return (threadIdx.x >> 5) - wid(); }  // its first warp
   static __device__ __forceinline__ float* table() {
     float* t = reinterpret_cast<float*>(dyn_smem + BS_WARPS * sizeof(BWarp));
     if (GW == BS_WARPS) return t;
@@ -511,7 +511,8 @@ __device__ void process_small(const BatchArgs& a, uint32_t gi, uint32_t m) {
   if (a.phases & PH_BFS) {
     uint32_t* depth = a.depth + G.vbase;
     uint32_t* vis = reinterpret_cast<uint32_t*>(tab);
-    uint32_t *fr = vis + nwd, *nx = fr + nwd;
+    const uint32_t words = GW == BS_WARPS ? BS_WORDS : nwd;
+    uint32_t *fr = vis + words, *nx = fr + words;
     // a team shares each level's new bitmap through one of three global ones:
     // written in a level, read after its barrier, cleared after the next one
     uint32_t* shared_nx[3] = {a.q0 + G.vbase, a.q1 + G.vbase, reinterpret_cast<uint32_t*>(a.c0 + G.vbase)};
